@@ -673,6 +673,7 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     s.sys.Hacc = reinterpret_cast<unsigned long long *const *>(g->d_tab + 7 * n_sys);
     s.sys.np = g->d_sys_np;
     s.n_rgrid = g->n_rgrid;
+    s.max_ppad = (g->max_P + NAO_PPAD - 1) / NAO_PPAD * NAO_PPAD;
     s.r0 = g->r0;
     s.inv_delta = 1.0 / g->delta;
     s.step_m1 = std::expm1(g->delta);

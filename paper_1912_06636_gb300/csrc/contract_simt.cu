@@ -14,33 +14,60 @@
 //
 // FP32: products accumulate in FP32 over chunks of 32 terms; each chunk sum is folded into an
 // FP32 (hi, lo) pair with Knuth's TwoSum, and hi + lo is widened to FP64 for the scatter.
-// FP64 work of any kind is ~60x slower than FP32 on this GPU, which rules out an FP64
-// accumulator per chunk.
+//
+// What bounds them: the FP64 pipe (two lanes per clock and SM, 1/64 of the FP32 rate), which FP64
+// products use by definition and which every conversion between FP64 and a 32-bit type uses as
+// well. So (1) a CTA's 64 x 64 tile is cut into small subtiles, one or two per warp, and a warp
+// leaves out the subtiles that lie below the diagonal, beyond the batch's functions or beyond its
+// points: 16 x 16 in FP64 and 32 x 16 in FP32 (with smaller ones the operands' loads would be too many
+// for the FP32 rate). Which warp takes which subtile turns with the CTA's index, so that the idle ones
+// spread over the SM's four schedulers. (2) The FP32 kernels convert with integer instructions and
+// keep their sums over functions as float-float pairs.
+#include "ff.h"
 #include "nao_internal.h"
 
 namespace {
 
 constexpr int T_ = NAO_TILE;  // 64
 
+// Subtile of a warp: 8 x 4 lanes of MR rows x 4 columns, SR = 8 MR rows x 16 columns; KC: K chunk
+// (128 bytes of an operand row).
 template <typename T> struct Cfg;
-template <> struct Cfg<double> { static constexpr int KC = 16; };
-template <> struct Cfg<float> { static constexpr int KC = 32; };
+template <> struct Cfg<double> { static constexpr int KC = 16, MR = 2, SR = 16, NU = 2; };
+template <> struct Cfg<float> { static constexpr int KC = 32, MR = 4, SR = 32, NU = 1; };
 
-__device__ __forceinline__ void load_vec(const double *p, double (&v)[4]) {
-    const double2 a = *reinterpret_cast<const double2 *>(p), b = *reinterpret_cast<const double2 *>(p + 2);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+template <typename T> struct Vec16;  // 16 bytes of T
+template <> struct Vec16<double> { using type = double2; };
+template <> struct Vec16<float> { using type = float4; };
+__device__ __forceinline__ double vget(const double2 &v, int e) { return e == 0 ? v.x : v.y; }
+__device__ __forceinline__ float vget(const float4 &v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
+__device__ __forceinline__ double2 vmul(double2 v, double2 w) { return make_double2(v.x * w.x, v.y * w.y); }
+__device__ __forceinline__ float4 vmul(float4 v, float4 w) { return make_float4(v.x * w.x, v.y * w.y, v.z * w.z, v.w * w.w); }
+
+// 16 bytes global -> shared, asynchronously; zeros when !ok (nothing is read then).
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
 }
-__device__ __forceinline__ void load_vec(const float *p, float (&v)[8]) {
-    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// FP64 -> FP32, round to nearest even, with integer instructions (the conversion instruction runs on
+// the FP64 pipe). Values outside FP32's normal range take the conversion.
+__device__ __forceinline__ float to_f32(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu;
+    if (e - 897u > 253u) return __double2float_rn(x);
+    const uint32_t m = (hi << 12) | (lo >> 20);  // the 32 leading bits of the fraction
+    const uint32_t tail = (m & 0x1FFu) << 1 | ((lo & 0xFFFFFu) != 0u ? 1u : 0u);  // the 29 dropped bits, the last one sticky
+    const uint32_t f = (hi & 0x80000000u) | ((e - 896u) << 23) | (m >> 9);
+    return __uint_as_float(f + (tail + 0x1FFu + (f & 1u) >= 0x400u ? 1u : 0u));
 }
-__device__ __forceinline__ void lds4(const double *p, double (&v)[4]) {
-    const double2 a = *reinterpret_cast<const double2 *>(p), b = *reinterpret_cast<const double2 *>(p + 2);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-__device__ __forceinline__ void lds4(const float *p, float (&v)[4]) {
-    const float4 a = *reinterpret_cast<const float4 *>(p);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+// FP32 -> FP64, exactly, with integer instructions where the FP32 is normal.
+__device__ __forceinline__ double to_f64(float x) {
+    const uint32_t b = __float_as_uint(x), a = b & 0x7FFFFFFFu;
+    if (a - 0x00800000u >= 0x7F000000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 // (hi, lo) += x with Knuth's TwoSum (exact transformation of hi + x).
@@ -52,113 +79,185 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
     lo = __fadd_rn(lo, err);
 }
 
-// 4 x 4 block accumulator: FP64 accumulates directly; FP32 keeps a chunk sum and a (hi, lo) pair.
-template <typename T>
-struct Block {
-    T c[4][4];
-    T hi[4][4], lo[4][4];
+// The lane's accumulators of one subtile: FP64 accumulates directly; FP32 keeps a chunk sum and a
+// (hi, lo) pair.
+template <typename T> struct Block;
+template <> struct Block<double> {
+    double c[2][4];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int a = 0; a < 2; a++)
+#pragma unroll
+            for (int b = 0; b < 4; b++) c[a][b] = 0.0;
+    }
+    __device__ __forceinline__ void fold() {}
+    __device__ __forceinline__ double value(int a, int b) const { return c[a][b]; }
+};
+template <> struct Block<float> {
+    float c[4][4], hi[4][4], lo[4][4];
     __device__ __forceinline__ void zero() {
 #pragma unroll
         for (int a = 0; a < 4; a++)
 #pragma unroll
-            for (int b = 0; b < 4; b++) c[a][b] = hi[a][b] = lo[a][b] = T(0);
+            for (int b = 0; b < 4; b++) c[a][b] = hi[a][b] = lo[a][b] = 0.0f;
     }
     __device__ __forceinline__ void fold() {
-        if constexpr (std::is_same<T, float>::value) {
 #pragma unroll
-            for (int a = 0; a < 4; a++)
+        for (int a = 0; a < 4; a++)
 #pragma unroll
-                for (int b = 0; b < 4; b++) {
-                    two_sum_acc(hi[a][b], lo[a][b], c[a][b]);
-                    c[a][b] = 0.0f;
-                }
-        }
+            for (int b = 0; b < 4; b++) {
+                two_sum_acc(hi[a][b], lo[a][b], c[a][b]);
+                c[a][b] = 0.0f;
+            }
     }
-    __device__ __forceinline__ double value(int a, int b) const {
-        if constexpr (std::is_same<T, float>::value) return (double)hi[a][b] + (double)lo[a][b];
-        else return c[a][b];
-    }
-    __device__ __forceinline__ void mma_chunk(const T (*As)[T_], const T (*Bs)[T_], int ty, int tx, int kc) {
-#pragma unroll 8
-        for (int kk = 0; kk < kc; kk++) {
-            T ra[4], rb[4];
-            lds4(&As[kk][ty * 4], ra);
-            lds4(&Bs[kk][tx * 4], rb);
-#pragma unroll
-            for (int a = 0; a < 4; a++)
-#pragma unroll
-                for (int b = 0; b < 4; b++) c[a][b] = fma(ra[a], rb[b], c[a][b]);
-        }
-    }
+    __device__ __forceinline__ double value(int a, int b) const { return __dadd_rn(to_f64(hi[a][b]), to_f64(lo[a][b])); }
 };
 
+// Shared-memory row of one K chunk: 128 bytes and 16 more, so that the eight rows that a warp reads at
+// once (one per lane group) lie in different banks.
+template <typename T> struct HTile {
+    static constexpr int LD = 144 / sizeof(T);
+    T a[2][T_][LD], b[2][T_][LD];
+};
+
+// One CTA per tile pair. Per K chunk of 128 bytes the rows of tile I come by cp.async and those of
+// tile J through registers, where they take their weights; two buffers, one barrier per chunk. The
+// chunks stay row-major (K along the row): a lane reads 16 bytes, 2 or 4 terms, of each of its rows
+// (ly + 8 a) and columns (lx + 4 b).
+// Whole 64 x 64 tiles computed 2.5 times the wanted triangle on the 8-atom cluster (batches of 75
+// functions on average) and 1.9 times on the 64-atom one, the subtiles 1.3 and 1.3 times. Measured with
+// the density below, H + n: 8 atoms FP64 13.7 -> 8.9 ms, 64 atoms FP32 15.7 -> 12.0 ms (H 6.7 -> 4.2, n
+// 3.7 -> 2.4).
 template <typename T>
-__global__ void __launch_bounds__(256) h_simt_kernel(DevSystem s, const HWork *__restrict__ work,
-                                                    const T *__restrict__ scratch, uint32_t terms) {
-    constexpr int KC = Cfg<T>::KC;
-    constexpr int VL = KC / 4;  // elements each thread loads per row segment
-    __shared__ __align__(16) T As[KC][T_];
-    __shared__ __align__(16) T Bs[KC][T_];
-    __shared__ T dv[NAO_MAX_BATCH], dk[NAO_MAX_BATCH];  // weights of the potential and kinetic parts
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
+    h_simt_kernel(const __grid_constant__ DevSystem s, const HWork *__restrict__ work, const T *__restrict__ scratch,
+                  uint32_t terms) {
+    using V = typename Vec16<T>::type;
+    constexpr int KC = Cfg<T>::KC, MR = Cfg<T>::MR, SR = Cfg<T>::SR, NU = Cfg<T>::NU, VK = 16 / sizeof(T);
+    constexpr int NS = (T_ / SR) * 4;  // subtiles of the tile
+    __shared__ __align__(16) HTile<T> sm;
+    extern __shared__ __align__(16) unsigned char dyn[];
     const HWork it = work[blockIdx.x];
     const int b = it.batch, m = s.sys.bmol[b];
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
     const int N = s.rel_off[b + 1] - s.rel_off[b];
+    T *wt = reinterpret_cast<T *>(dyn);  // [2][Ppad]: weights of the potential part, of the gradient parts
     const int64_t ld = 4 * (int64_t)Ppad;
     const T *E = scratch + s.scr_off[b];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int tid = threadIdx.x, lane = tid & 31, lx = lane & 3, ly = lane >> 2;
 
     for (int q = tid; q < Ppad; q += blockDim.x) {
         const double w = q < P ? s.pw[p0 + q] : 0.0;
         const double vv = q < P ? v_at(s, m, p0 + q) : 1.0;
-        dv[q] = T((terms & NAO_TERM_POTENTIAL) ? w * vv : 0.0);
+        wt[q] = T((terms & NAO_TERM_POTENTIAL) ? w * vv : 0.0);
         const double kin = (terms & NAO_TERM_KINETIC) ? 1.0 : 0.0;
-        dk[q] = T(0.5 * w * ((terms & NAO_TERM_TAU) && q < P ? kin + vt_at(s, m, p0 + q) : kin));
+        wt[Ppad + q] = T(0.5 * w * ((terms & NAO_TERM_TAU) && q < P ? kin + vt_at(s, m, p0 + q) : kin));
     }
 
     const int i0 = it.ti * T_, j0 = it.tj * T_;
-    const int lrow = tid >> 2, lk = (tid & 3) * VL;
-    const bool arow_ok = i0 + lrow < N, brow_ok = j0 + lrow < N;
-    const T *Arow = E + (int64_t)(i0 + lrow) * ld + lk;
-    const T *Brow = E + (int64_t)(j0 + lrow) * ld + lk;
-
-    Block<T> acc;
-    acc.zero();
-    __syncthreads();
-    const int K = 4 * Ppad;
-    for (int k0 = 0; k0 < K; k0 += KC) {
-        T av[VL], bv[VL];
+    const bool diag = it.ti == it.tj;
+    // this warp's subtiles: every eighth of the active ones (-1: none)
+    int sub[NU];
+    {
+        int k = 0;
+        const int w = ((tid >> 5) + blockIdx.x) & 7;
 #pragma unroll
-        for (int u = 0; u < VL; u++) av[u] = bv[u] = T(0);
-        if (arow_ok) load_vec(Arow + k0, av);
-        if (brow_ok) load_vec(Brow + k0, bv);
+        for (int u = 0; u < NU; u++) sub[u] = -1;
+        for (int x = 0; x < NS; x++) {
+            const int r = x >> 2, c = x & 3;
+            if (i0 + r * SR >= N || j0 + c * 16 >= N || (diag && c * 16 + 15 < r * SR)) continue;
 #pragma unroll
-        for (int u = 0; u < VL; u++) {
-            // column k of E belongs to component k / Ppad (phi, d/dx, d/dy, d/dz) of point k % Ppad;
-            // a chunk may straddle two components when Ppad is not a multiple of KC
-            const int k = k0 + lk + u, comp = k / Ppad, q = k - comp * Ppad;
-            As[lk + u][lrow] = av[u];
-            Bs[lk + u][lrow] = bv[u] * (comp == 0 ? dv[q] : dk[q]);
+            for (int u = 0; u < NU; u++)
+                if (k == w + 8 * u) sub[u] = x;
+            k++;
         }
-        __syncthreads();
-        acc.mma_chunk(As, Bs, ty, tx, KC);
-        acc.fold();
-        __syncthreads();
+    }
+    Block<T> acc[NU];
+#pragma unroll
+    for (int u = 0; u < NU; u++) acc[u].zero();
+
+    const int lv = tid & 7, lr = tid >> 3;  // loader: 16-byte vector lv of rows lr and lr + 32
+    const T *Ar[2], *Br[2];
+    bool aok[2], bok[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int r = lr + 32 * h;
+        aok[h] = i0 + r < N;
+        bok[h] = j0 + r < N;
+        Ar[h] = E + (int64_t)(aok[h] ? i0 + r : 0) * ld + lv * VK;
+        Br[h] = E + (int64_t)(bok[h] ? j0 + r : 0) * ld + lv * VK;
+    }
+    V bv[2];
+    int wq = lv * VK, comp = 0;  // the point and component (phi, d/dx, d/dy, d/dz) of this vector's column
+    auto load = [&](int k0, int buf) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            cp16(&sm.a[buf][lr + 32 * h][lv * VK], Ar[h] + k0, aok[h]);
+            if (bok[h]) bv[h] = *reinterpret_cast<const V *>(Br[h] + k0);
+        }
+    };
+    auto store = [&](int buf) {
+        while (wq >= Ppad) {
+            wq -= Ppad;
+            comp++;
+        }
+        const V w = *reinterpret_cast<const V *>(wt + (comp == 0 ? 0 : Ppad) + wq);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            V x{};
+            if (bok[h]) x = vmul(bv[h], w);
+            *reinterpret_cast<V *>(&sm.b[buf][lr + 32 * h][lv * VK]) = x;
+        }
+        wq += KC;
+    };
+    const int nk = 4 * Ppad / KC;
+    load(0, 0);
+    __syncthreads();  // the weights are written
+    store(0);
+    for (int kc = 0; kc < nk; kc++) {
+        const int buf = kc & 1;
+        cp_wait_all();
+        __syncthreads();  // this chunk is complete, and every warp has left the other buffer
+        if (kc + 1 < nk) load((kc + 1) * KC, buf ^ 1);
+#pragma unroll
+        for (int u = 0; u < NU; u++) {
+            if (sub[u] < 0) continue;
+            const T *a = &sm.a[buf][(sub[u] >> 2) * SR + ly][0], *bb = &sm.b[buf][(sub[u] & 3) * 16 + lx][0];
+#pragma unroll
+            for (int kv = 0; kv < KC; kv += VK) {
+                V ra[MR], rb[4];
+#pragma unroll
+                for (int x = 0; x < MR; x++) ra[x] = *reinterpret_cast<const V *>(a + 8 * x * HTile<T>::LD + kv);
+#pragma unroll
+                for (int y = 0; y < 4; y++) rb[y] = *reinterpret_cast<const V *>(bb + 4 * y * HTile<T>::LD + kv);
+#pragma unroll
+                for (int e = 0; e < VK; e++)
+#pragma unroll
+                    for (int x = 0; x < MR; x++)
+#pragma unroll
+                        for (int y = 0; y < 4; y++) acc[u].c[x][y] = fma(vget(ra[x], e), vget(rb[y], e), acc[u].c[x][y]);
+            }
+            acc[u].fold();
+        }
+        if (kc + 1 < nk) store(buf ^ 1);
     }
 
     const int32_t *rel = s.rel_idx + s.rel_off[b];
-    const bool diag = it.ti == it.tj;
 #pragma unroll
-    for (int a = 0; a < 4; a++) {
-        const int i = i0 + ty * 4 + a;
-        if (i >= N) continue;
-        const int64_t gi = rel[i];
+    for (int u = 0; u < NU; u++) {
+        if (sub[u] < 0) continue;
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const int j = j0 + tx * 4 + c;
-            if (j >= N || (diag && j < i)) continue;
-            h_add(s, m, gi, rel[j], acc.value(a, c));
+        for (int x = 0; x < MR; x++) {
+            const int i = i0 + (sub[u] >> 2) * SR + ly + 8 * x;
+            if (i >= N) continue;
+            const int64_t gi = rel[i];
+#pragma unroll
+            for (int y = 0; y < 4; y++) {
+                const int j = j0 + (sub[u] & 3) * 16 + lx + 4 * y;
+                if (j >= N || (diag && j < i)) continue;
+                h_add(s, m, gi, rel[j], acc[u].value(x, y));
+            }
         }
     }
 }
@@ -211,18 +310,46 @@ __global__ void __launch_bounds__(256) zero_h_kernel(DevSystem s, const int4 *__
     for (int i = threadIdx.x; i < tk.z; i += blockDim.x) H[i] = 0.0;
 }
 
+// Sums over functions of T_qj f_qj: in FP64, or as a float-float on the FP32 path (T there is a
+// (hi, lo) pair and f an FP32; the products are exact but for the 2^-48 terms).
+template <typename T> struct PointSum;
+template <> struct PointSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(const Block<double> &t, int a, int b, double f) { s += t.c[a][b] * f; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct PointSum<float> {
+    float h = 0.0f, l = 0.0f;
+    __device__ __forceinline__ void add(const Block<float> &t, int a, int b, float f) {
+        const float p = __fmul_rn(t.hi[a][b], f);
+        const float e = __fmaf_rn(t.lo[a][b], f, __fmaf_rn(t.hi[a][b], f, -p));
+        two_sum_acc(h, l, p);
+        l = __fadd_rn(l, e);
+    }
+    __device__ __forceinline__ double value() const { return __dadd_rn(to_f64(h), to_f64(l)); }
+};
+
 // GRADN: the density gradient too (Sec. 2; grad n = 2 sum_ij grad phi_i P_ij phi_j): with
 // T_qj = sum_i phi_qi P_ij over all of P (no tile-pair symmetry), n_q = sum_j T_qj phi_qj and
 // grad n_q = 2 sum_j T_qj grad phi_qj; the scratch rows then hold [phi | d/dx | d/dy | d/dz].
+// One CTA per 64-point tile; per 64-function tile J the K chunks of rows i are staged K-major (phi by
+// cp.async, P' through registers), two buffers and one barrier per chunk. A warp keeps one
+// 16-function column group and one or two groups of points for the whole tile loop, so that a point's
+// sums over functions stay in registers until the end. In FP64 the symmetry c_IJ is taken in blocks of
+// 16 functions instead of 64 (a warp leaves out the chunks below its column group's diagonal block).
 template <typename T, bool GRADN>
-__global__ void __launch_bounds__(256) density_simt_kernel(DevSystem s, const DWork *__restrict__ work, int32_t w0,
-                                                          const T *__restrict__ scratch, double *__restrict__ ne_part) {
-    constexpr int KC = Cfg<T>::KC;
-    constexpr int RPT = (KC * T_) / 256;     // elements each thread loads per tile
-    __shared__ __align__(16) T As[KC][T_];  // phi[i][q]
-    __shared__ __align__(16) T Bs[KC][T_];  // c_IJ P[rel_i][rel_j]
-    __shared__ double nacc[T_];
-    __shared__ double gacc[GRADN ? 3 : 1][T_];
+__global__ void __launch_bounds__(256, sizeof(T) == 8 && !GRADN ? 3 : 2)
+    density_simt_kernel(const __grid_constant__ DevSystem s, const DWork *__restrict__ work, int32_t w0,
+                        const T *__restrict__ scratch, double *__restrict__ ne_part) {
+    using V = typename Vec16<T>::type;
+    constexpr int KC = Cfg<T>::KC, MR = Cfg<T>::MR, SR = Cfg<T>::SR, NU = Cfg<T>::NU, VK = 16 / sizeof(T);
+    constexpr bool FP = std::is_same<T, double>::value;
+    constexpr int NC = GRADN ? 4 : 1;          // sums per point: n, grad n
+    constexpr int VR = T_ / VK;                // vectors per row of phi
+    constexpr int BR = KC / 8;                 // rows of P' per warp and chunk
+    __shared__ __align__(16) T As[2][KC][T_];  // phi[i][q]
+    __shared__ __align__(16) T Bs[2][KC][T_];  // c_IJ P[rel_i][rel_j]
+    __shared__ double part[4][NC][T_];
     __shared__ double red[8];
     const DWork it = work[w0 + blockIdx.x];
     const int b = it.batch, m = s.sys.bmol[b];
@@ -233,91 +360,160 @@ __global__ void __launch_bounds__(256) density_simt_kernel(DevSystem s, const DW
     const T *E = scratch + s.scr_off[b];  // row stride Ppad (phi only) or 4 Ppad (GRADN)
     const int64_t ld = GRADN ? 4 * (int64_t)Ppad : (int64_t)Ppad;
     const int32_t *rel = s.rel_idx + s.rel_off[b];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int32_t bo = s.sys.boff[m];
+    const int64_t nbm = s.sys.nbm[m];
+    const double *Pm = s.sys.P[m];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lx = lane & 3, ly = lane >> 2;
+    const int role = (warp + blockIdx.x) & 7, cg = role & 3;  // column group
     const int nt = (N + T_ - 1) / T_;
-    if (tid < T_) {
-        nacc[tid] = 0.0;
-        if (GRADN) gacc[0][tid] = gacc[GRADN ? 1 : 0][tid] = gacc[GRADN ? 2 : 0][tid] = 0.0;
+    int row[NU];  // first point (of the tile) of each of the warp's point groups, -1: beyond the batch
+#pragma unroll
+    for (int u = 0; u < NU; u++) {
+        row[u] = SR * ((role >> 2) + 2 * u);
+        if (q0 + row[u] >= P) row[u] = -1;
     }
+    PointSum<T> sum[NU][MR][NC];
 
-    // loader mapping: row lk of the chunk, RPT consecutive columns starting at lc
-    const int lk = tid / (T_ / RPT), lc = (tid % (T_ / RPT)) * RPT;
     for (int tj = 0; tj < nt; tj++) {
-        Block<T> acc;
-        acc.zero();
-        for (int ti = 0; ti < (GRADN ? nt : tj + 1); ti++) {
-            const double scale = (!GRADN && ti < tj) ? 2.0 : 1.0;
-            for (int k0 = 0; k0 < T_; k0 += KC) {
-                const int i = ti * T_ + k0 + lk;
-                T fv[RPT];
+        Block<T> acc[NU];
 #pragma unroll
-                for (int u = 0; u < RPT; u++) fv[u] = T(0);
-                if (i < N && q0 + lc < Ppad) load_vec(E + (int64_t)i * ld + q0 + lc, fv);
+        for (int u = 0; u < NU; u++) acc[u].zero();
+        const int kend = GRADN ? N : min(N, (tj + 1) * T_);
+        const int nk = (kend + KC - 1) / KC;
+        const bool live = row[0] >= 0 && tj * T_ + cg * 16 < N;
+        int64_t gj[2];  // the columns of P' that this lane loads: lane and lane + 32
+        bool jok[2];
 #pragma unroll
-                for (int u = 0; u < RPT; u++) {
-                    As[lk][lc + u] = fv[u];
-                    const int j = tj * T_ + lc + u;
-                    T pv = T(0);
-                    if (i < N && j < N) {
-                        int64_t gi = rel[i], gj = rel[j];
-                        if (gi > gj) { const int64_t t = gi; gi = gj; gj = t; }
-                        pv = T(scale * p_elem(s, m, gi, gj));
+        for (int c = 0; c < 2; c++) {
+            const int j = tj * T_ + lane + 32 * c;
+            jok[c] = j < N;
+            gj[c] = jok[c] ? rel[j] - bo : 0;
+        }
+        double pv[BR][2];
+        auto load = [&](int kc, int buf) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int x = tid + 256 * h, kk = x / VR, v = (x % VR) * VK, i = kc * KC + kk;
+                const bool ok = i < N && q0 + v < Ppad;
+                cp16(&As[buf][kk][v], ok ? E + (int64_t)i * ld + q0 + v : E, ok);
+            }
+#pragma unroll
+            for (int r = 0; r < BR; r++) {
+                const int i = kc * KC + warp * BR + r;
+                const int64_t gi = i < N ? rel[i] - bo : 0;
+#pragma unroll
+                for (int c = 0; c < 2; c++)
+                    if (i < N && jok[c]) pv[r][c] = gi <= gj[c] ? Pm[gi * nbm + gj[c]] : Pm[gj[c] * nbm + gi];
+            }
+        };
+        auto store = [&](int kc, int buf) {
+#pragma unroll
+            for (int r = 0; r < BR; r++) {
+                const int i = kc * KC + warp * BR + r;
+#pragma unroll
+                for (int c = 0; c < 2; c++) {
+                    const int j = tj * T_ + lane + 32 * c;
+                    // c_IJ = 2 above the diagonal blocks, 1 on them (those below are not used); FP64
+                    // blocks of 16 functions, FP32 blocks of 64
+                    const bool two = !GRADN && (FP ? (i >> 4) < (j >> 4) : (i >> 6) < tj);
+                    T x = T(0);
+                    if (i < N && jok[c]) {
+                        if constexpr (FP) x = pv[r][c];
+                        else x = to_f32(pv[r][c]);
+                        if (two) x += x;
                     }
-                    Bs[lk][lc + u] = pv;
+                    Bs[buf][warp * BR + r][lane + 32 * c] = x;
                 }
-                __syncthreads();
-                acc.mma_chunk(As, Bs, ty, tx, KC);
-                acc.fold();
-                __syncthreads();
+            }
+        };
+        load(0, 0);
+        store(0, 0);
+        for (int kc = 0; kc < nk; kc++) {
+            const int buf = kc & 1;
+            cp_wait_all();
+            __syncthreads();  // this chunk is complete, and every warp has left the other buffer
+            if (kc + 1 < nk) load(kc + 1, buf ^ 1);
+            if (live && !(FP && !GRADN && kc > tj * 4 + cg)) {
+#pragma unroll
+                for (int u = 0; u < NU; u++) {
+                    if (row[u] < 0) continue;
+                    const T *a = &As[buf][0][row[u] + ly * MR], *bb = &Bs[buf][0][cg * 16 + lx * 4];
+#pragma unroll 8
+                    for (int kk = 0; kk < KC; kk++) {
+                        T ra[MR], rb[4];
+#pragma unroll
+                        for (int x = 0; x < MR; x += VK) {
+                            const V v = *reinterpret_cast<const V *>(a + kk * T_ + x);
+#pragma unroll
+                            for (int e = 0; e < VK; e++) ra[x + e] = vget(v, e);
+                        }
+#pragma unroll
+                        for (int y = 0; y < 4; y += VK) {
+                            const V v = *reinterpret_cast<const V *>(bb + kk * T_ + y);
+#pragma unroll
+                            for (int e = 0; e < VK; e++) rb[y + e] = vget(v, e);
+                        }
+#pragma unroll
+                        for (int x = 0; x < MR; x++)
+#pragma unroll
+                            for (int y = 0; y < 4; y++) acc[u].c[x][y] = fma(ra[x], rb[y], acc[u].c[x][y]);
+                    }
+                    acc[u].fold();
+                }
+            }
+            if (kc + 1 < nk) store(kc + 1, buf ^ 1);
+        }
+        // n_q += sum_{j in J} T_qj phi_jq (and grad n): this lane's points and four columns
+#pragma unroll
+        for (int u = 0; u < NU; u++) {
+            const int q = q0 + row[u] + ly * MR;
+            if (row[u] < 0 || q >= Ppad) continue;
+#pragma unroll
+            for (int y = 0; y < 4; y++) {
+                const int j = tj * T_ + cg * 16 + lx * 4 + y;
+                if (j >= N) continue;
+#pragma unroll
+                for (int d = 0; d < NC; d++)
+#pragma unroll
+                    for (int x = 0; x < MR; x += VK) {
+                        const V f = *reinterpret_cast<const V *>(E + (int64_t)j * ld + d * Ppad + q + x);
+#pragma unroll
+                        for (int e = 0; e < VK; e++) sum[u][x + e][d].add(acc[u], x + e, y, vget(f, e));
+                    }
             }
         }
-        // n_q += sum_{j in J} T_qj phi_jq  (rows q = ty*4 + a of the tile, columns j = tx*4 + c)
-#pragma unroll
-        for (int a = 0; a < 4; a++) {
-            const int q = q0 + ty * 4 + a;
-            double part = 0.0, gp[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const int j = tj * T_ + tx * 4 + c;
-                const bool ok = j < N && q < Ppad;
-                const double tv = acc.value(a, c);
-                part += tv * (ok ? (double)E[(int64_t)j * ld + q] : 0.0);
-                if (GRADN)
-#pragma unroll
-                    for (int d = 0; d < 3; d++) gp[d] += tv * (ok ? (double)E[(int64_t)j * ld + (d + 1) * Ppad + q] : 0.0);
-            }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {
-                part += __shfl_xor_sync(0xffffffffu, part, o);
-                if (GRADN)
-#pragma unroll
-                    for (int d = 0; d < 3; d++) gp[d] += __shfl_xor_sync(0xffffffffu, gp[d], o);
-            }
-            if (tx == 0) {
-                nacc[ty * 4 + a] += part;
-                if (GRADN)
-#pragma unroll
-                    for (int d = 0; d < 3; d++) gacc[d][ty * 4 + a] += 2.0 * gp[d];
-            }
-        }
-        __syncthreads();
+        __syncthreads();  // the next tile's first chunk goes into buffer 0
     }
+    for (int x = tid; x < 4 * NC * T_; x += blockDim.x) (&part[0][0][0])[x] = 0.0;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < NU; u++)
+#pragma unroll
+        for (int x = 0; x < MR; x++)
+#pragma unroll
+            for (int d = 0; d < NC; d++) {
+                double t = sum[u][x][d].value();
+                t += __shfl_xor_sync(0xffffffffu, t, 1);
+                t += __shfl_xor_sync(0xffffffffu, t, 2);
+                if (lx == 0 && row[u] >= 0) part[cg][d][row[u] + ly * MR + x] = t;
+            }
     __syncthreads();
     double wn = 0.0;
     if (tid < T_) {
         const int q = q0 + tid;
         if (q < P) {
-            const double nv = nacc[tid];
+            auto total = [&](int d) { return (part[0][d][tid] + part[1][d][tid]) + (part[2][d][tid] + part[3][d][tid]); };
+            const double nv = total(0);
             *n_at(s, m, p0 + q) = nv;
             if (GRADN)
 #pragma unroll
-                for (int d = 0; d < 3; d++) *gn_at(s, m, p0 + q, d) = gacc[d][tid];
+                for (int d = 0; d < 3; d++) *gn_at(s, m, p0 + q, d) = 2.0 * total(GRADN ? 1 + d : 0);
             wn = s.pw[p0 + q] * nv;
         }
     }
     // fixed-order block sum of w n over the tile
     for (int o = 16; o > 0; o >>= 1) wn += __shfl_xor_sync(0xffffffffu, wn, o);
-    if ((tid & 31) == 0) red[tid >> 5] = wn;
+    if (lane == 0) red[warp] = wn;
     __syncthreads();
     if (tid == 0) {
         double t = 0.0;
@@ -370,14 +566,24 @@ __global__ void __launch_bounds__(64) zero_n_kernel(DevSystem s, const DWork *__
 
 }  // namespace
 
+template <typename T>
+static cudaError_t launch_h_simt_t(const DevSystem &s, const HWork *work, int32_t n_work, const T *scratch, uint32_t terms,
+                                   cudaStream_t st) {
+    const size_t dyn = 2 * (size_t)s.max_ppad * sizeof(T);  // the weights
+    if (dyn + sizeof(HTile<T>) > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(h_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * NAO_MAX_BATCH * (int)sizeof(T));
+        if (e != cudaSuccess) return e;
+    }
+    h_simt_kernel<T><<<n_work, 256, dyn, st>>>(s, work, scratch, terms);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_h_simt(const DevSystem &s, nao_precision prec, const HWork *work, int32_t n_work,
                           const double *scratch, uint32_t terms, cudaStream_t st) {
     if (n_work <= 0) return cudaSuccess;
-    if (prec == NAO_FP32)
-        h_simt_kernel<float><<<n_work, 256, 0, st>>>(s, work, reinterpret_cast<const float *>(scratch), terms);
-    else
-        h_simt_kernel<double><<<n_work, 256, 0, st>>>(s, work, scratch, terms);
-    return cudaGetLastError();
+    if (prec == NAO_FP32) return launch_h_simt_t(s, work, n_work, reinterpret_cast<const float *>(scratch), terms, st);
+    return launch_h_simt_t(s, work, n_work, scratch, terms, st);
 }
 
 cudaError_t launch_zero_h(const DevSystem &s, const int4 *tasks, int32_t n_tasks, cudaStream_t st) {
