@@ -742,7 +742,9 @@ int default_tn(int S, int F) { return nao_split_tn(S, F); }
 nao_status split_lists(nao_grid *g) {
     const int S = g->split_S, F = g->split_F;
     g->split_lists_ver++;
-    std::vector<HWork> hw[2], nw[2];
+    std::vector<HTask> hw[2];
+    BlockPairs pairs;
+    std::vector<HWork> nw[2];
     for (auto &c : g->split_chunks) {
         for (int k = 0; k < 2; k++) {
             c.hw0[k] = (int32_t)hw[k].size();
@@ -753,21 +755,21 @@ nao_status split_lists(nao_grid *g) {
             if (N == 0) continue;
             const int TN = g->split_tn[b], k = TN == 48 ? 0 : 1;
             const SplitGeom G(P, N, S, TN, F);
-            nao_split_h_items(b, P, N, TN, S, hw[k], F);
+            nao_split_h_items(b, P, N, TN, S, hw[k], pairs, F);
             for (int Q = 0; Q < G.n_qt; Q++) nw[k].push_back({b, Q, G.n_jtN, 0});  // all J tiles in one CTA
         }
         // the persistent contraction kernels take items round-robin: heaviest first (H: longest
         // K, i.e. most K chunks in the item's segment; density: most function tiles), so that
         // every CTA gets a similar share
-        auto item_kc = [&](const HWork &x) {
+        auto item_kc = [&](const HTask &x) {
             const SplitGeom G(g->Pb[x.batch], g->Nb[x.batch], S, 0, F);
             int kc0, kc1;
-            nao_split_h_seg_range(G.n_kc, nao_split_h_nseg(g->Pb[x.batch], S, F), x.pad, S, kc0, kc1, F);
+            nao_split_h_seg_range(G.n_kc, nao_split_h_nseg(g->Pb[x.batch], S, F), x.seg(), S, kc0, kc1, F);
             return kc1 - kc0;
         };
         for (int k = 0; k < 2; k++) {
             std::stable_sort(hw[k].begin() + c.hw0[k], hw[k].end(),
-                             [&](const HWork &x, const HWork &y) { return item_kc(x) > item_kc(y); });
+                             [&](const HTask &x, const HTask &y) { return item_kc(x) > item_kc(y); });
             std::stable_sort(nw[k].begin() + c.nw0[k], nw[k].end(),
                              [](const HWork &x, const HWork &y) { return x.tj > y.tj; });
             c.hw1[k] = (int32_t)hw[k].size();
@@ -787,11 +789,9 @@ nao_status split_lists(nao_grid *g) {
     hw[0].insert(hw[0].end(), hw[1].begin(), hw[1].end());
     nw[0].insert(nw[0].end(), nw[1].begin(), nw[1].end());
     if (!hw[0].empty())
-        NAO_CUDA(copy_async(g->d_split_hw, hw[0].data(), hw[0].size() * sizeof(HWork), cudaMemcpyHostToDevice, g->setup));
+        NAO_CUDA(copy_async(g->d_split_hw, hw[0].data(), hw[0].size() * sizeof(HTask), cudaMemcpyHostToDevice, g->setup));
     if (!nw[0].empty())
         NAO_CUDA(copy_async(g->d_split_nw, nw[0].data(), nw[0].size() * sizeof(HWork), cudaMemcpyHostToDevice, g->setup));
-    NAO_CUDA(copy_async(g->d_split_tn, g->split_tn.data(), g->split_tn.size() * sizeof(int32_t),
-                             cudaMemcpyHostToDevice, g->setup));
     NAO_CUDA(cudaStreamSynchronize(g->setup));
     g->n_split_hw = nh;
     g->n_split_nw = nn;
@@ -833,6 +833,8 @@ nao_status split_setup(nao_grid *g) {
         std::max<int64_t>(3 * (g->opt.scratch_bytes > 0 ? g->opt.scratch_bytes : kDefaultScratch), int64_t(1) << 20);
     std::vector<int64_t> off_h(g->n_batches, 0), off_n(g->n_batches, 0);
     int64_t max_used = 0, cap_h = 0, cap_n = 0;
+    BlockPairs pairs;
+    std::vector<HTask> tmp;
     g->split_tn.assign(g->n_batches, 32);
     for (const Chunk &c : g->chunks) {
         nao_grid::SplitChunk cur{};
@@ -861,8 +863,8 @@ nao_status split_setup(nao_grid *g) {
                 int64_t best_h = 0;
                 for (int TN : {48, 32}) {
                     if (TN == 48 && nao_split_tn(S, F) != 48) continue;
-                    std::vector<HWork> tmp;
-                    nao_split_h_items(b, P, N, TN, S, tmp, F);
+                    tmp.clear();
+                    nao_split_h_items(b, P, N, TN, S, tmp, pairs, F);
                     best_h = std::max(best_h, (int64_t)tmp.size());
                 }
                 cap_h += best_h;
@@ -880,7 +882,6 @@ nao_status split_setup(nao_grid *g) {
         (st = dev_alloc(g, &g->d_expo_q, (size_t)g->n_points)) ||
         (st = dev_alloc(g, &g->d_expo_b, (size_t)g->n_batches)) ||
         (st = dev_alloc(g, &g->d_neg16, (size_t)g->n_batches)) ||
-        (st = dev_alloc(g, &g->d_split_tn, (size_t)g->n_batches)) ||
         (st = dev_alloc(g, &g->d_split_hw, (size_t)std::max<int64_t>(cap_h, 1))) ||
         (st = dev_alloc(g, &g->d_split_nw, (size_t)std::max<int64_t>(cap_n, 1))))
         return st;
@@ -920,6 +921,7 @@ nao_status split_tune(nao_grid *g, uint32_t terms, cudaStream_t st) {
     const int S = g->split_S;
     const DevSystem &s = g->sys;
     constexpr int kBuckets = kTnBuckets, kChunks = 3;
+    BlockPairs pairs;
     std::vector<int> bucket(g->n_batches, -1), total(kBuckets, 0);
     for (int64_t b = 0; b < g->n_batches; b++)
         if (g->Nb[b] > 0) {
@@ -951,24 +953,24 @@ nao_status split_tune(nao_grid *g, uint32_t terms, cudaStream_t st) {
             int64_t base48 = 0;
             for (int32_t b = c.b0; b < c.b1; b++) {
                 if (bucket[b] != k) continue;
-                std::vector<HWork> tmp;
-                nao_split_h_items(b, g->Pb[b], g->Nb[b], 48, S, tmp);
+                std::vector<HTask> tmp;
+                nao_split_h_items(b, g->Pb[b], g->Nb[b], 48, S, tmp, pairs, g->split_F);
                 base48 += (int64_t)tmp.size();
             }
             const int64_t reps = base48 > 0 ? (8 * 152 + base48 - 1) / base48 : 0;
             for (int w = 0; w < 2 && rs == NAO_OK && reps > 0; w++) {
                 const int TN = w == 0 ? 48 : 32;
-                std::vector<HWork> items;
+                std::vector<HTask> items;
                 for (int64_t r = 0; r < reps; r++)
                     for (int32_t b = c.b0; b < c.b1; b++)
-                        if (bucket[b] == k) nao_split_h_items(b, g->Pb[b], g->Nb[b], TN, S, items);
+                        if (bucket[b] == k) nao_split_h_items(b, g->Pb[b], g->Nb[b], TN, S, items, pairs, g->split_F);
                 n_items = (int64_t)items.size();
                 if (items.empty()) break;
                 if ((int64_t)items.size() > g->cap_tune_hw) {
                     if ((rs = dev_alloc(g, &g->d_tune_hw, items.size()))) break;
                     g->cap_tune_hw = (int64_t)items.size();
                 }
-                ce = copy_async(g->d_tune_hw, items.data(), items.size() * sizeof(HWork), cudaMemcpyHostToDevice,
+                ce = copy_async(g->d_tune_hw, items.data(), items.size() * sizeof(HTask), cudaMemcpyHostToDevice,
                                      g->setup);
                 if (ce == cudaSuccess) ce = cudaStreamSynchronize(g->setup);
                 ms[w] = 1e30f;
@@ -1086,7 +1088,7 @@ nao_status enqueue_n(nao_grid *g, nao_precision prec, bool want_ne, bool grad, c
             }));
             NAO_CUDA(timed(g, NAO_K_SLICE_N, st, [&] {
                 return launch_slice_n(s, c.b0, c.b1, c.max_qt, c.max_rt, g->d_scratch, g->d_slices, g->d_sl_off_n,
-                                      g->d_expo_q, g->d_expo_b, g->d_split_tn, S, g->split_F, grad, st);
+                                      g->d_expo_q, g->d_expo_b, S, g->split_F, grad, st);
             }));
             for (int k = 0; k < 2; k++)
                 if (c.nw1[k] > c.nw0[k])
@@ -1623,7 +1625,7 @@ nao_status nao_update_density_hessian(nao_grid *g, const double *P_dev, nao_prec
                     const int32_t *eq = g->d_expo4 + (size_t)comp * (size_t)g->n_points;
                     NAO_CUDA(launch_slice_n_hess(sys, sub.b0, sub.b1, sub.max_qt, sub.max_rt, g->d_scratch,
                                                  g->d_hess_off, comp, g->d_slices, g->d_sl_off_n, eq, g->d_expo_b,
-                                                 g->d_split_tn, S, F, s));
+                                                 S, F, s));
                     for (int k = 0; k < 2; k++)
                         NAO_CUDA(launch_n_tc_hess(sys, g->d_hess_nw, sub.nw0[k], sub.nw1[k] - sub.nw0[k], g->d_slices,
                                                   g->d_sl_off_n, eq, g->d_expo_b, g->d_scratch, g->d_hess_off, comp,

@@ -63,13 +63,6 @@ __device__ __forceinline__ float to_f32(double x) {
     const uint32_t f = (hi & 0x80000000u) | ((e - 896u) << 23) | (m >> 9);
     return __uint_as_float(f + (tail + 0x1FFu + (f & 1u) >= 0x400u ? 1u : 0u));
 }
-// FP32 -> FP64, exactly, with integer instructions where the FP32 is normal.
-__device__ __forceinline__ double to_f64(float x) {
-    const uint32_t b = __float_as_uint(x), a = b & 0x7FFFFFFFu;
-    if (a - 0x00800000u >= 0x7F000000u) return (double)x;
-    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
-}
-
 // (hi, lo) += x with Knuth's TwoSum (exact transformation of hi + x).
 __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
     const float s = __fadd_rn(hi, x);
@@ -110,7 +103,7 @@ template <> struct Block<float> {
                 c[a][b] = 0.0f;
             }
     }
-    __device__ __forceinline__ double value(int a, int b) const { return __dadd_rn(to_f64(hi[a][b]), to_f64(lo[a][b])); }
+    __device__ __forceinline__ double value(int a, int b) const { return __dadd_rn(ffa::widen(hi[a][b]), ffa::widen(lo[a][b])); }
 };
 
 // Shared-memory row of one K chunk: 128 bytes and 16 more, so that the eight rows that a warp reads at
@@ -326,7 +319,7 @@ template <> struct PointSum<float> {
         two_sum_acc(h, l, p);
         l = __fadd_rn(l, e);
     }
-    __device__ __forceinline__ double value() const { return __dadd_rn(to_f64(h), to_f64(l)); }
+    __device__ __forceinline__ double value() const { return __dadd_rn(ffa::widen(h), ffa::widen(l)); }
 };
 
 // GRADN: the density gradient too (Sec. 2; grad n = 2 sum_ij grad phi_i P_ij phi_j): with

@@ -20,6 +20,7 @@
 
 #ifdef __CUDACC__
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace ffa {
 
@@ -34,6 +35,14 @@ __device__ __forceinline__ F make(float h, float l) { return F{h, l}; }
 __device__ __forceinline__ F from_double(double x) {
     const float h = __double2float_rn(x);
     return F{h, __double2float_rn(__dsub_rn(x, (double)h))};
+}
+
+// FP32 -> FP64, exactly, with integer instructions where the FP32 is normal (the conversion instruction
+// runs on the FP64 pipe).
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), a = b & 0x7FFFFFFFu;
+    if (a - 0x00800000u >= 0x7F000000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 __device__ __forceinline__ double to_double(F x) { return __dadd_rn((double)x.h, (double)x.l); }

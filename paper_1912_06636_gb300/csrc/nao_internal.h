@@ -203,7 +203,20 @@ struct SplitGeom {
 };
 
 struct HWork {  // one upper-triangular tile pair of one batch's h[B] (Eq. batch_matrix_mult)
-    int32_t batch, ti, tj, pad;  // split H items: pad = the K segment (below)
+    int32_t batch, ti, tj, pad;
+};
+
+// One item of the split H contraction: 128 x TN elements of one batch's h[B], over one K segment
+// (below). The 128 rows are four blocks of 32 functions, any four of the batch (kNoRows: none), and the
+// columns the TN-function tile tj.
+constexpr uint32_t kNoRows = 0xFFFFu;
+struct HTask {
+    int32_t batch;
+    uint32_t tj_seg;    // tj | segment << 16
+    uint32_t r01, r23;  // row blocks 0 | 1 << 16, 2 | 3 << 16
+    __host__ __device__ int tj() const { return (int)(tj_seg & 0xFFFFu); }
+    __host__ __device__ int seg() const { return (int)(tj_seg >> 16); }
+    __host__ __device__ uint32_t row(int x) const { return ((x < 2 ? r01 : r23) >> (16 * (x & 1))) & 0xFFFFu; }
 };
 
 // K segments of the split H contraction. A slice-order group's FP32 accumulator sums K products
@@ -235,16 +248,18 @@ __host__ __device__ inline void nao_split_h_seg_range(int n_kc, int nseg, int se
     kc1 = kc0 + kcs < n_kc ? kc0 + kcs : n_kc;
 }
 
-// Split H work items of one batch (P points, N functions) for tile width TN and S slices: per
-// 128-row tile I, the TN-column tiles J >= floor(128 I / TN) (those reaching the upper
-// triangle), once per K segment.
-inline void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HWork> &out,
-                              int F = NAO_DIGITS_BF16) {
-    const int nI = (N + 127) / 128, nJ = (N + TN - 1) / TN, nseg = nao_split_h_nseg(P, S, F);
-    for (int I = 0; I < nI; I++)
-        for (int J = (I * 128) / TN; J < nJ; J++)
-            for (int q = 0; q < nseg; q++) out.push_back({b, I, J, q});
-}
+// Split H items of one batch (P points, N functions) for tile width TN and S slices, once per K
+// segment (partition.cpp). h is symmetric, so every unordered pair of functions is wanted once.
+// TN = 48: per 128-row tile I the column tiles J >= floor(128 I / TN) (those reaching the upper triangle).
+// TN = 32: rows and columns are cut into the same 32-function blocks, and every pair of blocks {a, b} is
+// given to one of the two columns, a or b, so that the columns' row counts (their own block included) fill
+// their items of four: max(n, ceil(n (n + 1) / 8)) items for n blocks, against sum_I (n - 4 I) when
+// every pair went to the later block's column (N = 200: 7 against 10).
+// kept: the assignments made so far, by n (one list's scratch).
+using BlockPairs = std::map<int, std::vector<std::vector<int>>>;
+void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HTask> &out, BlockPairs &kept, int F);
+// The rows of each of n blocks' columns in that assignment, its own block first, then in cyclic order.
+std::vector<std::vector<int>> nao_block_pairs(int n);
 struct DWork {  // one tile of points of one batch for the density
     int32_t batch, tp;
 };
@@ -331,17 +346,17 @@ struct nao_grid {
     // tile width (MMA N) of every batch on the split path: a fixed rule until the autotuner has
     // timed both widths per (N_b, P_b) bucket of the batch-size histogram
     std::vector<int32_t> split_tn;
-    int32_t *d_split_tn = nullptr;
     bool split_tuned = false;
     int32_t tune_buckets = 0;      // buckets the autotuner timed
     int64_t cap_split_hw = 0, cap_split_nw = 0;
-    HWork *d_tune_hw = nullptr;    // scratch work list of the autotuner
+    HTask *d_tune_hw = nullptr;    // scratch work list of the autotuner
     int64_t cap_tune_hw = 0;
     uint8_t *d_slices = nullptr;
     int64_t *d_sl_off_h = nullptr, *d_sl_off_n = nullptr;
     int32_t *d_expo_h = nullptr, *d_expo_q = nullptr, *d_expo_b = nullptr;
     int32_t *d_neg16 = nullptr;  // per batch: leading negative-weight K steps of 16 columns
-    HWork *d_split_hw = nullptr, *d_split_nw = nullptr;
+    HTask *d_split_hw = nullptr;
+    HWork *d_split_nw = nullptr;   // density items: (batch, 128-point tile, function tiles)
     int64_t n_split_hw = 0, n_split_nw = 0;
     // kernel timing (nao_profile_enable)
     bool profiling = false;
@@ -417,24 +432,22 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
                            uint32_t terms, uint8_t *slices, const int64_t *sl_off, int32_t *expo, int32_t *neg16, int S,
                            int F, cudaStream_t st);
 // tn: tile width 48 (bf16 digits, S <= 10 only) or 32; scatter = 0 skips the H scatter (autotuner timing).
-// work: items (batch, 128-row tile I, TN-column tile J) of nao_split_h_items; a persistent kernel
-// (one CTA per SM) walks them
-cudaError_t launch_h_tc(const DevSystem &s, const HWork *work, int32_t w0, int32_t n_work, const uint8_t *slices,
+// work: items of nao_split_h_items; a persistent kernel (one CTA per SM) walks them
+cudaError_t launch_h_tc(const DevSystem &s, const HTask *work, int32_t w0, int32_t n_work, const uint8_t *slices,
                         const int64_t *sl_off, const int32_t *expo, const int32_t *neg16, int S, int F, int tn,
                         int scatter, int32_t *err, cudaStream_t st);
-// tn_b: per-batch tile width (the P' tiles of the density follow it). grad: the scratch rows hold
+// grad: the scratch rows hold
 // [phi | grad phi] (4 Ppad) and P' = P over all tiles (density gradient)
 cudaError_t launch_slice_n(const DevSystem &s, int32_t b0, int32_t b1, int32_t max_qt, int32_t max_rt,
                            const double *scratch, uint8_t *slices, const int64_t *sl_off, const int32_t *expo_q,
-                           int32_t *expo_b, const int32_t *tn_b, int S, int F, bool grad, cudaStream_t st);
+                           int32_t *expo_b, int S, int F, bool grad, cudaStream_t st);
 // The density Hessian on the split path (passes comp = 0..3 over the 10-row FP64 evaluation at
 // hoff: A = phi, then the gradient components; P' sliced with the first pass): slicing, the
 // four A operands' point exponents (expo4[comp n_points + p]) and the contraction passes
 // (comp 0 writes n, grad n and hess; comp a adds hess_(a, b), b >= a).
 cudaError_t launch_slice_n_hess(const DevSystem &s, int32_t b0, int32_t b1, int32_t max_qt, int32_t max_rt,
                                 const double *scratch, const int64_t *hoff, int comp, uint8_t *slices,
-                                const int64_t *sl_off, const int32_t *expo_q, int32_t *expo_b, const int32_t *tn_b, int S,
-                                int F, cudaStream_t st);
+                                const int64_t *sl_off, const int32_t *expo_q, int32_t *expo_b, int S, int F, cudaStream_t st);
 cudaError_t launch_hess_point_expo(const DevSystem &s, int32_t b0, int32_t b1, const double *scratch, const int64_t *hoff,
                                    int32_t *expo4, int64_t n_points, cudaStream_t st);
 cudaError_t launch_n_tc_hess(const DevSystem &s, const HWork *work, int32_t w0, int32_t n_work, const uint8_t *slices,

@@ -97,3 +97,87 @@ void nao_spline_coefficients(const double *y, int32_t n, double *coef) {
         c[3] = (M[(size_t)k + 1] - M[(size_t)k]) / 6.0;
     }
 }
+
+// Every pair of the complete graph on n blocks goes to one of its two ends; column j takes at most
+// cap[j] = 4 m_j - 1 pairs beside its own block, with sum_j m_j items in all. m_j is the same for every
+// column but for one more in the first few, and any k columns can hold their k (k - 1) / 2 inner pairs,
+// so an assignment exists. Pairs are placed by increasing cyclic distance d at the column d before
+// (so that a column's rows are mostly consecutive), else at the other end, else by moving pairs along a
+// path of full columns to one with room.
+std::vector<std::vector<int>> nao_block_pairs(int n) {
+    const int total = std::max(n, (n * (n + 1) / 2 + 3) / 4);
+    const int m = total / n, more = total - m * n;
+    std::vector<int> room(n);
+    for (int j = 0; j < n; j++) room[j] = 4 * (m + (j < more ? 1 : 0)) - 1;
+    std::vector<int> owner((size_t)n * n, -1);  // of the pair {a, b}: at both (a, b) and (b, a)
+    auto give = [&](int a, int b, int to) { owner[(size_t)a * n + b] = owner[(size_t)b * n + a] = to; };
+    for (int d = 1; d <= n / 2; d++)
+        for (int j = 0; j < n; j++) {
+            const int o = (j + d) % n;
+            if (owner[(size_t)j * n + o] >= 0) continue;  // n even, d = n / 2: the pair's other end came first
+            // a column with room that j or o reaches by moving pairs: breadth first
+            std::vector<int> from(n, -2), queue;
+            int end = -1;
+            for (int x : {j, o}) {
+                if (from[x] != -2) continue;
+                from[x] = -1;
+                queue.push_back(x);
+            }
+            for (size_t h = 0; h < queue.size() && end < 0; h++) {
+                const int x = queue[h];
+                if (room[x] > 0) {
+                    end = x;
+                    break;
+                }
+                for (int y = 0; y < n; y++)
+                    if (y != x && from[y] == -2 && owner[(size_t)x * n + y] == x) {  // x could pass {x, y} to y
+                        from[y] = x;
+                        queue.push_back(y);
+                    }
+            }
+            if (end < 0) end = j;  // cannot happen (see above); the column then takes one item more
+            room[end]--;
+            int x = end;
+            while (from[x] >= 0) {
+                give(from[x], x, x);
+                x = from[x];
+            }
+            give(j, o, x);
+        }
+    std::vector<std::vector<int>> rows(n);
+    for (int j = 0; j < n; j++)
+        for (int d = 0; d < n; d++) {
+            const int o = (j + d) % n;
+            if (d == 0 || owner[(size_t)j * n + o] == j) rows[j].push_back(o);
+        }
+    return rows;
+}
+
+void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HTask> &out, BlockPairs &kept, int F) {
+    const int nseg = nao_split_h_nseg(P, S, F);
+    auto add = [&](int j, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+        for (int q = 0; q < nseg; q++)
+            out.push_back({b, (uint32_t)j | (uint32_t)q << 16, r0 | r1 << 16, r2 | r3 << 16});
+    };
+    const int nr = (N + 31) / 32;
+    if (TN != 32) {
+        const int nJ = (N + TN - 1) / TN;
+        for (int I = 0; 128 * I < N; I++)
+            for (int J = (I * 128) / TN; J < nJ; J++) {
+                uint32_t r[4];
+                for (int x = 0; x < 4; x++) r[x] = 4 * I + x < nr ? (uint32_t)(4 * I + x) : kNoRows;
+                add(J, r[0], r[1], r[2], r[3]);
+            }
+        return;
+    }
+    auto it = kept.find(nr);
+    if (it == kept.end()) it = kept.emplace(nr, nao_block_pairs(nr)).first;
+    for (int j = 0; j < nr; j++) {
+        const std::vector<int> &rows = it->second[j];
+        for (size_t k = 0; k < rows.size(); k += 4) {
+            uint32_t r[4];
+            for (size_t x = 0; x < 4; x++) r[x] = k + x < rows.size() ? (uint32_t)rows[k + x] : kNoRows;
+            add(j, r[0], r[1], r[2], r[3]);
+        }
+    }
+}

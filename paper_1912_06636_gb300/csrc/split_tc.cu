@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(256, S <= 10 ? 5 : 4) slice_h_kernel(DevSystem
 // per lane, one 128-byte row segment per slice). CTAs with blockIdx.y = 0 instead reduce the batch's
 // exponent of P' (the upper-triangle tile pairs, read along rows of P).
 // ----------------------------------------------------------------------------------------
-__device__ __forceinline__ int tile_of(int i, int TN) { return i / TN; }
+// The symmetry c_IJ of P' is taken between groups of GW = nao_split_tn(S, F) functions, whatever width the
+// contraction's tiles have: the digits, and so n, do not depend on the tuned width.
 
 template <typename V>
 struct StageOf {  // shared-memory staging type of the density slicer's input
@@ -377,10 +378,12 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
                                                         const int64_t *__restrict__ eoff, int coff,
                                                         uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off,
                                                         const int32_t *__restrict__ expo_q, int32_t *__restrict__ expo_b,
-                                                        const int32_t *__restrict__ tn_b, int ld_mult, int full, int pexp) {
-    constexpr int C = nao_chunk_cols(F), LC = C / 32;
+                                                        int ld_mult, int full, int pexp) {
+    constexpr int C = nao_chunk_cols(F), LC = C / 32, GW = nao_split_tn(S, F);
     using TT = typename StageOf<V>::type;
-    __shared__ TT t[32][C + 1];
+    constexpr int KS = nao_kstep_cols(F);
+    // 8 more columns per K step: the two K steps that a half-warp reads at once lie in different banks
+    __shared__ TT t[32][C + 8 * (C / KS) + 1];
     __shared__ int red[8];
     const int b = b0 + blockIdx.x;
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
@@ -393,7 +396,7 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
         if (!pexp) return;
         // max |P'_ij| over i <= j (P' is P on the diagonal tiles, 2 P off them, 0 below unless
         // full): the exponent field of |P| plus one off the diagonal tiles
-        const int m = s.sys.bmol[b], TN = tn_b[b];
+        const int m = s.sys.bmol[b];
         const int32_t *rel = s.rel_idx + s.rel_off[b];
         int mk = 0;
         for (int i = warp; i < N; i += 8) {
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
             for (int j = (full ? 0 : i) + lane; j < N; j += 32) {
                 const int64_t gj = rel[j];
                 const int eb = split_bits::biased_exponent(abs_bits(gi <= gj ? p_elem(s, m, gi, gj) : p_elem(s, m, gj, gi)));
-                if (eb != 0) mk = max(mk, eb + ((!full && tile_of(i, TN) < tile_of(j, TN)) ? 1 : 0));
+                if (eb != 0) mk = max(mk, eb + ((!full && i / GW < j / GW) ? 1 : 0));
             }
         }
         mk = __reduce_max_sync(0xffffffffu, mk);
@@ -429,20 +432,22 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
 #pragma unroll
         for (int h = 0; h < C / 8; h++) {
             const int i = kc * C + warp + 8 * h;
-            t[lane][warp + 8 * h] = (i < N && qin) ? StageOf<V>::get(E[(int64_t)i * ld + q0 + lane]) : StageOf<V>::zero();
+            const int k = warp + 8 * h;
+            t[lane][k + 8 * (k / KS)] = (i < N && qin) ? StageOf<V>::get(E[(int64_t)i * ld + q0 + lane]) : StageOf<V>::zero();
         }
         __syncthreads();
 #pragma unroll
         for (int h = 0; h < 4; h++) {
             const int ql = warp * 4 + h, q = q0 + ql;
             if (q >= G.P16) break;
-            // lane L packs functions L, L + 32 (, L + 64, L + 96) of the chunk into its word: both
-            // operands of the density's product (this A and slice_np_kernel's B) order K this way
-            // inside each chunk, which leaves every slice product unchanged and reads the staging
-            // rows without bank conflicts
+            // within each K step (KS functions, the words of 8 lanes) lane l packs functions l, l + 8
+            // (, l + 16, l + 24): both operands of the density's product (this A and
+            // slice_np_kernel's B) order K this way inside each K step, which leaves every slice
+            // product unchanged; K steps hold consecutive functions, so that n_tc_kernel can stop
+            // at a tile's last one
             TT x[LC];
 #pragma unroll
-            for (int c = 0; c < LC; c++) x[c] = t[ql][lane + 32 * c];
+            for (int c = 0; c < LC; c++) x[c] = t[ql][(KS + 8) * (lane >> 3) + (lane & 7) + 8 * c];
             uint32_t wd[S];
             lane_digit_words<S, F>(x, eq[h], wd);
             const uint32_t off = tc::sw128_byte((uint32_t)q, (uint32_t)(4 * lane));
@@ -453,25 +458,24 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
     }
 }
 
-// P'_ij = c_IJ P[rel_i][rel_j] over TN-function tiles I = i/TN <= J = j/TN (c_II = 1,
+// P'_ij = c_IJ P[rel_i][rel_j] over GW-function groups I = i/GW <= J = j/GW (c_II = 1,
 // c_IJ = 2; every (i, j) with c = 1 when full), read from P's upper triangle, with the batch's
 // exponent from slice_nphi_kernel. One CTA per (batch, 16 rows j), one warp per row, 2 or 4
-// functions i per lane (i = lane + 32 c inside the chunk; one 128-byte row segment per slice).
+// functions i per lane (slice_nphi_kernel's K order; one 128-byte row segment per slice).
 template <int S, int F>
 __global__ void __launch_bounds__(256) slice_np_kernel(DevSystem s, int32_t b0, uint8_t *__restrict__ slices,
                                                       const int64_t *__restrict__ sl_off,
-                                                      const int32_t *__restrict__ expo_b,
-                                                      const int32_t *__restrict__ tn_b, int full) {
+                                                      const int32_t *__restrict__ expo_b, int full) {
     const int b = b0 + blockIdx.x, m = s.sys.bmol[b];
     const int P = s.batch_off[b + 1] - s.batch_off[b];
     const int N = s.rel_off[b + 1] - s.rel_off[b];
     if (N == 0) return;
-    constexpr int C = nao_chunk_cols(F), LC = C / 32;
+    constexpr int C = nao_chunk_cols(F), KS = nao_kstep_cols(F), LC = C / 32, GW = nao_split_tn(S, F);
     const SplitGeom G(P, N, S, 0, F);
     const int j0 = blockIdx.y * 16;
     if (j0 >= G.R16) return;
     const int32_t *rel = s.rel_idx + s.rel_off[b];
-    const int TN = tn_b[b], e = expo_b[b];
+    const int e = expo_b[b];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *base = slices + sl_off[b];
 #pragma unroll 1
@@ -479,20 +483,20 @@ __global__ void __launch_bounds__(256) slice_np_kernel(DevSystem s, int32_t b0, 
         const int j = j0 + warp * 2 + h;  // < R16: R16 is a multiple of 16
         const bool jin = j < N;
         const int64_t gj = jin ? rel[j] : 0;
-        const int tj = tile_of(j, TN);
+        const int group = j / GW;
         for (int kc = 0; kc < G.n_kcN; kc++) {
             double xp[LC];
 #pragma unroll
             for (int hh = 0; hh < LC; hh++) {
-                const int i = C * kc + lane + 32 * hh;  // the K order of slice_nphi_kernel
+                const int i = C * kc + KS * (lane >> 3) + (lane & 7) + 8 * hh;
                 double x = 0.0;
-                if (jin && i < N && (full || tile_of(i, TN) <= tj)) {
+                if (jin && i < N && (full || i / GW <= group)) {
                     const int64_t gi = rel[i];
                     x = gi <= gj ? p_elem(s, m, gi, gj) : p_elem(s, m, gj, gi);
                     // c_IJ = 2 off the diagonal tiles: exact, as one more in the exponent field
                     // (zero and subnormal values, which give no digits, are left as they are)
                     const long long pb = __double_as_longlong(x);
-                    if (!full && tile_of(i, TN) < tj && split_bits::biased_exponent(pb) != 0)
+                    if (!full && i / GW < group && split_bits::biased_exponent(pb) != 0)
                         x = __longlong_as_double(pb + (1LL << 52));
                 }
                 xp[hh] = x;
@@ -507,16 +511,24 @@ __global__ void __launch_bounds__(256) slice_np_kernel(DevSystem s, int32_t b0, 
 }
 
 // ----------------------------------------------------------------------------------------
-// Slice-product pipeline of the persistent contraction kernels. Shared memory: a ring of
-// ring_slots(S) A-tile buffers (128 rows x 64 bf16, 16 KB, one slice of one K chunk each) and two sets of S
-// B-tile buffers (TN rows, TN x 128 B). Producer (one lane): for each K chunk, the S B slices
-// into B set kc % 2, then the S A slices one by one into the ring, each copy a single bulk
-// (TMA) transfer completing on a "full" mbarrier. MMA issuer (one lane): for each A slice s,
-// the pairs (s, t) with s + t < S as one 128 x TN(S-s) x 16 tcgen05.mma per K step (two where
-// TN(S-s) > 256) into accumulator groups s .. S-1 (tensor-memory columns TN s ...); commits
-// release A buffers and B sets back to the producer through "empty" mbarriers. The phases of
-// the ring and of the B sets continue over all the accumulations a CTA runs. Every wait is
-// bounded; on a timeout the CTA records NAO_ERR_TIMEOUT and skips the rest of its work.
+// Slice-product pipeline of the persistent contraction kernels, ten warps. Shared memory: a ring of
+// ring_slots(S) A-tile buffers (128 rows of 128 B, 16 KB, one slice of one K chunk each) and two sets
+// of S B-tile buffers (TN rows, TN x 128 B). Producer (warp 8, one lane): for each K chunk, the S B
+// slices into B set kc % 2, then the S A slices one by one into the ring, each copy a bulk (TMA)
+// transfer completing on a "full" mbarrier. MMA issuer (warp 9): for each A slice s, the pairs (s, t)
+// with s + t < S as one 128 x TN(S-s) MMA per K step (two where TN(S-s) > 256) into accumulator groups
+// s .. S-1 (tensor-memory columns TN s ...); commits release A buffers and B sets back to the producer
+// through "empty" mbarriers. Warps 0-7 read the accumulators: warp w the rows of quadrant w % 4 and half
+// w / 4 of the TN columns. The phases of the ring and of the B sets continue over all the
+// accumulations a CTA runs. Every wait is bounded; on a timeout the CTA records NAO_ERR_TIMEOUT and
+// skips the rest of its work.
+// What bounds them: an earlier form (one issuing thread, four reading warps, 64-bit integer and FP64
+// arithmetic) took 18.3 ms for H and 9.2 ms for n on a slab of 75 atoms (14 e4m3 slices); 18.0 and 9.1
+// without any copies, 15.0 and 4.4 without the readers' work, 11.8 and 3.5 with the copies alone. So the
+// MMA issue and the serial part of the readers (tensor memory holds one accumulator set) decided, not the
+// operands' supply: the issuer runs with its whole warp, so that descriptors stay in uniform registers,
+// and eight warps read with 32-bit integer and FP32 arithmetic. With the H items of nao_split_h_items and
+// the density's K in whole steps: 10.8 and 3.8 ms.
 // ----------------------------------------------------------------------------------------
 constexpr int kMaxRing = 8;
 constexpr size_t kSmemOptin = 232448;  // shared memory a CTA may opt into on this GPU (227 KB)
@@ -540,43 +552,86 @@ static_assert(pipe_smem_bytes(12, 0) + kStaticSmem <= kSmemOptin && pipe_smem_by
                   pipe_smem_bytes(16, 1) + kStaticSmem <= kSmemOptin,
               "split pipeline exceeds shared memory");
 
-// Integer recombination of the S group accumulators M_g (|M_g| < 2^24, exact) for 16 columns of
-// this thread's row, in units of 2^(e_i + e_j):
-//   bf16 (base 64): hi = sum_{g<=6} M_g 64^(6-g) [units 2^-48], lo = sum_{7<=g<=9} M_g 64^(9-g)
-//     [2^-66], lo2 = sum_{g>=10} M_g 64^(12-g) [2^-84] (S = 11, 12 only);
-//   e4m3 (base 32): hi = sum_{g<=7} M_g 32^(7-g) [units 2^-45], lo = sum_{g>=8} M_g 32^(15-g)
-//     [2^-85] (S <= 16); lo2 stays 0.
-// Every part is exact in 64 bits (below 2^60.1).
-struct Parts16 {
-    long long hi[16], lo[16], lo2[16];
-};
+// The S group accumulators M_g (exact integers, |M_g| < 2^24) of one element, neighbouring groups
+// joined in 32-bit integers P = M_g 2^B + M_(g+1) (below 2^30.1):
+//   e4m3 (base 32): P_k of groups 2k, 2k + 1, k = 0..7;
+//   bf16 (base 64): P_0..P_2 of groups (0, 1), (2, 3), (4, 5), P_3 = M_6, P_4 of (7, 8), P_5 = M_9, P_6 of
+//     (10, 11).
+// Groups g >= S count as zero.
+template <int F>
+__host__ __device__ constexpr int n_pairs() { return F == NAO_DIGITS_E4M3 ? 8 : 7; }
 
-template <int TN, int F>
-__device__ __forceinline__ void combine16(uint32_t tm_row, int c0, int S, Parts16 &v) {
-    constexpr int B = nao_digit_bits(F), GH = F == NAO_DIGITS_E4M3 ? 7 : 6, GL = F == NAO_DIGITS_E4M3 ? 15 : 9;
+// The joined integers of 8 columns of this thread's row. SMALL: every |M_g| <= 2^22, so that adding
+// 1.5 2^23 leaves the integer in the significand (one FP32 addition; the conversion instruction has a
+// quarter of its rate).
+template <int TN, int F, bool SMALL>
+__device__ __forceinline__ void read_pairs8(uint32_t tm_col, int S, int (&p)[n_pairs<F>()][8]) {
+    constexpr int B = nao_digit_bits(F), GB = F == NAO_DIGITS_E4M3 ? 8 : 6;  // groups per wait
+    constexpr int kMagic = 0x4B400000;  // 1.5 2^23
 #pragma unroll
-    for (int jj = 0; jj < 16; jj++) v.hi[jj] = v.lo[jj] = v.lo2[jj] = 0;
-    // three groups' loads in flight per wait
-    for (int g0 = 0; g0 < S; g0 += 3) {
-        uint32_t r[3][16];
+    for (int h = 0; h < 2; h++) {
+        uint32_t r[GB][8];
 #pragma unroll
-        for (int d = 0; d < 3; d++)
-            if (g0 + d < S) tc::tmem_ld16(tm_row + (uint32_t)((g0 + d) * TN + c0), r[d]);
-        tc::tmem_ld_wait();
+        for (int q = 0; q < GB; q++) {
+            const int g = h * GB + q;
+            if (g < S) {
+                tc::tmem_ld8(tm_col + (uint32_t)(g * TN), r[q]);
+            } else {
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const int g = g0 + d;
-            if (g >= S) break;
-            const int part = g <= GH ? 0 : (g <= GL ? 1 : 2);
-            const long long w = 1LL << (B * (part == 0 ? GH - g : (part == 1 ? GL - g : 12 - g)));
-#pragma unroll
-            for (int jj = 0; jj < 16; jj++) {
-                const long long m = (long long)__float2int_rn(__uint_as_float(r[d][jj]));
-                if (part == 0) v.hi[jj] += m * w;
-                else if (part == 1) v.lo[jj] += m * w;
-                else v.lo2[jj] += m * w;
+                for (int c = 0; c < 8; c++) r[q][c] = 0;
             }
         }
+        tc::tmem_ld_wait();
+        auto integer = [&](int q, int c) {
+            const float x = __uint_as_float(r[q][c]);
+            return SMALL ? __float_as_int(__fadd_rn(x, 12582912.0f)) - kMagic : __float2int_rn(x);
+        };
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            auto join = [&](int q) { return integer(q, c) * (1 << B) + integer(q + 1, c); };
+            if constexpr (F == NAO_DIGITS_E4M3) {
+#pragma unroll
+                for (int k = 0; k < 4; k++) p[4 * h + k][c] = join(2 * k);
+            } else if (h == 0) {
+                p[0][c] = join(0);
+                p[1][c] = join(2);
+                p[2][c] = join(4);
+            } else {
+                p[3][c] = integer(0, c);
+                p[4][c] = join(1);
+                p[5][c] = integer(3, c);
+                p[6][c] = join(4);
+            }
+        }
+    }
+}
+template <int TN, int F>
+__device__ __forceinline__ void read_pairs8(uint32_t tm_col, int S, bool small, int (&p)[n_pairs<F>()][8]) {
+    if (small) read_pairs8<TN, F, true>(tm_col, S, p);
+    else read_pairs8<TN, F, false>(tm_col, S, p);
+}
+// Whether an accumulation over K columns keeps every |M_g| <= K S 2^(2 B - 2) at or below 2^22.
+template <int F>
+__device__ __forceinline__ bool small_groups(int K, int S) {
+    return (long long)K * S <= (1LL << (24 - 2 * nao_digit_bits(F)));
+}
+
+// The parts of one element in units of 2^(e_i + e_j), each exact in 64 bits (below 2^60.1):
+//   bf16: hi = sum_{g<=6} M_g 64^(6-g) [units 2^-48], lo = sum_{7<=g<=9} M_g 64^(9-g) [2^-66],
+//     lo2 = sum_{g>=10} M_g 64^(12-g) [2^-84] (S = 11, 12 only);
+//   e4m3: hi = sum_{g<=7} M_g 32^(7-g) [units 2^-45], lo = sum_{g>=8} M_g 32^(15-g) [2^-85] (S <= 16);
+//     lo2 stays 0.
+template <int F>
+__device__ __forceinline__ void pair_parts(const int (&p)[n_pairs<F>()][8], int c, long long &hi, long long &lo,
+                                           long long &lo2) {
+    if constexpr (F == NAO_DIGITS_E4M3) {
+        hi = (long long)p[0][c] * (1 << 30) + ((long long)p[1][c] * (1 << 20) + ((long long)p[2][c] * (1 << 10) + p[3][c]));
+        lo = (long long)p[4][c] * (1 << 30) + ((long long)p[5][c] * (1 << 20) + ((long long)p[6][c] * (1 << 10) + p[7][c]));
+        lo2 = 0;
+    } else {
+        hi = (long long)p[0][c] * (1 << 30) + ((long long)p[1][c] * (1 << 18) + ((long long)p[2][c] * (1 << 6) + p[3][c]));
+        lo = (long long)p[4][c] * (1 << 6) + p[5][c];
+        lo2 = (long long)p[6][c] * (1 << 6);
     }
 }
 
@@ -615,108 +670,79 @@ template <int F>
 __device__ __forceinline__ int h_unit(int t) {
     return F == NAO_DIGITS_BF16 ? (t == 0 ? 66 : 50) : (t == 0 ? 85 : (t == 1 ? 67 : 47));
 }
-// A density T element as one 64-bit integer in units of 2^(e_q + e_b - n_unit<F>): 4 hi +
-// round(lo' / 2^16) (bf16, unit 50) or 4 hi + round(lo / 2^38) (e4m3, unit 47); |4 hi| < 2^62.1,
-// rounded by at most half a unit.
+// A density T element from its joined integers, as a float-float in units of 2^(e_q + e_b - n_unit<F>):
+// v + f / 2^10 with the 64-bit integer v = floor(4 hi + lo' / 2^16) (bf16; lo' = lo + lo2 / 2^18) or
+// floor(4 hi + lo / 2^38) (e4m3), |v| < 2^62.1, and the next ten bits f. v's three 21-bit pieces and f
+// become FP32s exactly. n_unit: 50 and 47 bits below, and 21 more because the float-float counts in 2^21.
 template <int F>
-__device__ __forceinline__ long long n_int(long long hi, long long lo, long long lo2) {
-    if constexpr (F == NAO_DIGITS_BF16) {
-        const long long l = lo + ((lo2 + (1LL << 17)) >> 18);
-        return (hi << 2) + ((l + (1LL << 15)) >> 16);
+__device__ __forceinline__ ffa::F pair_ff(const int (&p)[n_pairs<F>()][8], int c) {
+    long long w;
+    int r;  // lo' or lo in units of 2^-10 of v's (their part above)
+    if constexpr (F == NAO_DIGITS_E4M3) {
+        r = p[4][c] * 4 + (p[5][c] >> 8);
+        w = (long long)p[1][c] * (1 << 22) + ((long long)p[2][c] * (1 << 12) + (p[3][c] * 4 + (r >> 10)));
     } else {
-        return (hi << 2) + ((lo + (1LL << 37)) >> 38);
+        r = p[4][c] + (p[5][c] >> 6) + (p[6][c] >> 18);
+        w = (long long)p[1][c] * (1 << 20) + ((long long)p[2][c] * (1 << 8) + (p[3][c] * 4 + (r >> 10)));
     }
+    const uint32_t lo = (uint32_t)w;
+    const int hi = (int)((uint32_t)(w >> 32) + (uint32_t)p[0][c]);  // v = hi 2^32 + lo
+    auto small = [](uint32_t x) { return __fsub_rn(__uint_as_float(0x4B000000u | x), 8388608.0f); };  // x < 2^23
+    const float f2 = __fsub_rn(__int_as_float(0x4B400000 + (hi >> 10)), 12582912.0f);
+    const float f1 = small(__funnelshift_r(lo, (uint32_t)hi, 21) & 0x1FFFFFu), f0 = small(lo & 0x1FFFFFu);
+    const ffa::F a = ffa::quick(__fmul_rn(f2, 2097152.0f), f1);
+    const float low = __fmaf_rn(small((uint32_t)r & 1023u), 1.0f / 1024.0f, f0);
+    return ffa::quick(a.h, __fmaf_rn(low, 1.0f / 2097152.0f, a.l));
 }
 template <int F>
-__host__ __device__ constexpr int n_unit() { return F == NAO_DIGITS_BF16 ? 50 : 47; }
+__host__ __device__ constexpr int n_unit() { return (F == NAO_DIGITS_BF16 ? 50 : 47) - 21; }
+
+// A float-float of an FP64 from its bit pattern (the FP64 pipe's conversions would bound the Hessian's
+// epilogue): the 24 leading bits and the next 23, truncated; zero below 2^-100 (of no weight in a density).
+__device__ __forceinline__ ffa::F ff_of_bits(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu;
+    if (e < 923u || e > 1100u) return e < 923u ? ffa::F{0.0f, 0.0f} : ffa::from_double(x);
+    const uint32_t sg = hi & 0x80000000u, fe = (e - 896u) << 23;
+    const float h = __uint_as_float(sg | fe | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+    // the next 23 bits as the fraction of a number in [1, 2) 2^(E-23), E the exponent of x, less that power
+    const uint32_t base = sg | (fe - (23u << 23));
+    const float l = __fsub_rn(__uint_as_float(base | ((lo >> 6) & 0x7FFFFFu)), __uint_as_float(base));
+    return ffa::F{h, l};
+}
+__device__ __forceinline__ ffa::F ff_of_value(const FF2 &v) { return v.f(); }
+__device__ __forceinline__ ffa::F ff_of_value(double v) { return ff_of_bits(v); }
+
+// acc += a b (float-floats): the product to 2^-48, added to the unevaluated sum.
+__device__ __forceinline__ void ff_mac(ffa::F &acc, ffa::F a, ffa::F b) {
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
+    const ffa::F t = ffa::two_sum(acc.h, p);
+    acc.h = t.h;
+    acc.l = __fadd_rn(acc.l, __fadd_rn(t.l, e));
+}
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
     return reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
-// Persistent, warp-specialised H contraction: one CTA per SM walks the work items w =
-// blockIdx.x, blockIdx.x + gridDim.x, ... Warp 4 (lane 0) loads the operands into the A ring and
-// the two B sets, its phases continuing over all items; warp 5 (lane 0) issues the MMAs of one
-// item after the other into the single accumulator set; warps 0-3 (128 threads, one accumulator
-// row each) read an item's accumulators into registers, hand tensor memory back to the MMA warp
-// ("acc_empty") and then scatter into H while the next item's MMAs run, so the scatter, the
-// tensor-memory reads and the next item's first loads overlap the MMAs.
-// The B tiles t = 0 .. nb-1 of one A slice as MMA pieces: one piece of nb TN columns up to
-// N = 256, else two halves of ceil(nb / 2) and floor(nb / 2) tiles (each at most 256 columns,
-// since nb TN <= 512, the tensor memory of one accumulator set). Every piece starts on a whole
-// tile, so on a multiple of 8 rows (one 128-byte swizzle atom). Two halves, issued alternately,
-// write disjoint accumulator columns: an MMA that accumulates into the columns of the one just
-// issued waits for it (about 97 cycles at this size, against about 60 for other columns), and
-// equal halves leave no narrow piece whose fixed cost exceeds its work.
-struct MmaPieces {
-    int n, c0[2], cols[2];
-    __device__ __forceinline__ MmaPieces(int nb, int TN) {
-        if (nb * TN <= 256) {
-            n = 1;
-            c0[0] = 0;
-            cols[0] = nb * TN;
-            c0[1] = cols[1] = 0;
-        } else {
-            const int h = (nb + 1) / 2;
-            n = 2;
-            c0[0] = 0;
-            cols[0] = h * TN;
-            c0[1] = h * TN;
-            cols[1] = (nb - h) * TN;
-        }
-    }
-};
+constexpr int kReaders = 8;                        // accumulator-reading warps
+constexpr int kTcThreads = 32 * (kReaders + 2);    // and the producer and MMA warps
 
 struct PPipe {
     uint64_t fullA[kMaxRing], emptyA[kMaxRing], fullB[2], emptyB[2];
     uint64_t acc_full, acc_empty, fin;
+    uint64_t part_full[4], part_empty[4];  // n: the exchange of the two column halves' sums, per quadrant
+    double part[4][32];
     uint32_t tmem;
     int abort;
 };
+static_assert(sizeof(PPipe) <= kStaticSmem, "barriers exceed their share of shared memory");
 
-struct HItem {  // geometry of one H work item
-    const uint8_t *a0, *b0;
-    size_t blk;
-    uint32_t a_bytes, b_bytes;
-    int n_kc, kc0, kc1, neg16, b, m, N, ti, tj;  // K chunks [kc0, kc1) of the item's segment
-};
-
-template <int TN, int F>
-__device__ __forceinline__ HItem h_item(const DevSystem &s, const HWork *work, int32_t w, const uint8_t *slices,
-                                        const int64_t *sl_off, const int32_t *neg16, int S) {
-    HItem h;
-    const HWork it = work[w];
-    h.b = it.batch;
-    h.ti = it.ti;
-    h.tj = it.tj;
-    h.m = s.sys.bmol[h.b];
-    const int P = s.batch_off[h.b + 1] - s.batch_off[h.b];
-    h.N = s.rel_off[h.b + 1] - s.rel_off[h.b];
-    const SplitGeom G(P, h.N, S, TN, F);
-    const uint8_t *base = slices + sl_off[h.b];
-    h.blk = (size_t)G.R16 * 128;
-    h.a0 = base + (size_t)it.ti * 128 * 128;
-    h.b0 = base + (size_t)it.tj * TN * 128;
-    h.a_bytes = (uint32_t)min(128, G.R16 - it.ti * 128) * 128u;
-    h.b_bytes = (uint32_t)min(TN, G.R16 - it.tj * TN) * 128u;
-    h.n_kc = G.n_kc;
-    nao_split_h_seg_range(G.n_kc, nao_split_h_nseg(P, S, F), it.pad, S, h.kc0, h.kc1, F);
-    h.neg16 = neg16[h.b];
-    return h;
-}
-
-template <int TN, int F>
-__global__ void __launch_bounds__(192, 1)
-    h_tc_kernel(DevSystem s, const HWork *__restrict__ work, int32_t w0, int32_t n_work, const uint8_t *__restrict__ slices,
-                const int64_t *__restrict__ sl_off, const int32_t *__restrict__ expo,
-                const int32_t *__restrict__ neg16, int S, int scatter, int32_t *__restrict__ err) {
-    constexpr uint32_t B_BLOCK = TN * 128;
-    extern __shared__ uint8_t smem_dyn[];
-    __shared__ PPipe pp;
-    uint8_t *smem = align1024(smem_dyn);
-    const int RING = ring_slots(S, F);
-    uint8_t *sA = smem, *sB = smem + (size_t)RING * 16384;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Barriers, tensor memory; returns its base address. RING: the A ring's slots.
+__device__ __forceinline__ uint32_t pipe_setup(PPipe &pp, int RING, const int32_t *err) {
+    const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         for (int i = 0; i < RING; i++) {
             tc::mbar_init(&pp.fullA[i], 1);
@@ -726,11 +752,15 @@ __global__ void __launch_bounds__(192, 1)
             tc::mbar_init(&pp.fullB[i], 1);
             tc::mbar_init(&pp.emptyB[i], 1);
         }
+        for (int i = 0; i < 4; i++) {
+            tc::mbar_init(&pp.part_full[i], 1);
+            tc::mbar_init(&pp.part_empty[i], 1);
+        }
         tc::mbar_init(&pp.acc_full, 1);
-        tc::mbar_init(&pp.acc_empty, 4);  // one arrival per accumulator-reading warp
+        tc::mbar_init(&pp.acc_empty, kReaders);  // one arrival per accumulator-reading warp
         tc::mbar_init(&pp.fin, 1);
         tc::fence_mbar_init();
-        pp.abort = *(volatile int32_t *)err != 0 ? 1 : 0;  // a timeout earlier in this launch
+        pp.abort = *(const volatile int32_t *)err != 0 ? 1 : 0;  // a timeout earlier in this launch
     }
     __syncwarp();
     if (warp == 0) {
@@ -740,29 +770,165 @@ __global__ void __launch_bounds__(192, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tm = pp.tmem;
+    return pp.tmem;
+}
+
+// A bounded wait of a whole warp (the outcome is the same on every lane).
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, kWaitCycles));
+}
+
+// Position in the A ring: slot and the parity of its current use.
+struct RingPos {
+    int a = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int RING) {
+        if (++a == RING) {
+            a = 0;
+            ph ^= 1u;
+        }
+    }
+};
+
+// The MMAs of one K chunk: for each A slice sa the pairs (sa, t = 0 .. S-1-sa), one MMA per K step over
+// the S - sa B tiles, or, above N = 256, two halves of them (ceil and floor of (S - sa) / 2 tiles: each at
+// most 256 columns, starting on a whole tile, so on a swizzle atom), issued K step by K step so that
+// consecutive MMAs alternate between the halves' columns: an MMA that accumulates into the columns of the
+// one just issued waits for it (about 97 cycles at this size, against about 60 for other columns), and
+// equal halves leave no narrow piece whose fixed cost exceeds its work. nks: K steps of this chunk;
+// negm: bit ks set: B negated on K step ks; first: the chunk's first MMA overwrites the accumulators.
+template <int TN, int F>
+__device__ __forceinline__ bool mma_chunk(PPipe &pp, uint32_t lead, uint32_t tm, uint32_t sA, uint32_t bset, int S, int RING,
+                                          RingPos &pos, int nks, uint32_t negm, bool first) {
+    const uint64_t bd = tc::sdesc_sw128(bset);
+    for (int sa = 0; sa < S; sa++) {
+        if (!warp_wait(&pp.fullA[pos.a], pos.ph)) return false;
+        tc::fence_after_sync();
+        const uint64_t ad = tc::sdesc_sw128(sA + (uint32_t)pos.a * 16384u);
+        const uint32_t d0 = tm + (uint32_t)(sa * TN);
+        const int nb = S - sa;
+        if (nb * TN <= 256) {
+            const uint32_t id = tc::idesc_digits<F>(128, nb * TN);
+#pragma unroll
+            for (int ks = 0; ks < 4; ks++)
+                if (ks < nks)
+                    tc::mma_digits<F>(lead, d0, ad + 2 * ks, bd + 2 * ks, id | ((negm >> ks & 1u) << 14),
+                                      (first && sa == 0 && ks == 0) ? 0u : 1u);
+        } else {
+            const int h = (nb + 1) / 2;
+            const uint32_t id0 = tc::idesc_digits<F>(128, h * TN), id1 = tc::idesc_digits<F>(128, (nb - h) * TN);
+            const uint32_t d1 = d0 + (uint32_t)(h * TN);
+            const uint64_t bd1 = bd + (uint64_t)(h * TN * 128 / 16);
+#pragma unroll
+            for (int ks = 0; ks < 4; ks++)
+                if (ks < nks) {
+                    const uint32_t neg = (negm >> ks & 1u) << 14, acc = (first && sa == 0 && ks == 0) ? 0u : 1u;
+                    tc::mma_digits<F>(lead, d0, ad + 2 * ks, bd + 2 * ks, id0 | neg, acc);
+                    tc::mma_digits<F>(lead, d1, ad + 2 * ks, bd1 + 2 * ks, id1 | neg, acc);
+                }
+        }
+        tc::mma_commit(lead, &pp.emptyA[pos.a]);
+        pos.next(RING);
+    }
+    return true;
+}
+
+// The common end: the timeout, and tensor memory back (every issued MMA has completed by then).
+__device__ __forceinline__ void pipe_end(PPipe &pp, uint32_t tm, int32_t *err) {
+    if (*(volatile int *)&pp.abort && threadIdx.x == 0) atomicExch(err, (int)NAO_ERR_TIMEOUT);
+    tc::fence_before_sync();
+    __syncthreads();
+    if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(tm, 512);
+}
+
+struct HItem {  // geometry of one H work item
+    const uint8_t *base, *b0;
+    size_t blk;
+    uint32_t b_bytes;
+    int n_kc, kc0, kc1, neg16, b, m, N, tj, R16;  // K chunks [kc0, kc1) of the item's segment
+    HTask task;
+};
+
+template <int TN, int F>
+__device__ __forceinline__ HItem h_item(const DevSystem &s, const HTask *work, int32_t w, const uint8_t *slices,
+                                        const int64_t *sl_off, const int32_t *neg16, int S) {
+    HItem h;
+    const HTask it = work[w];
+    h.task = it;
+    h.b = it.batch;
+    h.tj = it.tj();
+    h.m = s.sys.bmol[h.b];
+    const int P = s.batch_off[h.b + 1] - s.batch_off[h.b];
+    h.N = s.rel_off[h.b + 1] - s.rel_off[h.b];
+    const SplitGeom G(P, h.N, S, TN, F);
+    h.R16 = G.R16;
+    h.base = slices + sl_off[h.b];
+    h.blk = (size_t)G.R16 * 128;
+    h.b0 = h.base + (size_t)h.tj * TN * 128;
+    h.b_bytes = (uint32_t)min(TN, G.R16 - h.tj * TN) * 128u;
+    h.n_kc = G.n_kc;
+    nao_split_h_seg_range(G.n_kc, nao_split_h_nseg(P, S, F), it.seg(), S, h.kc0, h.kc1, F);
+    h.neg16 = neg16[h.b];
+    return h;
+}
+
+// Persistent, warp-specialised H contraction: one CTA per SM walks the work items w =
+// blockIdx.x, blockIdx.x + gridDim.x, ... The readers take an item's accumulators into registers, hand
+// tensor memory back to the MMA warp ("acc_empty") and then scatter into H while the next item's MMAs
+// run, so the scatter and the next item's first loads overlap the MMAs. A quadrant of the readers has one
+// of the item's four row blocks.
+template <int TN, int F>
+__global__ void __launch_bounds__(kTcThreads, 1)
+    h_tc_kernel(const __grid_constant__ DevSystem s, const HTask *__restrict__ work, int32_t w0, int32_t n_work,
+                const uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off, const int32_t *__restrict__ expo,
+                const int32_t *__restrict__ neg16, int S, int scatter, int32_t *__restrict__ err) {
+    constexpr uint32_t B_BLOCK = TN * 128;
+    constexpr int HC = TN / 2, NB8 = HC / 8;  // columns per reader thread, in blocks of 8
+    extern __shared__ uint8_t smem_dyn[];
+    __shared__ PPipe pp;
+    uint8_t *smem = align1024(smem_dyn);
+    const int RING = ring_slots(S, F);
+    uint8_t *sA = smem, *sB = smem + (size_t)RING * 16384;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t tm = pipe_setup(pp, RING, err);
     volatile int *abort = &pp.abort;
 
-    if (warp == 4) {
+    if (warp == kReaders) {
         // ---- producer ----
         if (lane == 0) {
             int gk = 0;
+            RingPos pos;
+            pos.ph = 1u;  // the parity that an unused slot's "empty" barrier passes
             for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x) {
                 const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
-                const bool more = w + (int)gridDim.x < n_work;
-                HItem hn = h;
-                if (more) hn = h_item<TN, F>(s, work, w0 + w + gridDim.x, slices, sl_off, neg16, S);
-                for (int kc = h.kc0; kc < h.kc1; kc++, gk++) {
-                    // the next K chunk's slices (or the next item's first) towards L2, so that the
-                    // ring's copies come from L2
-                    if (kc + 1 < h.kc1 || more) {
-                        const HItem &hp = kc + 1 < h.kc1 ? h : hn;
-                        const int kp = kc + 1 < h.kc1 ? kc + 1 : hn.kc0;
-                        for (int t = 0; t < S; t++) {
-                            tc::bulk_prefetch_l2(hp.b0 + ((size_t)t * hp.n_kc + kp) * hp.blk, hp.b_bytes);
-                            tc::bulk_prefetch_l2(hp.a0 + ((size_t)t * hp.n_kc + kp) * hp.blk, hp.a_bytes);
+                // the A tile's row blocks as runs of consecutive ones: tile offset, source offset, bytes
+                uint32_t run_to[4], run_at[4], run_n[4], a_bytes = 0;
+                int nrun = 0;
+#pragma unroll
+                for (int x = 0; x < 4; x++) {
+                    run_to[x] = run_at[x] = run_n[x] = 0;
+                    const uint32_t r = h.task.row(x);
+                    if (r == kNoRows) continue;
+                    const uint32_t at = r * 4096u, n = (uint32_t)min(32, h.R16 - (int)r * 32) * 128u;
+                    a_bytes += n;
+                    bool joined = false;
+#pragma unroll
+                    for (int y = 0; y < 4; y++)
+                        if (y == nrun - 1 && run_at[y] + run_n[y] == at && run_to[y] + run_n[y] == x * 4096u) {
+                            run_n[y] += n;
+                            joined = true;
                         }
-                    }
+                    if (joined) continue;
+#pragma unroll
+                    for (int y = 0; y < 4; y++)
+                        if (y == nrun) {
+                            run_to[y] = x * 4096u;
+                            run_at[y] = at;
+                            run_n[y] = n;
+                        }
+                    nrun++;
+                }
+                for (int kc = h.kc0; kc < h.kc1; kc++, gk++) {
                     const int bb = gk & 1, ub = gk >> 1;
                     if (ub >= 1 && !tc::mbar_wait(&pp.emptyB[bb], (ub - 1) & 1, kWaitCycles)) { *abort = 1; break; }
                     tc::mbar_arrive_expect_tx(&pp.fullB[bb], (uint32_t)S * h.b_bytes);
@@ -770,130 +936,117 @@ __global__ void __launch_bounds__(192, 1)
                         tc::bulk_g2s(sB + ((size_t)bb * S + t) * B_BLOCK, h.b0 + ((size_t)t * h.n_kc + kc) * h.blk,
                                      h.b_bytes, &pp.fullB[bb]);
                     for (int sa = 0; sa < S; sa++) {
-                        const int idx = gk * S + sa, a = idx % RING, ua = idx / RING;
-                        if (ua >= 1 && !tc::mbar_wait(&pp.emptyA[a], (ua - 1) & 1, kWaitCycles)) { *abort = 1; break; }
-                        tc::mbar_arrive_expect_tx(&pp.fullA[a], h.a_bytes);
-                        tc::bulk_g2s(sA + (size_t)a * 16384, h.a0 + ((size_t)sa * h.n_kc + kc) * h.blk, h.a_bytes,
-                                     &pp.fullA[a]);
+                        if (!tc::mbar_wait(&pp.emptyA[pos.a], pos.ph, kWaitCycles)) { *abort = 1; break; }
+                        tc::mbar_arrive_expect_tx(&pp.fullA[pos.a], a_bytes);
+                        const uint8_t *src = h.base + ((size_t)sa * h.n_kc + kc) * h.blk;
+                        uint8_t *dst = sA + (size_t)pos.a * 16384;
+#pragma unroll
+                        for (int y = 0; y < 4; y++)
+                            if (y < nrun) tc::bulk_g2s(dst + run_to[y], src + run_at[y], run_n[y], &pp.fullA[pos.a]);
+                        pos.next(RING);
                     }
                     if (*abort) break;
                 }
             }
         }
-    } else if (warp == 5) {
-        // ---- MMA issuer ----
-        if (lane == 0) {
-            int gk = 0, t = 0;
-            for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x, t++) {
-                const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
-                // the accumulators of the previous item have been read
-                if (t >= 1 && !tc::mbar_wait(&pp.acc_empty, (t - 1) & 1, kWaitCycles)) { *abort = 1; break; }
-                tc::fence_after_sync();
-                for (int kc = h.kc0; kc < h.kc1 && !*abort; kc++, gk++) {
-                    const int bb = gk & 1, ub = gk >> 1;
-                    if (!tc::mbar_wait(&pp.fullB[bb], ub & 1, kWaitCycles)) { *abort = 1; break; }
-                    const uint8_t *bset = sB + (size_t)bb * S * B_BLOCK;
-                    const int first = kc == h.kc0 ? 0 : 1;  // the segment's first chunk overwrites the accumulators
-                    for (int sa = 0; sa < S; sa++) {
-                        const int idx = gk * S + sa, a = idx % RING, ua = idx / RING;
-                        if (!tc::mbar_wait(&pp.fullA[a], ua & 1, kWaitCycles)) { *abort = 1; break; }
-                        tc::fence_after_sync();
-                        const uint64_t ad = tc::sdesc_sw128(tc::smem_addr(sA + (size_t)a * 16384));
-                        // pairs (sa, t = 0 .. S-1-sa): one MMA per K step over the S - sa B tiles,
-                        // or two halves of them above N = 256 (mma_pieces), issued K step by K
-                        // step so that consecutive MMAs alternate between the halves' columns
-                        const MmaPieces pc(S - sa, TN);
-#pragma unroll
-                        for (int ks = 0; ks < 4; ks++) {
-                            const bool neg = kc * 4 + ks < h.neg16;
-                            const uint32_t acc = (first | sa | ks) ? 1u : 0u;
-                            for (int p = 0; p < pc.n; p++) {
-                                const uint32_t idesc = tc::idesc_digits<F>(128, pc.cols[p]);
-                                const uint64_t bd = tc::sdesc_sw128(tc::smem_addr(bset + (size_t)pc.c0[p] * 128));
-                                tc::mma_digits<F>(tm + (uint32_t)(sa * TN + pc.c0[p]), ad + 2 * ks, bd + 2 * ks,
-                                                  neg ? (idesc | (1u << 14)) : idesc, acc);
-                            }
-                        }
-                        tc::mma_commit(&pp.emptyA[a]);
-                    }
-                    tc::mma_commit(&pp.emptyB[bb]);
-                }
-                if (*abort) break;
-                tc::mma_commit(&pp.acc_full);  // this item's accumulators are complete
+        __syncwarp();
+    } else if (warp == kReaders + 1) {
+        // ---- MMA issuer (the whole warp; one lane's tcgen05 instructions take effect) ----
+        const uint32_t lead = tc::elect_one();
+        const uint32_t sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
+        int gk = 0;
+        uint32_t t = 0;
+        RingPos pos;
+        bool ok = __all_sync(0xffffffffu, *abort == 0);
+        for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, t++) {
+            const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
+            // the accumulators of the previous item have been read
+            if (t >= 1) ok = warp_wait(&pp.acc_empty, (t - 1) & 1u);
+            tc::fence_after_sync();
+            for (int kc = h.kc0; kc < h.kc1 && ok; kc++, gk++) {
+                const int bb = gk & 1;
+                ok = warp_wait(&pp.fullB[bb], (uint32_t)(gk >> 1) & 1u);
+                if (!ok) break;
+                const int nn = min(max(h.neg16 - kc * 4, 0), 4);  // negated K steps of this chunk
+                ok = mma_chunk<TN, F>(pp, lead, tm, sA_addr, sB_addr + (uint32_t)bb * S * B_BLOCK, S, RING, pos, 4,
+                                      (1u << nn) - 1u, kc == h.kc0);
+                if (ok) tc::mma_commit(lead, &pp.emptyB[bb]);
             }
-            // every issued MMA has completed before tensor memory is released
-            tc::mma_commit(&pp.fin);
-            if (!tc::mbar_wait(&pp.fin, 0, kWaitCycles)) *abort = 1;
+            if (ok) tc::mma_commit(lead, &pp.acc_full);  // this item's accumulators are complete
+            ok = ok && __all_sync(0xffffffffu, *abort == 0);
         }
+        if (!ok && lane == 0) *abort = 1;
+        // every issued MMA has completed before tensor memory is released
+        tc::mma_commit(lead, &pp.fin);
+        if (!warp_wait(&pp.fin, 0) && lane == 0) *abort = 1;
     } else {
-        // ---- accumulator readers and scatter (warps 0-3) ----
-        int t = 0;
-        const uint32_t tm_row = tm + ((uint32_t)(warp * 32) << 16);
+        // ---- accumulator readers and scatter ----
+        uint32_t t = 0;
+        const int quad = warp & 3, half = warp >> 2;
+        const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HC);
         for (int w = blockIdx.x; w < n_work; w += gridDim.x, t++) {
             const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
-            if (*abort || !tc::mbar_wait(&pp.acc_full, t & 1, kWaitCycles)) { *abort = 1; break; }
-            tc::fence_after_sync();
-            const int i = h.ti * 128 + warp * 32 + lane;
-            const bool row_ok = i < h.N;
+            const uint32_t rb = h.task.row(quad);
+            const int i = (int)rb * 32 + lane;
+            const bool row_ok = rb != kNoRows && i < h.N;
             const int32_t *rel = s.rel_idx + s.rel_off[h.b];
             const int32_t *ex = expo + s.rel_off[h.b];
             const int ei = row_ok ? ex[i] : -10000;
-            // h_ij as one 64-bit integer v and a tier t (h_int: exact where the high part is
-            // small, else relative error <= 2^-43), formed before tensor memory is handed back;
-            // the conversion and the product by 2^(e_i + e_j - h_unit(t)) after.
-            long long val[TN];
-            uint64_t t1_mask = 0, t2_mask = 0;
+            const int64_t gi = row_ok ? rel[i] : 0;
+            if (*abort || !tc::mbar_wait(&pp.acc_full, t & 1u, kWaitCycles)) *abort = 1;
+            if (__any_sync(0xffffffffu, *abort != 0)) break;
+            tc::fence_after_sync();
+            int p[NB8][n_pairs<F>()][8];
+            if (rb != kNoRows) {
+                const bool small = small_groups<F>((h.kc1 - h.kc0) * nao_chunk_cols(F), S);
 #pragma unroll
-            for (int c0 = 0; c0 < TN; c0 += 16) {
-                Parts16 v;
-                combine16<TN, F>(tm_row, c0, S, v);
-#pragma unroll
-                for (int jj = 0; jj < 16; jj++) {
-                    int t;
-                    val[c0 + jj] = h_int<F>(v.hi[jj], v.lo[jj], v.lo2[jj], t);
-                    t1_mask |= (uint64_t)(t == 1) << (c0 + jj);
-                    t2_mask |= (uint64_t)(t == 2) << (c0 + jj);
-                }
+                for (int c8 = 0; c8 < NB8; c8++) read_pairs8<TN, F>(tm_row + 8 * c8, S, small, p[c8]);
             }
             // tensor memory is free for the next item
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&pp.acc_empty);
             if (scatter && row_ok) {
-                const int64_t gi = rel[i];
+                // 48-wide tiles lie on or above the diagonal; the 32-wide ones are whole blocks off it
+                // (either triangle) and the upper triangle on it
+                const bool whole = TN == 32 && (int)rb != h.tj;
 #pragma unroll
-                for (int jj = 0; jj < TN; jj++) {
-                    const int j = h.tj * TN + jj;
-                    if (j < h.N && j >= i) {
+                for (int c8 = 0; c8 < NB8; c8++)
+#pragma unroll
+                    for (int c = 0; c < 8; c++) {
+                        const int j = h.tj * TN + half * HC + 8 * c8 + c;
+                        if (j >= h.N || (!whole && j < i)) continue;
                         const int ej = ex[j];
-                        const int t = ((t1_mask >> jj) & 1) ? 1 : (((t2_mask >> jj) & 1) ? 2 : 0);
-                        const double x = (ei > -10000 && ej > -10000) ? (double)val[jj] * pow2(ei + ej - h_unit<F>(t)) : 0.0;
-                        h_add(s, h.m, gi, rel[j], x);
+                        long long hi, lo, lo2;
+                        pair_parts<F>(p[c8], c, hi, lo, lo2);
+                        int tier;
+                        const long long v = h_int<F>(hi, lo, lo2, tier);
+                        const double x = (ei > -10000 && ej > -10000) ? (double)v * pow2(ei + ej - h_unit<F>(tier)) : 0.0;
+                        const int64_t gj = rel[j];
+                        h_add(s, h.m, gi < gj ? gi : gj, gi < gj ? gj : gi, x);
                     }
-                }
             }
+            __syncwarp();
         }
     }
-    if (*abort && threadIdx.x == 0) atomicExch(err, (int)NAO_ERR_TIMEOUT);
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tm, 512);
+    pipe_end(pp, tm, err);
 }
 
 // Density contraction, persistent and warp-specialised as h_tc_kernel: one CTA per SM walks
 // the work items (batch, 128-point tile, nJ TN-function tiles) w = blockIdx.x, blockIdx.x +
 // gridDim.x, ...; each item is nJ accumulations T_qJ = Phi_q P'_J (K = the functions up to
-// tile J, where P' is nonzero), one after another through the single accumulator set. Warps
-// 0-3 (one point each) read tile J's accumulators, hand tensor memory back and then add
-// sum_j T_qj phi_qj to the point's n in registers while tile J+1's MMAs run; after the last
-// tile they store n (no atomics: one item owns each point).
+// tile J's group, where P' is nonzero, in whole K steps), one after another through the single accumulator set.
+// The readers take tile J's accumulators, hand tensor memory back and then add sum_j T_qj phi_qj to
+// the point's sums in registers while tile J+1's MMAs run (products and their sums over eight functions
+// as float-floats: on the FP64 pipe, two lanes per clock, this took longer than the MMAs); after the last tile the two column halves are added and
+// stored (no atomics: one item owns each point).
 // GRADN (density gradient, Sec. 2): P' = P over all of K, and the epilogue also forms
 // grad n_q = 2 sum_j T_qj grad phi_qj from the rows [phi | grad phi] of 4 Ppad.
 struct NItem {  // geometry of one density work item
     const uint8_t *a0, *b0;  // A: slice 0, chunk 0 of the point tile; B: slice 0, chunk 0, tile 0
     size_t a_s, a_kc, b_s, b_kc;
     uint32_t a_bytes;
-    int nJ, n_kcN, R16, b, m, p0, P, Ppad, N, ti;
+    int nJ, n_ks, R16, b, m, p0, P, Ppad, N, ti;  // n_ks: K steps of all functions
 };
 
 template <int TN, int F>
@@ -918,18 +1071,19 @@ __device__ __forceinline__ NItem n_item(const DevSystem &s, const HWork *work, i
     h.b_s = (size_t)G.n_kcN * G.R16 * 128;
     h.b_kc = (size_t)G.R16 * 128;
     h.a_bytes = (uint32_t)min(128, G.P16 - it.ti * 128) * 128u;
-    h.n_kcN = G.n_kcN;
+    constexpr int KS = nao_kstep_cols(F);
+    h.n_ks = (h.N + KS - 1) / KS;
     h.R16 = G.R16;
     return h;
 }
 
-// K chunks of tile J: P' is zero for basis functions beyond tile J, so K stops at TN (J + 1)
+// K steps of tile J: P' is zero for basis functions beyond the GW-function group of the tile's last one
 // (all of K for GRADN)
 template <int TN, bool GRADN, int F>
-__device__ __forceinline__ int n_item_kc(const NItem &h, int J) {
-    constexpr int C = nao_chunk_cols(F);
-    const int nk = GRADN ? h.n_kcN : ((J + 1) * TN + C - 1) / C;
-    return nk < h.n_kcN ? nk : h.n_kcN;
+__device__ __forceinline__ int n_item_ks(const NItem &h, int J, int S) {
+    constexpr int KS = nao_kstep_cols(F);
+    const int GW = nao_split_tn(S, F);
+    return GRADN ? h.n_ks : min(h.n_ks, (((J + 1) * TN + GW - 1) / GW * GW + KS - 1) / KS);
 }
 
 // MODE 0: n; 1: n and grad n (GRADN); 2: the density Hessian's first pass (A = Phi: n, grad n and
@@ -937,72 +1091,41 @@ __device__ __forceinline__ int n_item_kc(const NItem &h, int J) {
 // 2 sum_j T_qj d_b phi_qj for b >= hc). Modes 0, 1 read the float-float evaluation at scr_off,
 // modes 2, 3 the Hessian's 10-row FP64 evaluation at eoff.
 template <int TN, int MODE, int F>
-__global__ void __launch_bounds__(192, 1)
-    n_tc_kernel(DevSystem s, const HWork *__restrict__ work, int32_t w0, int32_t n_work, const uint8_t *__restrict__ slices,
-                const int64_t *__restrict__ sl_off, const int32_t *__restrict__ expo_q,
+__global__ void __launch_bounds__(kTcThreads, 1)
+    n_tc_kernel(const __grid_constant__ DevSystem s, const HWork *__restrict__ work, int32_t w0, int32_t n_work,
+                const uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off, const int32_t *__restrict__ expo_q,
                 const int32_t *__restrict__ expo_b, const void *__restrict__ scratch_v,
                 const int64_t *__restrict__ eoff, int S, int hc, double *__restrict__ hess,
                 int32_t *__restrict__ err) {
     constexpr bool GRADN = MODE >= 1;  // P' over all of K
+    constexpr int NC = MODE == 0 ? 1 : (MODE == 1 ? 4 : (MODE == 2 ? 10 : 3));  // sums per point
+    constexpr int R0 = MODE == 3 ? 1 : 0;  // the first row of the evaluation that they take
     using V = typename std::conditional<(MODE >= 2), double, FF2>::type;
     const V *scratch = static_cast<const V *>(scratch_v);
     constexpr uint32_t B_BLOCK = TN * 128;
+    constexpr int HC = TN / 2, NB8 = HC / 8;
     extern __shared__ uint8_t smem_dyn[];
     __shared__ PPipe pp;
     uint8_t *smem = align1024(smem_dyn);
     const int RING = ring_slots(S, F);
     uint8_t *sA = smem, *sB = smem + (size_t)RING * 16384;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < RING; i++) {
-            tc::mbar_init(&pp.fullA[i], 1);
-            tc::mbar_init(&pp.emptyA[i], 1);
-        }
-        for (int i = 0; i < 2; i++) {
-            tc::mbar_init(&pp.fullB[i], 1);
-            tc::mbar_init(&pp.emptyB[i], 1);
-        }
-        tc::mbar_init(&pp.acc_full, 1);
-        tc::mbar_init(&pp.acc_empty, 4);  // one arrival per accumulator-reading warp
-        tc::mbar_init(&pp.fin, 1);
-        tc::fence_mbar_init();
-        pp.abort = *(volatile int32_t *)err != 0 ? 1 : 0;  // a timeout earlier in this launch
-    }
-    __syncwarp();
-    if (warp == 0) {
-        tc::tmem_alloc(&pp.tmem, 512);
-        tc::tmem_relinquish();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tm = pp.tmem;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t tm = pipe_setup(pp, RING, err);
     volatile int *abort = &pp.abort;
 
-    if (warp == 4) {
+    if (warp == kReaders) {
         // ---- producer ----
         if (lane == 0) {
             int gk = 0;
+            RingPos pos;
+            pos.ph = 1u;
             for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x) {
                 const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
                 for (int J = 0; J < h.nJ && !*abort; J++) {
-                    const int nk = n_item_kc<TN, (MODE >= 1), F>(h, J);
+                    const int nk = (n_item_ks<TN, GRADN, F>(h, J, S) + 3) / 4;
                     const uint8_t *bJ = h.b0 + (size_t)J * TN * 128;
                     const uint32_t b_bytes = (uint32_t)min(TN, h.R16 - J * TN) * 128u;
                     for (int kc = 0; kc < nk; kc++, gk++) {
-                        // the next K chunk of this tile (or the next tile's first) towards L2
-                        {
-                            const bool same = kc + 1 < nk;
-                            const int Jp = same ? J : J + 1, kp = same ? kc + 1 : 0;
-                            if (Jp < h.nJ) {
-                                const uint8_t *bp = h.b0 + (size_t)Jp * TN * 128;
-                                const uint32_t bpb = (uint32_t)min(TN, h.R16 - Jp * TN) * 128u;
-                                for (int t = 0; t < S; t++) {
-                                    tc::bulk_prefetch_l2(bp + t * h.b_s + kp * h.b_kc, bpb);
-                                    tc::bulk_prefetch_l2(h.a0 + t * h.a_s + kp * h.a_kc, h.a_bytes);
-                                }
-                            }
-                        }
                         const int bb = gk & 1, ub = gk >> 1;
                         if (ub >= 1 && !tc::mbar_wait(&pp.emptyB[bb], (ub - 1) & 1, kWaitCycles)) { *abort = 1; break; }
                         tc::mbar_arrive_expect_tx(&pp.fullB[bb], (uint32_t)S * b_bytes);
@@ -1010,150 +1133,169 @@ __global__ void __launch_bounds__(192, 1)
                             tc::bulk_g2s(sB + ((size_t)bb * S + t) * B_BLOCK, bJ + t * h.b_s + kc * h.b_kc, b_bytes,
                                          &pp.fullB[bb]);
                         for (int sa = 0; sa < S; sa++) {
-                            const int idx = gk * S + sa, a = idx % RING, ua = idx / RING;
-                            if (ua >= 1 && !tc::mbar_wait(&pp.emptyA[a], (ua - 1) & 1, kWaitCycles)) { *abort = 1; break; }
-                            tc::mbar_arrive_expect_tx(&pp.fullA[a], h.a_bytes);
-                            tc::bulk_g2s(sA + (size_t)a * 16384, h.a0 + sa * h.a_s + kc * h.a_kc, h.a_bytes, &pp.fullA[a]);
+                            if (!tc::mbar_wait(&pp.emptyA[pos.a], pos.ph, kWaitCycles)) { *abort = 1; break; }
+                            tc::mbar_arrive_expect_tx(&pp.fullA[pos.a], h.a_bytes);
+                            tc::bulk_g2s(sA + (size_t)pos.a * 16384, h.a0 + sa * h.a_s + kc * h.a_kc, h.a_bytes,
+                                         &pp.fullA[pos.a]);
+                            pos.next(RING);
                         }
                         if (*abort) break;
                     }
                 }
             }
         }
-    } else if (warp == 5) {
+        __syncwarp();
+    } else if (warp == kReaders + 1) {
         // ---- MMA issuer ----
-        if (lane == 0) {
-            int gk = 0, t = 0;
-            for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x) {
-                const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
-                for (int J = 0; J < h.nJ && !*abort; J++, t++) {
-                    const int nk = n_item_kc<TN, (MODE >= 1), F>(h, J);
-                    // the accumulators of the previous tile have been read
-                    if (t >= 1 && !tc::mbar_wait(&pp.acc_empty, (t - 1) & 1, kWaitCycles)) { *abort = 1; break; }
-                    tc::fence_after_sync();
-                    for (int kc = 0; kc < nk && !*abort; kc++, gk++) {
-                        const int bb = gk & 1, ub = gk >> 1;
-                        if (!tc::mbar_wait(&pp.fullB[bb], ub & 1, kWaitCycles)) { *abort = 1; break; }
-                        const uint8_t *bset = sB + (size_t)bb * S * B_BLOCK;
-                        for (int sa = 0; sa < S; sa++) {
-                            const int idx = gk * S + sa, a = idx % RING, ua = idx / RING;
-                            if (!tc::mbar_wait(&pp.fullA[a], ua & 1, kWaitCycles)) { *abort = 1; break; }
-                            tc::fence_after_sync();
-                            const uint64_t ad = tc::sdesc_sw128(tc::smem_addr(sA + (size_t)a * 16384));
-                            // pairs (sa, t = 0 .. S-1-sa), issued as in h_tc_kernel
-                            const MmaPieces pc(S - sa, TN);
-#pragma unroll
-                            for (int ks = 0; ks < 4; ks++) {
-                                const uint32_t acc = (kc | sa | ks) ? 1u : 0u;
-                                for (int p = 0; p < pc.n; p++) {
-                                    const uint32_t idesc = tc::idesc_digits<F>(128, pc.cols[p]);
-                                    const uint64_t bd = tc::sdesc_sw128(tc::smem_addr(bset + (size_t)pc.c0[p] * 128));
-                                    tc::mma_digits<F>(tm + (uint32_t)(sa * TN + pc.c0[p]), ad + 2 * ks, bd + 2 * ks, idesc,
-                                                      acc);
-                                }
-                            }
-                            tc::mma_commit(&pp.emptyA[a]);
-                        }
-                        tc::mma_commit(&pp.emptyB[bb]);
-                    }
-                    if (*abort) break;
-                    tc::mma_commit(&pp.acc_full);  // tile J's accumulators are complete
-                }
-            }
-            // every issued MMA has completed before tensor memory is released
-            tc::mma_commit(&pp.fin);
-            if (!tc::mbar_wait(&pp.fin, 0, kWaitCycles)) *abort = 1;
-        }
-    } else {
-        // ---- accumulator readers and the n epilogue (warps 0-3) ----
-        int t = 0;
-        const uint32_t tm_row = tm + ((uint32_t)(warp * 32) << 16);
-        for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x) {
+        const uint32_t lead = tc::elect_one();
+        const uint32_t sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
+        int gk = 0;
+        uint32_t t = 0;
+        RingPos pos;
+        bool ok = __all_sync(0xffffffffu, *abort == 0);
+        for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
             const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
-            const int q = h.ti * 128 + warp * 32 + lane;
-            const bool row_ok = q < h.P;
-            const V *E = scratch + eoff[h.b];
-            const int64_t ld = MODE >= 2 ? 10 * (int64_t)h.Ppad : (GRADN ? 4 * (int64_t)h.Ppad : (int64_t)h.Ppad);
-            // sum_j T_qj phi_qj (and grad phi) in units of 2^(e_q + e_b - n_unit): each T_qj as one
-            // 64-bit integer in those units (n_int: 2^-50 with bf16 digits, 2^-47 with e4m3),
-            // rounded by at most half a unit: about the split's own truncation at 10 bf16 slices
-            // (the dropped groups g >= S reach K (S + 1) 2^(e_q + e_b - 6S - 2)) and below the FP64
-            // evaluation's rounding in n. Then one conversion and one FMA per product, all integer
-            // work done before tensor memory is handed back (no FP64 arithmetic on that path).
-            double part = 0.0, gpart[3] = {0.0, 0.0, 0.0}, hpart[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            for (int J = 0; J < h.nJ; J++, t++) {
-                if (*abort || !tc::mbar_wait(&pp.acc_full, t & 1, kWaitCycles)) { *abort = 1; break; }
+            for (int J = 0; J < h.nJ && ok; J++, t++) {
+                const int ks = n_item_ks<TN, GRADN, F>(h, J, S);
+                // the accumulators of the previous tile have been read
+                if (t >= 1) ok = warp_wait(&pp.acc_empty, (t - 1) & 1u);
                 tc::fence_after_sync();
-                long long val[TN];
-#pragma unroll
-                for (int c0 = 0; c0 < TN; c0 += 16) {
-                    Parts16 v;
-                    combine16<TN, F>(tm_row, c0, S, v);
-#pragma unroll
-                    for (int jj = 0; jj < 16; jj++) val[c0 + jj] = n_int<F>(v.hi[jj], v.lo[jj], v.lo2[jj]);
+                for (int kc = 0; 4 * kc < ks && ok; kc++, gk++) {
+                    const int bb = gk & 1;
+                    ok = warp_wait(&pp.fullB[bb], (uint32_t)(gk >> 1) & 1u);
+                    if (!ok) break;
+                    ok = mma_chunk<TN, F>(pp, lead, tm, sA_addr, sB_addr + (uint32_t)bb * S * B_BLOCK, S, RING, pos,
+                                          min(4, ks - 4 * kc), 0u, kc == 0);
+                    if (ok) tc::mma_commit(lead, &pp.emptyB[bb]);
                 }
+                if (ok) tc::mma_commit(lead, &pp.acc_full);  // tile J's accumulators are complete
+                ok = ok && __all_sync(0xffffffffu, *abort == 0);
+            }
+        }
+        if (!ok && lane == 0) *abort = 1;
+        // every issued MMA has completed before tensor memory is released
+        tc::mma_commit(lead, &pp.fin);
+        if (!warp_wait(&pp.fin, 0) && lane == 0) *abort = 1;
+    } else {
+        // ---- accumulator readers and the n epilogue ----
+        uint32_t t = 0, x = 0;  // accumulations read, exchanges made
+        const int quad = warp & 3, half = warp >> 2;
+        const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HC);
+        bool ok = true;
+        for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
+            const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
+            const int q = h.ti * 128 + quad * 32 + lane;
+            const bool row_ok = q < h.P;
+            const bool any_row = h.ti * 128 + quad * 32 < h.P;
+            const int64_t ld = MODE >= 2 ? 10 * (int64_t)h.Ppad : (GRADN ? 4 * (int64_t)h.Ppad : (int64_t)h.Ppad);
+            const V *E = scratch + eoff[h.b] + (int64_t)R0 * h.Ppad + (row_ok ? q : 0);
+            const bool small = small_groups<F>(h.n_ks * nao_kstep_cols(F), S);
+            double tot[NC];
+#pragma unroll
+            for (int d = 0; d < NC; d++) tot[d] = 0.0;
+            for (int J = 0; J < h.nJ && ok; J++, t++) {
+                const int j0 = J * TN + half * HC, jn = min(HC, h.N - j0);
+                // this tile's rows of phi towards L2 while its MMAs run
+                if (row_ok)
+                    for (int jj = 0; jj < jn; jj++) asm volatile("prefetch.global.L2 [%0];" ::"l"(E + (j0 + jj) * ld));
+                if (*abort || !tc::mbar_wait(&pp.acc_full, t & 1u, kWaitCycles)) *abort = 1;
+                if (__any_sync(0xffffffffu, *abort != 0)) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after_sync();
+                // the joined integers of all columns before tensor memory is handed back, the float-floats
+                // after; beside several sums, or with 24 columns, the integers do not fit in registers
+                // and become float-floats at once
+                constexpr bool NOW = NB8 > 2 || NC > 1;
+                ffa::F tv[HC];
+                int p[NB8][n_pairs<F>()][8];
+                if (any_row)
+#pragma unroll
+                    for (int c8 = 0; c8 < NB8; c8++) {
+                        read_pairs8<TN, F>(tm_row + 8 * c8, S, small, p[c8]);
+                        if (NOW)
+#pragma unroll
+                            for (int c = 0; c < 8; c++) tv[8 * c8 + c] = pair_ff<F>(p[c8], c);
+                    }
                 // tensor memory is free for the next tile
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&pp.acc_empty);
+                if (any_row && !NOW)
+#pragma unroll
+                    for (int c = 0; c < HC; c++) tv[c] = pair_ff<F>(p[c / 8], c % 8);
                 if (row_ok) {
-                    // the next tile's rows of phi towards L2 while this tile's products run
-                    if (J + 1 < h.nJ) {
-                        const V *fn = E + (int64_t)(J + 1) * TN * ld + q;
-                        const int jn1 = min(TN, h.N - (J + 1) * TN);
-                        for (int jj = 0; jj < jn1; jj++) asm volatile("prefetch.global.L2 [%0];" ::"l"(fn + jj * ld));
-                    }
-                    const int jn = min(TN, h.N - J * TN);
-                    const V *f = E + (int64_t)J * TN * ld + q;
+                    const V *f = E + (int64_t)j0 * ld;
+                    // eight columns' products are summed as float-floats, and these in FP64
+                    constexpr int CB = NC == 1 ? 8 : (NC <= 4 ? 4 : 2);  // columns whose loads are in flight together
 #pragma unroll
-                    for (int jj = 0; jj < TN; jj++) {
-                        if (jj < jn) {
-                            const double vj = (double)val[jj];
-                            const V *fj = f + jj * ld;
-                            if (MODE <= 2) part = fma(vj, double(fj[0]), part);
-                            if (MODE == 1 || MODE == 2)
+                    for (int c8 = 0; c8 < HC; c8 += 8) {
+                        ffa::F sum[NC];
 #pragma unroll
-                                for (int d = 0; d < 3; d++) gpart[d] = fma(vj, double(fj[(d + 1) * h.Ppad]), gpart[d]);
-                            if (MODE == 2)
+                        for (int d = 0; d < NC; d++) sum[d] = ffa::F{0.0f, 0.0f};
 #pragma unroll
-                                for (int k = 0; k < 6; k++) hpart[k] = fma(vj, double(fj[(4 + k) * h.Ppad]), hpart[k]);
-                            if (MODE == 3)  // T^hc_qj d_b phi_qj, b = 1..3 in hpart[b - 1]
+                        for (int c = c8; c < c8 + 8; c += CB) {
+                            V fv[CB][NC];
 #pragma unroll
-                                for (int d = 0; d < 3; d++) hpart[d] = fma(vj, double(fj[(d + 1) * h.Ppad]), hpart[d]);
+                            for (int y = 0; y < CB; y++)
+#pragma unroll
+                                for (int d = 0; d < NC; d++) fv[y][d] = c + y < jn ? f[(c + y) * ld + d * h.Ppad] : V(0);
+#pragma unroll
+                            for (int y = 0; y < CB; y++)
+#pragma unroll
+                                for (int d = 0; d < NC; d++)
+                                    if (c + y < jn) ff_mac(sum[d], tv[c + y], ff_of_value(fv[y][d]));
                         }
+#pragma unroll
+                        for (int d = 0; d < NC; d++) tot[d] += __dadd_rn(ffa::widen(sum[d].h), ffa::widen(sum[d].l));
                     }
                 }
+                __syncwarp();
             }
-            if (*abort) break;
-            if (row_ok) {
+            if (!ok) break;
+            // the second half's sums to the first half's warp of the quadrant, one after another
+#pragma unroll
+            for (int d = 0; d < NC; d++, x++) {
+                if (half == 1) {
+                    if (!tc::mbar_wait(&pp.part_empty[quad], (x & 1u) ^ 1u, kWaitCycles)) *abort = 1;
+                    pp.part[quad][lane] = tot[d];
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&pp.part_full[quad]);
+                } else {
+                    if (!tc::mbar_wait(&pp.part_full[quad], x & 1u, kWaitCycles)) *abort = 1;
+                    tot[d] += pp.part[quad][lane];
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&pp.part_empty[quad]);
+                }
+            }
+            if (__any_sync(0xffffffffu, *abort != 0)) break;
+            if (half == 0 && row_ok) {
                 const int eq = expo_q[h.p0 + q], eb = expo_b[h.b];
                 const bool live = eq > -10000 && eb > -10000;
                 const double sc = pow2(eq + eb - n_unit<F>());
-                if (MODE <= 2) *n_at(s, h.m, h.p0 + q) = live ? part * sc : 0.0;
+                if (MODE <= 2) *n_at(s, h.m, h.p0 + q) = live ? tot[0] * sc : 0.0;
                 if (MODE == 1 || MODE == 2)
 #pragma unroll
-                    for (int d = 0; d < 3; d++) *gn_at(s, h.m, h.p0 + q, d) = live ? 2.0 * gpart[d] * sc : 0.0;
+                    for (int d = 0; d < 3; d++) *gn_at(s, h.m, h.p0 + q, d) = live ? 2.0 * tot[NC > 3 ? 1 + d : 0] * sc : 0.0;
                 if (MODE >= 2) {
                     // hess: component-major (xx, xy, xz, yy, yz, zz), the system's original point order
                     const int64_t np = s.sys.np[h.m], o = s.perm[h.p0 + q] - s.sys.poff[h.m];
                     if (MODE == 2) {
 #pragma unroll
-                        for (int k = 0; k < 6; k++) hess[k * np + o] = live ? 2.0 * hpart[k] * sc : 0.0;
+                        for (int k = 0; k < 6; k++) hess[k * np + o] = live ? 2.0 * tot[NC > 9 ? 4 + k : 0] * sc : 0.0;
                     } else {
                         // pair (hc, b) of components 1..3 -> 0, 1, 2 (x.), 3, 4 (y.), 5 (zz)
                         const int kb = (hc - 1) * 3 - ((hc - 1) * (hc - 2)) / 2 - hc;
 #pragma unroll
                         for (int d = 0; d < 3; d++)
-                            if (d + 1 >= hc && live) hess[(kb + d + 1) * np + o] += 2.0 * hpart[d] * sc;
+                            if (d + 1 >= hc && live) hess[(kb + d + 1) * np + o] += 2.0 * tot[NC > 2 ? d : 0] * sc;
                     }
                 }
             }
         }
     }
-    if (*abort && threadIdx.x == 0) atomicExch(err, (int)NAO_ERR_TIMEOUT);
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tm, 512);
+    pipe_end(pp, tm, err);
 }
 
 // sum over each density tile of 64 points of w n (then the deterministic final reduction)
@@ -1284,18 +1426,18 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
     return cudaGetLastError();
 }
 
-cudaError_t launch_h_tc(const DevSystem &s, const HWork *work, int32_t w0, int32_t n_work, const uint8_t *slices,
+cudaError_t launch_h_tc(const DevSystem &s, const HTask *work, int32_t w0, int32_t n_work, const uint8_t *slices,
                         const int64_t *sl_off, const int32_t *expo, const int32_t *neg16, int S, int F, int tn,
                         int scatter, int32_t *err, cudaStream_t st) {
     if (n_work <= 0) return cudaSuccess;
     const int grid = n_work < sm_count() ? n_work : sm_count();  // persistent: one CTA per SM
     const size_t sm = split_smem_bytes(S, F);
     if (F == NAO_DIGITS_E4M3 && tn == 32)
-        h_tc_kernel<32, 1><<<grid, 192, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
+        h_tc_kernel<32, 1><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
     else if (F == NAO_DIGITS_BF16 && tn == 48 && S <= 10)
-        h_tc_kernel<48, 0><<<grid, 192, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
+        h_tc_kernel<48, 0><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
     else if (F == NAO_DIGITS_BF16 && tn == 32)
-        h_tc_kernel<32, 0><<<grid, 192, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
+        h_tc_kernel<32, 0><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
@@ -1303,20 +1445,20 @@ cudaError_t launch_h_tc(const DevSystem &s, const HWork *work, int32_t w0, int32
 
 cudaError_t launch_slice_n(const DevSystem &s, int32_t b0, int32_t b1, int32_t max_qt, int32_t max_rt,
                            const double *scratch, uint8_t *slices, const int64_t *sl_off, const int32_t *expo_q,
-                           int32_t *expo_b, const int32_t *tn_b, int S, int F, bool grad, cudaStream_t st) {
+                           int32_t *expo_b, int S, int F, bool grad, cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
     const FF2 *ev = reinterpret_cast<const FF2 *>(scratch);
     // y = 0: the exponent of P'; y >= 1: 32-point tiles (128 max_qt >= P16)
 #define NAO_SLICE_NPHI(SS, FF)                                                                            \
     slice_nphi_kernel<SS, FF, FF2><<<dim3(b1 - b0, 4 * max_qt + 1), 256, 0, st>>>(                        \
-        s, b0, ev, s.scr_off, 0, slices, sl_off, expo_q, expo_b, tn_b, grad ? 4 : 1, grad ? 1 : 0, 1)
+        s, b0, ev, s.scr_off, 0, slices, sl_off, expo_q, expo_b, grad ? 4 : 1, grad ? 1 : 0, 1)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NPHI)
 #undef NAO_SLICE_NPHI
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || max_rt <= 0) return e;
     // 16 rows per CTA (64 max_rt >= R16)
 #define NAO_SLICE_NP(SS, FF) \
-    slice_np_kernel<SS, FF><<<dim3(b1 - b0, 4 * max_rt), 256, 0, st>>>(s, b0, slices, sl_off, expo_b, tn_b, grad ? 1 : 0)
+    slice_np_kernel<SS, FF><<<dim3(b1 - b0, 4 * max_rt), 256, 0, st>>>(s, b0, slices, sl_off, expo_b, grad ? 1 : 0)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NP)
 #undef NAO_SLICE_NP
     return cudaGetLastError();
@@ -1324,19 +1466,18 @@ cudaError_t launch_slice_n(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
 
 cudaError_t launch_slice_n_hess(const DevSystem &s, int32_t b0, int32_t b1, int32_t max_qt, int32_t max_rt,
                                 const double *scratch, const int64_t *hoff, int comp, uint8_t *slices,
-                                const int64_t *sl_off, const int32_t *expo_q, int32_t *expo_b, const int32_t *tn_b, int S,
-                                int F, cudaStream_t st) {
+                                const int64_t *sl_off, const int32_t *expo_q, int32_t *expo_b, int S, int F, cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
     const int first = comp == 0 ? 1 : 0;  // P' (its exponent and its slices) once, with the first pass
 #define NAO_SLICE_NPHI(SS, FF)                                                                                   \
     slice_nphi_kernel<SS, FF, double><<<dim3(b1 - b0, 4 * max_qt + 1), 256, 0, st>>>(                            \
-        s, b0, scratch, hoff, comp, slices, sl_off, expo_q, expo_b, tn_b, 10, 1, first)
+        s, b0, scratch, hoff, comp, slices, sl_off, expo_q, expo_b, 10, 1, first)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NPHI)
 #undef NAO_SLICE_NPHI
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !first || max_rt <= 0) return e;
 #define NAO_SLICE_NP(SS, FF) \
-    slice_np_kernel<SS, FF><<<dim3(b1 - b0, 4 * max_rt), 256, 0, st>>>(s, b0, slices, sl_off, expo_b, tn_b, 1)
+    slice_np_kernel<SS, FF><<<dim3(b1 - b0, 4 * max_rt), 256, 0, st>>>(s, b0, slices, sl_off, expo_b, 1)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NP)
 #undef NAO_SLICE_NP
     return cudaGetLastError();
@@ -1359,7 +1500,7 @@ static cudaError_t launch_n_tc_mode(const DevSystem &s, const HWork *work, int32
     const size_t sm = split_smem_bytes(S, F);
     const int grid = n_work < sm_count() ? n_work : sm_count();  // persistent: one CTA per SM
 #define NAO_N_TC(TNV, M, FF)                                                                                  \
-    n_tc_kernel<TNV, M, FF><<<grid, 192, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo_q, expo_b, ev, eoff, S, hc, \
+    n_tc_kernel<TNV, M, FF><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo_q, expo_b, ev, eoff, S, hc, \
                                                    hess, err)
 #define NAO_N_TC_MODES(TNV, FF)             \
     switch (mode) {                         \
