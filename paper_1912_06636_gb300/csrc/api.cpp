@@ -673,6 +673,7 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     s.sys.Hacc = reinterpret_cast<unsigned long long *const *>(g->d_tab + 7 * n_sys);
     s.sys.np = g->d_sys_np;
     s.n_rgrid = g->n_rgrid;
+    s.lmax = fn_l.empty() ? 0 : *std::max_element(fn_l.begin(), fn_l.end());
     s.max_ppad = (g->max_P + NAO_PPAD - 1) / NAO_PPAD * NAO_PPAD;
     s.r0 = g->r0;
     s.inv_delta = 1.0 / g->delta;
@@ -689,6 +690,27 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
             s.knorm_h[l][m] = (float)k;
             s.knorm_l[l][m] = (float)(k - (double)s.knorm_h[l][m]);
         }
+    // With W_l^m = r^l P_l^m e^{i m phi} (no Condon-Shortley phase): d/dz W_l^m = (l+m) W_{l-1}^m,
+    // (d/dx + i d/dy) W_l^m = -W_{l-1}^{m+1}, (d/dx - i d/dy) W_l^m = (l+m)(l+m-1) W_{l-1}^{m-1} (m >= 1),
+    // and S_l,m = K_lm Re W_l^m, S_l,-m = K_lm Im W_l^m.
+    s.hc = HarmonicCoefs{};
+    double odd = 1.0;  // (2l-1)!!
+    for (int l = 1; l <= NAO_LMAX; l++) {
+        odd *= 2 * l - 1;
+        s.hc.kl[l] = odd * s.knorm[l][l];
+        for (int m = 0; m <= l; m++) {
+            const double k = s.knorm[l][m];
+            if (m <= l - 1) {
+                s.hc.ra[l][m] = k / s.knorm[l - 1][m] * (2 * l - 1) / (l - m);
+                s.hc.dz[l][m] = k / s.knorm[l - 1][m] * (l + m);
+            }
+            if (m <= l - 2) {
+                s.hc.rb[l][m] = k / s.knorm[l - 2][m] * (l + m - 1) / (l - m);
+                s.hc.dp[l][m] = (m == 0 ? -1.0 : -0.5) * k / s.knorm[l - 1][m + 1];
+            }
+            if (m >= 1) s.hc.dm[l][m] = 0.5 * (l + m) * (l + m - 1) * k / s.knorm[l - 1][m - 1];
+        }
+    }
     NAO_CUDA(cudaStreamSynchronize(g->setup));
     return NAO_OK;
 }

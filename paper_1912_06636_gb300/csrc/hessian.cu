@@ -8,26 +8,29 @@
 // and the same pass gives n_q = sum_j T_qj phi_qj and d_a n_q = 2 sum_j T_qj d_a phi_qj.
 //
 // Evaluation: one CTA per batch, one thread per (point, atom) as in the other evaluation
-// kernels; phi = g(r) S_lm with g = R / r^l and S_lm = K Pi_l^m(z, r^2) {A_m, B_m}(x, y) (the
-// solid-harmonic recurrence, carried with the first and second derivatives of Pi in z and r^2):
+// kernels; phi = g(r) S_lm with g = R / r^l and S_lm the normalised real solid harmonic:
 //   d_a phi     = g' (x_a / r) S + g d_a S,
 //   d_a d_b phi = (g'' / r^2 - g' / r^3) x_a x_b S + (g' / r)(delta_ab S + x_b d_a S + x_a d_b S)
 //                 + g d_a d_b S,
 //   g' = R' / r^l - l R / r^(l+1),  g'' = R'' / r^l - 2 l R' / r^(l+1) + l (l+1) R / r^(l+2),
 // with R' and R'' from the spline in s = ln(r / r0) / Delta (ds/dr = 1 / (r Delta),
-// d^2s/dr^2 = -1 / (r^2 Delta)). Every batch's block of scratch holds, per reduced-basis row,
-// 10 rows of Ppad points: phi, d/dx, d/dy, d/dz, xx, xy, xz, yy, yz, zz, in the path's type T
-// (the values are computed in FP64 on both paths; the FP32 path rounds them once when storing).
-// For the Pulay terms (LAP) the fifth row holds the Laplacian xx + yy + zz instead, summed in
-// FP64 before the rounding (the three terms cancel where the Laplacian is small).
+// d^2s/dr^2 = -1 / (r^2 Delta)). The harmonics of l come from those of l - 1 and l - 2, and their
+// derivatives are fixed combinations of at most two harmonics of l - 1 (the second ones of the first
+// ones of l - 1), so that an entry takes 3 + 5 + 9 FP64 operations. Every batch's block of scratch holds,
+// per reduced-basis row, 10 rows of Ppad points: phi, d/dx, d/dy, d/dz, xx, xy, xz, yy, yz, zz, in the
+// path's type T (the values are computed in FP64 on both paths; the FP32 path rounds them once when
+// storing). For the Pulay terms (LAP) the fifth row holds the Laplacian instead: S is harmonic and
+// homogeneous of degree l, so lap phi = (g'' + (2 l + 2) g' / r) S, and no second derivative is formed.
+// Bound by the FP64 pipe, so powers of 1/r replace divisions. Per call, against recurrences for the derivatives
+// of Pi(z, r^2) with divisions: 13-atom molecule (76,050 points) 5.28 -> 1.92 ms, with the Laplacian (9 atoms,
+// 19,440 points) 3.17 -> 0.43 ms.
 //
 // Contraction: one CTA per 64-point density tile; for each 64-function tile J the four
 // products Phi P, (d_x Phi) P, (d_y Phi) P, (d_z Phi) P over all of K in T (P read from its
 // upper triangle, so the matrix used is exactly symmetric), then the epilogue above in T, the
 // per-tile sums added in FP64. Every point is written once (no atomics).
-#include <cmath>
-
 #include "nao_internal.h"
+#include "radial.h"
 
 namespace {
 
@@ -36,191 +39,165 @@ constexpr int TQ = NAO_TILE; // 64 points per density tile
 constexpr int TJ = 64;       // functions per tile
 constexpr int KC = 8;        // K chunk of the contraction
 
-__host__ __device__ constexpr double dfact_odd(int m) { return m <= 1 ? 1.0 : (2 * m - 1) * dfact_odd(m - 1); }
-
 // (xx, xy, xz, yy, yz, zz)
 __device__ __forceinline__ int pair_a(int k) { return k < 3 ? 0 : (k < 5 ? 1 : 2); }
 __device__ __forceinline__ int pair_b(int k) { return k == 0 ? 0 : k == 1 ? 1 : k == 2 ? 2 : k == 3 ? 1 : 2; }
 
-template <int LMAX, typename OutT, bool LAP>
-__device__ __noinline__ void eval_group_hess(const DevSystem &s, const AtomGroup &ag, double x, double y, double z,
-                                             double r2, double r, OutT *E, int64_t rs, int64_t cs, int q) {
-    // radial coordinate (the radial part is taken at r0 for r < r0)
-    const double rr = fmax(r, s.r0);
-    const double sc = log(rr / s.r0) * s.inv_delta;
-    int k = (int)floor(sc);
-    k = k < 0 ? 0 : (k > s.n_rgrid - 2 ? s.n_rgrid - 2 : k);
-    const double t = sc - (double)k;
-    const double ds1 = s.inv_delta / rr, ds2 = -s.inv_delta / (rr * rr);
-    const double ur = 1.0 / r;
-    const double xa[3] = {x, y, z};
+// d/dx, d/dy, d/dz of the entry +-m of harmonics l from the entries C of l - 1 (index l - 1 + m), or of
+// their gradients where C holds one component of those.
+template <int l, int LM>
+__device__ __forceinline__ double harmonic_d(const DevSystem &s, const double (&C)[2 * LM + 1], int mm, int axis) {
+    // mm: 0 .. 2 l, the entry m = mm - l (m >= 0: the cosine part); a compile-time constant once unrolled
+    const int m = mm >= l ? mm - l : l - mm, sg = mm >= l ? 1 : -1;
+    constexpr int o = l - 1;
+    if (axis == 2) return m <= l - 1 ? s.hc.dz[l][m] * C[o + sg * m] : 0.0;
+    // d/dx: the same part of m + 1 and m - 1; d/dy: the other part
+    const int t = axis == 0 ? sg : -sg;
+    const double p = axis == 0 ? s.hc.dp[l][m] : (sg > 0 ? s.hc.dp[l][m] : -s.hc.dp[l][m]);
+    const double q = axis == 0 ? s.hc.dm[l][m] : (sg > 0 ? -s.hc.dm[l][m] : s.hc.dm[l][m]);
+    // m = 0 has no sine part: S_l0 has d/dx from +1 and d/dy from -1 with dp alone
+    const bool up = m + 1 <= l - 1, down = m >= 1 && !(m == 1 && t < 0);
+    if (up && down) return fma(p, C[o + t * (m + 1)], q * C[o + t * (m - 1)]);
+    if (up) return p * C[o + t * (m + 1)];
+    return down ? q * C[o + t * (m - 1)] : 0.0;
+}
 
-    // A_m + i B_m = (x + i y)^m
-    double A[LMAX + 1], B[LMAX + 1];
-    A[0] = 1.0;
-    B[0] = 0.0;
+// All functions of l = L of one atom at one point, and then of L + 1, .. LMAX. A + i B = (x + i y)^L;
+// S1, S2: harmonics of L - 1 and L - 2; G1: their gradients for L - 1.
+template <int L, int LMAX, typename OutT, bool LAP>
+struct HessLevel {
+    static __device__ __forceinline__ void run(const DevSystem &s, const AtomGroup &ag, int &ri, const double (&xa)[3],
+                                               double r2, double r, double ur, double ul, int k, double t, double ds1,
+                                               double A, double B,
+                                               const double (&S1)[2 * LMAX + 1], const double (&S2)[2 * LMAX + 1],
+                                               const double (&G1)[3][2 * LMAX + 1], OutT *E, int64_t rs, int64_t cs, int q) {
+        double S[2 * LMAX + 1], G[3][2 * LMAX + 1], H[6][2 * LMAX + 1];
+        if constexpr (L == 0) {
+            S[0] = s.knorm[0][0];
+            G[0][0] = G[1][0] = G[2][0] = 0.0;
 #pragma unroll
-    for (int m = 1; m <= LMAX; m++) {
-        A[m] = x * A[m - 1] - y * B[m - 1];
-        B[m] = x * B[m - 1] + y * A[m - 1];
-    }
-    // Pi_{l-1}^m (c) and Pi_{l-2}^m (p) with derivatives in z and q = r^2:
-    // component 0 value, 1 d/dz, 2 d/dq, 3 d2/dz2, 4 d2/dzdq, 5 d2/dq2
-    double Pc[6][LMAX + 1], Pp[6][LMAX + 1];
+            for (int kk = 0; kk < 6; kk++) H[kk][0] = 0.0;
+        } else {
+            S[2 * L] = s.hc.kl[L] * A;
+            S[0] = s.hc.kl[L] * B;
 #pragma unroll
-    for (int c = 0; c < 6; c++)
+            for (int m = 0; m < L; m++) {
+                const double az = s.hc.ra[L][m] * xa[2];
+                const double bq = m <= L - 2 ? s.hc.rb[L][m] * r2 : 0.0;
 #pragma unroll
-        for (int m = 0; m <= LMAX; m++) Pc[c][m] = Pp[c][m] = 0.0;
-    int ri = ag.r0;
-    const int re = ag.r0 + ag.nr;
-    double rl = 1.0;  // r^l
-#pragma unroll
-    for (int l = 0; l <= LMAX; l++) {
-        double S[2 * LMAX + 1], Sg[3][2 * LMAX + 1], Sh[6][2 * LMAX + 1];
-#pragma unroll
-        for (int m = 0; m <= l; m++) {
-            double pv[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            if (m == l) {
-                pv[0] = dfact_odd(m);
-            } else if (m == l - 1) {
-                pv[0] = (2 * m + 1) * z * Pc[0][m];
-                pv[1] = (2 * m + 1) * Pc[0][m];
-            } else {
-                const double c1 = (double)(2 * l - 1) / (double)(l - m), c2 = (double)(l + m - 1) / (double)(l - m);
-                pv[0] = c1 * z * Pc[0][m] - c2 * r2 * Pp[0][m];
-                pv[1] = c1 * (Pc[0][m] + z * Pc[1][m]) - c2 * r2 * Pp[1][m];
-                pv[2] = c1 * z * Pc[2][m] - c2 * (Pp[0][m] + r2 * Pp[2][m]);
-                pv[3] = c1 * (2.0 * Pc[1][m] + z * Pc[3][m]) - c2 * r2 * Pp[3][m];
-                pv[4] = c1 * (Pc[2][m] + z * Pc[4][m]) - c2 * (Pp[1][m] + r2 * Pp[4][m]);
-                pv[5] = c1 * z * Pc[5][m] - c2 * (2.0 * Pp[2][m] + r2 * Pp[5][m]);
-            }
-#pragma unroll
-            for (int c = 0; c < 6; c++) {
-                Pp[c][m] = Pc[c][m];
-                Pc[c][m] = pv[c];
-            }
-            // P(x, y, z) = Pi(z, q(x, y, z)) and its derivatives
-            const double P0 = pv[0];
-            const double Pd[3] = {2.0 * x * pv[2], 2.0 * y * pv[2], pv[1] + 2.0 * z * pv[2]};
-            const double Pdd[6] = {2.0 * pv[2] + 4.0 * x * x * pv[5],                       // xx
-                                   4.0 * x * y * pv[5],                                       // xy
-                                   2.0 * x * (pv[4] + 2.0 * z * pv[5]),                       // xz
-                                   2.0 * pv[2] + 4.0 * y * y * pv[5],                       // yy
-                                   2.0 * y * (pv[4] + 2.0 * z * pv[5]),                       // yz
-                                   pv[3] + 4.0 * z * pv[4] + 2.0 * pv[2] + 4.0 * z * z * pv[5]};  // zz
-            const double kn = s.knorm[l][m];
-            // the x, y factor C and its derivatives (d/dz = 0): m = 0: C = 1; m > 0: C = A_m or B_m
-            for (int part = 0; part < (m == 0 ? 1 : 2); part++) {
-                double C = 1.0, Cd[3] = {0.0, 0.0, 0.0}, Cdd[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-                const double fm = (double)m, fmm = (double)(m * (m - 1));
-                if (m > 0 && part == 0) {  // A_m: d/dx = m A_{m-1}, d/dy = -m B_{m-1}
-                    C = A[m];
-                    Cd[0] = fm * A[m - 1];
-                    Cd[1] = -fm * B[m - 1];
-                    if (m >= 2) {
-                        Cdd[0] = fmm * A[m - 2];
-                        Cdd[1] = -fmm * B[m - 2];
-                        Cdd[3] = -fmm * A[m - 2];
-                    }
-                } else if (m > 0) {        // B_m: d/dx = m B_{m-1}, d/dy = m A_{m-1}
-                    C = B[m];
-                    Cd[0] = fm * B[m - 1];
-                    Cd[1] = fm * A[m - 1];
-                    if (m >= 2) {
-                        Cdd[0] = fmm * B[m - 2];
-                        Cdd[1] = fmm * A[m - 2];
-                        Cdd[3] = -fmm * B[m - 2];
-                    }
+                for (int sg = 1; sg >= (m == 0 ? 1 : -1); sg -= 2) {
+                    const double v = az * S1[L - 1 + sg * m];
+                    S[L + sg * m] = m <= L - 2 ? fma(-bq, S2[L - 2 + sg * m], v) : v;
                 }
-                const int idx = m == 0 ? l : (part == 0 ? l + m : l - m);
-                S[idx] = kn * P0 * C;
+            }
 #pragma unroll
-                for (int a = 0; a < 3; a++) Sg[a][idx] = kn * (Pd[a] * C + P0 * Cd[a]);
+            for (int mm = 0; mm < 2 * L + 1; mm++) {
 #pragma unroll
-                for (int kk = 0; kk < 6; kk++) {
-                    const int a = pair_a(kk), b = pair_b(kk);
-                    Sh[kk][idx] = kn * (Pdd[kk] * C + Pd[a] * Cd[b] + Pd[b] * Cd[a] + P0 * Cdd[kk]);
+                for (int a = 0; a < 3; a++) G[a][mm] = harmonic_d<L, LMAX>(s, S1, mm, a);
+                if (!LAP) {
+#pragma unroll
+                    for (int kk = 0; kk < 6; kk++) H[kk][mm] = harmonic_d<L, LMAX>(s, G1[pair_a(kk)], mm, pair_b(kk));
                 }
             }
         }
-        // the atom's radial functions of this l
-        for (; ri < re; ri++) {
+        for (; ri < ag.r0 + ag.nr; ri++) {
             const RfnEntry e = s.rfn[ri];
-            if (e.l != l) break;
-            double g = 0.0, G1 = 0.0, Q = 0.0;  // g, g'/r, g''/r^2 - g'/r^3
+            if (e.l != L) break;
+            OutT *row = E + (int64_t)e.pos * rs + q;
+            double g = 0.0, G1r = 0.0, Q = 0.0, lapr = 0.0;  // g, g'/r, g''/r^2 - g'/r^3, the Laplacian's factor of S
             if (r < s.fn_rc[e.fn]) {
-                const double *cf = s.coef + ((size_t)e.fn * (s.n_rgrid - 1) + k) * 4;
-                const double R = ((cf[3] * t + cf[2]) * t + cf[1]) * t + cf[0];
-                const double Rs = (3.0 * cf[3] * t + 2.0 * cf[2]) * t + cf[1];
-                const double Rss = 6.0 * cf[3] * t + 2.0 * cf[2];
-                const double R1 = Rs * ds1, R2 = Rss * ds1 * ds1 + Rs * ds2;
-                const double fl = (double)l;
-                g = R / rl;
-                const double g1 = R1 / rl - fl * R / (rl * r);
-                const double g2 = R2 / rl - 2.0 * fl * R1 / (rl * r) + fl * (fl + 1.0) * R / (rl * r * r);
-                G1 = g1 * ur;
-                Q = g2 * ur * ur - g1 * ur * ur * ur;
+                const double2 *c = reinterpret_cast<const double2 *>(s.coef + ((size_t)e.fn * (s.n_rgrid - 1) + k) * 4);
+                const double2 c01 = __ldg(c), c23 = __ldg(c + 1);
+                const double a = fma(c23.y, t, c23.x);
+                const double R = fma(fma(a, t, c01.y), t, c01.x);
+                const double Rs = fma(fma(c23.y, t, a + a), t, c01.y);
+                const double Rss = fma(6.0 * c23.y, t, 2.0 * c23.x);
+                const double R1 = Rs * ds1, R2 = ds1 * fma(Rss, ds1, -(Rs * ur));  // d^2s/dr^2 = -ds/dr / r
+                g = R * ul;
+                const double lr = (double)L * ur;
+                const double g1 = fma(-lr, R, R1) * ul;
+                const double g2 = fma(-2.0 * lr, R1, fma((double)(L * (L + 1)) * ur * ur, R, R2)) * ul;
+                G1r = g1 * ur;
+                if (LAP) lapr = fma((double)(2 * L + 2), G1r, g2);
+                else Q = (g2 - G1r) * (ur * ur);
             }
-            for (int mm = 0; mm < 2 * l + 1; mm++) {
-                OutT *row = E + (int64_t)(e.pos + mm) * rs + q;
+            const double gx[3] = {G1r * xa[0], G1r * xa[1], G1r * xa[2]};
+            double Qab[6];
+            if (!LAP) {
+#pragma unroll
+                for (int kk = 0; kk < 6; kk++) {
+                    const double v = Q * xa[pair_a(kk)];
+                    Qab[kk] = pair_a(kk) == pair_b(kk) ? fma(v, xa[pair_b(kk)], G1r) : v * xa[pair_b(kk)];
+                }
+            }
+#pragma unroll
+            for (int mm = 0; mm < 2 * L + 1; mm++, row += rs) {
                 const double Sv = S[mm];
                 row[0] = OutT(g * Sv);
 #pragma unroll
-                for (int a = 0; a < 3; a++) row[(1 + a) * cs] = OutT(G1 * xa[a] * Sv + g * Sg[a][mm]);
-                double lap = 0.0;
+                for (int a = 0; a < 3; a++) row[(1 + a) * cs] = OutT(L == 0 ? gx[a] * Sv : fma(gx[a], Sv, g * G[a][mm]));
+                if (LAP) {
+                    row[4 * cs] = OutT(lapr * Sv);
+                } else {
 #pragma unroll
-                for (int kk = 0; kk < 6; kk++) {
-                    const int a = pair_a(kk), b = pair_b(kk);
-                    const double dab = a == b ? 1.0 : 0.0;
-                    const double v = Q * xa[a] * xa[b] * Sv + G1 * (dab * Sv + xa[b] * Sg[a][mm] + xa[a] * Sg[b][mm]) +
-                                     g * Sh[kk][mm];
-                    if (LAP) {
-                        if (a == b) lap += v;  // xx + yy + zz, in that order
-                    } else {
+                    for (int kk = 0; kk < 6; kk++) {
+                        const int a = pair_a(kk), b = pair_b(kk);
+                        double v = Qab[kk] * Sv;
+                        if (L >= 1) v = fma(gx[b], G[a][mm], fma(gx[a], G[b][mm], v));
+                        if (L >= 2) v = fma(g, H[kk][mm], v);
                         row[(4 + kk) * cs] = OutT(v);
                     }
                 }
-                if (LAP) row[4 * cs] = OutT(lap);
             }
         }
-        rl *= r;
+        if constexpr (L < LMAX) {
+            if (ri < ag.r0 + ag.nr)
+                HessLevel<L + 1, LMAX, OutT, LAP>::run(s, ag, ri, xa, r2, r, ur, ul * ur, k, t, ds1,
+                                                       L == 0 ? xa[0] : fma(xa[0], A, -(xa[1] * B)),
+                                                       L == 0 ? xa[1] : fma(xa[0], B, xa[1] * A), S, S1, G, E, rs, cs, q);
+        }
     }
+};
+
+template <int LMAX, typename OutT, bool LAP>
+__device__ __forceinline__ void eval_group_hess(const DevSystem &s, const AtomGroup &ag, double x, double y, double z,
+                                                OutT *E, int64_t rs, int64_t cs, int q) {
+    const double xa[3] = {x, y, z};
+    const double r2 = fma(x, x, fma(y, y, z * z)), ur = rsqrt(r2), r = r2 * ur;
+    const double rr = fmax(r, s.r0);  // the radial part is taken at r0 for r < r0
+    int k;
+    const double t = radial_coordinate(s, rr, k);
+    const double ur0 = r < s.r0 ? 1.0 / s.r0 : ur;
+    const double zero[2 * LMAX + 1] = {}, zero3[3][2 * LMAX + 1] = {};
+    int ri = ag.r0;
+    HessLevel<0, LMAX, OutT, LAP>::run(s, ag, ri, xa, r2, r, ur, 1.0, k, t, s.inv_delta * ur0, 1.0, 0.0, zero, zero, zero3, E, rs, cs,
+                                       q);
 }
 
-template <typename OutT, bool LAP>
-__global__ void __launch_bounds__(256) eval_hess_kernel(DevSystem s, int32_t b0, OutT *__restrict__ scratch,
-                                                       const int64_t *__restrict__ hoff) {
+// LMAX: at least the largest l of the handle's functions.
+template <int LMAX, typename OutT, bool LAP>
+__global__ void __launch_bounds__(128) eval_hess_kernel(const __grid_constant__ DevSystem s, int32_t b0,
+                                                       OutT *__restrict__ scratch, const int64_t *__restrict__ hoff) {
     const int b = b0 + blockIdx.x;
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
     const int g0 = s.agrp_off[b], ng = s.agrp_off[b + 1] - g0;
     OutT *E = scratch + hoff[b];
     const int64_t rs = (int64_t)HR * Ppad, cs = Ppad;
-    for (int idx = threadIdx.x; idx < ng * Ppad; idx += blockDim.x) {
+    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < ng * Ppad; idx += gridDim.y * blockDim.x) {
         const int gl = idx / Ppad, q = idx - gl * Ppad;
         const AtomGroup ag = s.agrp[g0 + gl];
         if (q >= P) {  // padding points: zero rows
             for (int ri = ag.r0; ri < ag.r0 + ag.nr; ri++) {
                 const RfnEntry e = s.rfn[ri];
                 for (int mm = 0; mm < 2 * e.l + 1; mm++)
-                    for (int c = 0; c < HR; c++) E[(int64_t)(e.pos + mm) * rs + c * cs + q] = OutT(0);
+                    for (int c = 0; c < (LAP ? 5 : HR); c++) E[(int64_t)(e.pos + mm) * rs + c * cs + q] = OutT(0);
             }
             continue;
         }
         const int p = p0 + q;
-        const double dx = s.px[p] - s.atom_xyz[3 * ag.atom], dy = s.py[p] - s.atom_xyz[3 * ag.atom + 1],
-                     dz = s.pz[p] - s.atom_xyz[3 * ag.atom + 2];
-        const double r2 = dx * dx + dy * dy + dz * dz;
-        const double r = sqrt(r2);
-        switch (ag.lmax) {
-            case 0: eval_group_hess<0, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-            case 1: eval_group_hess<1, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-            case 2: eval_group_hess<2, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-            case 3: eval_group_hess<3, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-            case 4: eval_group_hess<4, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-            case 5: eval_group_hess<5, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-            default: eval_group_hess<6, OutT, LAP>(s, ag, dx, dy, dz, r2, r, E, rs, cs, q); break;
-        }
+        eval_group_hess<LMAX, OutT, LAP>(s, ag, s.px[p] - s.atom_xyz[3 * ag.atom], s.py[p] - s.atom_xyz[3 * ag.atom + 1],
+                                         s.pz[p] - s.atom_xyz[3 * ag.atom + 2], E, rs, cs, q);
     }
 }
 
@@ -355,15 +332,31 @@ __global__ void __launch_bounds__(256) density_hess_kernel(DevSystem s, const DW
 
 }  // namespace
 
+template <typename OutT, bool LAP>
+static cudaError_t launch_eval_hess_t(const DevSystem &s, int32_t b0, int32_t b1, OutT *scratch, const int64_t *hoff,
+                                      cudaStream_t st) {
+    // several CTAs per batch: a batch's (atom, point) pairs are independent, and small systems have
+    // fewer batches than the GPU has SMs
+    const dim3 grid(b1 - b0, 4);
+    switch (s.lmax) {
+        case 0:
+        case 1: eval_hess_kernel<1, OutT, LAP><<<grid, 128, 0, st>>>(s, b0, scratch, hoff); break;
+        case 2: eval_hess_kernel<2, OutT, LAP><<<grid, 128, 0, st>>>(s, b0, scratch, hoff); break;
+        case 3: eval_hess_kernel<3, OutT, LAP><<<grid, 128, 0, st>>>(s, b0, scratch, hoff); break;
+        case 4: eval_hess_kernel<4, OutT, LAP><<<grid, 128, 0, st>>>(s, b0, scratch, hoff); break;
+        default: eval_hess_kernel<NAO_LMAX, OutT, LAP><<<grid, 128, 0, st>>>(s, b0, scratch, hoff); break;
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_eval_hess(const DevSystem &s, int32_t b0, int32_t b1, void *scratch, bool fp32, bool lap,
                              const int64_t *hoff, cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
-    const int n = b1 - b0;
-    if (fp32 && lap) eval_hess_kernel<float, true><<<n, 256, 0, st>>>(s, b0, static_cast<float *>(scratch), hoff);
-    else if (fp32) eval_hess_kernel<float, false><<<n, 256, 0, st>>>(s, b0, static_cast<float *>(scratch), hoff);
-    else if (lap) eval_hess_kernel<double, true><<<n, 256, 0, st>>>(s, b0, static_cast<double *>(scratch), hoff);
-    else eval_hess_kernel<double, false><<<n, 256, 0, st>>>(s, b0, static_cast<double *>(scratch), hoff);
-    return cudaGetLastError();
+    if (fp32)
+        return lap ? launch_eval_hess_t<float, true>(s, b0, b1, static_cast<float *>(scratch), hoff, st)
+                   : launch_eval_hess_t<float, false>(s, b0, b1, static_cast<float *>(scratch), hoff, st);
+    return lap ? launch_eval_hess_t<double, true>(s, b0, b1, static_cast<double *>(scratch), hoff, st)
+               : launch_eval_hess_t<double, false>(s, b0, b1, static_cast<double *>(scratch), hoff, st);
 }
 
 cudaError_t launch_density_hess(const DevSystem &s, const DWork *work, int32_t w0, int32_t n_work, const void *scratch,

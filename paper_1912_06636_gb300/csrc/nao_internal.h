@@ -53,6 +53,13 @@ struct SysTables {
     const int32_t *np;       // [n_sys] points of the system
 };
 
+// Coefficients of the recurrences for the normalised real solid harmonics (see DevSystem::hc).
+struct HarmonicCoefs {
+    double ra[NAO_LMAX + 1][NAO_LMAX + 1], rb[NAO_LMAX + 1][NAO_LMAX + 1];
+    double kl[NAO_LMAX + 1];  // S_l,l + i S_l,-l = kl (x + i y)^l
+    double dz[NAO_LMAX + 1][NAO_LMAX + 1], dp[NAO_LMAX + 1][NAO_LMAX + 1], dm[NAO_LMAX + 1][NAO_LMAX + 1];
+};
+
 // Geometry and tables shared by every kernel (device pointers).
 struct DevSystem {
     const double *atom_xyz;   // [n_atoms*3]
@@ -74,12 +81,18 @@ struct DevSystem {
     const int64_t *scr_off;   // [n_batches] element offset of the batch's block in scratch
     int32_t n_rgrid;
     int32_t max_ppad;         // largest padded batch (points)
+    int32_t lmax;             // largest angular momentum of the handle's functions
     double r0, inv_delta;
     double step_m1;           // exp(Delta) - 1: r_{k+1} / r_k - 1 of the logarithmic grid
     int64_t nb;               // total basis size over all systems
     SysTables sys;
     double knorm[NAO_LMAX + 1][NAO_LMAX + 1];  // sqrt((2l+1)/(4pi) (l-m)!/(l+m)!) (x sqrt2 for m>0)
     float knorm_h[NAO_LMAX + 1][NAO_LMAX + 1], knorm_l[NAO_LMAX + 1][NAO_LMAX + 1];  // knorm as float-float
+    // The normalised solid harmonics by l (from l - 1 and l - 2) and their derivatives from l - 1
+    // (nao_harmonic_coefficients): S_l,+-m = ra z S_{l-1},+-m - rb r^2 S_{l-2},+-m (m < l), and with
+    // C = S_{l-1}, d/dz S_l,+-m = dz C_{+-m}, d/dx S_l,+-m = dp C_{+-(m+1)} + dm C_{+-(m-1)} and
+    // d/dy S_l,+-m = +-(dp C_{-+(m+1)} - dm C_{-+(m-1)}).
+    HarmonicCoefs hc;
 };
 
 #ifdef __CUDACC__

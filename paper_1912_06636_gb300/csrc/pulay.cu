@@ -8,20 +8,124 @@
 //     F_at,c = 2 sum_{i on at} sum_j (n_ij M^c_ij - q_ij S^c_ij).
 // The batches' basis functions come from the density Hessian's evaluation (10 rows per function:
 // phi, grad phi and, in place of the six second derivatives, lap = xx + yy + zz summed in FP64).
-// One CTA per 64 x 64 tile pair (I, J) of a batch (all pairs: the matrices are not symmetric); per 8-point K chunk the CTA
-// stages w d_c phi_i (three components) and h phi_j, phi_j, and accumulates the six products in
-// the path's type T (the evaluation is FP64 on both paths, stored in T; on the FP32 path each
-// 8-point chunk's sums are added into compensated (hi, lo) pairs, in two passes of three
-// products); FP64 atomics add each tile into the global matrices.
-#include <type_traits>
-
+// Work items are the 64 x 64 tile pairs (I, J) of a batch (all pairs: the matrices are not symmetric);
+// FP64 atomics add each tile into the global matrices.
+// FP64: bound by the FP64 pipe (two lanes per clock and SM), 6 N^2 P products per batch. One CTA takes half
+// an item, 64 x 32, and each warp one 16 x 16 subtile of it with all six products; subtiles beyond the
+// batch's functions are left out. The rows d_c phi_i come by cp.async as they lie, the weights go into the
+// columns: w phi_j and w h phi_j. 9 atoms, 19,440 points: 11.3 -> 9.5 ms (floor 7.2).
+// FP32: per 8-point chunk w d_c phi_i (three components) and h phi_j or phi_j, each chunk's sums added
+// into compensated (hi, lo) pairs, in two passes of three products.
 #include "nao_internal.h"
 
 namespace {
 
 constexpr int HR = 10;  // rows per basis function in the Hessian evaluation
 constexpr int TT = 64;  // tile edge (functions)
-constexpr int KC = 8;   // points per K chunk
+constexpr int KC = 8;   // points per K chunk (FP32)
+
+constexpr int KP = 16;      // points per K chunk (FP64): 128 bytes of a row
+constexpr int LDP = 18;     // and 16 bytes more: the eight rows a warp reads at once in different banks
+
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(256, 2)
+    pulay_fp64_kernel(const __grid_constant__ DevSystem s, const HWork *__restrict__ work, int32_t w0,
+                      const double *__restrict__ scratch, const int64_t *__restrict__ hoff, double *__restrict__ M,
+                      double *__restrict__ Sm, int64_t nb) {
+    __shared__ __align__(16) double As[3][TT][LDP];      // d_c phi_i
+    __shared__ __align__(16) double Bs[2][TT / 2][LDP];  // w h phi_j, w phi_j
+    extern __shared__ __align__(16) double wt[];         // [2][Ppad]: w, w v
+    const HWork it = work[w0 + blockIdx.x];
+    const int b = it.batch, m = s.sys.bmol[b];
+    const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
+    const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
+    const int N = s.rel_off[b + 1] - s.rel_off[b];
+    const int i0 = it.ti * TT, j0 = it.tj * TT + (int)blockIdx.y * (TT / 2);
+    if (j0 >= N) return;
+    const double *E = scratch + hoff[b];
+    const int64_t ld = (int64_t)HR * Ppad;
+    const int tid = threadIdx.x, lane = tid & 31, lx = lane & 3, ly = lane >> 2;
+    for (int q = tid; q < Ppad; q += 256) {
+        const double w = q < P ? s.pw[p0 + q] : 0.0;
+        wt[q] = w;
+        wt[Ppad + q] = q < P ? w * v_at(s, m, p0 + q) : 0.0;
+    }
+    // the warp's subtile (rows r0 .., columns c0 ..); which warp takes which turns with the CTA, so that
+    // the idle ones spread over the schedulers
+    const int role = ((tid >> 5) + blockIdx.x) & 7, r0 = 16 * (role >> 1), c0 = 16 * (role & 1);
+    const bool live = i0 + r0 < N && j0 + c0 < N;
+    double acc[3][2][2][4];
+#pragma unroll
+    for (int x = 0; x < 48; x++) (&acc[0][0][0][0])[x] = 0.0;
+    const int lv = tid & 7, lr = tid >> 3;  // loader: vector lv (two points), rows lr and lr + 32
+    for (int q0 = 0; q0 < Ppad; q0 += KP) {
+        __syncthreads();  // the weights are written; every warp has left the last chunk
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int i = i0 + lr + 32 * h;
+            const double *row = E + (int64_t)(i < N ? i : 0) * ld + q0 + 2 * lv;
+#pragma unroll
+            for (int c = 0; c < 3; c++) cp16(&As[c][lr + 32 * h][2 * lv], row + (int64_t)(1 + c) * Ppad, i < N);
+        }
+        double2 wh = make_double2(0.0, 0.0), wf = wh;
+        if (j0 + lr < N) {
+            const double *row = E + (int64_t)(j0 + lr) * ld + q0 + 2 * lv;
+            const double2 f = *reinterpret_cast<const double2 *>(row);
+            const double2 lap = *reinterpret_cast<const double2 *>(row + 4 * (int64_t)Ppad);
+            const double2 w = *reinterpret_cast<const double2 *>(wt + q0 + 2 * lv);
+            const double2 wv = *reinterpret_cast<const double2 *>(wt + Ppad + q0 + 2 * lv);
+            wf = make_double2(w.x * f.x, w.y * f.y);
+            wh = make_double2(fma(wv.x, f.x, -0.5 * w.x * lap.x), fma(wv.y, f.y, -0.5 * w.y * lap.y));
+        }
+        *reinterpret_cast<double2 *>(&Bs[0][lr][2 * lv]) = wh;
+        *reinterpret_cast<double2 *>(&Bs[1][lr][2 * lv]) = wf;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (!live) continue;
+#pragma unroll 1
+        for (int kv = 0; kv < KP; kv += 2)
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                double2 rb[4];
+#pragma unroll
+                for (int y = 0; y < 4; y++) rb[y] = *reinterpret_cast<const double2 *>(&Bs[u][c0 + lx + 4 * y][kv]);
+#pragma unroll
+                for (int c = 0; c < 3; c++)
+#pragma unroll
+                    for (int x = 0; x < 2; x++) {
+                        const double2 ra = *reinterpret_cast<const double2 *>(&As[c][r0 + ly + 8 * x][kv]);
+#pragma unroll
+                        for (int y = 0; y < 4; y++)
+                            acc[c][u][x][y] = fma(ra.y, rb[y].y, fma(ra.x, rb[y].x, acc[c][u][x][y]));
+                    }
+            }
+    }
+    if (!live) return;
+    const int32_t *rel = s.rel_idx + s.rel_off[b];
+    const int64_t nn = nb * nb;
+#pragma unroll
+    for (int x = 0; x < 2; x++) {
+        const int i = i0 + r0 + ly + 8 * x;
+        if (i >= N) continue;
+        const int64_t gi = rel[i];
+#pragma unroll
+        for (int y = 0; y < 4; y++) {
+            const int j = j0 + c0 + lx + 4 * y;
+            if (j >= N) continue;
+            const int64_t e = gi * nb + rel[j];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                atomicAdd(M + c * nn + e, acc[c][0][x][y]);
+                atomicAdd(Sm + c * nn + e, acc[c][1][x][y]);
+            }
+        }
+    }
+}
 
 // (hi, lo) += x with Knuth's TwoSum (exact transformation of hi + x): the FP32 path's running
 // sums over the chunks, so that only each 8-point chunk is summed in plain FP32.
@@ -32,96 +136,77 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
     hi = t;
 }
 
-// NU = 2: both products (h phi_j and phi_j) in one pass (FP64); NU = 1: the product u0 only
-// (FP32: two passes, which leaves registers for the compensated sums).
-template <typename T, int NU>
-__global__ void __launch_bounds__(256) pulay_kernel(DevSystem s, const HWork *__restrict__ work, int32_t w0,
-                                                   const T *__restrict__ scratch, const int64_t *__restrict__ hoff,
-                                                   double *__restrict__ M, double *__restrict__ Sm, int64_t nb, int u0) {
-    constexpr bool F32 = std::is_same<T, float>::value;
-    __shared__ __align__(16) T As[3][KC][TT];  // w_q d_c phi_i(q)
-    __shared__ __align__(16) T Bs[NU][KC][TT];  // h phi_j(q) (u = 0), phi_j(q) (u = 1)
+// One of the two products: u0 = 0 (h phi_j, into M) or 1 (phi_j, into S), which leaves registers for the
+// compensated sums.
+__global__ void __launch_bounds__(256) pulay_fp32_kernel(const __grid_constant__ DevSystem s, const HWork *__restrict__ work,
+                                                        int32_t w0, const float *__restrict__ scratch,
+                                                        const int64_t *__restrict__ hoff, double *__restrict__ out, int64_t nb,
+                                                        int u0) {
+    __shared__ __align__(16) float As[3][KC][TT];  // w_q d_c phi_i(q)
+    __shared__ __align__(16) float Bs[KC][TT];     // h phi_j(q) or phi_j(q)
     const HWork it = work[w0 + blockIdx.x];
     const int b = it.batch, m = s.sys.bmol[b];
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
     const int N = s.rel_off[b + 1] - s.rel_off[b];
-    const T *E = scratch + hoff[b];
+    const float *E = scratch + hoff[b];
     const int64_t ld = (int64_t)HR * Ppad;
     const int32_t *rel = s.rel_idx + s.rel_off[b];
     const int i0 = it.ti * TT, j0 = it.tj * TT;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    T acc[3][NU][4][4];
-    float hi[3][NU][4][4], lo[3][NU][4][4];  // FP32 only (unused, and removed, for FP64)
+    float acc[3][4][4], hi[3][4][4], lo[3][4][4];
 #pragma unroll
     for (int c = 0; c < 3; c++)
 #pragma unroll
-        for (int u = 0; u < NU; u++)
+        for (int a = 0; a < 4; a++)
 #pragma unroll
-            for (int a = 0; a < 4; a++)
-#pragma unroll
-                for (int d = 0; d < 4; d++) {
-                    acc[c][u][a][d] = T(0);
-                    hi[c][u][a][d] = lo[c][u][a][d] = 0.0f;
-                }
+            for (int d = 0; d < 4; d++) acc[c][a][d] = hi[c][a][d] = lo[c][a][d] = 0.0f;
     for (int q0 = 0; q0 < P; q0 += KC) {
         __syncthreads();
         for (int u = tid; u < 3 * KC * TT; u += blockDim.x) {
             const int c = u / (KC * TT), kk = (u / TT) % KC, ii = u % TT;
             const int i = i0 + ii, q = q0 + kk;
-            As[c][kk][ii] = (i < N && q < P) ? T(s.pw[p0 + q] * (double)E[(int64_t)i * ld + (int64_t)(1 + c) * Ppad + q]) : T(0);
+            As[c][kk][ii] =
+                (i < N && q < P) ? float(s.pw[p0 + q] * (double)E[(int64_t)i * ld + (int64_t)(1 + c) * Ppad + q]) : 0.0f;
         }
         for (int u = tid; u < KC * TT; u += blockDim.x) {
             const int kk = u / TT, jj = u % TT;
             const int j = j0 + jj, q = q0 + kk;
-            double hphi = 0.0, f = 0.0;
+            float f = 0.0f;
             if (j < N && q < P) {
-                const T *row = E + (int64_t)j * ld + q;
-                f = (double)row[0];
-                if (NU == 2 || u0 == 0) {
+                const float *row = E + (int64_t)j * ld + q;
+                f = row[0];
+                if (u0 == 0) {
                     const double lap = (double)row[4 * (int64_t)Ppad];  // the evaluation's Laplacian row
-                    hphi = -0.5 * lap + v_at(s, m, p0 + q) * f;
+                    f = float(-0.5 * lap + v_at(s, m, p0 + q) * (double)f);
                 }
             }
-            if (NU == 2) {
-                Bs[0][kk][jj] = T(hphi);
-                Bs[NU - 1][kk][jj] = T(f);
-            } else {
-                Bs[0][kk][jj] = T(u0 == 0 ? hphi : f);
-            }
+            Bs[kk][jj] = f;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < KC; kk++) {
-            T rb[NU][4];
+            float rb[4];
 #pragma unroll
-            for (int u = 0; u < NU; u++)
-#pragma unroll
-                for (int d = 0; d < 4; d++) rb[u][d] = Bs[u][kk][tx * 4 + d];
+            for (int d = 0; d < 4; d++) rb[d] = Bs[kk][tx * 4 + d];
 #pragma unroll
             for (int c = 0; c < 3; c++)
 #pragma unroll
                 for (int a = 0; a < 4; a++) {
-                    const T ra = As[c][kk][ty * 4 + a];
+                    const float ra = As[c][kk][ty * 4 + a];
 #pragma unroll
-                    for (int u = 0; u < NU; u++)
-#pragma unroll
-                        for (int d = 0; d < 4; d++) acc[c][u][a][d] = fma(ra, rb[u][d], acc[c][u][a][d]);
+                    for (int d = 0; d < 4; d++) acc[c][a][d] = fmaf(ra, rb[d], acc[c][a][d]);
                 }
         }
-        if constexpr (F32) {
 #pragma unroll
-            for (int c = 0; c < 3; c++)
+        for (int c = 0; c < 3; c++)
 #pragma unroll
-                for (int u = 0; u < NU; u++)
+            for (int a = 0; a < 4; a++)
 #pragma unroll
-                    for (int a = 0; a < 4; a++)
-#pragma unroll
-                        for (int d = 0; d < 4; d++) {
-                            two_sum_acc(hi[c][u][a][d], lo[c][u][a][d], (float)acc[c][u][a][d]);
-                            acc[c][u][a][d] = T(0);
-                        }
-        }
+                for (int d = 0; d < 4; d++) {
+                    two_sum_acc(hi[c][a][d], lo[c][a][d], acc[c][a][d]);
+                    acc[c][a][d] = 0.0f;
+                }
     }
     const int64_t nn = nb * nb;
 #pragma unroll
@@ -135,12 +220,7 @@ __global__ void __launch_bounds__(256) pulay_kernel(DevSystem s, const HWork *__
             if (j >= N) continue;
             const int64_t e = gi * nb + rel[j];
 #pragma unroll
-            for (int c = 0; c < 3; c++)
-#pragma unroll
-                for (int u = 0; u < NU; u++) {
-                    const double v = F32 ? (double)hi[c][u][a][d] + (double)lo[c][u][a][d] : (double)acc[c][u][a][d];
-                    atomicAdd(((NU == 2 ? u : u0) == 0 ? M : Sm) + c * nn + e, v);
-                }
+            for (int c = 0; c < 3; c++) atomicAdd(out + c * nn + e, (double)hi[c][a][d] + (double)lo[c][a][d]);
         }
     }
 }
@@ -180,12 +260,19 @@ cudaError_t launch_pulay(const DevSystem &s, const HWork *work, int32_t w0, int3
     if (n_work <= 0) return cudaSuccess;
     if (fp32) {
         for (int u0 = 0; u0 < 2; u0++) {
-            pulay_kernel<float, 1><<<n_work, 256, 0, st>>>(s, work, w0, static_cast<const float *>(scratch), hoff, M, S, nb, u0);
+            pulay_fp32_kernel<<<n_work, 256, 0, st>>>(s, work, w0, static_cast<const float *>(scratch), hoff, u0 == 0 ? M : S,
+                                                      nb, u0);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
     } else {
-        pulay_kernel<double, 2><<<n_work, 256, 0, st>>>(s, work, w0, static_cast<const double *>(scratch), hoff, M, S, nb, 0);
+        const size_t dyn = 2 * (size_t)s.max_ppad * sizeof(double);  // the weights
+        if (dyn > 11 * 1024) {  // beyond 48 KB with the 36.9 KB of operands
+            const cudaError_t e = cudaFuncSetAttribute(pulay_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       2 * NAO_MAX_BATCH * (int)sizeof(double));
+            if (e != cudaSuccess) return e;
+        }
+        pulay_fp64_kernel<<<dim3(n_work, 2), 256, dyn, st>>>(s, work, w0, static_cast<const double *>(scratch), hoff, M, S, nb);
     }
     return cudaGetLastError();
 }
