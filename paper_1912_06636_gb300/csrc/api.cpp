@@ -679,6 +679,8 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     s.inv_delta = 1.0 / g->delta;
     s.step_m1 = std::expm1(g->delta);
     s.nb = g->nb;
+    // K_lm = sqrt((2l+1)/(4pi) (l-m)!/(l+m)!), times sqrt 2 for m > 0
+    double knorm[NAO_LMAX + 1][NAO_LMAX + 1] = {};
     for (int l = 0; l <= NAO_LMAX; l++)
         for (int m = 0; m <= NAO_LMAX; m++) {
             double k = 0.0;
@@ -686,10 +688,11 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
                 k = std::sqrt((2.0 * l + 1.0) / (4.0 * M_PI) * factorial(l - m) / factorial(l + m));
                 if (m > 0) k *= std::sqrt(2.0);
             }
-            s.knorm[l][m] = k;
-            s.knorm_h[l][m] = (float)k;
-            s.knorm_l[l][m] = (float)(k - (double)s.knorm_h[l][m]);
+            knorm[l][m] = k;
         }
+    s.s00 = knorm[0][0];
+    s.s00_h = (float)s.s00;
+    s.s00_l = (float)(s.s00 - (double)s.s00_h);
     // With W_l^m = r^l P_l^m e^{i m phi} (no Condon-Shortley phase): d/dz W_l^m = (l+m) W_{l-1}^m,
     // (d/dx + i d/dy) W_l^m = -W_{l-1}^{m+1}, (d/dx - i d/dy) W_l^m = (l+m)(l+m-1) W_{l-1}^{m-1} (m >= 1),
     // and S_l,m = K_lm Re W_l^m, S_l,-m = K_lm Im W_l^m.
@@ -697,20 +700,28 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     double odd = 1.0;  // (2l-1)!!
     for (int l = 1; l <= NAO_LMAX; l++) {
         odd *= 2 * l - 1;
-        s.hc.kl[l] = odd * s.knorm[l][l];
+        s.hc.kl[l] = odd * knorm[l][l];
         for (int m = 0; m <= l; m++) {
-            const double k = s.knorm[l][m];
+            const double k = knorm[l][m];
             if (m <= l - 1) {
-                s.hc.ra[l][m] = k / s.knorm[l - 1][m] * (2 * l - 1) / (l - m);
-                s.hc.dz[l][m] = k / s.knorm[l - 1][m] * (l + m);
+                s.hc.ra[l][m] = k / knorm[l - 1][m] * (2 * l - 1) / (l - m);
+                s.hc.dz[l][m] = k / knorm[l - 1][m] * (l + m);
             }
             if (m <= l - 2) {
-                s.hc.rb[l][m] = k / s.knorm[l - 2][m] * (l + m - 1) / (l - m);
-                s.hc.dp[l][m] = (m == 0 ? -1.0 : -0.5) * k / s.knorm[l - 1][m + 1];
+                s.hc.rb[l][m] = k / knorm[l - 2][m] * (l + m - 1) / (l - m);
+                s.hc.dp[l][m] = (m == 0 ? -1.0 : -0.5) * k / knorm[l - 1][m + 1];
             }
-            if (m >= 1) s.hc.dm[l][m] = 0.5 * (l + m) * (l + m - 1) * k / s.knorm[l - 1][m - 1];
+            if (m >= 1) s.hc.dm[l][m] = 0.5 * (l + m) * (l + m - 1) * k / knorm[l - 1][m - 1];
         }
     }
+    for (int l = 0; l <= NAO_LMAX; l++)
+        for (int m = 0; m <= NAO_LMAX; m++) {
+            const double c[6] = {s.hc.ra[l][m], s.hc.rb[l][m], s.hc.dz[l][m], s.hc.dp[l][m], s.hc.dm[l][m], m == 0 ? s.hc.kl[l] : 0.0};
+            for (int i = 0; i < 6; i++) {
+                s.hcf[i][l][m][0] = (float)c[i];
+                s.hcf[i][l][m][1] = (float)(c[i] - (double)s.hcf[i][l][m][0]);
+            }
+        }
     NAO_CUDA(cudaStreamSynchronize(g->setup));
     return NAO_OK;
 }
@@ -1106,7 +1117,7 @@ nao_status enqueue_n(nao_grid *g, nao_precision prec, bool want_ne, bool grad, c
         NAO_CUDA(launch_zero_n(s, g->d_dwork, (int32_t)g->n_dwork, grad, st));
         for (const auto &c : g->split_chunks) {
             NAO_CUDA(timed(g, grad ? NAO_K_EVAL_GRAD : NAO_K_EVAL_PHI, st, [&] {
-                return launch_eval_split(s, c.b0, c.b1, grad, g->d_scratch, g->d_expo_q, 128 * c.max_qt, st);
+                return launch_eval_split(s, c.b0, c.b1, grad, g->d_scratch, g->d_expo_q, g->d_expo_b, st);
             }));
             NAO_CUDA(timed(g, NAO_K_SLICE_N, st, [&] {
                 return launch_slice_n(s, c.b0, c.b1, c.max_qt, c.max_rt, g->d_scratch, g->d_slices, g->d_sl_off_n,

@@ -45,6 +45,19 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
 }
 
+// The same from the bit pattern, with integer instructions and one integer-to-float conversion (the four
+// FP64 ones of from_double run on the FP64 pipe): the 24 leading bits rounded to nearest, and the signed
+// 29-bit rest rounded to FP32, so to 2^-49 of x. Outside 2^-72 .. 2^104, and for zero, from_double.
+__device__ __forceinline__ F from_double_bits(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu, sg = hi & 0x80000000u;
+    if (e - 951u > 176u) return from_double(x);
+    const uint32_t rest = lo & 0x1FFFFFFFu, up = rest >> 28;
+    const float h = __uint_as_float((sg | ((e - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29)) + up);
+    const float l = __int2float_rn((int)rest - (int)(up << 29));
+    return F{h, __fmul_rn(l, __uint_as_float(sg | ((e - 948u) << 23)))};
+}
+
 __device__ __forceinline__ double to_double(F x) { return __dadd_rn((double)x.h, (double)x.l); }
 
 // s + e = a + b exactly, for |a| >= |b| (or a = 0)

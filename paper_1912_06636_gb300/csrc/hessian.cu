@@ -73,7 +73,7 @@ struct HessLevel {
                                                const double (&G1)[3][2 * LMAX + 1], OutT *E, int64_t rs, int64_t cs, int q) {
         double S[2 * LMAX + 1], G[3][2 * LMAX + 1], H[6][2 * LMAX + 1];
         if constexpr (L == 0) {
-            S[0] = s.knorm[0][0];
+            S[0] = s.s00;
             G[0][0] = G[1][0] = G[2][0] = 0.0;
 #pragma unroll
             for (int kk = 0; kk < 6; kk++) H[kk][0] = 0.0;

@@ -86,13 +86,14 @@ struct DevSystem {
     double step_m1;           // exp(Delta) - 1: r_{k+1} / r_k - 1 of the logarithmic grid
     int64_t nb;               // total basis size over all systems
     SysTables sys;
-    double knorm[NAO_LMAX + 1][NAO_LMAX + 1];  // sqrt((2l+1)/(4pi) (l-m)!/(l+m)!) (x sqrt2 for m>0)
-    float knorm_h[NAO_LMAX + 1][NAO_LMAX + 1], knorm_l[NAO_LMAX + 1][NAO_LMAX + 1];  // knorm as float-float
+    double s00;               // S_00 = 1 / sqrt(4 pi)
+    float s00_h, s00_l;       // and as a float-float
     // The normalised solid harmonics by l (from l - 1 and l - 2) and their derivatives from l - 1
     // (nao_harmonic_coefficients): S_l,+-m = ra z S_{l-1},+-m - rb r^2 S_{l-2},+-m (m < l), and with
     // C = S_{l-1}, d/dz S_l,+-m = dz C_{+-m}, d/dx S_l,+-m = dp C_{+-(m+1)} + dm C_{+-(m-1)} and
     // d/dy S_l,+-m = +-(dp C_{-+(m+1)} - dm C_{-+(m-1)}).
     HarmonicCoefs hc;
+    float hcf[6][NAO_LMAX + 1][NAO_LMAX + 1][2];  // ra, rb, dz, dp, dm and kl (at m = 0) as float-floats
 };
 
 #ifdef __CUDACC__
@@ -397,10 +398,10 @@ cudaError_t launch_relevance_minr2(const double *atom_xyz, const int32_t *bmol, 
                                    int64_t n_batches, double *minr2, cudaStream_t st);
 cudaError_t launch_eval(const DevSystem &s, int32_t b0, int32_t b1, nao_precision prec, bool grad, double *scratch,
                         cudaStream_t st);
-// Split path, the density's evaluation (FP64 values; phi, with grad phi when grad) and the
-// point exponents of the slicing into expo (by batch-ordered point; n_red >= P_b).
+// Split path, the density's evaluation (float-float values; phi, with grad phi when grad) and the
+// point exponents of the slicing into expo (by batch-ordered point); expo_b[b] = 0 for the P' exponents.
 cudaError_t launch_eval_split(const DevSystem &s, int32_t b0, int32_t b1, bool grad, double *scratch, int32_t *expo,
-                              int32_t n_red, cudaStream_t st);
+                              int32_t *expo_b, cudaStream_t st);
 // Density Hessian (FP64, or FP32 with fp32): evaluation of phi, grad phi and the six second
 // derivatives (computed in FP64, stored as double or float: 10 rows of Ppad per function at
 // scratch + hoff[b] elements; lap: the fifth row holds the Laplacian, for the Pulay terms) and
