@@ -1651,7 +1651,7 @@ nao_status nao_update_density_hessian(nao_grid *g, const double *P_dev, nao_prec
         size_t k_sub = 0;
         for (const auto &c : g->hess_chunks) {
             NAO_CUDA(launch_eval_hess(sys, c.b0, c.b1, g->d_scratch, false, false, g->d_hess_off, s));
-            NAO_CUDA(launch_hess_point_expo(sys, c.b0, c.b1, g->d_scratch, g->d_hess_off, g->d_expo4, g->n_points, s));
+            NAO_CUDA(launch_hess_point_expo(sys, c.b0, c.b1, g->d_scratch, g->d_hess_off, g->d_expo4, g->n_points, g->d_expo_b, s));
             for (; k_sub < g->hess_split.size() && g->hess_split[k_sub].b0 < c.b1; k_sub++) {
                 const auto &sub = g->hess_split[k_sub];
                 for (int comp = 0; comp < 4; comp++) {

@@ -463,7 +463,7 @@ cudaError_t launch_slice_n_hess(const DevSystem &s, int32_t b0, int32_t b1, int3
                                 const double *scratch, const int64_t *hoff, int comp, uint8_t *slices,
                                 const int64_t *sl_off, const int32_t *expo_q, int32_t *expo_b, int S, int F, cudaStream_t st);
 cudaError_t launch_hess_point_expo(const DevSystem &s, int32_t b0, int32_t b1, const double *scratch, const int64_t *hoff,
-                                   int32_t *expo4, int64_t n_points, cudaStream_t st);
+                                   int32_t *expo4, int64_t n_points, int32_t *expo_b, cudaStream_t st);
 cudaError_t launch_n_tc_hess(const DevSystem &s, const HWork *work, int32_t w0, int32_t n_work, const uint8_t *slices,
                              const int64_t *sl_off, const int32_t *expo_q, const int32_t *expo_b, const double *scratch,
                              const int64_t *hoff, int comp, double *hess, int S, int F, int tn, int32_t *err,

@@ -35,6 +35,7 @@
 namespace {
 
 constexpr long long kWaitCycles = 400000000LL;  // ~0.2 s at 2 GHz: bounded mbarrier waits
+constexpr size_t kSmemOptin = 232448;           // shared memory a CTA may opt into on this GPU (227 KB)
 
 
 // Digit extraction works on FP64 bit patterns with integer instructions: on this GPU the FP64
@@ -44,150 +45,107 @@ using split_bits::abs_bits;
 
 // S balanced base-2^B digits (B = 6: base 64, |d| <= 32, bf16; B = 5: base 32, |d| <= 16, e4m3;
 // most significant first in dig[0]) of X = round(x 2^(BS-e)), |x 2^-e| < 1/2, as exact
-// small-integer floats. From x's bits x = +-m 2^(E-1075) (53-bit m): |X| = m 2^-sh with
-// sh = 1075 + e - BS - E, rounded half up when sh > 0, held as a 128-bit integer (hi:lo; more
-// than 64 bits only for BS > 64). |X| is cut into chunks of D digits (3 x 6 = 18 or 4 x 5 = 20
-// bits; the fourth chunk takes the remaining 23 bits), exact in FP32, and the digits are peeled
-// off from the bottom in FP32: q = rint(v / 2^B), d = v - 2^B q in [-2^(B-1), 2^(B-1)], v <- q,
-// the carry q (0 or 1 after a chunk's digits) joining the next chunk. The top digit keeps
-// whatever remains, which the bound on |X| keeps in range. Subnormal x and e = -10000 give zeros.
-// |X| = round(|x| 2^(BS-e)) as a 128-bit integer (hi:lo) from the bits of x, and the sign of x.
-template <int S, int B>
-__device__ __forceinline__ void digit_integer(double x, int e, unsigned long long &lo, unsigned long long &hi,
-                                              float &sgn) {
-    const long long bits = __double_as_longlong(x);
-    const int eb = (int)((bits >> 52) & 0x7FF);
-    lo = 0;
-    hi = 0;
-    if (eb != 0 && e > -10000) {
-        const unsigned long long m = ((unsigned long long)bits & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
-        const int sh = 1075 + e - B * S - eb;
-        if (sh > 0) {
-            lo = sh >= 63 ? 0ULL : (m + (1ULL << (sh - 1))) >> sh;
-        } else {
-            const int k = -sh;  // <= B S - 54: 18 for 12 bf16 slices, 26 for 16 e4m3 slices
-            lo = m << k;
-            hi = k > 0 ? m >> (64 - k) : 0ULL;
-        }
+// small-integer floats, for two values at once (.x and .y) in packed FP32x2 arithmetic.
+//
+// x comes as two or three FP32 parts, each scaled exactly by 2^(BS-e). A part is cut into balanced chunks
+// of CB = D B bits (3 x 6 or 4 x 5) from the top: q = rint(R 2^-(c CB)), R <- R - q 2^(c CB), for
+// c = 3, 2, 1, then u_0 = rint(R). Every step is exact (R keeps a subset of the part's 24 significand
+// bits; |R 2^-(c CB)| < 2^22 keeps the rounding by 1.5 2^23 valid, and an FMA forms the product and
+// that rounding at once), so sum_c u_c 2^(c CB) is the part rounded to an integer. The parts' chunks are
+// added per chunk, and the digits are peeled off the chunks from the bottom: q = rint(v / 2^B),
+// d = v - 2^B q in [-2^(B-1), 2^(B-1)], v <- q, the carry q joining the next chunk. The top digit keeps
+// whatever remains, which the bound on |X| keeps in range. The result is within one unit of
+// round(|x| 2^(BS-e)).
+constexpr float kRint = 12582912.0f;  // 1.5 2^23: y + kRint - kRint = rint(y) for |y| < 2^22
+
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+
+// u_c += the chunks of part R (|R| < 2^(TOP CB + 22)), c = TOP .. 0.
+template <int CB, int TOP>
+__device__ __forceinline__ void add_chunks(float2 R, float2 (&u)[4]) {
+#pragma unroll
+    for (int c = TOP; c >= 1; c--) {
+        const float w = c == 3 ? (float)(1ULL << CB) * (float)(1ULL << CB) * (float)(1ULL << CB)
+                      : c == 2 ? (float)(1ULL << CB) * (float)(1ULL << CB) : (float)(1ULL << CB);
+        const float2 q = __fadd2_rn(__ffma2_rn(R, f2(1.0f / w), f2(kRint)), f2(-kRint));
+        R = __ffma2_rn(q, f2(-w), R);
+        u[c] = __fadd2_rn(u[c], q);
     }
-    sgn = bits < 0 ? -1.0f : 1.0f;
+    u[0] = __fadd2_rn(u[0], __fadd2_rn(__fadd2_rn(R, f2(kRint)), f2(-kRint)));
 }
 
-// Chunk c of |X| = (hi:lo): c = 0, 1, 2 the CB-bit fields (CB = 3 x 6 or 4 x 5 bits), c = 3 the
-// 23 bits from bit 3 CB.
-template <int B>
-__device__ __forceinline__ uint32_t digit_chunk(unsigned long long lo, unsigned long long hi, int c) {
-    constexpr int CB = B == 6 ? 18 : 20;
-    constexpr unsigned long long M = (1ULL << CB) - 1;
-    return c == 0 ? (uint32_t)(lo & M)
-         : c == 1 ? (uint32_t)((lo >> CB) & M)
-         : c == 2 ? (uint32_t)((lo >> (2 * CB)) & M)
-                  : (uint32_t)(((lo >> (3 * CB)) | (hi << (64 - 3 * CB))) & 0x7FFFFFULL);
-}
-
-// The S digits of two values x0, x1 at once (.x and .y of dig[s]) with packed FP32x2 arithmetic.
-// The sign is carried in the running value: v starts as sgn (|X| mod 2^CB) (sgn (2^23 + u) - sgn 2^23,
-// one packed FMA, exact), every later chunk enters as + sgn u at its digit position, and the
-// peeling q = rint(v / 2^B), d = v - 2^B q works on signed v as well: rint is odd-symmetric, so
-// the digits are those of |X| times the sign.
+// The digits from the chunks.
 template <int S, int B>
-__device__ __forceinline__ void digits2(double x0, double x1, int e, float2 (&dig)[S]) {
+__device__ __forceinline__ void peel(const float2 (&u)[4], float2 (&dig)[S]) {
     constexpr int D = B == 6 ? 3 : 4;  // digits per chunk
-    unsigned long long lo0, hi0, lo1, hi1;
-    float s0, s1;
-    digit_integer<S, B>(x0, e, lo0, hi0, s0);
-    digit_integer<S, B>(x1, e, lo1, hi1, s1);
-    const float2 sgn = make_float2(s0, s1), nb = make_float2(-8388608.0f * s0, -8388608.0f * s1);
-    const float2 inv = make_float2(1.0f / (1 << B), 1.0f / (1 << B)), big = make_float2(12582912.0f, 12582912.0f);
-    const float2 nbig = make_float2(-12582912.0f, -12582912.0f), mb = make_float2(-(float)(1 << B), -(float)(1 << B));
-    auto chunk = [&](int c) {  // sgn u, u < 2^23, exactly
-        const float2 u = make_float2(__int_as_float(0x4B000000 | (int)digit_chunk<B>(lo0, hi0, c)),
-                                     __int_as_float(0x4B000000 | (int)digit_chunk<B>(lo1, hi1, c)));
-        return __ffma2_rn(sgn, u, nb);
-    };
-    float2 v = chunk(0);
+    const float2 inv = f2(1.0f / (1 << B)), mb = f2(-(float)(1 << B));
+    float2 v = u[0];
 #pragma unroll
     for (int s = S - 1; s >= 0; s--) {
         const int t = S - 1 - s;  // digits already taken
-        if (t > 0 && t % D == 0) v = __fadd2_rn(v, chunk(t / D));
+        if (t > 0 && t % D == 0) v = __fadd2_rn(v, u[t / D]);
         if (s == 0) {
             dig[0] = v;
         } else {
-            const float2 q = __fadd2_rn(__ffma2_rn(v, inv, big), nbig);  // rint(v / 2^B)
+            const float2 q = __fadd2_rn(__ffma2_rn(v, inv, f2(kRint)), f2(-kRint));  // rint(v / 2^B)
             dig[s] = __ffma2_rn(q, mb, v);
             v = q;
         }
     }
 }
 
-// The digits of a float-float value without 128-bit integers: x = h + l is scaled by 2^(BS-e)
-// through its exponent fields (H = h 2^(BS-e), L = l 2^(BS-e), exact), and each part is cut into
-// balanced chunks of CB bits from the top in FP32: q = rint(R 2^-(c CB)), R <- R - q 2^(c CB),
-// for c = 3, 2, 1, then u_0 = rint(R). Every step is exact (R keeps a subset of the part's 24
-// significand bits; |R 2^-(c CB)| < 2^22 keeps the rounding by 1.5 2^23 valid), so
-// sum_c u_c 2^(c CB) = round(H) and the chunks of round(H) + round(L), summed per chunk (each at
-// most 2^(CB-1) in magnitude), feed the digit peeling below; the result is within one unit of
-// round(|h + l| 2^(BS-e)). A part below the FP32 normal range after scaling counts as zero.
-__device__ __forceinline__ float ff_scale_pow2(float v, int k) {
-    const int b = __float_as_int(v);
-    const int ex = (b >> 23) & 0xFF;
-    if (ex == 0 || ex + k <= 0) return 0.0f;
-    return __int_as_float(b + (k << 23));
-}
-
-__device__ __forceinline__ float rint_small(float y) {  // |y| < 2^22
-    return __fsub_rn(__fadd_rn(y, 12582912.0f), 12582912.0f);
-}
-
-template <int CB>
-__device__ __forceinline__ void ff_part_chunks(float P, float (&u)[4]) {
-    constexpr float W1 = (float)(1ULL << CB), W2 = W1 * W1, W3 = W2 * W1;
-    constexpr float I1 = 1.0f / W1, I2 = I1 * I1, I3 = I2 * I1;
-    float R = P;
-    const float q3 = rint_small(__fmul_rn(R, I3));
-    R = __fmaf_rn(-q3, W3, R);
-    const float q2 = rint_small(__fmul_rn(R, I2));
-    R = __fmaf_rn(-q2, W2, R);
-    const float q1 = rint_small(__fmul_rn(R, I1));
-    R = __fmaf_rn(-q1, W1, R);
-    u[0] += rint_small(R);
-    u[1] += q1;
-    u[2] += q2;
-    u[3] += q3;
-}
-
+// 2^(BS-e) as the product of two FP32 powers (the exponent itself may exceed FP32's range); both zero
+// for a row that counts as zero (e <= -10000).
 template <int S, int B>
-__device__ __forceinline__ void ff_chunks(ffa::F x, int e, float (&u)[4]) {
-    constexpr int D = B == 6 ? 3 : 4, CB = D * B;
-    u[0] = u[1] = u[2] = u[3] = 0.0f;
-    if (e <= -10000) return;
-    const int k = B * S - e;
-    ff_part_chunks<CB>(ff_scale_pow2(x.h, k), u);
-    ff_part_chunks<CB>(ff_scale_pow2(x.l, k), u);
-}
-
-// The S digits of two float-float values at once (packed FP32x2 peeling, as for FP64 values).
-template <int S, int B>
-__device__ __forceinline__ void digits2(ffa::F x0, ffa::F x1, int e, float2 (&dig)[S]) {
-    constexpr int D = B == 6 ? 3 : 4;
-    float u0[4], u1[4];
-    ff_chunks<S, B>(x0, e, u0);
-    ff_chunks<S, B>(x1, e, u1);
-    const float2 inv = make_float2(1.0f / (1 << B), 1.0f / (1 << B)), big = make_float2(12582912.0f, 12582912.0f);
-    const float2 nbig = make_float2(-12582912.0f, -12582912.0f), mb = make_float2(-(float)(1 << B), -(float)(1 << B));
-    float2 v = make_float2(u0[0], u1[0]);
-#pragma unroll
-    for (int s = S - 1; s >= 0; s--) {
-        const int t = S - 1 - s;
-        if (t > 0 && t % D == 0) v = __fadd2_rn(v, make_float2(u0[t / D], u1[t / D]));
-        if (s == 0) {
-            dig[0] = v;
-        } else {
-            const float2 q = __fadd2_rn(__ffma2_rn(v, inv, big), nbig);
-            dig[s] = __ffma2_rn(q, mb, v);
-            v = q;
-        }
+struct Scale {
+    float2 a, b;
+    __device__ __forceinline__ explicit Scale(int e) {
+        const int k = B * S - e, k1 = k >> 1;
+        a = f2(e <= -10000 ? 0.0f : __int_as_float((127 + k1) << 23));
+        b = f2(e <= -10000 ? 0.0f : __int_as_float((127 + k - k1) << 23));
     }
+    __device__ __forceinline__ float2 operator()(float2 v) const { return __fmul2_rn(__fmul2_rn(v, a), b); }
+};
+
+// Of two float-floats. The low part is below 2^-24 of the high one, so below 2^(2 CB + 22).
+template <int S, int B>
+__device__ __forceinline__ void digits2(ffa::F x0, ffa::F x1, const Scale<S, B> &sc, float2 (&dig)[S]) {
+    constexpr int CB = (B == 6 ? 3 : 4) * B;
+    static_assert(B * S - 25 < 2 * CB + 22, "the low part reaches the top chunk");
+    float2 u[4] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
+    add_chunks<CB, 3>(sc(make_float2(x0.h, x1.h)), u);
+    add_chunks<CB, 2>(sc(make_float2(x0.l, x1.l)), u);
+    peel<S, B>(u, dig);
+}
+
+// An FP64's 53 bits as three FP32s (24, 23 and 6 bits, all of its sign), scaled by 2^(BS-e) through the exponent
+// field: no FP64 instruction (the FP64 pipe has 1/64 of the FP32 rate). FP64s below 2^-900 count as zero.
+template <int S, int B>
+__device__ __forceinline__ void f64_parts(double x, int e, float &h, float &m, float &l) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int eb = (int)((hi >> 20) & 0x7FF), ex = eb - 1023 + B * S - e;  // |x| 2^(BS-e) in [2^ex, 2^(ex+1))
+    const uint32_t sg = hi & 0x80000000u;
+    h = m = l = 0.0f;
+    if (eb == 0 || e <= -10000 || ex < -30) return;  // below half a unit
+    const uint32_t b1 = sg | (uint32_t)(127 + ex) << 23;
+    h = __uint_as_float(b1 | (hi & 0xFFFFFu) << 3 | lo >> 29);
+    // the next bits as the fraction of a number of that binade, less its leading one
+    const uint32_t b2 = sg | (uint32_t)(127 + ex - 23) << 23;
+    m = __fsub_rn(__uint_as_float(b2 | ((lo >> 6) & 0x7FFFFFu)), __uint_as_float(b2));
+    const uint32_t b3 = sg | (uint32_t)(127 + ex - 46) << 23;
+    l = __fsub_rn(__uint_as_float(b3 | (lo & 0x3Fu) << 17), __uint_as_float(b3));
+}
+// Of two FP64s.
+template <int S, int B>
+__device__ __forceinline__ void digits2(double x0, double x1, int e, float2 (&dig)[S]) {
+    constexpr int CB = (B == 6 ? 3 : 4) * B;
+    float2 p[3], u[4] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
+    f64_parts<S, B>(x0, e, p[0].x, p[1].x, p[2].x);
+    f64_parts<S, B>(x1, e, p[0].y, p[1].y, p[2].y);
+    add_chunks<CB, 3>(p[0], u);
+    add_chunks<CB, 2>(p[1], u);
+    add_chunks<CB, 1>(p[2], u);
+    peel<S, B>(u, dig);
 }
 
 // bf16 bit patterns of two small integers held exactly in floats (their low halves are zero).
@@ -205,9 +163,10 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
 }
 
 // Digits of the 128-byte row segment a lane owns in one K chunk: values x[0..LC-1] of its LC
-// columns (2 for bf16, 4 for e4m3; FP64 or float-float), packed per slice into one 32-bit word.
-template <int S, int F, typename V>
-__device__ __forceinline__ void lane_digit_words(const V *x, int e, uint32_t (&w)[S]) {
+// columns (2 for bf16, 4 for e4m3; FP64 with the exponent, or float-float with its scale), packed per
+// slice into one 32-bit word.
+template <int S, int F, typename V, typename E>
+__device__ __forceinline__ void lane_digit_words(const V *x, const E &e, uint32_t (&w)[S]) {
     constexpr int B = nao_digit_bits(F);
     float2 d0[S];
     digits2<S, B>(x[0], x[1], e, d0);
@@ -221,6 +180,11 @@ __device__ __forceinline__ void lane_digit_words(const V *x, int e, uint32_t (&w
         for (int sl = 0; sl < S; sl++) w[sl] = pack_e4m3x4(d0[sl].x, d0[sl].y, d1[sl].x, d1[sl].y);
     }
 }
+// What lane_digit_words takes for a row's exponent, by value type.
+template <int S, int F>
+__device__ __forceinline__ Scale<S, nao_digit_bits(F)> digit_scale(const ffa::F *, int e) { return Scale<S, nao_digit_bits(F)>(e); }
+template <int S, int F>
+__device__ __forceinline__ int digit_scale(const double *, int e) { return e; }
 
 // 2^E as an FP64 (0 below the normal range).
 __device__ __forceinline__ double pow2(int E) {
@@ -235,61 +199,77 @@ __device__ __forceinline__ double pow2(int E) {
 // reordered: the negative-weight ones (v < 0 on the potential part) first, padded to a whole
 // MMA K step (16 bf16 or 32 e4m3 columns), then the rest, so that B = A and the sign is applied
 // per K step.
-// One warp per row: the row's exponent (a pass over the row's K float-float values), then its
-// digits (a second pass, served from L2: the slices are written with evict-first stores so that
-// they do not push the rows out). Within each K step, lane l of the 8 lanes that write the
-// step's 32 bytes takes logical columns l, l + 8 (, l + 16, l + 24) of the step: a permutation
-// inside the K step, the same for every row (A and B of H are the same digit rows, so every
-// product is unchanged, and each K step keeps its sign), which keeps each load instruction of the
-// second pass on a few 64-byte runs of the row.
+// One warp per row: the largest magnitude of the row times the column scales sqrt|d_k| (a pass over the row's
+// K float-float values), then its digits (a second pass, served from L2: the slices are written with
+// evict-first stores so that they do not push the rows out), one 128-byte segment per slice and K chunk.
+// Within each K step, lane l of the 8 lanes that write the step's 32 bytes takes the logical columns 2 l,
+// 2 l + 1 (, 16 + 2 l, 17 + 2 l): a permutation inside the K step, the same for every row (A and B of H are the
+// same digit rows, so every product is unchanged, and each K step keeps its sign), which keeps each load
+// instruction of the second pass on a few 64-byte runs of the row.
+// Bound by HBM (8 bytes read and 14 or 24 written per value: 4.8 and 5.3 TB/s of the copy's 6.8): 75-atom slab,
+// 14 e4m3 slices, 5.89 -> 5.17 ms with the packed digit code; 12 bf16 slices 6.85 -> 6.33 ms. Keeping the scaled
+// rows in shared memory between the passes cost more in occupancy than the second read.
 // ----------------------------------------------------------------------------------------
+constexpr int kSliceWarps = 8;
+// Shared memory of slice_h_kernel for a batch of Ppad padded points: column scales, order, signs.
+__host__ __device__ constexpr size_t slice_h_smem(int Ppad, int F) {
+    return (size_t)4 * Ppad * (8 + 1) + 32 +
+           (size_t)2 * ((4 * Ppad + nao_kstep_cols(F) + nao_chunk_cols(F) - 1) / nao_chunk_cols(F) * nao_chunk_cols(F));
+}
+
 template <int S, int F>
-__global__ void __launch_bounds__(256, S <= 10 ? 5 : 4) slice_h_kernel(DevSystem s, int32_t b0, const FF2 *__restrict__ scratch,
-                                                        uint32_t terms, uint8_t *__restrict__ slices,
-                                                        const int64_t *__restrict__ sl_off, int32_t *__restrict__ expo,
-                                                        int32_t *__restrict__ neg16) {
-    __shared__ ffa::F sd[4 * NAO_SPLIT_MAX_PPAD];    // column scale as a float-float
-    __shared__ int sd_eb[4 * NAO_SPLIT_MAX_PPAD];    // biased exponent of sd (0: zero weight)
-    __shared__ float sd_m[4 * NAO_SPLIT_MAX_PPAD];   // significand of sd in [1, 2)
-    __shared__ short src[4 * NAO_SPLIT_MAX_PPAD + 128];
-    __shared__ unsigned char negf[4 * NAO_SPLIT_MAX_PPAD];
-    __shared__ int wsum[8];
+__global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __grid_constant__ DevSystem s, int32_t b0,
+                                                                  const FF2 *__restrict__ scratch, uint32_t terms,
+                                                                  uint8_t *__restrict__ slices,
+                                                                  const int64_t *__restrict__ sl_off,
+                                                                  int32_t *__restrict__ expo, int32_t *__restrict__ neg16) {
+    extern __shared__ __align__(16) unsigned char slice_sh[];
+    __shared__ int wsum[kSliceWarps];
     const int b = b0 + blockIdx.x, rt = blockIdx.y, m = s.sys.bmol[b];
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
     const int N = s.rel_off[b + 1] - s.rel_off[b];
-    constexpr int C = nao_chunk_cols(F), KS = nao_kstep_cols(F), LC = C / 32;  // columns per lane
+    constexpr int C = nao_chunk_cols(F), KS = nao_kstep_cols(F), LC = C / 32, B = nao_digit_bits(F);  // LC: columns per lane
     const SplitGeom G(P, N, S, 0, F);
     if (N == 0 || rt >= G.h_slice_tiles()) return;
-    const int K = 4 * Ppad, Kp = C * G.n_kc;
+    const int K = 4 * Ppad, Kp = C * G.n_kc, T = 32 * kSliceWarps;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float2 *sd = reinterpret_cast<float2 *>(slice_sh);              // [K] column scale sqrt|d| as a float-float
+    short *src = reinterpret_cast<short *>(sd + K);                 // [Kp] the column at each logical place (-1: none)
+    unsigned char *negf = reinterpret_cast<unsigned char *>(src + Kp);  // [K]
     const FF2 *E = scratch + s.scr_off[b];
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const int c = k / Ppad, q = k - c * Ppad;
-        const double d = q < P ? split_bits::h_column_weight(s, m, p0 + q, c, terms) : 0.0;
-        // sqrt|d| as a float-float: the FP32 square root s0 and one Newton correction
-        // (|d| - s0^2) / (2 s0), the residual formed exactly by one FP64 FMA (|d| below the FP32
-        // range counts as a zero weight)
-        const float a = __double2float_rn(fabs(d));
-        ffa::F sdf{0.0f, 0.0f};
-        if (a >= 1.17549435e-38f) {
-            const float s0 = __fsqrt_rn(a);
-            const double r = fma(-(double)s0, (double)s0, fabs(d));
-            sdf = ffa::quick(s0, __fmul_rn(__double2float_rn(r), __fdiv_rn(0.5f, s0)));
+    for (int q = threadIdx.x; q < Ppad; q += T) {
+        float2 sq[2];
+        bool ng[2];
+#pragma unroll
+        for (int c = 0; c < 2; c++) {  // the potential part, the gradient parts
+            const double d = q < P ? split_bits::h_column_weight(s, m, p0 + q, c, terms) : 0.0;
+            // sqrt|d| as a float-float: the FP32 square root s0 and one Newton correction
+            // (|d| - s0^2) / (2 s0), the residual formed exactly by one FP64 FMA (|d| below the FP32
+            // range counts as a zero weight)
+            const float a = __double2float_rn(fabs(d));
+            sq[c] = make_float2(0.0f, 0.0f);
+            if (a >= 1.17549435e-38f) {
+                const float s0 = __fsqrt_rn(a);
+                const double r = fma(-(double)s0, (double)s0, fabs(d));
+                const ffa::F f = ffa::quick(s0, __fmul_rn(__double2float_rn(r), __fdiv_rn(0.5f, s0)));
+                sq[c] = make_float2(f.h, f.l);
+            }
+            ng[c] = d < 0.0;
         }
-        sd[k] = sdf;
-        const int sb = __float_as_int(sdf.h);
-        sd_eb[k] = sdf.h != 0.0f ? ((sb >> 23) & 0xFF) + 896 : 0;  // biased exponent on the FP64 scale
-        sd_m[k] = __int_as_float(0x3F800000 | (sb & 0x7FFFFF));
-        negf[k] = d < 0.0 ? 1 : 0;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            sd[c * Ppad + q] = sq[c == 0 ? 0 : 1];
+            negf[c * Ppad + q] = ng[c == 0 ? 0 : 1] ? 1 : 0;
+        }
     }
-    for (int k = threadIdx.x; k < Kp; k += blockDim.x) src[k] = -1;
+    for (int k = threadIdx.x; k < Kp; k += T) src[k] = -1;
     __syncthreads();
     // exclusive scan of the negative flags: thread t owns columns [t*per, t*per + per)
-    const int per = (K + 255) / 256;
-    const int kb = threadIdx.x * per, ke = min(K, kb + per);
+    const int per = (K + T - 1) / T;
+    const int kb = min(K, (int)threadIdx.x * per), ke = min(K, kb + per);
     int cnt = 0;
     for (int k = kb; k < ke; k++) cnt += negf[k];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -299,46 +279,48 @@ __global__ void __launch_bounds__(256, S <= 10 ? 5 : 4) slice_h_kernel(DevSystem
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
     int before = 0, total = 0;
-    for (int w = 0; w < 8; w++) {
+    for (int w = 0; w < kSliceWarps; w++) {
         if (w < warp) before += wsum[w];
         total += wsum[w];
     }
     before += incl - cnt;
     const int negpad = (total + KS - 1) / KS * KS;  // a whole MMA K step
     for (int k = kb; k < ke; k++) {
-        const int pos = negf[k] ? before : negpad + k - before;
+        src[negf[k] ? before : negpad + k - before] = (short)k;
         before += negf[k];
-        src[pos] = (short)k;
     }
     if (rt == 0 && threadIdx.x == 0) neg16[b] = negpad / KS;  // negated K steps
     __syncthreads();
     uint8_t *base = slices + sl_off[b];
-    // the logical column of this lane's value c inside a chunk (see above)
-    const int lcol = KS * (lane >> 3) + (lane & 7);
-    for (int lr = warp; lr < 64; lr += 8) {
+    for (int lr = warp; lr < 64; lr += kSliceWarps) {
         const int r = rt * 64 + lr;
         if (r >= G.R16) break;
         const float2 *row = reinterpret_cast<const float2 *>(E + (int64_t)(r < N ? r : 0) * K);
-        int mk = 0;
+        auto scaled = [&](int k) {
+            const float2 v = row[k], w = sd[k];
+            return ffa::mul(ffa::F{v.x, v.y}, ffa::F{w.x, w.y});
+        };
+        int mx = 0;
         if (r < N)
-            for (int k = lane; k < K; k += 32) mk = max(mk, split_bits::h_row_key_ff(row[k].x, sd_eb[k], sd_m[k]));
-        mk = __reduce_max_sync(0xffffffffu, mk);
-        const int e = r < N ? split_bits::h_row_exponent(mk) : -10000;
+#pragma unroll 4
+            for (int k = lane; k < K; k += 32) mx = max(mx, __float_as_int(scaled(k).h) & 0x7FFFFFFF);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        // |x.h| <= (2 - 2^-23) 2^k and |x.l| <= 2^-24 2^(k+1): |x| < 2^(k+1), and |x 2^-e| < 1/2 with e = k + 2
+        const int e = (mx >> 23) != 0 ? (mx >> 23) - 127 + 2 : -10000;
         if (lane == 0 && r < N) expo[s.rel_off[b] + r] = e;
+        const Scale<S, B> sc(e);
         for (int kc = 0; kc < G.n_kc; kc++) {
             ffa::F x[LC];
 #pragma unroll
-            for (int c = 0; c < LC; c++) {
-                const int kk = src[C * kc + lcol + 8 * c];
-                if (kk >= 0 && e > -10000) {
-                    const float2 v = __ldcs(row + kk);
-                    x[c] = ffa::mul(ffa::F{v.x, v.y}, sd[kk]);
-                } else {
-                    x[c] = ffa::F{0.0f, 0.0f};
-                }
+            for (int c = 0; c < LC; c += 2) {
+                // bf16: columns 2 lane, 2 lane + 1 of the chunk; e4m3: 32 (lane / 8) + 2 (lane % 8) + {0, 1, 16, 17}
+                const int at = C * kc + (F == NAO_DIGITS_BF16 ? 2 * lane : KS * (lane >> 3) + 2 * (lane & 7) + 8 * c);
+                const short2 kk = *reinterpret_cast<const short2 *>(src + at);
+                x[c] = kk.x >= 0 ? scaled(kk.x) : ffa::F{0.0f, 0.0f};
+                x[c + 1] = kk.y >= 0 ? scaled(kk.y) : ffa::F{0.0f, 0.0f};
             }
             uint32_t wd[S];
-            lane_digit_words<S, F>(x, e, wd);
+            lane_digit_words<S, F>(x, sc, wd);
             const uint32_t off = tc::sw128_byte((uint32_t)r, (uint32_t)(4 * lane));
 #pragma unroll
             for (int sl = 0; sl < S; sl++) __stcs(reinterpret_cast<unsigned int *>(base + G.h_block(sl, kc) + off), wd[sl]);
@@ -351,11 +333,13 @@ __global__ void __launch_bounds__(256, S <= 10 ? 5 : 4) slice_h_kernel(DevSystem
 // Phi^T: one CTA (8 warps) per (batch, 32-point tile), the point exponents from the
 // evaluation. Per K chunk (64 or 128 functions) the CTA stages phi[i][q] (chunk x 32, read along
 // the points) in shared memory and each warp writes its points' rows along K (2 or 4 functions
-// per lane, one 128-byte row segment per slice). CTAs with blockIdx.y = 0 instead reduce the batch's
-// exponent of P' (the upper-triangle tile pairs, read along rows of P).
+// per lane, one 128-byte row segment per slice). The first kPexpCtas
+// CTAs of a batch instead reduce its exponent of P' (read along rows of P), as a biased exponent.
 // ----------------------------------------------------------------------------------------
 // The symmetry c_IJ of P' is taken between groups of GW = nao_split_tn(S, F) functions, whatever width the
 // contraction's tiles have: the digits, and so n, do not depend on the tuned width.
+
+constexpr int kPexpCtas = 4;  // CTAs per batch that reduce the exponent of P'
 
 template <typename V>
 struct StageOf {  // shared-memory staging type of the density slicer's input
@@ -372,9 +356,9 @@ struct StageOf<double> {
 
 // V = FF2: the split path's float-float phi (rows of ld_mult Ppad at scr_off[b]); V = double: the
 // density Hessian's FP64 evaluation (rows of 10 Ppad at eoff[b]), component row coff (phi or one
-// gradient component). pexp = 0 leaves the P' exponent (blockIdx.y = 0) to another launch.
+// gradient component). pexp = 0 leaves the P' exponent to another launch.
 template <int S, int F, typename V>
-__global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0, const V *__restrict__ scratch,
+__global__ void __launch_bounds__(256) slice_nphi_kernel(const __grid_constant__ DevSystem s, int32_t b0, const V *__restrict__ scratch,
                                                         const int64_t *__restrict__ eoff, int coff,
                                                         uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off,
                                                         const int32_t *__restrict__ expo_q, int32_t *__restrict__ expo_b,
@@ -384,7 +368,6 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
     constexpr int KS = nao_kstep_cols(F);
     // 8 more columns per K step: the two K steps that a half-warp reads at once lie in different banks
     __shared__ TT t[32][C + 8 * (C / KS) + 1];
-    __shared__ int red[8];
     const int b = b0 + blockIdx.x;
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
@@ -392,31 +375,28 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
     if (N == 0) return;
     const SplitGeom G(P, N, S, 0, F);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (blockIdx.y == 0) {
+    if (blockIdx.y < kPexpCtas) {
         if (!pexp) return;
-        // max |P'_ij| over i <= j (P' is P on the diagonal tiles, 2 P off them, 0 below unless
-        // full): the exponent field of |P| plus one off the diagonal tiles
+        // max |P'_ij| over i <= j (P' is P on the diagonal groups, 2 P off them, 0 below unless
+        // full): the exponent field of |P| plus one off the diagonal groups; each CTA takes every
+        // kPexpCtas-th set of eight rows (expo_b[b] is zero before: the evaluation clears it)
         const int m = s.sys.bmol[b];
         const int32_t *rel = s.rel_idx + s.rel_off[b];
         int mk = 0;
-        for (int i = warp; i < N; i += 8) {
+        for (int i = warp + 8 * (int)blockIdx.y; i < N; i += 8 * kPexpCtas) {
             const int64_t gi = rel[i];
+#pragma unroll 4
             for (int j = (full ? 0 : i) + lane; j < N; j += 32) {
                 const int64_t gj = rel[j];
                 const int eb = split_bits::biased_exponent(abs_bits(gi <= gj ? p_elem(s, m, gi, gj) : p_elem(s, m, gj, gi)));
-                if (eb != 0) mk = max(mk, eb + ((!full && i / GW < j / GW) ? 1 : 0));
+                mk = max(mk, eb + ((eb != 0 && !full && i / GW < j / GW) ? 1 : 0));
             }
         }
         mk = __reduce_max_sync(0xffffffffu, mk);
-        if (lane == 0) red[warp] = mk;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < 8; w++) mk = max(mk, red[w]);
-            expo_b[b] = split_bits::exponent_of_binade(mk);
-        }
+        if (lane == 0 && mk > 0) atomicMax(expo_b + b, mk);
         return;
     }
-    const int q0 = (blockIdx.y - 1) * 32;
+    const int q0 = ((int)blockIdx.y - kPexpCtas) * 32;
     if (q0 >= G.P16) return;
     const V *E = scratch + eoff[b] + (int64_t)coff * Ppad;  // row i at E + i ld_mult Ppad
     const int64_t ld = (int64_t)ld_mult * Ppad;
@@ -449,7 +429,7 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
 #pragma unroll
             for (int c = 0; c < LC; c++) x[c] = t[ql][(KS + 8) * (lane >> 3) + (lane & 7) + 8 * c];
             uint32_t wd[S];
-            lane_digit_words<S, F>(x, eq[h], wd);
+            lane_digit_words<S, F>(x, digit_scale<S, F>(x, eq[h]), wd);
             const uint32_t off = tc::sw128_byte((uint32_t)q, (uint32_t)(4 * lane));
 #pragma unroll
             for (int sl = 0; sl < S; sl++) *reinterpret_cast<uint32_t *>(base + G.nA_block(sl, kc) + off) = wd[sl];
@@ -463,7 +443,7 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(DevSystem s, int32_t b0
 // exponent from slice_nphi_kernel. One CTA per (batch, 16 rows j), one warp per row, 2 or 4
 // functions i per lane (slice_nphi_kernel's K order; one 128-byte row segment per slice).
 template <int S, int F>
-__global__ void __launch_bounds__(256) slice_np_kernel(DevSystem s, int32_t b0, uint8_t *__restrict__ slices,
+__global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ DevSystem s, int32_t b0, uint8_t *__restrict__ slices,
                                                       const int64_t *__restrict__ sl_off,
                                                       const int32_t *__restrict__ expo_b, int full) {
     const int b = b0 + blockIdx.x, m = s.sys.bmol[b];
@@ -475,7 +455,7 @@ __global__ void __launch_bounds__(256) slice_np_kernel(DevSystem s, int32_t b0, 
     const int j0 = blockIdx.y * 16;
     if (j0 >= G.R16) return;
     const int32_t *rel = s.rel_idx + s.rel_off[b];
-    const int e = expo_b[b];
+    const int e = split_bits::exponent_of_binade(expo_b[b]);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *base = slices + sl_off[b];
 #pragma unroll 1
@@ -531,7 +511,6 @@ __global__ void __launch_bounds__(256) slice_np_kernel(DevSystem s, int32_t b0, 
 // the density's K in whole steps: 10.8 and 3.8 ms.
 // ----------------------------------------------------------------------------------------
 constexpr int kMaxRing = 8;
-constexpr size_t kSmemOptin = 232448;  // shared memory a CTA may opt into on this GPU (227 KB)
 constexpr size_t kStaticSmem = 2048;   // room for the CTA's static shared memory (the PPipe barriers)
 
 // A-ring slots: as many 16 KB A tiles as fit beside the two B sets (S tiles of TN rows each),
@@ -1271,7 +1250,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (__any_sync(0xffffffffu, *abort != 0)) break;
             if (half == 0 && row_ok) {
-                const int eq = expo_q[h.p0 + q], eb = expo_b[h.b];
+                const int eq = expo_q[h.p0 + q], eb = split_bits::exponent_of_binade(expo_b[h.b]);
                 const bool live = eq > -10000 && eb > -10000;
                 const double sc = pow2(eq + eb - n_unit<F>());
                 if (MODE <= 2) *n_at(s, h.m, h.p0 + q) = live ? tot[0] * sc : 0.0;
@@ -1332,20 +1311,33 @@ __global__ void wait_timeout_probe_kernel(long long max_cycles, int32_t *__restr
 
 // Point exponents of the Hessian's four A operands (phi and the three gradient components, rows
 // c = 0..3 of the 10-row FP64 evaluation): expo4[c n_points + batch_off[b] + q] from the binade
-// of max_i |row c of function i at point q|. One CTA per batch.
-__global__ void __launch_bounds__(256) hess_point_expo_kernel(DevSystem s, int32_t b0, const double *__restrict__ scratch,
+// of max_i |row c of function i at point q|. Clears the batch's exponent of P' for slice_nphi_kernel.
+__global__ void __launch_bounds__(256) hess_point_expo_kernel(const __grid_constant__ DevSystem s, int32_t b0,
+                                                             const double *__restrict__ scratch,
                                                              const int64_t *__restrict__ hoff, int32_t *__restrict__ expo4,
-                                                             int64_t n_points) {
+                                                             int64_t n_points, int32_t *__restrict__ expo_b) {
     const int b = b0 + blockIdx.x;
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
     const int N = s.rel_off[b + 1] - s.rel_off[b];
     const double *E = scratch + hoff[b];
     const int64_t ld = 10 * (int64_t)Ppad;
-    for (int idx = threadIdx.x; idx < 4 * P; idx += blockDim.x) {
-        const int c = idx / P, q = idx - c * P;
-        int mx = 0;
-        for (int i = 0; i < N; i++) mx = max(mx, split_bits::biased_exponent(abs_bits(E[i * ld + (int64_t)c * Ppad + q])));
+    // blockIdx.y: component and 32-point tile; the eight warps share the rows, a lane per point
+    __shared__ int red[8][32];
+    const int c = blockIdx.y & 3, q = 32 * (blockIdx.y >> 2) + (threadIdx.x & 31), warp = threadIdx.x >> 5;
+    if (blockIdx.y == 0 && threadIdx.x == 0) expo_b[b] = 0;
+    if (32 * (int)(blockIdx.y >> 2) >= P) return;
+    int mx = 0;
+    if (q < P) {
+        const double *col = E + (int64_t)c * Ppad + q;
+#pragma unroll 8
+        for (int i = warp; i < N; i += 8) mx = max(mx, split_bits::biased_exponent(abs_bits(__ldg(col + i * ld))));
+    }
+    red[warp][threadIdx.x & 31] = mx;
+    __syncthreads();
+    if (warp == 0 && q < P) {
+#pragma unroll
+        for (int w = 1; w < 8; w++) mx = max(mx, red[w][threadIdx.x]);
         expo4[c * n_points + p0 + q] = split_bits::exponent_of_binade(mx);
     }
 }
@@ -1419,11 +1411,21 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
                            int32_t *neg16, int S, int F, cudaStream_t st) {
     if (b1 <= b0 || max_rt <= 0) return cudaSuccess;
     const FF2 *ev = reinterpret_cast<const FF2 *>(scratch);  // the split path's evaluation: float-float values
-#define NAO_SLICE_H(SS, FF) \
-    slice_h_kernel<SS, FF><<<dim3(b1 - b0, max_rt), 256, 0, st>>>(s, b0, ev, terms, slices, sl_off, expo, neg16)
+    const size_t sm = slice_h_smem(s.max_ppad, F);
+    static_assert(slice_h_smem(NAO_SPLIT_MAX_PPAD, 0) + 1024 <= kSmemOptin && slice_h_smem(NAO_SPLIT_MAX_PPAD, 1) + 1024 <= kSmemOptin,
+                  "the H slicer's rows exceed shared memory");
+    cudaError_t e = cudaSuccess;
+#define NAO_SLICE_H(SS, FF)                                                                                          \
+    {                                                                                                                \
+        if (sm > 48 * 1024)                                                                                          \
+            e = cudaFuncSetAttribute(slice_h_kernel<SS, FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);  \
+        if (e == cudaSuccess)                                                                                        \
+            slice_h_kernel<SS, FF><<<dim3(b1 - b0, max_rt), 32 * kSliceWarps, sm, st>>>(s, b0, ev, terms, slices, sl_off, expo, \
+                                                                                         neg16);                    \
+    }
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_H)
 #undef NAO_SLICE_H
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_h_tc(const DevSystem &s, const HTask *work, int32_t w0, int32_t n_work, const uint8_t *slices,
@@ -1448,9 +1450,9 @@ cudaError_t launch_slice_n(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
                            int32_t *expo_b, int S, int F, bool grad, cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
     const FF2 *ev = reinterpret_cast<const FF2 *>(scratch);
-    // y = 0: the exponent of P'; y >= 1: 32-point tiles (128 max_qt >= P16)
+    // y < kPexpCtas: the exponent of P'; above: 32-point tiles (128 max_qt >= P16)
 #define NAO_SLICE_NPHI(SS, FF)                                                                            \
-    slice_nphi_kernel<SS, FF, FF2><<<dim3(b1 - b0, 4 * max_qt + 1), 256, 0, st>>>(                        \
+    slice_nphi_kernel<SS, FF, FF2><<<dim3(b1 - b0, 4 * max_qt + kPexpCtas), 256, 0, st>>>(                        \
         s, b0, ev, s.scr_off, 0, slices, sl_off, expo_q, expo_b, grad ? 4 : 1, grad ? 1 : 0, 1)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NPHI)
 #undef NAO_SLICE_NPHI
@@ -1470,7 +1472,7 @@ cudaError_t launch_slice_n_hess(const DevSystem &s, int32_t b0, int32_t b1, int3
     if (b1 <= b0) return cudaSuccess;
     const int first = comp == 0 ? 1 : 0;  // P' (its exponent and its slices) once, with the first pass
 #define NAO_SLICE_NPHI(SS, FF)                                                                                   \
-    slice_nphi_kernel<SS, FF, double><<<dim3(b1 - b0, 4 * max_qt + 1), 256, 0, st>>>(                            \
+    slice_nphi_kernel<SS, FF, double><<<dim3(b1 - b0, 4 * max_qt + kPexpCtas), 256, 0, st>>>(                            \
         s, b0, scratch, hoff, comp, slices, sl_off, expo_q, expo_b, 10, 1, first)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NPHI)
 #undef NAO_SLICE_NPHI
@@ -1484,9 +1486,10 @@ cudaError_t launch_slice_n_hess(const DevSystem &s, int32_t b0, int32_t b1, int3
 }
 
 cudaError_t launch_hess_point_expo(const DevSystem &s, int32_t b0, int32_t b1, const double *scratch, const int64_t *hoff,
-                                   int32_t *expo4, int64_t n_points, cudaStream_t st) {
+                                   int32_t *expo4, int64_t n_points, int32_t *expo_b, cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
-    hess_point_expo_kernel<<<b1 - b0, 256, 0, st>>>(s, b0, scratch, hoff, expo4, n_points);
+    hess_point_expo_kernel<<<dim3(b1 - b0, 4 * ((s.max_ppad + 31) / 32)), 256, 0, st>>>(s, b0, scratch, hoff, expo4, n_points,
+                                                                                      expo_b);
     return cudaGetLastError();
 }
 
