@@ -777,50 +777,29 @@ nao_status split_lists(nao_grid *g) {
     g->split_lists_ver++;
     std::vector<HTask> hw[2];
     BlockPairs pairs;
-    int sms = 1;
-    NAO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device));
     std::vector<HWork> nw[2];
     for (auto &c : g->split_chunks) {
         for (int k = 0; k < 2; k++) {
             c.hw0[k] = (int32_t)hw[k].size();
             c.nw0[k] = (int32_t)nw[k].size();
         }
-        auto add_h = [&](int segments) {
-            for (int k = 0; k < 2; k++) hw[k].resize(c.hw0[k]);
-            for (int32_t b = c.b0; b < c.b1; b++) {
-                const int TN = g->split_tn[b], k = TN == 48 ? 0 : 1;
-                if (g->Nb[b] > 0) nao_split_h_items(b, g->Pb[b], g->Nb[b], TN, S, hw[k], pairs, F, segments);
-            }
-            return (int64_t)(hw[0].size() - c.hw0[0] + hw[1].size() - c.hw0[1]);
-        };
-        // A launch of few items leaves SMs idle in its last (or only) wave: K is cut into as many
-        // segments (up to 4) as make ceil(items / SMs) waves of 1 / segments of an item's length
-        // shortest, with a tenth of an item for each segment's read-out and scatter. Measured on the
-        // 3-atom molecule (58 items): its H contraction 0.063 -> 0.045 ms.
-        const int64_t items = add_h(1);
-        if (items < 4 * sms) {
-            int best = 1;
-            double cost = 1e300;
-            for (int q = 1; q <= 4; q++) {
-                const double t = (double)((items * q + sms - 1) / sms) * (1.0 / q + 0.1);
-                if (t < cost) {
-                    cost = t;
-                    best = q;
-                }
-            }
-            if (best > 1) add_h(best);
-        }
         for (int32_t b = c.b0; b < c.b1; b++) {
             const int P = g->Pb[b], N = g->Nb[b];
             if (N == 0) continue;
             const int TN = g->split_tn[b], k = TN == 48 ? 0 : 1;
             const SplitGeom G(P, N, S, TN, F);
+            nao_split_h_items(b, P, N, TN, S, hw[k], pairs, F);
             for (int Q = 0; Q < G.n_qt; Q++) nw[k].push_back({b, Q, G.n_jtN, 0});  // all J tiles in one CTA
         }
         // the persistent contraction kernels take items round-robin: heaviest first (H: longest
         // K, i.e. most K chunks in the item's segment; density: most function tiles), so that
         // every CTA gets a similar share
-        auto item_kc = [](const HTask &x) { return x.kc1() - x.kc0(); };
+        auto item_kc = [&](const HTask &x) {
+            const SplitGeom G(g->Pb[x.batch], g->Nb[x.batch], S, 0, F);
+            int kc0, kc1;
+            nao_split_h_seg_range(G.n_kc, nao_split_h_nseg(g->Pb[x.batch], S, F), x.seg(), S, kc0, kc1, F);
+            return kc1 - kc0;
+        };
         for (int k = 0; k < 2; k++) {
             std::stable_sort(hw[k].begin() + c.hw0[k], hw[k].end(),
                              [&](const HTask &x, const HTask &y) { return item_kc(x) > item_kc(y); });
@@ -832,17 +811,8 @@ nao_status split_lists(nao_grid *g) {
     }
     // one array per list: width-48 items, then width-32 items (offsets shifted below)
     const int64_t nh = (int64_t)(hw[0].size() + hw[1].size()), nn = (int64_t)(nw[0].size() + nw[1].size());
-    // the lists grow when the tuned widths need more items; an outgrown one stays in g->allocs until the
-    // handle is destroyed, as kernels in flight may still read it
-    nao_status st;
-    if (nh > g->cap_split_hw || !g->d_split_hw) {
-        if ((st = dev_alloc(g, &g->d_split_hw, (size_t)std::max<int64_t>(nh, 1)))) return st;
-        g->cap_split_hw = std::max<int64_t>(nh, 1);
-    }
-    if (nn > g->cap_split_nw || !g->d_split_nw) {
-        if ((st = dev_alloc(g, &g->d_split_nw, (size_t)std::max<int64_t>(nn, 1)))) return st;
-        g->cap_split_nw = std::max<int64_t>(nn, 1);
-    }
+    if (nh > g->cap_split_hw || nn > g->cap_split_nw)
+        return fail(NAO_ERR_INTERNAL, "split work lists exceed their planned capacity");
     for (auto &c : g->split_chunks) {
         c.hw0[1] += (int32_t)hw[0].size();
         c.hw1[1] += (int32_t)hw[0].size();
@@ -895,7 +865,9 @@ nao_status split_setup(nao_grid *g) {
     const int64_t budget =
         std::max<int64_t>(3 * (g->opt.scratch_bytes > 0 ? g->opt.scratch_bytes : kDefaultScratch), int64_t(1) << 20);
     std::vector<int64_t> off_h(g->n_batches, 0), off_n(g->n_batches, 0);
-    int64_t max_used = 0;
+    int64_t max_used = 0, cap_h = 0, cap_n = 0;
+    BlockPairs pairs;
+    std::vector<HTask> tmp;
     g->split_tn.assign(g->n_batches, 32);
     for (const Chunk &c : g->chunks) {
         nao_grid::SplitChunk cur{};
@@ -920,6 +892,16 @@ nao_status split_setup(nao_grid *g) {
             if (N > 0) {
                 cur.max_rt = std::max<int32_t>(cur.max_rt, G.h_slice_tiles());
                 cur.max_qt = std::max<int32_t>(cur.max_qt, G.n_qt);
+                // list capacity: the larger of the two widths' item counts
+                int64_t best_h = 0;
+                for (int TN : {48, 32}) {
+                    if (TN == 48 && nao_split_tn(S, F) != 48) continue;
+                    tmp.clear();
+                    nao_split_h_items(b, P, N, TN, S, tmp, pairs, F);
+                    best_h = std::max(best_h, (int64_t)tmp.size());
+                }
+                cap_h += best_h;
+                cap_n += G.n_qt;
             }
         }
         cur.b1 = c.b1;
@@ -932,8 +914,12 @@ nao_status split_setup(nao_grid *g) {
         (st = dev_alloc(g, &g->d_expo_h, (size_t)std::max<int64_t>(g->rel_total, 1))) ||
         (st = dev_alloc(g, &g->d_expo_q, (size_t)g->n_points)) ||
         (st = dev_alloc(g, &g->d_expo_b, (size_t)g->n_batches)) ||
-        (st = dev_alloc(g, &g->d_neg16, (size_t)g->n_batches)))
+        (st = dev_alloc(g, &g->d_neg16, (size_t)g->n_batches)) ||
+        (st = dev_alloc(g, &g->d_split_hw, (size_t)std::max<int64_t>(cap_h, 1))) ||
+        (st = dev_alloc(g, &g->d_split_nw, (size_t)std::max<int64_t>(cap_n, 1))))
         return st;
+    g->cap_split_hw = cap_h;
+    g->cap_split_nw = cap_n;
     g->split_S = S;
     g->split_F = F;
     g->split_tuned = nao_split_tn(S, F) != 48 || !g->opt.autotune;  // only one width exists, or tuning is off

@@ -220,27 +220,25 @@ struct HWork {  // one upper-triangular tile pair of one batch's h[B] (Eq. batch
     int32_t batch, ti, tj, pad;
 };
 
-// One item of the split H contraction: 128 x TN elements of one batch's h[B], over the K chunks
-// [kc0, kc1) of one K segment (below). The 128 rows are four blocks of 32 functions, any four of the batch (kNoRows: none), and the
+// One item of the split H contraction: 128 x TN elements of one batch's h[B], over one K segment
+// (below). The 128 rows are four blocks of 32 functions, any four of the batch (kNoRows: none), and the
 // columns the TN-function tile tj.
 constexpr uint32_t kNoRows = 0xFFFFu;
 struct HTask {
     int32_t batch;
-    uint32_t tj_kc;     // tj | kc0 << 16 | kc1 << 24
+    uint32_t tj_seg;    // tj | segment << 16
     uint32_t r01, r23;  // row blocks 0 | 1 << 16, 2 | 3 << 16
-    __host__ __device__ int tj() const { return (int)(tj_kc & 0xFFFFu); }
-    __host__ __device__ int kc0() const { return (int)(tj_kc >> 16 & 0xFFu); }
-    __host__ __device__ int kc1() const { return (int)(tj_kc >> 24); }
+    __host__ __device__ int tj() const { return (int)(tj_seg & 0xFFFFu); }
+    __host__ __device__ int seg() const { return (int)(tj_seg >> 16); }
     __host__ __device__ uint32_t row(int x) const { return ((x < 2 ? r01 : r23) >> (16 * (x & 1))) & 0xFFFFu; }
 };
 
 // K segments of the split H contraction. A slice-order group's FP32 accumulator sums K products
 // of at most 2^(2 bits - 2) for each of its g + 1 <= S slice pairs; it stays an exact integer
 // while K S 2^(2 bits - 2) < 2^24 (nao_exact_ks). A batch whose 4 Ppad weighted columns meet that
-// bound is one accumulation; a larger batch is accumulated in segments of at most nao_split_kc_seg(S, F)
+// bound is one accumulation; a larger batch is accumulated in segments of nao_split_kc_seg(S, F)
 // K chunks, each recombined and scattered into H on its own (H is a sum over K, so the segments'
-// FP64 partial sums simply add; Eq. H_decomp). Batches of a small system are cut into more segments, so
-// that their items fill the GPU (split_lists).
+// FP64 partial sums simply add; Eq. H_decomp).
 __host__ __device__ constexpr int nao_split_kc_seg(int S, int F = NAO_DIGITS_BF16) {
     return (nao_exact_ks(F) - 1) / (nao_chunk_cols(F) * S);
 }
@@ -251,18 +249,29 @@ __host__ __device__ inline int nao_split_h_nseg(int P, int S, int F = NAO_DIGITS
     const int n_kc = (4 * Ppad + nao_kstep_cols(F) + C - 1) / C, kcs = nao_split_kc_seg(S, F);
     return (n_kc + kcs - 1) / kcs;
 }
+// K chunks [kc0, kc1) of segment seg of a batch with n_kc chunks.
+__host__ __device__ inline void nao_split_h_seg_range(int n_kc, int nseg, int seg, int S, int &kc0, int &kc1,
+                                                      int F = NAO_DIGITS_BF16) {
+    if (nseg <= 1) {
+        kc0 = 0;
+        kc1 = n_kc;
+        return;
+    }
+    const int kcs = nao_split_kc_seg(S, F);
+    kc0 = seg * kcs;
+    kc1 = kc0 + kcs < n_kc ? kc0 + kcs : n_kc;
+}
+
 // Split H items of one batch (P points, N functions) for tile width TN and S slices, once per K
 // segment (partition.cpp). h is symmetric, so every unordered pair of functions is wanted once.
 // TN = 48: per 128-row tile I the column tiles J >= floor(128 I / TN) (those reaching the upper triangle).
 // TN = 32: rows and columns are cut into the same 32-function blocks, and every pair of blocks {a, b} is
 // given to one of the two columns, a or b, so that the columns' row counts (their own block included) fill
 // their items of four: max(n, ceil(n (n + 1) / 8)) items for n blocks, against sum_I (n - 4 I) when
-// every pair went to the later block's column (N = 200: 7 against 10). segments: at least so many K
-// segments (as far as there are K chunks).
+// every pair went to the later block's column (N = 200: 7 against 10).
 // kept: the assignments made so far, by n (one list's scratch).
 using BlockPairs = std::map<int, std::vector<std::vector<int>>>;
-void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HTask> &out, BlockPairs &kept, int F,
-                       int segments = 1);
+void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HTask> &out, BlockPairs &kept, int F);
 // The rows of each of n blocks' columns in that assignment, its own block first, then in cyclic order.
 std::vector<std::vector<int>> nao_block_pairs(int n);
 struct DWork {  // one tile of points of one batch for the density
@@ -353,7 +362,7 @@ struct nao_grid {
     std::vector<int32_t> split_tn;
     bool split_tuned = false;
     int32_t tune_buckets = 0;      // buckets the autotuner timed
-    int64_t cap_split_hw = 0, cap_split_nw = 0;  // entries that the lists below hold
+    int64_t cap_split_hw = 0, cap_split_nw = 0;
     HTask *d_tune_hw = nullptr;    // scratch work list of the autotuner
     int64_t cap_tune_hw = 0;
     uint8_t *d_slices = nullptr;

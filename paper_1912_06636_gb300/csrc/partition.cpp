@@ -153,13 +153,11 @@ std::vector<std::vector<int>> nao_block_pairs(int n) {
     return rows;
 }
 
-void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HTask> &out, BlockPairs &kept, int F,
-                       int segments) {
-    const int n_kc = SplitGeom(P, N, S, TN, F).n_kc;
-    const int nseg = std::min(n_kc, std::max(segments, nao_split_h_nseg(P, S, F))), per = (n_kc + nseg - 1) / nseg;
+void nao_split_h_items(int32_t b, int P, int N, int TN, int S, std::vector<HTask> &out, BlockPairs &kept, int F) {
+    const int nseg = nao_split_h_nseg(P, S, F);
     auto add = [&](int j, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
-        for (int k = 0; k < n_kc; k += per)  // segments of equal length, so none above the exact one
-            out.push_back({b, (uint32_t)j | (uint32_t)k << 16 | (uint32_t)std::min(n_kc, k + per) << 24, r0 | r1 << 16, r2 | r3 << 16});
+        for (int q = 0; q < nseg; q++)
+            out.push_back({b, (uint32_t)j | (uint32_t)q << 16, r0 | r1 << 16, r2 | r3 << 16});
     };
     const int nr = (N + 31) / 32;
     if (TN != 32) {

@@ -846,8 +846,7 @@ __device__ __forceinline__ HItem h_item(const DevSystem &s, const HTask *work, i
     h.b0 = h.base + (size_t)h.tj * TN * 128;
     h.b_bytes = (uint32_t)min(TN, G.R16 - h.tj * TN) * 128u;
     h.n_kc = G.n_kc;
-    h.kc0 = it.kc0();
-    h.kc1 = it.kc1();
+    nao_split_h_seg_range(G.n_kc, nao_split_h_nseg(P, S, F), it.seg(), S, h.kc0, h.kc1, F);
     h.neg16 = neg16[h.b];
     return h;
 }

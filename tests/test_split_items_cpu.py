@@ -1,5 +1,5 @@
 """The split Hamiltonian's work items (csrc/partition.cpp): every pair of functions of a batch is computed
-exactly once per K chunk, in no more items than the blocks need."""
+exactly once per K segment, in no more items than the blocks need."""
 import subprocess
 from pathlib import Path
 
@@ -13,20 +13,15 @@ MAIN = r"""
 #include <cstdlib>
 #include "nao_internal.h"
 int main(int argc, char **argv) {
-    const int TN = atoi(argv[1]), S = atoi(argv[2]), F = atoi(argv[3]), P = atoi(argv[4]), want = atoi(argv[5]);
+    const int TN = atoi(argv[1]), S = atoi(argv[2]), F = atoi(argv[3]), P = atoi(argv[4]);
     BlockPairs kept;
-    for (int a = 6; a < argc; a++) {
-        const int N = atoi(argv[a]), nr = (N + 31) / 32, n_kc = SplitGeom(P, N, S, TN, F).n_kc;
+    for (int a = 5; a < argc; a++) {
+        const int N = atoi(argv[a]), nseg = nao_split_h_nseg(P, S, F), nr = (N + 31) / 32;
         std::vector<HTask> items;
-        nao_split_h_items(7, P, N, TN, S, items, kept, F, want);
-        std::vector<unsigned char> hit((size_t)n_kc * N * N, 0);
-        int nseg = 0;
+        nao_split_h_items(7, P, N, TN, S, items, kept, F);
+        std::vector<unsigned char> hit((size_t)nseg * N * N, 0);
         for (const HTask &t : items) {
-            if (t.batch != 7 || t.kc0() < 0 || t.kc1() <= t.kc0() || t.kc1() > n_kc) return 2;
-            // exact FP32 sums: K S 2^(2 bits - 2) < 2^24
-            const int K = 4 * ((P + 15) / 16 * 16), k = (t.kc1() - t.kc0()) * nao_chunk_cols(F);
-            if ((k < K ? k : K) * S >= nao_exact_ks(F)) return 7;
-            if (t.kc0() == 0 && t.tj() == 0 && t.row(0) == 0) nseg = (n_kc + t.kc1() - 1) / t.kc1();
+            if (t.batch != 7 || t.seg() >= nseg) return 2;
             for (int x = 0; x < 4; x++) {
                 const uint32_t r = t.row(x);
                 if (r == kNoRows) continue;
@@ -35,12 +30,12 @@ int main(int argc, char **argv) {
                     for (int j = t.tj() * TN; j < (t.tj() + 1) * TN && j < N; j++) {
                         // the kernel's rule: off-diagonal blocks of the 32-wide form are whole, the rest j >= i
                         if (!(TN == 32 && (int)r != t.tj()) && j < i) continue;
-                        for (int k = t.kc0(); k < t.kc1(); k++)
-                            if (hit[((size_t)k * N + (i < j ? i : j)) * N + (i < j ? j : i)]++) return 4;
+                        unsigned char &h = hit[((size_t)t.seg() * N + (i < j ? i : j)) * N + (i < j ? j : i)];
+                        if (h++) return 4;
                     }
             }
         }
-        for (int q = 0; q < n_kc; q++)
+        for (int q = 0; q < nseg; q++)
             for (int i = 0; i < N; i++)
                 for (int j = i; j < N; j++)
                     if (hit[((size_t)q * N + i) * N + j] != 1) return 5;
@@ -63,11 +58,10 @@ def program(tmp_path_factory):
     return str(d / "items")
 
 
-@pytest.mark.parametrize("TN,S,F,P,segments", [(32, 14, 1, 200, 1), (32, 12, 0, 200, 1), (32, 12, 0, 512, 1), (48, 10, 0, 200, 1),
-                                               (48, 4, 0, 512, 1), (32, 14, 1, 200, 3), (32, 12, 0, 20, 4), (32, 12, 0, 512, 4)])
-def test_every_pair_once(program, TN, S, F, P, segments):
+@pytest.mark.parametrize("TN,S,F,P", [(32, 14, 1, 200), (32, 12, 0, 200), (32, 12, 0, 512), (48, 10, 0, 200), (48, 4, 0, 512)])
+def test_every_pair_once(program, TN, S, F, P):
     # edges of the 32- and 48-function blocks and of 128 rows, odd and even block counts, large bases
     sizes = [1, 15, 16, 31, 32, 33, 47, 48, 49, 64, 65, 95, 96, 97, 127, 128, 129, 160, 161, 200, 224, 225, 256, 257, 320, 384,
-             440, 510, 570, 768, 1000]
-    r = subprocess.run([program, str(TN), str(S), str(F), str(P), str(segments), *map(str, sizes)], capture_output=True)
+             440, 510, 570, 768, 1000, 1343]
+    r = subprocess.run([program, str(TN), str(S), str(F), str(P), *map(str, sizes)], capture_output=True)
     assert r.returncode == 0, r.returncode
