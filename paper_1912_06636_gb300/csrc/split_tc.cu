@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ D
 // ----------------------------------------------------------------------------------------
 // Slice-product pipeline of the persistent contraction kernels, ten warps. Shared memory: a ring of
 // ring_slots(S) A-tile buffers (128 rows of 128 B, 16 KB, one slice of one K chunk each) and two sets
-// of S B-tile buffers (TN rows, TN x 128 B). Producer (warp 8, one lane): for each K chunk, the S B
+// of S B-tile buffers (TN rows, TN x 128 B). Producer (warp 8): for each K chunk, the S B
 // slices into B set kc % 2, then the S A slices one by one into the ring, each copy a bulk (TMA)
 // transfer completing on a "full" mbarrier. MMA issuer (warp 9): for each A slice s, the pairs (s, t)
 // with s + t < S as one 128 x TN(S-s) MMA per K step (two where TN(S-s) > 256) into accumulator groups
@@ -508,7 +508,10 @@ __global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ D
 // MMA issue and the serial part of the readers (tensor memory holds one accumulator set) decided, not the
 // operands' supply: the issuer runs with its whole warp, so that descriptors stay in uniform registers,
 // and eight warps read with 32-bit integer and FP32 arithmetic. With the H items of nao_split_h_items and
-// the density's K in whole steps: 10.8 and 3.8 ms.
+// the density's K in whole steps: 10.9 and 3.8 ms. Of these 9.8 ms were the H producer's alone (9.4 with a
+// quarter of the bytes, 4.8 with one copy per slice): it was one lane of a diverged warp, where every operand of
+// a copy costs a loop over lanes. Issued by the converged warp the copies alone take 3.9 ms, H 8.6 and n 3.6 ms
+// (12 bf16 slices: H 18.1 -> 13.0); H is now at its MMAs, 8.3 ms without the readers' work.
 // ----------------------------------------------------------------------------------------
 constexpr int kMaxRing = 8;
 constexpr size_t kStaticSmem = 2048;   // room for the CTA's static shared memory (the PPipe barriers)
@@ -873,61 +876,71 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     volatile int *abort = &pp.abort;
 
     if (warp == kReaders) {
-        // ---- producer ----
-        if (lane == 0) {
-            int gk = 0;
-            RingPos pos;
-            pos.ph = 1u;  // the parity that an unused slot's "empty" barrier passes
-            for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x) {
-                const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
-                // the A tile's row blocks as runs of consecutive ones: tile offset, source offset, bytes
-                uint32_t run_to[4], run_at[4], run_n[4], a_bytes = 0;
-                int nrun = 0;
+        // ---- producer (the whole warp; one lane's copies take effect) ----
+        const uint32_t lead = tc::elect_one(), sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
+        const uint32_t fullA = tc::smem_addr(pp.fullA), fullB = tc::smem_addr(pp.fullB);
+        int gk = 0;
+        RingPos pos;
+        pos.ph = 1u;  // the parity that an unused slot's "empty" barrier passes
+        bool ok = __all_sync(0xffffffffu, *abort == 0);
+        for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
+            const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
+            // the A tile's row blocks as runs of consecutive ones: tile offset, source offset, bytes
+            uint32_t run_to[4], run_at[4], run_n[4], a_bytes = 0;
+            int nrun = 0;
 #pragma unroll
-                for (int x = 0; x < 4; x++) {
-                    run_to[x] = run_at[x] = run_n[x] = 0;
-                    const uint32_t r = h.task.row(x);
-                    if (r == kNoRows) continue;
-                    const uint32_t at = r * 4096u, n = (uint32_t)min(32, h.R16 - (int)r * 32) * 128u;
-                    a_bytes += n;
-                    bool joined = false;
+            for (int x = 0; x < 4; x++) {
+                run_to[x] = run_at[x] = run_n[x] = 0;
+                const uint32_t r = h.task.row(x);
+                if (r == kNoRows) continue;
+                const uint32_t at = r * 4096u, n = (uint32_t)min(32, h.R16 - (int)r * 32) * 128u;
+                a_bytes += n;
+                bool joined = false;
 #pragma unroll
-                    for (int y = 0; y < 4; y++)
-                        if (y == nrun - 1 && run_at[y] + run_n[y] == at && run_to[y] + run_n[y] == x * 4096u) {
-                            run_n[y] += n;
-                            joined = true;
-                        }
-                    if (joined) continue;
-#pragma unroll
-                    for (int y = 0; y < 4; y++)
-                        if (y == nrun) {
-                            run_to[y] = x * 4096u;
-                            run_at[y] = at;
-                            run_n[y] = n;
-                        }
-                    nrun++;
-                }
-                for (int kc = h.kc0; kc < h.kc1; kc++, gk++) {
-                    const int bb = gk & 1, ub = gk >> 1;
-                    if (ub >= 1 && !tc::mbar_wait(&pp.emptyB[bb], (ub - 1) & 1, kWaitCycles)) { *abort = 1; break; }
-                    tc::mbar_arrive_expect_tx(&pp.fullB[bb], (uint32_t)S * h.b_bytes);
-                    for (int t = 0; t < S; t++)
-                        tc::bulk_g2s(sB + ((size_t)bb * S + t) * B_BLOCK, h.b0 + ((size_t)t * h.n_kc + kc) * h.blk,
-                                     h.b_bytes, &pp.fullB[bb]);
-                    for (int sa = 0; sa < S; sa++) {
-                        if (!tc::mbar_wait(&pp.emptyA[pos.a], pos.ph, kWaitCycles)) { *abort = 1; break; }
-                        tc::mbar_arrive_expect_tx(&pp.fullA[pos.a], a_bytes);
-                        const uint8_t *src = h.base + ((size_t)sa * h.n_kc + kc) * h.blk;
-                        uint8_t *dst = sA + (size_t)pos.a * 16384;
-#pragma unroll
-                        for (int y = 0; y < 4; y++)
-                            if (y < nrun) tc::bulk_g2s(dst + run_to[y], src + run_at[y], run_n[y], &pp.fullA[pos.a]);
-                        pos.next(RING);
+                for (int y = 0; y < 4; y++)
+                    if (y == nrun - 1 && run_at[y] + run_n[y] == at && run_to[y] + run_n[y] == x * 4096u) {
+                        run_n[y] += n;
+                        joined = true;
                     }
-                    if (*abort) break;
+                if (joined) continue;
+#pragma unroll
+                for (int y = 0; y < 4; y++)
+                    if (y == nrun) {
+                        run_to[y] = x * 4096u;
+                        run_at[y] = at;
+                        run_n[y] = n;
+                    }
+                nrun++;
+            }
+            const size_t step = (size_t)h.n_kc * h.blk;  // from one slice to the next
+            for (int kc = h.kc0; kc < h.kc1 && ok; kc++, gk++) {
+                const int bb = gk & 1, ub = gk >> 1;
+                if (ub >= 1) ok = warp_wait(&pp.emptyB[bb], (ub - 1) & 1);
+                if (!ok) break;
+                tc::mbar_arrive_expect_tx(lead, fullB + 8u * bb, (uint32_t)S * h.b_bytes);
+                const uint8_t *src = h.b0 + (size_t)kc * h.blk;
+                uint32_t dst = sB_addr + (uint32_t)(bb * S) * B_BLOCK;
+                for (int t = 0; t < S; t++, src += step, dst += B_BLOCK)
+                    tc::bulk_g2s(lead, dst, src, h.b_bytes, fullB + 8u * bb);
+                src = h.base + (size_t)kc * h.blk;
+                for (int sa = 0; sa < S; sa++, src += step) {
+                    ok = warp_wait(&pp.emptyA[pos.a], pos.ph);
+                    if (!ok) break;
+                    const uint32_t bar = fullA + 8u * pos.a;
+                    dst = sA_addr + (uint32_t)pos.a * 16384u;
+                    tc::mbar_arrive_expect_tx(lead, bar, a_bytes);
+                    tc::bulk_g2s(lead, dst + run_to[0], src + run_at[0], run_n[0], bar);
+                    if (nrun > 1) {
+#pragma unroll
+                        for (int y = 1; y < 4; y++)
+                            if (y < nrun) tc::bulk_g2s(lead, dst + run_to[y], src + run_at[y], run_n[y], bar);
+                    }
+                    pos.next(RING);
                 }
             }
+            ok = ok && __all_sync(0xffffffffu, *abort == 0);
         }
+        if (!ok && lane == 0) *abort = 1;
         __syncwarp();
     } else if (warp == kReaders + 1) {
         // ---- MMA issuer (the whole warp; one lane's tcgen05 instructions take effect) ----
@@ -1094,35 +1107,41 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
     if (warp == kReaders) {
         // ---- producer ----
-        if (lane == 0) {
-            int gk = 0;
-            RingPos pos;
-            pos.ph = 1u;
-            for (int w = blockIdx.x; w < n_work && !*abort; w += gridDim.x) {
-                const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
-                for (int J = 0; J < h.nJ && !*abort; J++) {
-                    const int nk = (n_item_ks<TN, GRADN, F>(h, J, S) + 3) / 4;
-                    const uint8_t *bJ = h.b0 + (size_t)J * TN * 128;
-                    const uint32_t b_bytes = (uint32_t)min(TN, h.R16 - J * TN) * 128u;
-                    for (int kc = 0; kc < nk; kc++, gk++) {
-                        const int bb = gk & 1, ub = gk >> 1;
-                        if (ub >= 1 && !tc::mbar_wait(&pp.emptyB[bb], (ub - 1) & 1, kWaitCycles)) { *abort = 1; break; }
-                        tc::mbar_arrive_expect_tx(&pp.fullB[bb], (uint32_t)S * b_bytes);
-                        for (int t = 0; t < S; t++)
-                            tc::bulk_g2s(sB + ((size_t)bb * S + t) * B_BLOCK, bJ + t * h.b_s + kc * h.b_kc, b_bytes,
-                                         &pp.fullB[bb]);
-                        for (int sa = 0; sa < S; sa++) {
-                            if (!tc::mbar_wait(&pp.emptyA[pos.a], pos.ph, kWaitCycles)) { *abort = 1; break; }
-                            tc::mbar_arrive_expect_tx(&pp.fullA[pos.a], h.a_bytes);
-                            tc::bulk_g2s(sA + (size_t)pos.a * 16384, h.a0 + sa * h.a_s + kc * h.a_kc, h.a_bytes,
-                                         &pp.fullA[pos.a]);
-                            pos.next(RING);
-                        }
-                        if (*abort) break;
+        const uint32_t lead = tc::elect_one(), sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
+        const uint32_t fullA = tc::smem_addr(pp.fullA), fullB = tc::smem_addr(pp.fullB);
+        int gk = 0;
+        RingPos pos;
+        pos.ph = 1u;
+        bool ok = __all_sync(0xffffffffu, *abort == 0);
+        for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
+            const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
+            for (int J = 0; J < h.nJ && ok; J++) {
+                const int nk = (n_item_ks<TN, GRADN, F>(h, J, S) + 3) / 4;
+                const uint8_t *bJ = h.b0 + (size_t)J * TN * 128;
+                const uint32_t b_bytes = (uint32_t)min(TN, h.R16 - J * TN) * 128u;
+                for (int kc = 0; kc < nk && ok; kc++, gk++) {
+                    const int bb = gk & 1, ub = gk >> 1;
+                    if (ub >= 1) ok = warp_wait(&pp.emptyB[bb], (ub - 1) & 1);
+                    if (!ok) break;
+                    tc::mbar_arrive_expect_tx(lead, fullB + 8u * bb, (uint32_t)S * b_bytes);
+                    const uint8_t *src = bJ + kc * h.b_kc;
+                    uint32_t dst = sB_addr + (uint32_t)(bb * S) * B_BLOCK;
+                    for (int t = 0; t < S; t++, src += h.b_s, dst += B_BLOCK)
+                        tc::bulk_g2s(lead, dst, src, b_bytes, fullB + 8u * bb);
+                    src = h.a0 + kc * h.a_kc;
+                    for (int sa = 0; sa < S; sa++, src += h.a_s) {
+                        ok = warp_wait(&pp.emptyA[pos.a], pos.ph);
+                        if (!ok) break;
+                        const uint32_t bar = fullA + 8u * pos.a;
+                        tc::mbar_arrive_expect_tx(lead, bar, h.a_bytes);
+                        tc::bulk_g2s(lead, sA_addr + (uint32_t)pos.a * 16384u, src, h.a_bytes, bar);
+                        pos.next(RING);
                     }
                 }
+                ok = ok && __all_sync(0xffffffffu, *abort == 0);
             }
         }
+        if (!ok && lane == 0) *abort = 1;
         __syncwarp();
     } else if (warp == kReaders + 1) {
         // ---- MMA issuer ----
@@ -1160,7 +1179,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         uint32_t t = 0, x = 0;  // accumulations read, exchanges made
         const int quad = warp & 3, half = warp >> 2;
         const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HC);
-        bool ok = true;
+        bool ok = __all_sync(0xffffffffu, *abort == 0);
         for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
             const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
             const int q = h.ti * 128 + quad * 32 + lane;
