@@ -206,7 +206,7 @@ __device__ __forceinline__ double pow2(int E) {
 // 2 l + 1 (, 16 + 2 l, 17 + 2 l): a permutation inside the K step, the same for every row (A and B of H are the
 // same digit rows, so every product is unchanged, and each K step keeps its sign), which keeps each load
 // instruction of the second pass on a few 64-byte runs of the row.
-// Bound by HBM (8 bytes read and 14 or 24 written per value: 4.8 and 5.3 TB/s of the copy's 6.8): 75-atom slab,
+// Bound by HBM (8 bytes read and 14 or 24 written per value: 4.8 and 5.3 TB/s of the copy's 6.8): 45-atom slab,
 // 14 e4m3 slices, 5.89 -> 5.17 ms with the packed digit code; 12 bf16 slices 6.85 -> 6.33 ms. Keeping the scaled
 // rows in shared memory between the passes cost more in occupancy than the second read.
 // ----------------------------------------------------------------------------------------
@@ -493,21 +493,21 @@ __global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ D
 // ----------------------------------------------------------------------------------------
 // Slice-product pipeline of the persistent contraction kernels, ten warps. Shared memory: a ring of
 // ring_slots(S) A-tile buffers (128 rows of 128 B, 16 KB, one slice of one K chunk each) and two sets
-// of S B-tile buffers (TN rows, TN x 128 B). Producer (warp 8): for each K chunk, the S B
+// of S B-tile buffers (TN rows, TN x 128 B). Producer (second last warp): for each K chunk, the S B
 // slices into B set kc % 2, then the S A slices one by one into the ring, each copy a bulk (TMA)
-// transfer completing on a "full" mbarrier. MMA issuer (warp 9): for each A slice s, the pairs (s, t)
+// transfer completing on a "full" mbarrier. MMA issuer (last warp): for each A slice s, the pairs (s, t)
 // with s + t < S as one 128 x TN(S-s) MMA per K step (two where TN(S-s) > 256) into accumulator groups
 // s .. S-1 (tensor-memory columns TN s ...); commits release A buffers and B sets back to the producer
-// through "empty" mbarriers. Warps 0-7 read the accumulators: warp w the rows of quadrant w % 4 and half
-// w / 4 of the TN columns. The phases of the ring and of the B sets continue over all the
+// through "empty" mbarriers. The other warps read the accumulators: warp w the rows of quadrant w % 4 and
+// part w / 4 of the TN columns. The phases of the ring and of the B sets continue over all the
 // accumulations a CTA runs. Every wait is bounded; on a timeout the CTA records NAO_ERR_TIMEOUT and
 // skips the rest of its work.
 // What bounds them: an earlier form (one issuing thread, four reading warps, 64-bit integer and FP64
-// arithmetic) took 18.3 ms for H and 9.2 ms for n on a slab of 75 atoms (14 e4m3 slices); 18.0 and 9.1
+// arithmetic) took 18.3 ms for H and 9.2 ms for n on a slab of 45 atoms (14 e4m3 slices); 18.0 and 9.1
 // without any copies, 15.0 and 4.4 without the readers' work, 11.8 and 3.5 with the copies alone. So the
 // MMA issue and the serial part of the readers (tensor memory holds one accumulator set) decided, not the
 // operands' supply: the issuer runs with its whole warp, so that descriptors stay in uniform registers,
-// and eight warps read with 32-bit integer and FP32 arithmetic. With the H items of nao_split_h_items and
+// and more warps read, with 32-bit integer and FP32 arithmetic. With the H items of nao_split_h_items and
 // the density's K in whole steps: 10.9 and 3.8 ms. Of these 9.8 ms were the H producer's alone (9.4 with a
 // quarter of the bytes, 4.8 with one copy per slice): it was one lane of a diverged warp, where every operand of
 // a copy costs a loop over lanes. Issued by the converged warp the copies alone take 3.9 ms, H 8.6 and n 3.6 ms
@@ -546,12 +546,21 @@ __host__ __device__ constexpr int n_pairs() { return F == NAO_DIGITS_E4M3 ? 8 : 
 // The joined integers of 8 columns of this thread's row. SMALL: every |M_g| <= 2^22, so that adding
 // 1.5 2^23 leaves the integer in the significand (one FP32 addition; the conversion instruction has a
 // quarter of its rate).
+// a += x, b += x as FP32s, in one instruction.
+__device__ __forceinline__ void add2(uint32_t &a, uint32_t &b, float x) {
+    asm("{\n\t.reg .b64 u, v;\n\t"
+        "mov.b64 u, {%0, %1};\n\tmov.b64 v, {%2, %2};\n\t"
+        "add.rn.f32x2 u, u, v;\n\t"
+        "mov.b64 {%0, %1}, u;\n\t}"
+        : "+r"(a), "+r"(b)
+        : "r"(__float_as_uint(x)));
+}
 template <int TN, int F, bool SMALL>
 __device__ __forceinline__ void read_pairs8(uint32_t tm_col, int S, int (&p)[n_pairs<F>()][8]) {
-    constexpr int B = nao_digit_bits(F), GB = F == NAO_DIGITS_E4M3 ? 8 : 6;  // groups per wait
+    constexpr int B = nao_digit_bits(F), GB = F == NAO_DIGITS_E4M3 ? 4 : 6;  // groups per wait
     constexpr int kMagic = 0x4B400000;  // 1.5 2^23
 #pragma unroll
-    for (int h = 0; h < 2; h++) {
+    for (int h = 0; h < (F == NAO_DIGITS_E4M3 ? 4 : 2); h++) {
         uint32_t r[GB][8];
 #pragma unroll
         for (int q = 0; q < GB; q++) {
@@ -564,24 +573,34 @@ __device__ __forceinline__ void read_pairs8(uint32_t tm_col, int S, int (&p)[n_p
             }
         }
         tc::tmem_ld_wait();
-        auto integer = [&](int q, int c) {
-            const float x = __uint_as_float(r[q][c]);
-            return SMALL ? __float_as_int(__fadd_rn(x, 12582912.0f)) - kMagic : __float2int_rn(x);
-        };
+        // in place: the integer of each group, offset by kMagic where SMALL
+#pragma unroll
+        for (int q = 0; q < GB; q++)
+#pragma unroll
+            for (int c = 0; c < 8; c += 2) {
+                if (SMALL) {
+                    add2(r[q][c], r[q][c + 1], 12582912.0f);
+                } else {
+                    r[q][c] = (uint32_t)__float2int_rn(__uint_as_float(r[q][c]));
+                    r[q][c + 1] = (uint32_t)__float2int_rn(__uint_as_float(r[q][c + 1]));
+                }
+            }
 #pragma unroll
         for (int c = 0; c < 8; c++) {
-            auto join = [&](int q) { return integer(q, c) * (1 << B) + integer(q + 1, c); };
+            constexpr uint32_t K1 = SMALL ? (uint32_t)kMagic : 0u, K2 = K1 * ((1u << B) + 1u);
+            auto integer = [&](int q) { return (int)(r[q][c] - K1); };
+            auto join = [&](int q) { return (int)(r[q][c] * (1u << B) + r[q + 1][c] - K2); };
             if constexpr (F == NAO_DIGITS_E4M3) {
-#pragma unroll
-                for (int k = 0; k < 4; k++) p[4 * h + k][c] = join(2 * k);
+                p[2 * h][c] = join(0);
+                p[2 * h + 1][c] = join(2);
             } else if (h == 0) {
                 p[0][c] = join(0);
                 p[1][c] = join(2);
                 p[2][c] = join(4);
             } else {
-                p[3][c] = integer(0, c);
+                p[3][c] = integer(0);
                 p[4][c] = join(1);
-                p[5][c] = integer(3, c);
+                p[5][c] = integer(3);
                 p[6][c] = join(4);
             }
         }
@@ -709,13 +728,23 @@ __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
     return reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
-constexpr int kReaders = 8;                        // accumulator-reading warps
-constexpr int kTcThreads = 32 * (kReaders + 2);    // and the producer and MMA warps
+// Accumulator-reading warps, four (one per quadrant of rows) for each part of the TN columns, 8 of them with
+// TN = 32 and 16 with 48; and the CTA's threads with the producer and MMA warps. Tensor memory holds one
+// accumulator set, so the MMAs stand still while it is read, and that is bound by latency: eight reading warps
+// with 16 and 24 columns took 3.59 ms for n on the slab of 45 atoms where sixteen take 3.19 (27 atoms
+// with grad n, 12 bf16 slices: 5.1 -> 4.5 ms; Hessian of a 13-atom molecule 5.4 -> 4.5 ms). More warps would
+// leave too few registers for a block of 8 columns.
+template <int TN>
+__host__ __device__ constexpr int n_parts() { return TN == 48 ? 3 : 4; }
+template <int TN>
+__host__ __device__ constexpr int n_readers() { return 4 * n_parts<TN>(); }
+template <int TN>
+__host__ __device__ constexpr int tc_threads() { return 32 * (n_readers<TN>() + 2); }
 
 struct PPipe {
     uint64_t fullA[kMaxRing], emptyA[kMaxRing], fullB[2], emptyB[2];
     uint64_t acc_full, acc_empty, fin;
-    uint64_t part_full[4], part_empty[4];  // n: the exchange of the two column halves' sums, per quadrant
+    uint64_t part_full[4][3], part_empty[4];  // n: the exchange of the column parts' sums, per quadrant
     double part[4][32];
     uint32_t tmem;
     int abort;
@@ -723,6 +752,7 @@ struct PPipe {
 static_assert(sizeof(PPipe) <= kStaticSmem, "barriers exceed their share of shared memory");
 
 // Barriers, tensor memory; returns its base address. RING: the A ring's slots.
+template <int TN>
 __device__ __forceinline__ uint32_t pipe_setup(PPipe &pp, int RING, const int32_t *err) {
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
@@ -735,11 +765,11 @@ __device__ __forceinline__ uint32_t pipe_setup(PPipe &pp, int RING, const int32_
             tc::mbar_init(&pp.emptyB[i], 1);
         }
         for (int i = 0; i < 4; i++) {
-            tc::mbar_init(&pp.part_full[i], 1);
+            for (int x = 0; x < 3; x++) tc::mbar_init(&pp.part_full[i][x], 1);
             tc::mbar_init(&pp.part_empty[i], 1);
         }
         tc::mbar_init(&pp.acc_full, 1);
-        tc::mbar_init(&pp.acc_empty, kReaders);  // one arrival per accumulator-reading warp
+        tc::mbar_init(&pp.acc_empty, n_readers<TN>());  // one arrival per accumulator-reading warp
         tc::mbar_init(&pp.fin, 1);
         tc::fence_mbar_init();
         pp.abort = *(const volatile int32_t *)err != 0 ? 1 : 0;  // a timeout earlier in this launch
@@ -860,22 +890,22 @@ __device__ __forceinline__ HItem h_item(const DevSystem &s, const HTask *work, i
 // run, so the scatter and the next item's first loads overlap the MMAs. A quadrant of the readers has one
 // of the item's four row blocks.
 template <int TN, int F>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(tc_threads<TN>(), 1)
     h_tc_kernel(const __grid_constant__ DevSystem s, const HTask *__restrict__ work, int32_t w0, int32_t n_work,
                 const uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off, const int32_t *__restrict__ expo,
                 const int32_t *__restrict__ neg16, int S, int scatter, int32_t *__restrict__ err) {
     constexpr uint32_t B_BLOCK = TN * 128;
-    constexpr int HC = TN / 2, NB8 = HC / 8;  // columns per reader thread, in blocks of 8
+    constexpr int HC = TN / n_parts<TN>(), NB8 = HC / 8;  // columns per reader thread, in blocks of 8
     extern __shared__ uint8_t smem_dyn[];
     __shared__ PPipe pp;
     uint8_t *smem = align1024(smem_dyn);
     const int RING = ring_slots(S, F);
     uint8_t *sA = smem, *sB = smem + (size_t)RING * 16384;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    const uint32_t tm = pipe_setup(pp, RING, err);
+    const uint32_t tm = pipe_setup<TN>(pp, RING, err);
     volatile int *abort = &pp.abort;
 
-    if (warp == kReaders) {
+    if (warp == n_readers<TN>()) {
         // ---- producer (the whole warp; one lane's copies take effect) ----
         const uint32_t lead = tc::elect_one(), sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
         const uint32_t fullA = tc::smem_addr(pp.fullA), fullB = tc::smem_addr(pp.fullB);
@@ -942,7 +972,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         if (!ok && lane == 0) *abort = 1;
         __syncwarp();
-    } else if (warp == kReaders + 1) {
+    } else if (warp == n_readers<TN>() + 1) {
         // ---- MMA issuer (the whole warp; one lane's tcgen05 instructions take effect) ----
         const uint32_t lead = tc::elect_one();
         const uint32_t sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
@@ -974,8 +1004,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     } else {
         // ---- accumulator readers and scatter ----
         uint32_t t = 0;
-        const int quad = warp & 3, half = warp >> 2;
-        const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HC);
+        const int quad = warp & 3, part = warp >> 2;
+        const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * HC);
         for (int w = blockIdx.x; w < n_work; w += gridDim.x, t++) {
             const HItem h = h_item<TN, F>(s, work, w0 + w, slices, sl_off, neg16, S);
             const uint32_t rb = h.task.row(quad);
@@ -1006,7 +1036,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 for (int c8 = 0; c8 < NB8; c8++)
 #pragma unroll
                     for (int c = 0; c < 8; c++) {
-                        const int j = h.tj * TN + half * HC + 8 * c8 + c;
+                        const int j = h.tj * TN + part * HC + 8 * c8 + c;
                         if (j >= h.N || (!whole && j < i)) continue;
                         const int ej = ex[j];
                         long long hi, lo, lo2;
@@ -1030,7 +1060,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // tile J's group, where P' is nonzero, in whole K steps), one after another through the single accumulator set.
 // The readers take tile J's accumulators, hand tensor memory back and then add sum_j T_qj phi_qj to
 // the point's sums in registers while tile J+1's MMAs run (products and their sums over eight functions
-// as float-floats: on the FP64 pipe, two lanes per clock, this took longer than the MMAs); after the last tile the two column halves are added and
+// as float-floats: on the FP64 pipe, two lanes per clock, this took longer than the MMAs); after the last tile the column parts' sums are added and
 // stored (no atomics: one item owns each point).
 // GRADN (density gradient, Sec. 2): P' = P over all of K, and the epilogue also forms
 // grad n_q = 2 sum_j T_qj grad phi_qj from the rows [phi | grad phi] of 4 Ppad.
@@ -1083,7 +1113,7 @@ __device__ __forceinline__ int n_item_ks(const NItem &h, int J, int S) {
 // 2 sum_j T_qj d_b phi_qj for b >= hc). Modes 0, 1 read the float-float evaluation at scr_off,
 // modes 2, 3 the Hessian's 10-row FP64 evaluation at eoff.
 template <int TN, int MODE, int F>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(tc_threads<TN>(), 1)
     n_tc_kernel(const __grid_constant__ DevSystem s, const HWork *__restrict__ work, int32_t w0, int32_t n_work,
                 const uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off, const int32_t *__restrict__ expo_q,
                 const int32_t *__restrict__ expo_b, const void *__restrict__ scratch_v,
@@ -1095,17 +1125,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     using V = typename std::conditional<(MODE >= 2), double, FF2>::type;
     const V *scratch = static_cast<const V *>(scratch_v);
     constexpr uint32_t B_BLOCK = TN * 128;
-    constexpr int HC = TN / 2, NB8 = HC / 8;
+    constexpr int PARTS = n_parts<TN>(), HC = TN / PARTS, NB8 = HC / 8;
     extern __shared__ uint8_t smem_dyn[];
     __shared__ PPipe pp;
     uint8_t *smem = align1024(smem_dyn);
     const int RING = ring_slots(S, F);
     uint8_t *sA = smem, *sB = smem + (size_t)RING * 16384;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    const uint32_t tm = pipe_setup(pp, RING, err);
+    const uint32_t tm = pipe_setup<TN>(pp, RING, err);
     volatile int *abort = &pp.abort;
 
-    if (warp == kReaders) {
+    if (warp == n_readers<TN>()) {
         // ---- producer ----
         const uint32_t lead = tc::elect_one(), sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
         const uint32_t fullA = tc::smem_addr(pp.fullA), fullB = tc::smem_addr(pp.fullB);
@@ -1143,7 +1173,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         if (!ok && lane == 0) *abort = 1;
         __syncwarp();
-    } else if (warp == kReaders + 1) {
+    } else if (warp == n_readers<TN>() + 1) {
         // ---- MMA issuer ----
         const uint32_t lead = tc::elect_one();
         const uint32_t sA_addr = tc::smem_addr(sA), sB_addr = tc::smem_addr(sB);
@@ -1177,8 +1207,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     } else {
         // ---- accumulator readers and the n epilogue ----
         uint32_t t = 0, x = 0;  // accumulations read, exchanges made
-        const int quad = warp & 3, half = warp >> 2;
-        const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HC);
+        const int quad = warp & 3, part = warp >> 2;
+        const uint32_t tm_row = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * HC);
         bool ok = __all_sync(0xffffffffu, *abort == 0);
         for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
             const NItem h = n_item<TN, F>(s, work, w0 + w, slices, sl_off, S);
@@ -1192,7 +1222,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
             for (int d = 0; d < NC; d++) tot[d] = 0.0;
             for (int J = 0; J < h.nJ && ok; J++, t++) {
-                const int j0 = J * TN + half * HC, jn = min(HC, h.N - j0);
+                const int j0 = J * TN + part * HC, jn = min(HC, h.N - j0);
                 // this tile's rows of phi towards L2 while its MMAs run
                 if (row_ok)
                     for (int jj = 0; jj < jn; jj++) asm volatile("prefetch.global.L2 [%0];" ::"l"(E + (j0 + jj) * ld));
@@ -1203,9 +1233,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 }
                 tc::fence_after_sync();
                 // the joined integers of all columns before tensor memory is handed back, the float-floats
-                // after; beside several sums, or with 24 columns, the integers do not fit in registers
+                // after; beside several sums, or with 16 columns, the integers do not fit in registers
                 // and become float-floats at once
-                constexpr bool NOW = NB8 > 2 || NC > 1;
+                constexpr bool NOW = NB8 > 1 || NC > 1;
                 ffa::F tv[HC];
                 int p[NB8][n_pairs<F>()][8];
                 if (any_row)
@@ -1252,23 +1282,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 __syncwarp();
             }
             if (!ok) break;
-            // the second half's sums to the first half's warp of the quadrant, one after another
+            // the parts' sums from the last part's warp of the quadrant to the first's, each adding its own
 #pragma unroll
             for (int d = 0; d < NC; d++, x++) {
-                if (half == 1) {
-                    if (!tc::mbar_wait(&pp.part_empty[quad], (x & 1u) ^ 1u, kWaitCycles)) *abort = 1;
-                    pp.part[quad][lane] = tot[d];
-                    __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(&pp.part_full[quad]);
-                } else {
-                    if (!tc::mbar_wait(&pp.part_full[quad], x & 1u, kWaitCycles)) *abort = 1;
+                if (part < PARTS - 1) {
+                    if (!tc::mbar_wait(&pp.part_full[quad][part], x & 1u, kWaitCycles)) *abort = 1;
                     tot[d] += pp.part[quad][lane];
-                    __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(&pp.part_empty[quad]);
+                } else if (!tc::mbar_wait(&pp.part_empty[quad], (x & 1u) ^ 1u, kWaitCycles)) {
+                    *abort = 1;
                 }
+                if (part > 0) pp.part[quad][lane] = tot[d];
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(part > 0 ? &pp.part_full[quad][part - 1] : &pp.part_empty[quad]);
             }
             if (__any_sync(0xffffffffu, *abort != 0)) break;
-            if (half == 0 && row_ok) {
+            if (part == 0 && row_ok) {
                 const int eq = expo_q[h.p0 + q], eb = split_bits::exponent_of_binade(expo_b[h.b]);
                 const bool live = eq > -10000 && eb > -10000;
                 const double sc = pow2(eq + eb - n_unit<F>());
@@ -1454,11 +1482,11 @@ cudaError_t launch_h_tc(const DevSystem &s, const HTask *work, int32_t w0, int32
     const int grid = n_work < sm_count() ? n_work : sm_count();  // persistent: one CTA per SM
     const size_t sm = split_smem_bytes(S, F);
     if (F == NAO_DIGITS_E4M3 && tn == 32)
-        h_tc_kernel<32, 1><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
+        h_tc_kernel<32, 1><<<grid, tc_threads<32>(), sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
     else if (F == NAO_DIGITS_BF16 && tn == 48 && S <= 10)
-        h_tc_kernel<48, 0><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
+        h_tc_kernel<48, 0><<<grid, tc_threads<48>(), sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
     else if (F == NAO_DIGITS_BF16 && tn == 32)
-        h_tc_kernel<32, 0><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
+        h_tc_kernel<32, 0><<<grid, tc_threads<32>(), sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
@@ -1522,7 +1550,7 @@ static cudaError_t launch_n_tc_mode(const DevSystem &s, const HWork *work, int32
     const size_t sm = split_smem_bytes(S, F);
     const int grid = n_work < sm_count() ? n_work : sm_count();  // persistent: one CTA per SM
 #define NAO_N_TC(TNV, M, FF)                                                                                  \
-    n_tc_kernel<TNV, M, FF><<<grid, kTcThreads, sm, st>>>(s, work, w0, n_work, slices, sl_off, expo_q, expo_b, ev, eoff, S, hc, \
+    n_tc_kernel<TNV, M, FF><<<grid, tc_threads<TNV>(), sm, st>>>(s, work, w0, n_work, slices, sl_off, expo_q, expo_b, ev, eoff, S, hc, \
                                                    hess, err)
 #define NAO_N_TC_MODES(TNV, FF)             \
     switch (mode) {                         \
