@@ -178,24 +178,32 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
         const int r = lr + 32 * h;
         aok[h] = i0 + r < N;
         bok[h] = j0 + r < N;
-        Ar[h] = E + (int64_t)(aok[h] ? i0 + r : 0) * ld + lv * VK;
-        Br[h] = E + (int64_t)(bok[h] ? j0 + r : 0) * ld + lv * VK;
+        Ar[h] = E + (int64_t)(aok[h] ? i0 + r : 0) * ld;
+        Br[h] = E + (int64_t)(bok[h] ? j0 + r : 0) * ld;
     }
     V bv[2];
-    int wq = lv * VK, comp = 0;  // the point and component (phi, d/dx, d/dy, d/dz) of this vector's column
-    auto load = [&](int k0, int buf) {
+    // this CTA's points [qa, qa + Ps) (see the launcher) and, of the next chunk's column of this vector, the
+    // point after qa and the component (phi, d/dx, d/dy, d/dz)
+    const int per = (Ppad / NAO_PPAD + (int)gridDim.y - 1) / (int)gridDim.y * NAO_PPAD;
+    const int qa = (int)blockIdx.y * per, Ps = min(Ppad - qa, per), nk = 4 * Ps / KC;
+    if (Ps <= 0) return;
+    int wq = lv * VK, comp = 0;
+    auto wrap = [&]() {
+        while (wq >= Ps) {
+            wq -= Ps;
+            comp++;
+        }
+    };
+    auto load = [&](int buf) {
+        const int k = comp * Ppad + qa + wq;
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            cp16(&sm.a[buf][lr + 32 * h][lv * VK], Ar[h] + k0, aok[h]);
-            if (bok[h]) bv[h] = *reinterpret_cast<const V *>(Br[h] + k0);
+            cp16(&sm.a[buf][lr + 32 * h][lv * VK], Ar[h] + k, aok[h]);
+            if (bok[h]) bv[h] = *reinterpret_cast<const V *>(Br[h] + k);
         }
     };
     auto store = [&](int buf) {
-        while (wq >= Ppad) {
-            wq -= Ppad;
-            comp++;
-        }
-        const V w = *reinterpret_cast<const V *>(wt + (comp == 0 ? 0 : Ppad) + wq);
+        const V w = *reinterpret_cast<const V *>(wt + (comp == 0 ? 0 : Ppad) + qa + wq);
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             V x{};
@@ -203,16 +211,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
             *reinterpret_cast<V *>(&sm.b[buf][lr + 32 * h][lv * VK]) = x;
         }
         wq += KC;
+        wrap();
     };
-    const int nk = 4 * Ppad / KC;
-    load(0, 0);
+    wrap();
+    load(0);
     __syncthreads();  // the weights are written
     store(0);
     for (int kc = 0; kc < nk; kc++) {
         const int buf = kc & 1;
         cp_wait_all();
         __syncthreads();  // this chunk is complete, and every warp has left the other buffer
-        if (kc + 1 < nk) load((kc + 1) * KC, buf ^ 1);
+        if (kc + 1 < nk) load(buf ^ 1);
 #pragma unroll
         for (int u = 0; u < NU; u++) {
             if (sub[u] < 0) continue;
@@ -568,7 +577,13 @@ static cudaError_t launch_h_simt_t(const DevSystem &s, const HWork *work, int32_
             cudaFuncSetAttribute(h_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * NAO_MAX_BATCH * (int)sizeof(T));
         if (e != cudaSuccess) return e;
     }
-    h_simt_kernel<T><<<n_work, 256, dyn, st>>>(s, work, scratch, terms);
+    // A tile pair of a few hundred points keeps an SM's FP64 pipe busy for most of a millisecond: with fewer than
+    // 20 FP64 items per SM their points are cut into up to four segments, or the last ones leave most SMs idle.
+    // Segments of points, not of K: a point's four components may cancel in phi_i phi_j d and the gradients'
+    // product, and a sum over points of h's terms has no larger partial sums than the magnitudes it is measured
+    // against. 8-atom cluster (490 batches): H 6.60 -> 5.33 ms.
+    const int kseg = sizeof(T) == 4 || n_work >= 20 * 152 ? 1 : (n_work >= 10 * 152 ? 2 : 4);
+    h_simt_kernel<T><<<dim3(n_work, kseg), 256, dyn, st>>>(s, work, scratch, terms);
     return cudaGetLastError();
 }
 

@@ -13,7 +13,8 @@
 // FP64: bound by the FP64 pipe (two lanes per clock and SM), 6 N^2 P products per batch. One CTA takes half
 // an item, 64 x 32, and each warp one 16 x 16 subtile of it with all six products; subtiles beyond the
 // batch's functions are left out. The rows d_c phi_i come by cp.async as they lie, the weights go into the
-// columns: w phi_j and w h phi_j. 9 atoms, 19,440 points: 11.3 -> 9.5 ms (floor 7.2).
+// columns: w phi_j and w h phi_j. 9 atoms, 19,440 points: 11.3 -> 9.5 ms, with
+// the points of an item in up to four CTAs 8.4 (floor 7.2).
 // FP32: per 8-point chunk w d_c phi_i (three components) and h phi_j or phi_j, each chunk's sums added
 // into compensated (hi, lo) pairs, in two passes of three products.
 #include "nao_internal.h"
@@ -63,7 +64,11 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
     for (int x = 0; x < 48; x++) (&acc[0][0][0][0])[x] = 0.0;
     const int lv = tid & 7, lr = tid >> 3;  // loader: vector lv (two points), rows lr and lr + 32
-    for (int q0 = 0; q0 < Ppad; q0 += KP) {
+    // this CTA's points (see the launcher)
+    const int chunks = Ppad / KP, per = (chunks + (int)gridDim.z - 1) / (int)gridDim.z;
+    const int qa = (int)blockIdx.z * per * KP, qb = min(Ppad, qa + per * KP);
+    if (qa >= qb) return;
+    for (int q0 = qa; q0 < qb; q0 += KP) {
         __syncthreads();  // the weights are written; every warp has left the last chunk
 #pragma unroll
         for (int h = 0; h < 2; h++) {
@@ -272,7 +277,10 @@ cudaError_t launch_pulay(const DevSystem &s, const HWork *work, int32_t w0, int3
                                                        2 * NAO_MAX_BATCH * (int)sizeof(double));
             if (e != cudaSuccess) return e;
         }
-        pulay_fp64_kernel<<<dim3(n_work, 2), 256, dyn, st>>>(s, work, w0, static_cast<const double *>(scratch), hoff, M, S, nb);
+        // few items: their points are cut into up to four segments, whose partial sums simply add (an item
+        // keeps an SM's FP64 pipe busy for most of a millisecond)
+        const int seg = n_work >= 10 * 152 ? 1 : (n_work >= 5 * 152 ? 2 : 4);
+        pulay_fp64_kernel<<<dim3(n_work, 2, seg), 256, dyn, st>>>(s, work, w0, static_cast<const double *>(scratch), hoff, M, S, nb);
     }
     return cudaGetLastError();
 }
