@@ -69,7 +69,8 @@ constexpr double kNearNucleus = 0.1;
 // The solid harmonics and their gradients are computed in H, the radial functions and the products in R.
 //   F64: both in FP64.
 //   F32: harmonics in float-float, rounded once to FP32 (their recurrences cancel near the nodes of
-//        cos(m phi), sin(m phi) and P_l^m(cos theta), where FP32 loses several ulps), the rest in FP32.
+//        cos(m phi), sin(m phi) and P_l^m(cos theta), where FP32 loses several ulps), the rest in FP32, but
+//        ill-conditioned spline segments (DevSystem::seg64) in float-float.
 //   FF:  the split path's evaluation, both in float-float (csrc/ff.h), ~48-bit significands on the FP32 pipe.
 // The geometry (d, r^2, 1/r) and the radial coordinate t stay in FP64 in all three. Points within
 // kNearNucleus of an atom take F64 in all three, and FF takes it for atoms with functions of l >= 5.
@@ -154,7 +155,8 @@ struct Point {
     typename A::H x[3], r2;
     typename A::R t, xr[3], u, dr;  // xr: x in R; u: 1/r; dr: dR/ds -> dR/dr
     int k;                          // spline segment
-    double r, xk;                   // xk (F32): r / r_k - 1, for segments evaluated from the FP64 coefficients
+    double r;
+    ffa::F tf;                      // t as a float-float (F32: for the ill-conditioned segments)
 };
 
 // (phi, phi' / r as the factors of S) of one radial function: g and gpu = g'(r) / r.
@@ -176,12 +178,15 @@ __device__ __forceinline__ void radial(const DevSystem &s, const Point<A> &pt, i
         const float t = pt.t;
         float R, dRds;
         if (__ldg(s.seg64 + seg)) {
-            // ill-conditioned segment: FP64 coefficients and FP64 t
-            const double t64 = log1p(pt.xk) * s.inv_delta;
-            const double2 *c = reinterpret_cast<const double2 *>(s.coef + seg * 4);
-            const double2 c01 = __ldg(c), c23 = __ldg(c + 1);
-            R = (float)fma(fma(fma(c23.y, t64, c23.x), t64, c01.y), t64, c01.x);
-            dRds = (float)fma(fma(3.0 * c23.y, t64, 2.0 * c23.x), t64, c01.y);
+            // ill-conditioned segment: coefficients, t and polynomials as float-floats, rounded once (in FP64
+            // they and a log1p per radial function took half of this path's evaluation: 64 atoms, phi and grad phi
+            // 2.28 -> 1.19 ms, phi alone 1.78 -> 0.76)
+            const float4 ch = __ldg(reinterpret_cast<const float4 *>(s.coef_f32 + seg * 4));
+            const float4 cl = __ldg(reinterpret_cast<const float4 *>(s.coef_lo + seg * 4));
+            const ffa::F c0{ch.x, cl.x}, c1{ch.y, cl.y}, c2{ch.z, cl.z}, c3{ch.w, cl.w};
+            const ffa::F a = ffa::fma(c3, pt.tf, c2);
+            R = ffa::fma(ffa::fma(a, pt.tf, c1), pt.tf, c0).h;
+            dRds = ffa::fma(ffa::fma(c3, pt.tf, ffa::twice(a)), pt.tf, c1).h;
         } else {
             const float4 c = __ldg(reinterpret_cast<const float4 *>(s.coef_f32 + seg * 4));
             R = fmaf(fmaf(fmaf(c.w, t, c.z), t, c.y), t, c.x);
@@ -321,7 +326,7 @@ __device__ __forceinline__ void eval_group(const DevSystem &s, const AtomGroup &
     const double rr = fmax(r, s.r0);
     const double dr = s.inv_delta * (r < s.r0 ? __ldg(s.inv_rk) : ur);  // dR/dr = dR/ds * inv_delta / rr
     pt.r = r;
-    pt.xk = 0.0;
+    pt.tf = ffa::F{0.0f, 0.0f};
     if constexpr (std::is_same<A, F32>::value) {
         // FP32 segment, refined as ln(r / r_k)/Delta = log1p(r * (1/r_k) - 1)/Delta with one FP64
         // FMA: t keeps ~1e-7 although a plain FP32 ln(r/r0) carries ~1e-6.
@@ -329,8 +334,9 @@ __device__ __forceinline__ void eval_group(const DevSystem &s, const AtomGroup &
         int k = (int)floorf(sa);
         k = k < 0 ? 0 : (k > s.n_rgrid - 2 ? s.n_rgrid - 2 : k);
         pt.k = k;
-        pt.xk = fma(rr, __ldg(s.inv_rk + k), -1.0);
-        pt.t = log1pf((float)pt.xk) * (float)s.inv_delta;
+        const double xk = fma(rr, __ldg(s.inv_rk + k), -1.0);
+        pt.t = log1pf((float)xk) * (float)s.inv_delta;
+        pt.tf = ffa::from_double_bits(log1p_small(xk, s.step_m1) * s.inv_delta);
         pt.u = float(ur);
         pt.dr = float(dr);
     } else {
