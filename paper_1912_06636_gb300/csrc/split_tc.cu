@@ -195,7 +195,7 @@ __device__ __forceinline__ double pow2(int E) {
 
 
 // ----------------------------------------------------------------------------------------
-// Hamiltonian slicing: one CTA per (batch, 64-row tile of basis functions). Columns are
+// Hamiltonian slicing: one CTA per (batch, tile of `tile` basis functions, 64 or 16). Columns are
 // reordered: the negative-weight ones (v < 0 on the potential part) first, padded to a whole
 // MMA K step (16 bf16 or 32 e4m3 columns), then the rest, so that B = A and the sign is applied
 // per K step.
@@ -218,7 +218,7 @@ __host__ __device__ constexpr size_t slice_h_smem(int Ppad, int F) {
 }
 
 template <int S, int F>
-__global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __grid_constant__ DevSystem s, int32_t b0,
+__global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __grid_constant__ DevSystem s, int32_t b0, int tile,
                                                                   const FF2 *__restrict__ scratch, uint32_t terms,
                                                                   uint8_t *__restrict__ slices,
                                                                   const int64_t *__restrict__ sl_off,
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __gr
     const int N = s.rel_off[b + 1] - s.rel_off[b];
     constexpr int C = nao_chunk_cols(F), KS = nao_kstep_cols(F), LC = C / 32, B = nao_digit_bits(F);  // LC: columns per lane
     const SplitGeom G(P, N, S, 0, F);
-    if (N == 0 || rt >= G.h_slice_tiles()) return;
+    if (N == 0 || rt * tile >= G.R16) return;
     const int K = 4 * Ppad, Kp = C * G.n_kc, T = 32 * kSliceWarps;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float2 *sd = reinterpret_cast<float2 *>(slice_sh);              // [K] column scale sqrt|d| as a float-float
@@ -292,8 +292,8 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __gr
     if (rt == 0 && threadIdx.x == 0) neg16[b] = negpad / KS;  // negated K steps
     __syncthreads();
     uint8_t *base = slices + sl_off[b];
-    for (int lr = warp; lr < 64; lr += kSliceWarps) {
-        const int r = rt * 64 + lr;
+    for (int lr = warp; lr < tile; lr += kSliceWarps) {
+        const int r = rt * tile + lr;
         if (r >= G.R16) break;
         const float2 *row = reinterpret_cast<const float2 *>(E + (int64_t)(r < N ? r : 0) * K);
         auto scaled = [&](int k) {
@@ -1459,6 +1459,10 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
     if (b1 <= b0 || max_rt <= 0) return cudaSuccess;
     const FF2 *ev = reinterpret_cast<const FF2 *>(scratch);  // the split path's evaluation: float-float values
     const size_t sm = slice_h_smem(s.max_ppad, F);
+    // 64 rows per CTA (max_rt such tiles cover the largest batch), 16 where that gives fewer than two CTAs per
+    // SM: a small system's launch is as long as one CTA (3-atom molecule, 66 batches: 41 -> 26 us)
+    const int tile = (int64_t)(b1 - b0) * max_rt < 2 * 152 ? 16 : 64;
+    const dim3 grid(b1 - b0, max_rt * (64 / tile));
     static_assert(slice_h_smem(NAO_SPLIT_MAX_PPAD, 0) + 1024 <= kSmemOptin && slice_h_smem(NAO_SPLIT_MAX_PPAD, 1) + 1024 <= kSmemOptin,
                   "the H slicer's rows exceed shared memory");
     cudaError_t e = cudaSuccess;
@@ -1467,8 +1471,7 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
         if (sm > 48 * 1024)                                                                                          \
             e = cudaFuncSetAttribute(slice_h_kernel<SS, FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);  \
         if (e == cudaSuccess)                                                                                        \
-            slice_h_kernel<SS, FF><<<dim3(b1 - b0, max_rt), 32 * kSliceWarps, sm, st>>>(s, b0, ev, terms, slices, sl_off, expo, \
-                                                                                         neg16);                    \
+            slice_h_kernel<SS, FF><<<grid, 32 * kSliceWarps, sm, st>>>(s, b0, tile, ev, terms, slices, sl_off, expo, neg16);                    \
     }
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_H)
 #undef NAO_SLICE_H
