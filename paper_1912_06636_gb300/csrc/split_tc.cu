@@ -330,44 +330,46 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __gr
 
 // ----------------------------------------------------------------------------------------
 // Density slicing.
-// Phi^T: one CTA (8 warps) per (batch, 32-point tile), the point exponents from the
-// evaluation. Per K chunk (64 or 128 functions) the CTA stages phi[i][q] (chunk x 32, read along
-// the points) in shared memory and each warp writes its points' rows along K (2 or 4 functions
-// per lane, one 128-byte row segment per slice). The first kPexpCtas
-// CTAs of a batch instead reduce its exponent of P' (read along rows of P), as a biased exponent.
+// Phi^T: one CTA (4 warps) per (batch, 16-point tile), the point exponents from the evaluation. A K chunk (64 or
+// 128 functions) of phi[i][q], read along the points, comes to shared memory while the chunk before it is cut
+// into digits; each warp writes its points' rows along K (2 or 4 functions per lane, one 128-byte row segment per
+// slice). The first kPexpCtas CTAs of a batch instead reduce its exponent of P' (read along rows of P), as a
+// biased exponent.
+// Bound by the latency of the loads (a batch has one to four chunks), and with 12 bf16 slices by HBM next (4.8 TB/s):
+// against 32 points by 8 warps with one buffer, loads and digits in turn, 64 atoms 1.37 -> 0.92 ms.
 // ----------------------------------------------------------------------------------------
 // The symmetry c_IJ of P' is taken between groups of GW = nao_split_tn(S, F) functions, whatever width the
 // contraction's tiles have: the digits, and so n, do not depend on the tuned width.
 
-constexpr int kPexpCtas = 4;  // CTAs per batch that reduce the exponent of P'
+constexpr int kPexpCtas = 8;  // CTAs per batch that reduce the exponent of P'
+constexpr int kNphiWarps = 4, kNphiPoints = 16;
 
-template <typename V>
-struct StageOf {  // shared-memory staging type of the density slicer's input
-    using type = ffa::F;
-    __device__ static ffa::F get(const FF2 &v) { return v.f(); }
-    __device__ static ffa::F zero() { return ffa::F{0.0f, 0.0f}; }
-};
-template <>
-struct StageOf<double> {
-    using type = double;
-    __device__ static double get(double v) { return v; }
-    __device__ static double zero() { return 0.0; }
-};
+// Row of function k of a chunk in shared memory: eight more per K step, so that the functions a half-warp reads
+// at once (eight each of two K steps) lie in different banks.
+template <int F>
+__device__ __forceinline__ int stage_row(int k) { return k + 8 * (k / nao_kstep_cols(F)); }
+template <int F>
+__host__ __device__ constexpr int stage_rows() { return nao_chunk_cols(F) + 8 * (nao_chunk_cols(F) / nao_kstep_cols(F)); }
+
+// 8 bytes global -> shared, zeros where !ok
+__device__ __forceinline__ void cp8(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_addr(dst)), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ ffa::F stage_value(const FF2 &v) { return v.f(); }
+__device__ __forceinline__ double stage_value(double v) { return v; }
 
 // V = FF2: the split path's float-float phi (rows of ld_mult Ppad at scr_off[b]); V = double: the
 // density Hessian's FP64 evaluation (rows of 10 Ppad at eoff[b]), component row coff (phi or one
 // gradient component). pexp = 0 leaves the P' exponent to another launch.
 template <int S, int F, typename V>
-__global__ void __launch_bounds__(256) slice_nphi_kernel(const __grid_constant__ DevSystem s, int32_t b0, const V *__restrict__ scratch,
+__global__ void __launch_bounds__(32 * kNphiWarps) slice_nphi_kernel(const __grid_constant__ DevSystem s, int32_t b0, const V *__restrict__ scratch,
                                                         const int64_t *__restrict__ eoff, int coff,
                                                         uint8_t *__restrict__ slices, const int64_t *__restrict__ sl_off,
                                                         const int32_t *__restrict__ expo_q, int32_t *__restrict__ expo_b,
                                                         int ld_mult, int full, int pexp) {
-    constexpr int C = nao_chunk_cols(F), LC = C / 32, GW = nao_split_tn(S, F);
-    using TT = typename StageOf<V>::type;
+    constexpr int C = nao_chunk_cols(F), LC = C / 32, GW = nao_split_tn(S, F), W = kNphiWarps, Q = kNphiPoints;
     constexpr int KS = nao_kstep_cols(F);
-    // 8 more columns per K step: the two K steps that a half-warp reads at once lie in different banks
-    __shared__ TT t[32][C + 8 * (C / KS) + 1];
+    __shared__ V t[2][stage_rows<F>()][Q + 1];
     const int b = b0 + blockIdx.x;
     const int p0 = s.batch_off[b], P = s.batch_off[b + 1] - p0;
     const int Ppad = (P + NAO_PPAD - 1) & ~(NAO_PPAD - 1);
@@ -379,11 +381,11 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(const __grid_constant__
         if (!pexp) return;
         // max |P'_ij| over i <= j (P' is P on the diagonal groups, 2 P off them, 0 below unless
         // full): the exponent field of |P| plus one off the diagonal groups; each CTA takes every
-        // kPexpCtas-th set of eight rows (expo_b[b] is zero before: the evaluation clears it)
+        // kPexpCtas-th set of W rows (expo_b[b] is zero before: the evaluation clears it)
         const int m = s.sys.bmol[b];
         const int32_t *rel = s.rel_idx + s.rel_off[b];
         int mk = 0;
-        for (int i = warp + 8 * (int)blockIdx.y; i < N; i += 8 * kPexpCtas) {
+        for (int i = warp + W * (int)blockIdx.y; i < N; i += W * kPexpCtas) {
             const int64_t gi = rel[i];
 #pragma unroll 4
             for (int j = (full ? 0 : i) + lane; j < N; j += 32) {
@@ -396,52 +398,62 @@ __global__ void __launch_bounds__(256) slice_nphi_kernel(const __grid_constant__
         if (lane == 0 && mk > 0) atomicMax(expo_b + b, mk);
         return;
     }
-    const int q0 = ((int)blockIdx.y - kPexpCtas) * 32;
+    const int q0 = ((int)blockIdx.y - kPexpCtas) * Q;
     if (q0 >= G.P16) return;
-    const V *E = scratch + eoff[b] + (int64_t)coff * Ppad;  // row i at E + i ld_mult Ppad
     const int64_t ld = (int64_t)ld_mult * Ppad;
-    const bool qin = q0 + lane < P;
-    int eq[4];
+    // this thread's point and its first function of a chunk; row i of phi at scratch + eoff[b] + coff Ppad + i ld
+    const int lq = threadIdx.x % Q, li = threadIdx.x / Q;
+    const bool qin = q0 + lq < P;
+    const V *E = scratch + eoff[b] + (int64_t)coff * Ppad + q0 + lq;
+    auto load = [&](int kc) {
 #pragma unroll
-    for (int h = 0; h < 4; h++) {
-        const int q = q0 + warp * 4 + h;
+        for (int h = 0; h < C * Q / (32 * W); h++) {
+            const int k = li + 32 * W / Q * h, i = kc * C + k;
+            const bool ok = i < N && qin;
+            cp8(&t[kc & 1][stage_row<F>(k)][lq], ok ? E + (int64_t)i * ld : scratch, ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int eq[Q / W];
+#pragma unroll
+    for (int h = 0; h < Q / W; h++) {
+        const int q = q0 + warp * (Q / W) + h;
         eq[h] = q < P ? expo_q[p0 + q] : -10000;
     }
     uint8_t *base = slices + sl_off[b];
+    load(0);
     for (int kc = 0; kc < G.n_kcN; kc++) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // this chunk is there, and every warp has left the other buffer
+        if (kc + 1 < G.n_kcN) load(kc + 1);
 #pragma unroll
-        for (int h = 0; h < C / 8; h++) {
-            const int i = kc * C + warp + 8 * h;
-            const int k = warp + 8 * h;
-            t[lane][k + 8 * (k / KS)] = (i < N && qin) ? StageOf<V>::get(E[(int64_t)i * ld + q0 + lane]) : StageOf<V>::zero();
-        }
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < 4; h++) {
-            const int ql = warp * 4 + h, q = q0 + ql;
-            if (q >= G.P16) break;
+        for (int h = 0; h < Q / W; h++) {
+            const int ql = warp * (Q / W) + h, q = q0 + ql;  // below P16, a multiple of Q
             // within each K step (KS functions, the words of 8 lanes) lane l packs functions l, l + 8
             // (, l + 16, l + 24): both operands of the density's product (this A and
             // slice_np_kernel's B) order K this way inside each K step, which leaves every slice
             // product unchanged; K steps hold consecutive functions, so that n_tc_kernel can stop
             // at a tile's last one
-            TT x[LC];
+            decltype(stage_value(V())) x[LC];
 #pragma unroll
-            for (int c = 0; c < LC; c++) x[c] = t[ql][(KS + 8) * (lane >> 3) + (lane & 7) + 8 * c];
+            for (int c = 0; c < LC; c++) x[c] = stage_value(t[kc & 1][(KS + 8) * (lane >> 3) + (lane & 7) + 8 * c][ql]);
             uint32_t wd[S];
             lane_digit_words<S, F>(x, digit_scale<S, F>(x, eq[h]), wd);
             const uint32_t off = tc::sw128_byte((uint32_t)q, (uint32_t)(4 * lane));
 #pragma unroll
             for (int sl = 0; sl < S; sl++) *reinterpret_cast<uint32_t *>(base + G.nA_block(sl, kc) + off) = wd[sl];
         }
-        __syncthreads();
     }
 }
 
 // P'_ij = c_IJ P[rel_i][rel_j] over GW-function groups I = i/GW <= J = j/GW (c_II = 1,
 // c_IJ = 2; every (i, j) with c = 1 when full), read from P's upper triangle, with the batch's
 // exponent from slice_nphi_kernel. One CTA per (batch, 16 rows j), one warp per row, 2 or 4
-// functions i per lane (slice_nphi_kernel's K order; one 128-byte row segment per slice).
+// functions i per lane (slice_nphi_kernel's K order; one 128-byte row segment per slice). Chunks that no
+// tile of the contraction reads (n_item_ks: those past the last function of the row's group) are not written.
+// Bound by integer and FP32 issue (the digits of FP64 values). Staging P's blocks in shared memory, read along
+// its rows, was slower (slab of 45 atoms 2.3 ms against 1.4; with all chunks written 2.0): P is in L2, and
+// neighbouring lanes' sectors are used by the next rows' warps.
 template <int S, int F>
 __global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ DevSystem s, int32_t b0, uint8_t *__restrict__ slices,
                                                       const int64_t *__restrict__ sl_off,
@@ -458,13 +470,16 @@ __global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ D
     const int e = split_bits::exponent_of_binade(expo_b[b]);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *base = slices + sl_off[b];
+    // functions that a 32- or GW-wide tile with these rows multiplies, in K steps
+    const int end = full ? N : ((j0 / 32 + 1) * 32 + GW - 1) / GW * GW;
+    const int nk = min(G.n_kcN, ((end + KS - 1) / KS + 3) / 4);
 #pragma unroll 1
     for (int h = 0; h < 2; h++) {
         const int j = j0 + warp * 2 + h;  // < R16: R16 is a multiple of 16
         const bool jin = j < N;
         const int64_t gj = jin ? rel[j] : 0;
         const int group = j / GW;
-        for (int kc = 0; kc < G.n_kcN; kc++) {
+        for (int kc = 0; kc < nk; kc++) {
             double xp[LC];
 #pragma unroll
             for (int hh = 0; hh < LC; hh++) {
@@ -1223,9 +1238,12 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
             for (int d = 0; d < NC; d++) tot[d] = 0.0;
             for (int J = 0; J < h.nJ && ok; J++, t++) {
                 const int j0 = J * TN + part * HC, jn = min(HC, h.N - j0);
-                // this tile's rows of phi towards L2 while its MMAs run
-                if (row_ok)
-                    for (int jj = 0; jj < jn; jj++) asm volatile("prefetch.global.L2 [%0];" ::"l"(E + (j0 + jj) * ld));
+                // a single sum's phi arrive while this tile's MMAs run (more sums' values would not fit in
+                // registers, and prefetching them to L2 costs more than it gives)
+                V f0[MODE == 0 ? HC : 1];
+                if constexpr (MODE == 0)
+#pragma unroll
+                    for (int c = 0; c < HC; c++) f0[c] = row_ok && c < jn ? E[(j0 + c) * ld] : V(0);
                 if (*abort || !tc::mbar_wait(&pp.acc_full, t & 1u, kWaitCycles)) *abort = 1;
                 if (__any_sync(0xffffffffu, *abort != 0)) {
                     ok = false;
@@ -1268,7 +1286,7 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
 #pragma unroll
                             for (int y = 0; y < CB; y++)
 #pragma unroll
-                                for (int d = 0; d < NC; d++) fv[y][d] = c + y < jn ? f[(c + y) * ld + d * h.Ppad] : V(0);
+                                for (int d = 0; d < NC; d++) fv[y][d] = MODE == 0 ? f0[MODE == 0 ? c + y : 0] : (c + y < jn ? f[(c + y) * ld + d * h.Ppad] : V(0));
 #pragma unroll
                             for (int y = 0; y < CB; y++)
 #pragma unroll
@@ -1500,9 +1518,9 @@ cudaError_t launch_slice_n(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
                            int32_t *expo_b, int S, int F, bool grad, cudaStream_t st) {
     if (b1 <= b0) return cudaSuccess;
     const FF2 *ev = reinterpret_cast<const FF2 *>(scratch);
-    // y < kPexpCtas: the exponent of P'; above: 32-point tiles (128 max_qt >= P16)
+    // y < kPexpCtas: the exponent of P'; above: tiles of kNphiPoints points (128 max_qt >= P16)
 #define NAO_SLICE_NPHI(SS, FF)                                                                            \
-    slice_nphi_kernel<SS, FF, FF2><<<dim3(b1 - b0, 4 * max_qt + kPexpCtas), 256, 0, st>>>(                        \
+    slice_nphi_kernel<SS, FF, FF2><<<dim3(b1 - b0, 128 / kNphiPoints * max_qt + kPexpCtas), 32 * kNphiWarps, 0, st>>>(                        \
         s, b0, ev, s.scr_off, 0, slices, sl_off, expo_q, expo_b, grad ? 4 : 1, grad ? 1 : 0, 1)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NPHI)
 #undef NAO_SLICE_NPHI
@@ -1522,7 +1540,7 @@ cudaError_t launch_slice_n_hess(const DevSystem &s, int32_t b0, int32_t b1, int3
     if (b1 <= b0) return cudaSuccess;
     const int first = comp == 0 ? 1 : 0;  // P' (its exponent and its slices) once, with the first pass
 #define NAO_SLICE_NPHI(SS, FF)                                                                                   \
-    slice_nphi_kernel<SS, FF, double><<<dim3(b1 - b0, 4 * max_qt + kPexpCtas), 256, 0, st>>>(                            \
+    slice_nphi_kernel<SS, FF, double><<<dim3(b1 - b0, 128 / kNphiPoints * max_qt + kPexpCtas), 32 * kNphiWarps, 0, st>>>(                            \
         s, b0, scratch, hoff, comp, slices, sl_off, expo_q, expo_b, 10, 1, first)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_NPHI)
 #undef NAO_SLICE_NPHI

@@ -127,7 +127,10 @@ def bloch_reference(h, fm, fi, cell, lat, k, nb):
     F = np.zeros((len(k), len(fm), nb), complex)
     for q in range(len(k)):
         F[q, np.arange(len(fm)), fm] = np.exp(1j * (T @ k[q]))
-    return np.einsum("qri,rs,qsj->qij", F.conj(), h, F), np.einsum("qri,rs,qsj->qij", np.abs(F), np.abs(h), np.abs(F)).real
+    def fold(G, x):
+        return np.swapaxes(G.conj(), 1, 2) @ (x @ G)
+
+    return fold(F, h), fold(np.abs(F), np.abs(h))
 
 
 # 2000 images: their phases for eight k points do not fit in shared memory, so the general form runs
