@@ -726,6 +726,18 @@ __device__ __forceinline__ ffa::F ff_of_bits(double x) {
     const float l = __fsub_rn(__uint_as_float(base | ((lo >> 6) & 0x7FFFFFu)), __uint_as_float(base));
     return ffa::F{h, l};
 }
+// A value that no other thread reads, past L1: shared memory, the same array, is what the MMAs read their operands
+// from (27 atoms with grad n: 4.43 -> 4.01 ms).
+__device__ __forceinline__ FF2 load_once(const FF2 *p) {
+    float h, l;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(h), "=f"(l) : "l"(p));
+    return FF2(ffa::F{h, l});
+}
+__device__ __forceinline__ double load_once(const double *p) {
+    double x;
+    asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(x) : "l"(p));
+    return x;
+}
 __device__ __forceinline__ ffa::F ff_of_value(const FF2 &v) { return v.f(); }
 __device__ __forceinline__ ffa::F ff_of_value(double v) { return ff_of_bits(v); }
 
@@ -1243,7 +1255,7 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
                 V f0[MODE == 0 ? HC : 1];
                 if constexpr (MODE == 0)
 #pragma unroll
-                    for (int c = 0; c < HC; c++) f0[c] = row_ok && c < jn ? E[(j0 + c) * ld] : V(0);
+                    for (int c = 0; c < HC; c++) f0[c] = row_ok && c < jn ? load_once(E + (j0 + c) * ld) : V(0);
                 if (*abort || !tc::mbar_wait(&pp.acc_full, t & 1u, kWaitCycles)) *abort = 1;
                 if (__any_sync(0xffffffffu, *abort != 0)) {
                     ok = false;
@@ -1286,7 +1298,7 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
 #pragma unroll
                             for (int y = 0; y < CB; y++)
 #pragma unroll
-                                for (int d = 0; d < NC; d++) fv[y][d] = MODE == 0 ? f0[MODE == 0 ? c + y : 0] : (c + y < jn ? f[(c + y) * ld + d * h.Ppad] : V(0));
+                                for (int d = 0; d < NC; d++) fv[y][d] = MODE == 0 ? f0[MODE == 0 ? c + y : 0] : (c + y < jn ? load_once(f + (c + y) * ld + d * h.Ppad) : V(0));
 #pragma unroll
                             for (int y = 0; y < CB; y++)
 #pragma unroll
