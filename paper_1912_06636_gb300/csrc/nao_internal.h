@@ -311,6 +311,7 @@ struct nao_grid {
     HWork *d_hwork = nullptr;
     DWork *d_dwork = nullptr;
     double *d_scratch = nullptr;
+    double *hess_scratch = nullptr;  // the Hessian's and Pulay terms' evaluation: d_scratch or a buffer of its own
     double *d_ne_part = nullptr;    // [n_dwork] per-tile sums of w n
     int32_t *d_err = nullptr;       // device error word
     // systems (molecules) of the handle
