@@ -1180,22 +1180,28 @@ nao_status hess_plan(nao_grid *g) {
     const int64_t nbat = g->n_batches;
     std::vector<int64_t> off((size_t)std::max<int64_t>(nbat, 1), 0);
     int64_t used = 0, dw = 0, need = 0;
-    for (int64_t b = 0; b < nbat; b++) need += (int64_t)g->Nb[b] * 10 * ((g->Pb[b] + NAO_PPAD - 1) / NAO_PPAD * NAO_PPAD);
+    for (int64_t b = 0; b < nbat; b++) {
+        const int64_t e = (int64_t)g->Nb[b] * 10 * ((g->Pb[b] + NAO_PPAD - 1) / NAO_PPAD * NAO_PPAD);
+        if (e > g->scratch_elems)
+            return fail(NAO_ERR_UNSUPPORTED, "density Hessian: batch " + std::to_string(b) +
+                                                 " needs more evaluation scratch than the handle has (raise scratch_bytes)");
+        need += e;
+    }
     // The evaluation scratch holds four values per function and point where the whole grid fits, so ten would
     // always make three chunks, of which each leaves the GPU partly idle at its end: a buffer of their own, where
     // both stay within scratch_bytes (Hessian of 13 atoms 7.2 -> 5.1 ms, Pulay terms of 9 atoms 8.9 -> 8.75).
     const int64_t limit = (g->opt.scratch_bytes > 0 ? g->opt.scratch_bytes : kDefaultScratch) / (int64_t)sizeof(double);
-    g->hess_scratch = g->d_scratch;
-    int64_t elems = g->scratch_elems;
-    if (need > elems && elems + need <= limit && dev_alloc(g, &g->hess_scratch, (size_t)need) == NAO_OK) elems = need;
+    if (!g->hess_scratch) {
+        g->hess_scratch = g->d_scratch;
+        g->hess_elems = g->scratch_elems;
+        if (need > g->scratch_elems && g->scratch_elems + need <= limit && dev_alloc(g, &g->hess_scratch, (size_t)need) == NAO_OK)
+            g->hess_elems = need;
+    }
     nao_grid::HessChunk cur{0, 0, 0, 0};
     for (int64_t b = 0; b < nbat; b++) {
         const int64_t Ppad = (g->Pb[b] + NAO_PPAD - 1) / NAO_PPAD * NAO_PPAD;
         const int64_t e = (int64_t)g->Nb[b] * 10 * Ppad;
-        if (e > g->scratch_elems)
-            return fail(NAO_ERR_UNSUPPORTED, "density Hessian: batch " + std::to_string(b) +
-                                                 " needs more evaluation scratch than the handle has (raise scratch_bytes)");
-        if (used + e > elems && b > cur.b0) {
+        if (used + e > g->hess_elems && b > cur.b0) {
             cur.b1 = (int32_t)b;
             cur.dw1 = (int32_t)dw;
             g->hess_chunks.push_back(cur);

@@ -312,6 +312,7 @@ struct nao_grid {
     DWork *d_dwork = nullptr;
     double *d_scratch = nullptr;
     double *hess_scratch = nullptr;  // the Hessian's and Pulay terms' evaluation: d_scratch or a buffer of its own
+    int64_t hess_elems = 0;          // its doubles
     double *d_ne_part = nullptr;    // [n_dwork] per-tile sums of w n
     int32_t *d_err = nullptr;       // device error word
     // systems (molecules) of the handle
