@@ -339,8 +339,10 @@ template <> struct PointSum<float> {
 // 16-function column group and one or two groups of points for the whole tile loop, so that a point's
 // sums over functions stay in registers until the end. In FP64 the symmetry c_IJ is taken in blocks of
 // 16 functions instead of 64 (a warp leaves out the chunks below its column group's diagonal block).
+// Three CTAs per SM without GRADN: with two the FP32 form had too few warps for its shared-memory latency (64 atoms
+// 2.44 -> 2.17 ms, in spite of some spills; the H kernel above is faster with two, 4.2 against 4.4).
 template <typename T, bool GRADN>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 && !GRADN ? 3 : 2)
+__global__ void __launch_bounds__(256, GRADN ? 2 : 3)
     density_simt_kernel(const __grid_constant__ DevSystem s, const DWork *__restrict__ work, int32_t w0,
                         const T *__restrict__ scratch, double *__restrict__ ne_part) {
     using V = typename Vec16<T>::type;

@@ -14,7 +14,7 @@
 // an item, 64 x 32, and each warp one 16 x 16 subtile of it with all six products; subtiles beyond the
 // batch's functions are left out. The rows d_c phi_i come by cp.async as they lie, the weights go into the
 // columns: w phi_j and w h phi_j. 9 atoms, 19,440 points: 11.3 -> 9.5 ms, with
-// the points of an item in up to four CTAs 8.4 (floor 7.2).
+// the points of an item in up to four CTAs 8.3 (floor 7.2).
 // FP32: per 8-point chunk w d_c phi_i (three components) and h phi_j or phi_j, each chunk's sums added
 // into compensated (hi, lo) pairs, in two passes of three products.
 #include "nao_internal.h"
@@ -278,8 +278,8 @@ cudaError_t launch_pulay(const DevSystem &s, const HWork *work, int32_t w0, int3
             if (e != cudaSuccess) return e;
         }
         // few items: their points are cut into up to four segments, whose partial sums simply add (an item
-        // keeps an SM's FP64 pipe busy for most of a millisecond)
-        const int seg = n_work >= 10 * 152 ? 1 : (n_work >= 5 * 152 ? 2 : 4);
+        // keeps an SM's FP64 pipe busy for most of a millisecond; at 900 items two segments took 8.44 ms, four 8.30)
+        const int seg = n_work >= 20 * 152 ? 1 : (n_work >= 10 * 152 ? 2 : 4);
         pulay_fp64_kernel<<<dim3(n_work, 2, seg), 256, dyn, st>>>(s, work, w0, static_cast<const double *>(scratch), hoff, M, S, nb);
     }
     return cudaGetLastError();
