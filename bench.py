@@ -223,13 +223,13 @@ TRAFFIC_PER_FLOP_H = {
     (1, "h_fp64", 0): ((359.834112e6 + 3.945472e6) / 4.6096304e9, "profiles/h_simt_kernel_diamond8_fp64.md"),
 }
 # DRAM bytes per issued tensor FLOP of the split H contraction, from one ncu capture of one launch
-# of the 125-atom slab (the first five layers of the 375-atom workload, the same batch shapes):
-# dram__bytes_read.sum + dram__bytes_write.sum over sm__ops_path_tensor_op_utcqmma_src_fp8_dst_fp32
-# (the slices are read from DRAM once and re-read from L2, so the traffic grows with the tiles
+# of a 45-atom slab (five layers of 3 x 3 atoms of the 375-atom workload's structure, 16 radial points):
+# dram__bytes_read.sum + dram__bytes_write.sum over the issued FLOP (h_item_area times two per slice
+# product; the slices are read from DRAM once and re-read from L2, so the traffic grows with the tiles
 # issued). Scaled by the issued FLOP of this run's average launch. Valid only for the kernel
 # version, digit format and slice count the capture was taken with (e4m3, 14 slices).
 TRAFFIC_PER_ISSUED_FLOP = {
-    (2, "h_split", 14): ((1.044792e9 + 5.37984e6) / 2.6126843904e12, "profiles/h_tc_kernel_slab125_e4m3.md"),
+    (2, "h_split", 14): ((3.789794816e9 + 3.8706944e7) / 8.60358180864e12, "profiles/kernels_slab45_e4m3.md"),
 }
 
 
@@ -377,6 +377,21 @@ def h_tile_area(n_basis, k_cols, tile_width, tile_rows: int = 128):
         for i0 in range(0, n, tile_rows):
             j_first = (i0 // tn) * tn  # the first column tile that reaches i0 <= j
             issued += k * tile_rows * tn * len(range(j_first, n, tn))
+    return issued, useful
+
+
+def h_item_area(n_basis, k_cols, tile_width):
+    """h_tile_area of the items the library issues: 48-wide tiles as there; 32-wide ones take the pairs of
+    32-function blocks four rows at a time, max(r, ceil(r (r + 1) / 8)) items of 128 x 32 for r blocks."""
+    wide = [(n, k, tn) for n, k, tn in zip(n_basis, k_cols, tile_width) if int(tn) != 32]
+    issued, useful = h_tile_area(*zip(*wide)) if wide else (0, 0)
+    for n, k, tn in zip(n_basis, k_cols, tile_width):
+        n, k = int(n), int(k)
+        if int(tn) != 32 or n <= 0:
+            continue
+        r = (n + 31) // 32
+        useful += k * n * (n + 1) // 2
+        issued += k * 128 * 32 * max(r, -(-r * (r + 1) // 8))
     return issued, useful
 
 
@@ -647,7 +662,7 @@ def main():
         tuning = {"buckets_timed": timed, "batches_tile48": int(np.sum(tw == 48)), "batches_tile32": int(np.sum(tw == 32))}
         if roofline is not None and fam == "h_split":
             try:  # the share of the issued MMA area that is the work FLOP_H counts
-                issued, useful = h_tile_area(Nb, 4 * Ppad, tw)
+                issued, useful = h_item_area(Nb, 4 * Ppad, tw)
                 roofline["useful_area_frac"] = useful / issued
                 roofline["issued_tflops"] = roofline["achieved"] * issued / useful
             except Exception as e:  # reported, never fatal
@@ -657,7 +672,7 @@ def main():
                 issued_per_launch = roofline["issued_tflops"] * 1e12 * roofline["avg_launch_ms"] / 1e3
                 roofline["traffic"] = per_flop * issued_per_launch
                 roofline["traffic_unit"] = "bytes per launch"
-                roofline["traffic_source"] = (src + " (DRAM bytes per issued tensor FLOP of one 125-atom slab launch "
+                roofline["traffic_source"] = (src + " (DRAM bytes per issued tensor FLOP of one 45-atom slab launch "
                                               "x this run's issued FLOP per launch)")
 
     line = {

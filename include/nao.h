@@ -114,7 +114,9 @@ typedef struct {
     int32_t device;           /* CUDA device ordinal; -1 = the calling thread's current device */
     int64_t scratch_bytes;    /* device scratch for evaluated basis functions; 0 = library default (8 GiB;
                                  the split path's slices take three times this). Memory is taken only
-                                 up to what the batches need; smaller values mean more, smaller launches */
+                                 up to what the batches need; smaller values mean more, smaller launches.
+                                 The density Hessian and the Pulay terms take a buffer of their own where it
+                                 fits beside the evaluation scratch within this figure */
     int32_t capture_graph;    /* 1: the first call of each (operation, precision, terms) records
                                  its kernel launches as a CUDA graph on a stream the handle
                                  owns; later calls upload that call's pointer tables and replay

@@ -15,13 +15,14 @@
 // pairs with s + t >= S are dropped (their weight is below 64^-S). The epilogue recombines the
 // groups as integers (three 64-bit parts) and scales once in FP64:
 //     x_i . y_j = 2^(e_i + e_j) sum_g M_g 64^-(g+2).
-// Tensor memory holds S groups x TN columns: TN = 48 for S <= 10, TN = 32 for S = 11, 12.
+// Tensor memory holds S groups x TN columns: TN = 48 for S <= 10 bf16 slices, else TN = 32.
 //
 // Hamiltonian: A = F (rows i, K = 4 Ppad: phi | d/dx | d/dy | d/dz weighted by sqrt|d_k|) and
-// B = sign(d_k) F (rows j), tiles of 128 x TN (S groups x TN FP32 columns, at most 480 of the
-// 512 tensor-memory columns), tile pairs crossing the upper triangle, FP64 atomic scatter.
-// Density: A = Phi^T (rows = points, K = basis), B = P' (rows j, P'_ij = c_IJ P_ij for TN-function
-// tiles I <= J with c_II = 1, c_IJ = 2, else 0) so that T_qj = sum_i phi_qi P'_ij and
+// B = sign(d_k) F (rows j), 128 x TN elements at a time (S groups x TN FP32 columns of tensor memory's 512):
+// with TN = 32 any four 32-row blocks against one column tile, so that each pair of blocks is computed once;
+// FP64 atomic scatter.
+// Density: A = Phi^T (rows = points, K = basis), B = P' (rows j, P'_ij = c_IJ P_ij for groups
+// I <= J of functions with c_II = 1, c_IJ = 2, else 0) so that T_qj = sum_i phi_qi P'_ij and
 // n_q = sum_j T_qj phi_qj; one per-batch exponent is used for P'.
 #include <algorithm>
 #include <cmath>
@@ -1354,23 +1355,25 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
     pipe_end(pp, tm, err);
 }
 
-// sum over each density tile of 64 points of w n (then the deterministic final reduction)
-__global__ void __launch_bounds__(256) wn_partial_kernel(DevSystem s, const DWork *__restrict__ work, int32_t w0,
-                                                        double *__restrict__ ne_part) {
-    __shared__ double red[8];
-    const DWork it = work[w0 + blockIdx.x];
-    const int p0 = s.batch_off[it.batch], P = s.batch_off[it.batch + 1] - p0;
-    const int q = it.tp * NAO_TILE + threadIdx.x;
-    double wn = 0.0;
-    if (threadIdx.x < NAO_TILE && q < P) wn = s.pw[p0 + q] * *n_at(s, s.sys.bmol[it.batch], p0 + q);
-    for (int o = 16; o > 0; o >>= 1) wn += __shfl_xor_sync(0xffffffffu, wn, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = wn;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; w++) t += red[w];
-        ne_part[w0 + blockIdx.x] = t;
+// sum over each density tile of 64 points of w n (then the deterministic final reduction), a warp per tile
+// (a CTA per tile: 78 us for 64 atoms, 1.2 million points; now 20)
+constexpr int kWnWarps = 8;
+__global__ void __launch_bounds__(32 * kWnWarps) wn_partial_kernel(const __grid_constant__ DevSystem s, const DWork *__restrict__ work,
+                                                                   int32_t w0, int32_t n_work, double *__restrict__ ne_part) {
+    const int w = blockIdx.x * kWnWarps + (threadIdx.x >> 5);
+    if (w >= n_work) return;
+    const DWork it = work[w0 + w];
+    const int p0 = s.batch_off[it.batch], P = s.batch_off[it.batch + 1] - p0, m = s.sys.bmol[it.batch];
+    double wn[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int q = it.tp * NAO_TILE + 32 * h + (int)(threadIdx.x & 31);
+        wn[h] = q < P ? s.pw[p0 + q] * *n_at(s, m, p0 + q) : 0.0;
     }
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+        for (int o = 16; o > 0; o >>= 1) wn[h] += __shfl_xor_sync(0xffffffffu, wn[h], o);
+    if ((threadIdx.x & 31) == 0) ne_part[w0 + w] = wn[0] + wn[1];
 }
 
 // The timeout path of the bounded waits, exercised without a stuck pipeline: one thread waits on
@@ -1618,6 +1621,6 @@ cudaError_t launch_n_tc_hess(const DevSystem &s, const HWork *work, int32_t w0, 
 cudaError_t launch_wn_partial(const DevSystem &s, const DWork *work, int32_t w0, int32_t n_work, double *ne_part,
                               cudaStream_t st) {
     if (n_work <= 0) return cudaSuccess;
-    wn_partial_kernel<<<n_work, 256, 0, st>>>(s, work, w0, ne_part);
+    wn_partial_kernel<<<(n_work + kWnWarps - 1) / kWnWarps, 32 * kWnWarps, 0, st>>>(s, work, w0, n_work, ne_part);
     return cudaGetLastError();
 }

@@ -158,12 +158,8 @@ __device__ __forceinline__ void mma_commit(uint32_t lead, uint64_t *bar) {
         : "memory");
 }
 
-// Byte offset of element (row r, k) inside a block of rows x 64 bf16 stored K-major with the
-// 128-byte swizzle: 16-byte chunk k/8 of row r is placed at chunk (k/8) ^ (r%8).
-__host__ __device__ __forceinline__ uint32_t sw128_offset(uint32_t r, uint32_t k) {
-    return (r >> 3) * 1024u + (r & 7u) * 128u + ((((k >> 3) ^ (r & 7u)) & 7u) << 4) + (k & 7u) * 2u;
-}
-// The same for byte kb of row r (any element size): 16-byte chunk kb/16 goes to (kb/16) ^ (r%8).
+// Byte offset of byte kb of row r inside a block of rows of 128 bytes stored K-major with the 128-byte
+// swizzle: 16-byte chunk kb/16 of row r is placed at chunk (kb/16) ^ (r%8).
 __host__ __device__ __forceinline__ uint32_t sw128_byte(uint32_t r, uint32_t kb) {
     return (r >> 3) * 1024u + (r & 7u) * 128u + ((((kb >> 4) ^ (r & 7u)) & 7u) << 4) + (kb & 15u);
 }
