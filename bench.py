@@ -220,7 +220,7 @@ def serving(n_requests: int, device: int, fp64_requests: int) -> dict:
 # FP64 contraction on the 8-atom profiling case (a launch's traffic grows with tiles x K, i.e. with
 # FLOP_H). Valid only for the kernel version and slice count the capture was taken with.
 TRAFFIC_PER_FLOP_H = {
-    (1, "h_fp64", 0): ((359.834112e6 + 3.945472e6) / 4.6096304e9, "profiles/h_simt_kernel_diamond8_fp64.md"),
+    (1, "h_fp64", 0): ((365.077504e6 + 3.158272e6) / 4.6096304e9, "profiles/h_simt_kernel_diamond8_fp64.md"),
 }
 # DRAM bytes per issued tensor FLOP of the split H contraction, from one ncu capture of one launch
 # of a 45-atom slab (five layers of 3 x 3 atoms of the 375-atom workload's structure, 16 radial points):
