@@ -17,10 +17,10 @@
 //
 // What bounds them: the FP64 pipe (two lanes per clock and SM, 1/64 of the FP32 rate), which FP64
 // products use by definition and which every conversion between FP64 and a 32-bit type uses as
-// well. So (1) a CTA's 64 x 64 tile is cut into small subtiles, one or two per warp, and a warp
+// well. So (1) a CTA's 64 x 64 tile is cut into small subtiles, up to eight per warp, and a warp
 // leaves out the subtiles that lie below the diagonal, beyond the batch's functions or beyond its
-// points: 16 x 16 in FP64 and 32 x 16 in FP32 (with smaller ones the operands' loads would be too many
-// for the FP32 rate). Which warp takes which subtile turns with the CTA's index, so that the idle ones
+// points: in FP64 8 x 8 (H) and 16 x 16 (density), in FP32 32 x 16 (with smaller ones the operands' loads
+// would be too many for the FP32 rate). Which warp takes which subtile turns with the CTA's index, so that the idle ones
 // spread over the SM's four schedulers. (2) The FP32 kernels convert with integer instructions and
 // keep their sums over functions as float-float pairs.
 #include "ff.h"
@@ -35,6 +35,11 @@ constexpr int T_ = NAO_TILE;  // 64
 template <typename T> struct Cfg;
 template <> struct Cfg<double> { static constexpr int KC = 16, MR = 2, SR = 16, NU = 2; };
 template <> struct Cfg<float> { static constexpr int KC = 32, MR = 4, SR = 32, NU = 1; };
+// The H kernel's: MR rows x MC columns per lane. In FP64 8 x 8 subtiles: the FP64 pipe is the limit, shared memory
+// far from it, and they compute 1.15 times the wanted triangle of the 8-atom cluster's batches where 16 x 16 ones
+// compute 1.30.
+template <typename T> struct HCfg : Cfg<T> { static constexpr int MC = 4; };
+template <> struct HCfg<double> { static constexpr int KC = 16, MR = 1, MC = 2, SR = 8, NU = 8; };
 
 template <typename T> struct Vec16;  // 16 bytes of T
 template <> struct Vec16<double> { using type = double2; };
@@ -74,31 +79,31 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
 
 // The lane's accumulators of one subtile: FP64 accumulates directly; FP32 keeps a chunk sum and a
 // (hi, lo) pair.
-template <typename T> struct Block;
-template <> struct Block<double> {
-    double c[2][4];
+template <typename T, int MR = Cfg<T>::MR, int MC = 4> struct Block;
+template <int MR, int MC> struct Block<double, MR, MC> {
+    double c[MR][MC];
     __device__ __forceinline__ void zero() {
 #pragma unroll
-        for (int a = 0; a < 2; a++)
+        for (int a = 0; a < MR; a++)
 #pragma unroll
-            for (int b = 0; b < 4; b++) c[a][b] = 0.0;
+            for (int b = 0; b < MC; b++) c[a][b] = 0.0;
     }
     __device__ __forceinline__ void fold() {}
     __device__ __forceinline__ double value(int a, int b) const { return c[a][b]; }
 };
-template <> struct Block<float> {
-    float c[4][4], hi[4][4], lo[4][4];
+template <int MR, int MC> struct Block<float, MR, MC> {
+    float c[MR][MC], hi[MR][MC], lo[MR][MC];
     __device__ __forceinline__ void zero() {
 #pragma unroll
-        for (int a = 0; a < 4; a++)
+        for (int a = 0; a < MR; a++)
 #pragma unroll
-            for (int b = 0; b < 4; b++) c[a][b] = hi[a][b] = lo[a][b] = 0.0f;
+            for (int b = 0; b < MC; b++) c[a][b] = hi[a][b] = lo[a][b] = 0.0f;
     }
     __device__ __forceinline__ void fold() {
 #pragma unroll
-        for (int a = 0; a < 4; a++)
+        for (int a = 0; a < MR; a++)
 #pragma unroll
-            for (int b = 0; b < 4; b++) {
+            for (int b = 0; b < MC; b++) {
                 two_sum_acc(hi[a][b], lo[a][b], c[a][b]);
                 c[a][b] = 0.0f;
             }
@@ -118,16 +123,16 @@ template <typename T> struct HTile {
 // chunks stay row-major (K along the row): a lane reads 16 bytes, 2 or 4 terms, of each of its rows
 // (ly + 8 a) and columns (lx + 4 b).
 // Whole 64 x 64 tiles computed 2.5 times the wanted triangle on the 8-atom cluster (batches of 75
-// functions on average) and 1.9 times on the 64-atom one, the subtiles 1.3 and 1.3 times. Measured with
-// the density below, H + n: 8 atoms FP64 13.7 -> 8.9 ms, 64 atoms FP32 15.7 -> 12.0 ms (H 6.7 -> 4.2, n
-// 3.7 -> 2.4).
+// functions on average) and 1.9 times on the 64-atom one, 16 x 16 and 32 x 16 subtiles 1.3 times. Measured
+// with the density below, H + n: 8 atoms FP64 13.7 -> 8.9 ms, 64 atoms FP32 15.7 -> 12.0 ms (H 6.7 -> 4.2, n
+// 3.7 -> 2.4). In FP64 (the FP64 pipe 98 % busy) 8 x 8 subtiles then took H from 5.33 to 4.75 ms.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
     h_simt_kernel(const __grid_constant__ DevSystem s, const HWork *__restrict__ work, const T *__restrict__ scratch,
                   uint32_t terms) {
     using V = typename Vec16<T>::type;
-    constexpr int KC = Cfg<T>::KC, MR = Cfg<T>::MR, SR = Cfg<T>::SR, NU = Cfg<T>::NU, VK = 16 / sizeof(T);
-    constexpr int NS = (T_ / SR) * 4;  // subtiles of the tile
+    constexpr int KC = HCfg<T>::KC, MR = HCfg<T>::MR, MC = HCfg<T>::MC, SR = HCfg<T>::SR, NU = HCfg<T>::NU, VK = 16 / sizeof(T);
+    constexpr int SC = 4 * MC, NSC = T_ / SC, NS = (T_ / SR) * NSC;  // a subtile's columns, subtiles across, of the tile
     __shared__ __align__(16) HTile<T> sm;
     extern __shared__ __align__(16) unsigned char dyn[];
     const HWork it = work[blockIdx.x];
@@ -158,15 +163,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
 #pragma unroll
         for (int u = 0; u < NU; u++) sub[u] = -1;
         for (int x = 0; x < NS; x++) {
-            const int r = x >> 2, c = x & 3;
-            if (i0 + r * SR >= N || j0 + c * 16 >= N || (diag && c * 16 + 15 < r * SR)) continue;
+            const int r = x / NSC, c = x % NSC;
+            if (i0 + r * SR >= N || j0 + c * SC >= N || (diag && c * SC + SC - 1 < r * SR)) continue;
 #pragma unroll
             for (int u = 0; u < NU; u++)
                 if (k == w + 8 * u) sub[u] = x;
             k++;
         }
     }
-    Block<T> acc[NU];
+    Block<T, MR, MC> acc[NU];
 #pragma unroll
     for (int u = 0; u < NU; u++) acc[u].zero();
 
@@ -225,20 +230,20 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
 #pragma unroll
         for (int u = 0; u < NU; u++) {
             if (sub[u] < 0) continue;
-            const T *a = &sm.a[buf][(sub[u] >> 2) * SR + ly][0], *bb = &sm.b[buf][(sub[u] & 3) * 16 + lx][0];
+            const T *a = &sm.a[buf][(sub[u] / NSC) * SR + ly][0], *bb = &sm.b[buf][(sub[u] % NSC) * SC + lx][0];
 #pragma unroll
             for (int kv = 0; kv < KC; kv += VK) {
-                V ra[MR], rb[4];
+                V ra[MR], rb[MC];
 #pragma unroll
                 for (int x = 0; x < MR; x++) ra[x] = *reinterpret_cast<const V *>(a + 8 * x * HTile<T>::LD + kv);
 #pragma unroll
-                for (int y = 0; y < 4; y++) rb[y] = *reinterpret_cast<const V *>(bb + 4 * y * HTile<T>::LD + kv);
+                for (int y = 0; y < MC; y++) rb[y] = *reinterpret_cast<const V *>(bb + 4 * y * HTile<T>::LD + kv);
 #pragma unroll
                 for (int e = 0; e < VK; e++)
 #pragma unroll
                     for (int x = 0; x < MR; x++)
 #pragma unroll
-                        for (int y = 0; y < 4; y++) acc[u].c[x][y] = fma(vget(ra[x], e), vget(rb[y], e), acc[u].c[x][y]);
+                        for (int y = 0; y < MC; y++) acc[u].c[x][y] = fma(vget(ra[x], e), vget(rb[y], e), acc[u].c[x][y]);
             }
             acc[u].fold();
         }
@@ -251,12 +256,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 2)
         if (sub[u] < 0) continue;
 #pragma unroll
         for (int x = 0; x < MR; x++) {
-            const int i = i0 + (sub[u] >> 2) * SR + ly + 8 * x;
+            const int i = i0 + (sub[u] / NSC) * SR + ly + 8 * x;
             if (i >= N) continue;
             const int64_t gi = rel[i];
 #pragma unroll
-            for (int y = 0; y < 4; y++) {
-                const int j = j0 + (sub[u] & 3) * 16 + lx + 4 * y;
+            for (int y = 0; y < MC; y++) {
+                const int j = j0 + (sub[u] % NSC) * SC + lx + 4 * y;
                 if (j >= N || (diag && j < i)) continue;
                 h_add(s, m, gi, rel[j], acc[u].value(x, y));
             }

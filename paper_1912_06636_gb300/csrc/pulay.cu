@@ -11,10 +11,10 @@
 // Work items are the 64 x 64 tile pairs (I, J) of a batch (all pairs: the matrices are not symmetric);
 // FP64 atomics add each tile into the global matrices.
 // FP64: bound by the FP64 pipe (two lanes per clock and SM), 6 N^2 P products per batch. One CTA takes half
-// an item, 64 x 32, and each warp one 16 x 16 subtile of it with all six products; subtiles beyond the
+// an item, 64 x 32, and each warp up to four 8 x 8 subtiles of it with all six products; subtiles beyond the
 // batch's functions are left out. The rows d_c phi_i come by cp.async as they lie, the weights go into the
 // columns: w phi_j and w h phi_j. 9 atoms, 19,440 points: 11.3 -> 9.5 ms, with
-// the points of an item in up to four CTAs 8.3 (floor 7.2).
+// the points of an item in up to four CTAs 8.3, with 8 x 8 subtiles instead of 16 x 16 7.96 (floor 7.2).
 // FP32: per 8-point chunk w d_c phi_i (three components) and h phi_j or phi_j, each chunk's sums added
 // into compensated (hi, lo) pairs, in two passes of three products.
 #include "nao_internal.h"
@@ -56,11 +56,16 @@ __global__ void __launch_bounds__(256, 2)
         wt[q] = w;
         wt[Ppad + q] = q < P ? w * v_at(s, m, p0 + q) : 0.0;
     }
-    // the warp's subtile (rows r0 .., columns c0 ..); which warp takes which turns with the CTA, so that
-    // the idle ones spread over the schedulers
-    const int role = ((tid >> 5) + blockIdx.x) & 7, r0 = 16 * (role >> 1), c0 = 16 * (role & 1);
-    const bool live = i0 + r0 < N && j0 + c0 < N;
-    double acc[3][2][2][4];
+    // this warp's 8 x 8 subtiles: every eighth of those within the batch's functions (the first nr x nc of 8 x 4), the
+    // first of which turns with the CTA; subtile k at row k / nc, column k % nc, -1: none
+    const int nr = min(8, (N - i0 + 7) / 8), nc = min(4, (N - j0 + 7) / 8);
+    int sub[4];
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+        const int k = (((tid >> 5) + (int)blockIdx.x) & 7) + 8 * t;
+        sub[t] = k < nr * nc ? 8 * (k / nc) | 8 * (k % nc) << 8 : -1;  // first row | first column << 8
+    }
+    double acc[4][3][2][2];
 #pragma unroll
     for (int x = 0; x < 48; x++) (&acc[0][0][0][0])[x] = 0.0;
     const int lv = tid & 7, lr = tid >> 3;  // loader: vector lv (two points), rows lr and lr + 32
@@ -91,42 +96,45 @@ __global__ void __launch_bounds__(256, 2)
         *reinterpret_cast<double2 *>(&Bs[1][lr][2 * lv]) = wf;
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        if (!live) continue;
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            if (sub[t] < 0) continue;
+            const double *a = &As[0][(sub[t] & 255) + ly][0], *bb = &Bs[0][(sub[t] >> 8) + lx][0];
 #pragma unroll 1
-        for (int kv = 0; kv < KP; kv += 2)
+            for (int kv = 0; kv < KP; kv += 2) {
+                double2 ra[3], rb[2][2];
 #pragma unroll
-            for (int u = 0; u < 2; u++) {
-                double2 rb[4];
+                for (int c = 0; c < 3; c++) ra[c] = *reinterpret_cast<const double2 *>(a + c * TT * LDP + kv);
 #pragma unroll
-                for (int y = 0; y < 4; y++) rb[y] = *reinterpret_cast<const double2 *>(&Bs[u][c0 + lx + 4 * y][kv]);
+                for (int u = 0; u < 2; u++)
+#pragma unroll
+                    for (int y = 0; y < 2; y++) rb[u][y] = *reinterpret_cast<const double2 *>(bb + (u * (TT / 2) + 4 * y) * LDP + kv);
 #pragma unroll
                 for (int c = 0; c < 3; c++)
 #pragma unroll
-                    for (int x = 0; x < 2; x++) {
-                        const double2 ra = *reinterpret_cast<const double2 *>(&As[c][r0 + ly + 8 * x][kv]);
+                    for (int u = 0; u < 2; u++)
 #pragma unroll
-                        for (int y = 0; y < 4; y++)
-                            acc[c][u][x][y] = fma(ra.y, rb[y].y, fma(ra.x, rb[y].x, acc[c][u][x][y]));
-                    }
+                        for (int y = 0; y < 2; y++)
+                            acc[t][c][u][y] = fma(ra[c].y, rb[u][y].y, fma(ra[c].x, rb[u][y].x, acc[t][c][u][y]));
             }
+        }
     }
-    if (!live) return;
     const int32_t *rel = s.rel_idx + s.rel_off[b];
     const int64_t nn = nb * nb;
 #pragma unroll
-    for (int x = 0; x < 2; x++) {
-        const int i = i0 + r0 + ly + 8 * x;
-        if (i >= N) continue;
+    for (int t = 0; t < 4; t++) {
+        const int i = i0 + (sub[t] & 255) + ly;
+        if (sub[t] < 0 || i >= N) continue;
         const int64_t gi = rel[i];
 #pragma unroll
-        for (int y = 0; y < 4; y++) {
-            const int j = j0 + c0 + lx + 4 * y;
+        for (int y = 0; y < 2; y++) {
+            const int j = j0 + (sub[t] >> 8) + lx + 4 * y;
             if (j >= N) continue;
             const int64_t e = gi * nb + rel[j];
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                atomicAdd(M + c * nn + e, acc[c][0][x][y]);
-                atomicAdd(Sm + c * nn + e, acc[c][1][x][y]);
+                atomicAdd(M + c * nn + e, acc[t][c][0][y]);
+                atomicAdd(Sm + c * nn + e, acc[t][c][1][y]);
             }
         }
     }
