@@ -343,7 +343,8 @@ template <> struct PointSum<float> {
 // cp.async, P' through registers), two buffers and one barrier per chunk. A warp keeps one
 // 16-function column group and one or two groups of points for the whole tile loop, so that a point's
 // sums over functions stay in registers until the end. In FP64 the symmetry c_IJ is taken in blocks of
-// 16 functions instead of 64 (a warp leaves out the chunks below its column group's diagonal block).
+// 8 functions instead of 64 (a warp leaves out the chunks below its column group's diagonal block, and on it a
+// quarter: 8 atoms 1.54 ms, with blocks of 16 1.68).
 // Three CTAs per SM without GRADN: with two the FP32 form had too few warps for its shared-memory latency (64 atoms
 // 2.44 -> 2.17 ms, in spite of some spills; the H kernel above is faster with two, 4.2 against 4.4).
 template <typename T, bool GRADN>
@@ -374,6 +375,9 @@ __global__ void __launch_bounds__(256, GRADN ? 2 : 3)
     const double *Pm = s.sys.P[m];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lx = lane & 3, ly = lane >> 2;
     const int role = (warp + blockIdx.x) & 7, cg = role & 3;  // column group
+    // column y of the lane in the group: in FP64 two in each half, so that on the diagonal block the warp leaves out
+    // the products of its second eight rows with the first half
+    auto col = [&](int y) { return FP && !GRADN ? 2 * lx + (y & 1) + 8 * (y >> 1) : 4 * lx + y; };
     const int nt = (N + T_ - 1) / T_;
     int row[NU];  // first point (of the tile) of each of the warp's point groups, -1: beyond the batch
 #pragma unroll
@@ -423,8 +427,8 @@ __global__ void __launch_bounds__(256, GRADN ? 2 : 3)
                 for (int c = 0; c < 2; c++) {
                     const int j = tj * T_ + lane + 32 * c;
                     // c_IJ = 2 above the diagonal blocks, 1 on them (those below are not used); FP64
-                    // blocks of 16 functions, FP32 blocks of 64
-                    const bool two = !GRADN && (FP ? (i >> 4) < (j >> 4) : (i >> 6) < tj);
+                    // blocks of 8 functions, FP32 blocks of 64
+                    const bool two = !GRADN && (FP ? (i >> 3) < (j >> 3) : (i >> 6) < tj);
                     T x = T(0);
                     if (i < N && jok[c]) {
                         if constexpr (FP) x = pv[r][c];
@@ -446,9 +450,8 @@ __global__ void __launch_bounds__(256, GRADN ? 2 : 3)
 #pragma unroll
                 for (int u = 0; u < NU; u++) {
                     if (row[u] < 0) continue;
-                    const T *a = &As[buf][0][row[u] + ly * MR], *bb = &Bs[buf][0][cg * 16 + lx * 4];
-#pragma unroll 8
-                    for (int kk = 0; kk < KC; kk++) {
+                    const T *a = &As[buf][0][row[u] + ly * MR], *bb = &Bs[buf][0][cg * 16];
+                    auto products = [&](int kk, int y0) {  // with the columns from y0 on
                         T ra[MR], rb[4];
 #pragma unroll
                         for (int x = 0; x < MR; x += VK) {
@@ -458,15 +461,24 @@ __global__ void __launch_bounds__(256, GRADN ? 2 : 3)
                         }
 #pragma unroll
                         for (int y = 0; y < 4; y += VK) {
-                            const V v = *reinterpret_cast<const V *>(bb + kk * T_ + y);
+                            if (y < y0) continue;
+                            const V v = *reinterpret_cast<const V *>(bb + kk * T_ + col(y));
 #pragma unroll
                             for (int e = 0; e < VK; e++) rb[y + e] = vget(v, e);
                         }
 #pragma unroll
                         for (int x = 0; x < MR; x++)
 #pragma unroll
-                            for (int y = 0; y < 4; y++) acc[u].c[x][y] = fma(ra[x], rb[y], acc[u].c[x][y]);
-                    }
+                            for (int y = 0; y < 4; y++)
+                                if (y >= y0) acc[u].c[x][y] = fma(ra[x], rb[y], acc[u].c[x][y]);
+                    };
+                    const bool half = FP && !GRADN && kc == tj * 4 + cg;
+                    const int k1 = half ? KC / 2 : KC;
+#pragma unroll 8
+                    for (int kk = 0; kk < k1; kk++) products(kk, 0);
+                    if (half)
+#pragma unroll
+                        for (int kk = KC / 2; kk < KC; kk++) products(kk, 2);
                     acc[u].fold();
                 }
             }
@@ -479,7 +491,7 @@ __global__ void __launch_bounds__(256, GRADN ? 2 : 3)
             if (row[u] < 0 || q >= Ppad) continue;
 #pragma unroll
             for (int y = 0; y < 4; y++) {
-                const int j = tj * T_ + cg * 16 + lx * 4 + y;
+                const int j = tj * T_ + cg * 16 + col(y);
                 if (j >= N) continue;
 #pragma unroll
                 for (int d = 0; d < NC; d++)
