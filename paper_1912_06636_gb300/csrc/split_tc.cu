@@ -210,6 +210,8 @@ __device__ __forceinline__ double pow2(int E) {
 // Bound by HBM (8 bytes read and 14 or 24 written per value: 4.8 and 5.3 TB/s of the copy's 6.8): 45-atom slab,
 // 14 e4m3 slices, 5.89 -> 5.17 ms with the packed digit code; 12 bf16 slices 6.85 -> 6.33 ms. Keeping the scaled
 // rows in shared memory between the passes cost more in occupancy than the second read.
+// The first pass has eight loads in flight per lane: 5.10 ms with four, 4.82 with eight, 4.73 to 5.14 with 13 to 20
+// (whose remainders cost other row lengths more); the next row's prefetch to L2 5.34.
 // ----------------------------------------------------------------------------------------
 constexpr int kSliceWarps = 8;
 // Shared memory of slice_h_kernel for a batch of Ppad padded points: column scales, order, signs.
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 4) slice_h_kernel(const __gr
         };
         int mx = 0;
         if (r < N)
-#pragma unroll 4
+#pragma unroll 8
             for (int k = lane; k < K; k += 32) mx = max(mx, __float_as_int(scaled(k).h) & 0x7FFFFFFF);
         mx = __reduce_max_sync(0xffffffffu, mx);
         // |x.h| <= (2 - 2^-23) 2^k and |x.l| <= 2^-24 2^(k+1): |x| < 2^(k+1), and |x 2^-e| < 1/2 with e = k + 2
