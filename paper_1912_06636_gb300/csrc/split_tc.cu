@@ -207,7 +207,7 @@ __device__ __forceinline__ double pow2(int E) {
 // 2 l + 1 (, 16 + 2 l, 17 + 2 l): a permutation inside the K step, the same for every row (A and B of H are the
 // same digit rows, so every product is unchanged, and each K step keeps its sign), which keeps each load
 // instruction of the second pass on a few 64-byte runs of the row.
-// Bound by HBM (8 bytes read and 14 or 24 written per value: 4.8 and 5.3 TB/s of the copy's 6.8): 45-atom slab,
+// Bound by HBM (8 bytes read and 14 or 24 written per value: 5.2 and 5.5 TB/s of the copy's 6.8): 45-atom slab,
 // 14 e4m3 slices, 5.89 -> 5.17 ms with the packed digit code; 12 bf16 slices 6.85 -> 6.33 ms. Keeping the scaled
 // rows in shared memory between the passes cost more in occupancy than the second read.
 // The first pass has eight loads in flight per lane: 5.10 ms with four, 4.82 with eight, 4.73 to 5.14 with 13 to 20
