@@ -14,7 +14,7 @@
 //                 + g d_a d_b S,
 //   g' = R' / r^l - l R / r^(l+1),  g'' = R'' / r^l - 2 l R' / r^(l+1) + l (l+1) R / r^(l+2),
 // with R' and R'' from the spline in s = ln(r / r0) / Delta (ds/dr = 1 / (r Delta),
-// d^2s/dr^2 = -1 / (r^2 Delta)). The harmonics of l come from those of l - 1 and l - 2, and their
+// d^2s/dr^2 = -1 / (r^2 Delta), all at r0 where r < r0). The harmonics of l come from those of l - 1 and l - 2, and their
 // derivatives are fixed combinations of at most two harmonics of l - 1 (the second ones of the first
 // ones of l - 1), so that an entry takes 3 + 5 + 9 FP64 operations. Every batch's block of scratch holds,
 // per reduced-basis row, 10 rows of Ppad points: phi, d/dx, d/dy, d/dz, xx, xy, xz, yy, yz, zz, in the
@@ -67,7 +67,7 @@ __device__ __forceinline__ double harmonic_d(const DevSystem &s, const double (&
 template <int L, int LMAX, typename OutT, bool LAP>
 struct HessLevel {
     static __device__ __forceinline__ void run(const DevSystem &s, const AtomGroup &ag, int &ri, const double (&xa)[3],
-                                               double r2, double r, double ur, double ul, int k, double t, double ds1,
+                                               double r2, double r, double ur, double ur0, double ul, int k, double t, double ds1,
                                                double A, double B,
                                                const double (&S1)[2 * LMAX + 1], const double (&S2)[2 * LMAX + 1],
                                                const double (&G1)[3][2 * LMAX + 1], OutT *E, int64_t rs, int64_t cs, int q) {
@@ -112,7 +112,7 @@ struct HessLevel {
                 const double R = fma(fma(a, t, c01.y), t, c01.x);
                 const double Rs = fma(fma(c23.y, t, a + a), t, c01.y);
                 const double Rss = fma(6.0 * c23.y, t, 2.0 * c23.x);
-                const double R1 = Rs * ds1, R2 = ds1 * fma(Rss, ds1, -(Rs * ur));  // d^2s/dr^2 = -ds/dr / r
+                const double R1 = Rs * ds1, R2 = ds1 * fma(Rss, ds1, -(Rs * ur0));  // d^2s/dr^2 = -ds/dr / max(r, r0)
                 g = R * ul;
                 const double lr = (double)L * ur;
                 const double g1 = fma(-lr, R, R1) * ul;
@@ -152,7 +152,7 @@ struct HessLevel {
         }
         if constexpr (L < LMAX) {
             if (ri < ag.r0 + ag.nr)
-                HessLevel<L + 1, LMAX, OutT, LAP>::run(s, ag, ri, xa, r2, r, ur, ul * ur, k, t, ds1,
+                HessLevel<L + 1, LMAX, OutT, LAP>::run(s, ag, ri, xa, r2, r, ur, ur0, ul * ur, k, t, ds1,
                                                        L == 0 ? xa[0] : fma(xa[0], A, -(xa[1] * B)),
                                                        L == 0 ? xa[1] : fma(xa[0], B, xa[1] * A), S, S1, G, E, rs, cs, q);
         }
@@ -164,14 +164,16 @@ __device__ __forceinline__ void eval_group_hess(const DevSystem &s, const AtomGr
                                                 OutT *E, int64_t rs, int64_t cs, int q) {
     const double xa[3] = {x, y, z};
     const double r2 = fma(x, x, fma(y, y, z * z)), ur = rsqrt(r2), r = r2 * ur;
-    const double rr = fmax(r, s.r0);  // the radial part is taken at r0 for r < r0
+    // for r < r0 R, R' and R'' are those at r0: both factors of d^2s/dr^2 take the clamped 1/r (ur0), while the
+    // powers of 1/r of phi = (R / r^l) S are those of r itself (ur)
+    const double rr = fmax(r, s.r0);
     int k;
     const double t = radial_coordinate(s, rr, k);
     const double ur0 = r < s.r0 ? 1.0 / s.r0 : ur;
     const double zero[2 * LMAX + 1] = {}, zero3[3][2 * LMAX + 1] = {};
     int ri = ag.r0;
-    HessLevel<0, LMAX, OutT, LAP>::run(s, ag, ri, xa, r2, r, ur, 1.0, k, t, s.inv_delta * ur0, 1.0, 0.0, zero, zero, zero3, E, rs, cs,
-                                       q);
+    HessLevel<0, LMAX, OutT, LAP>::run(s, ag, ri, xa, r2, r, ur, ur0, 1.0, k, t, s.inv_delta * ur0, 1.0, 0.0, zero, zero, zero3, E,
+                                       rs, cs, q);
 }
 
 // LMAX: at least the largest l of the handle's functions.
