@@ -144,8 +144,11 @@ __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restric
             if (j < nb)
 #pragma unroll
                 for (int q = 0; q < KQ; q++)
-                    if (k0 + q < n_k)
-                        reinterpret_cast<double2 *>(hk)[((int64_t)(k0 + q) * nb + row) * nb + j] = acc[q];
+                    if (k0 + q < n_k) {  // as two doubles: hk need not lie on a 16-byte boundary
+                        double *out = hk + 2 * (((int64_t)(k0 + q) * nb + row) * nb + j);
+                        out[0] = acc[q].x;
+                        out[1] = acc[q].y;
+                    }
         }
 }
 
