@@ -21,7 +21,7 @@ struct Lattice {
 };
 
 // Shared memory that the row form of the sum may take (227 KB less its static part).
-constexpr size_t kBlochSmem = 226 * 1024;
+constexpr size_t kBlochSmem = 225 * 1024;
 
 // e^{i k.T} of image (c0, c1, c2).
 __device__ __forceinline__ double2 image_phase(const Lattice &L, const int32_t *c, const double *k) {
@@ -32,6 +32,35 @@ __device__ __forceinline__ double2 image_phase(const Lattice &L, const int32_t *
     double sn, cs;
     sincos(ph, &sn, &cs);
     return make_double2(cs, sn);
+}
+
+// (h, l) += a b as an unevaluated sum: the product's and the addition's rounding errors go into l.
+__device__ __forceinline__ void add_product(double2 &s, double a, double b) {
+    const double p = __dmul_rn(a, b), e = fma(a, b, -p), t = __dadd_rn(s.x, p), bb = __dsub_rn(t, s.x);
+    s.y += (__dsub_rn(s.x, __dsub_rn(t, bb)) + __dsub_rn(p, bb)) + e;
+    s.x = t;
+}
+// k.a_c of one lattice vector.
+__device__ __forceinline__ double2 k_dot(const Lattice &L, int c, const double *k) {
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int d = 0; d < 3; d++) add_product(s, k[d], L.a[3 * c + d]);
+    return s;
+}
+// e^{i k.T} of image (c0, c1, c2) with the argument in twice the precision (ka: k.a_c): the row form multiplies the
+// phases of two images, whose arguments may be far larger than their difference, the only one the general form takes
+// (cells 1000 lattice vectors from the origin: h(k) to 4e-13 with the argument in FP64 as well, 5e-16 in both forms).
+__device__ __forceinline__ double2 image_phase2(const double2 *ka, const int32_t *c) {
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int x = 0; x < 3; x++) {
+        add_product(s, (double)c[x], ka[x].x);
+        s.y = fma((double)c[x], ka[x].y, s.y);
+    }
+    const double ph = __dadd_rn(s.x, s.y), lo = __dsub_rn(s.y, __dsub_rn(ph, s.x));
+    double sn, cs;
+    sincos(ph, &sn, &cs);
+    return make_double2(fma(-sn, lo, cs), fma(cs, lo, sn));
 }
 
 // The sum by rows of h(k): one CTA takes `rows` unit-cell functions i and KQ k points (blockIdx.y).
@@ -46,7 +75,8 @@ template <int KQ>
 __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restrict__ huc, int32_t n_rs,
                                                         const int32_t *__restrict__ fn_map,
                                                         const int32_t *__restrict__ fn_image,
-                                                        const int32_t *__restrict__ img_cell, int32_t n_images, Lattice L,
+                                                        const int32_t *__restrict__ img_cell, int32_t n_images,
+                                                        const __grid_constant__ Lattice L,
                                                         const double *__restrict__ kpts, int32_t n_k, int32_t nb, int32_t rows,
                                                         double *__restrict__ hk) {
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -55,6 +85,7 @@ __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restric
     int *cur = off + nb + 1;                                 // [nb] fill position
     int2 *ent = reinterpret_cast<int2 *>(cur + nb + ((2 * nb + 1) & 1));  // [n_rs] (real-space function, image)
     __shared__ int wsum[8];
+    __shared__ double2 ka[KQ][3];  // k.a_c
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k0 = blockIdx.y * KQ;
     auto valid = [&](int r, int &i, int &t) {
@@ -62,12 +93,13 @@ __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restric
         t = fn_image[r];
         return i >= 0 && i < nb && t >= 0 && t < n_images;
     };
-    for (int i = tid; i < nb; i += 256) cur[i] = 0;
-    for (int x = tid; x < n_images * KQ; x += 256) {
-        const int t = x / KQ, k = k0 + x % KQ;
-        ph[x] = k < n_k ? image_phase(L, img_cell + 3 * (int64_t)t, kpts + 3 * (int64_t)k) : make_double2(0.0, 0.0);
+    if (tid < 3 * KQ) {
+        const int q = tid / 3, c = tid % 3;
+        ka[q][c] = k0 + q < n_k ? k_dot(L, c, kpts + 3 * (int64_t)(k0 + q)) : make_double2(0.0, 0.0);
     }
+    for (int i = tid; i < nb; i += 256) cur[i] = 0;
     __syncthreads();
+    for (int x = tid; x < n_images * KQ; x += 256) ph[x] = image_phase2(ka[x % KQ], img_cell + 3 * (int64_t)(x / KQ));
     int i, t;
     for (int r = tid; r < n_rs; r += 256)
         if (valid(r, i, t)) atomicAdd(cur + i, 1);

@@ -1,4 +1,4 @@
-"""The Bloch sum against complex sums in numpy: an output array on any 8-byte boundary."""
+"""The Bloch sum against complex sums in numpy: an output array on any 8-byte boundary, images far from the origin."""
 import numpy as np
 import pytest
 
@@ -49,3 +49,14 @@ def test_output_on_an_odd_double(n_rs, nb, n_images, n_k):
     assert got[0] == 7.0 and got[-1] == 7.0  # and nothing beside the array is written
     got = got[1:-1].reshape(n_k, nb, nb, 2)
     assert np.max(np.abs(got[..., 0] + 1j * got[..., 1] - ref)) <= 1e-13 * A.max()
+
+
+@pytest.mark.parametrize("far", [0, 1000, -30000])
+def test_images_far_from_the_origin(far):
+    """h(k) depends on the images' differences alone: cells that all lie `far` lattice vectors away leave it as it is,
+    to the rounding of a few hundred terms."""
+    n_rs, nb, n_images, n_k = 120, 9, 6, 5
+    h, fm, fi, cell, lat, k = inputs(n_rs, nb, n_images, n_k)
+    ref, A = reference(h, fm, fi, cell, lat, k, nb)
+    hk = nao.nao_bloch_sum(cuda(h), cuda(fm), cuda(fi), cuda(cell + np.int32(far)), lat, cuda(k), nb).cpu().numpy()
+    assert np.max(np.abs(hk - ref) / A) <= 1e-14
