@@ -21,7 +21,8 @@ struct Lattice {
 };
 
 // Shared memory that the row form of the sum may take (227 KB less its static part).
-constexpr size_t kBlochSmem = 225 * 1024;
+constexpr size_t kBlochSmem = 222 * 1024;
+constexpr int kBlochThreads = 256;
 
 // e^{i k.T} of image (c0, c1, c2).
 __device__ __forceinline__ double2 image_phase(const Lattice &L, const int32_t *c, const double *k) {
@@ -64,28 +65,37 @@ __device__ __forceinline__ double2 image_phase2(const double2 *ka, const int32_t
 }
 
 // The sum by rows of h(k): one CTA takes `rows` unit-cell functions i and KQ k points (blockIdx.y).
-// It lists the real-space functions of every unit-cell function (a counting sort of fn_map in shared
+// It lists the real-space functions of every unit-cell function (a stable counting sort of fn_map in shared
 // memory) and the phases of every image, once. Then for each real-space function i' of i
 //     G_j = sum_{j' -> j} h^uc_{i'j'} e^{i k.T_j'}      (thread j; two FMAs per element and k point)
 // is multiplied by e^{-i k.T_i'} and added to h_ij(k) in registers: no atomics, every h(k) element is
-// written once. Bound by the FP64 pipe (two lanes per clock and SM); elements that are zero for the
-// whole warp are left out. Periodic silicon, N_rs = 2350, 64 k points: 0.78 ms, against 6.2 ms with one
-// sincos and two atomics per element and k point (bloch_kernel).
-template <int KQ>
-__global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restrict__ huc, int32_t n_rs,
-                                                        const int32_t *__restrict__ fn_map,
-                                                        const int32_t *__restrict__ fn_image,
-                                                        const int32_t *__restrict__ img_cell, int32_t n_images,
-                                                        const __grid_constant__ Lattice L,
-                                                        const double *__restrict__ kpts, int32_t n_k, int32_t nb, int32_t rows,
-                                                        double *__restrict__ hk) {
+// written once, and its terms are added in the same order on every call. Bound by the FP64 pipe (two lanes per clock
+// and SM); elements that are zero for the whole warp are left out. Periodic silicon, N_rs = 2350, 64 k points:
+// 0.8 ms, against 6.2 ms with one sincos and two atomics per element and k point (bloch_kernel).
+// With at most 128 unit-cell functions a thread takes every parts-th i' only, parts = 256 / nb, and the parts' sums
+// are added in order: a small cell has long lists (N_rs / nb entries each) and few functions. One thread per j, as
+// with more functions, walked all (N_rs / nb)^2 elements by itself:
+//     nb = 4, N_rs = 1600, 1 / 8 k points     44.3 / 113 -> 1.01 / 3.16 ms (bloch_kernel 2.70 / 19.9)
+//     nb = 13, N_rs = 1300, 1 / 8 k points    3.00 / 7.38 -> 0.33 / 0.81 ms (0.48 / 2.63)
+//     nb = 25, N_rs = 2500, 1 / 8 k points    3.07 / 7.40 -> 0.47 / 1.31 ms (0.63 / 4.07)
+//     nb = 50, N_rs = 2500, 1 / 8 k points    0.90 / 1.99 -> 0.33 / 0.76 ms (0.63 / 4.06)
+// (whole calls through the Python binding, about 0.15 ms of them on the host).
+template <int KQ, bool PARTS>
+__global__ void __launch_bounds__(kBlochThreads) bloch_rows_kernel(const double *__restrict__ huc, int32_t n_rs,
+                                                                  const int32_t *__restrict__ fn_map,
+                                                                  const int32_t *__restrict__ fn_image,
+                                                                  const int32_t *__restrict__ img_cell, int32_t n_images,
+                                                                  const __grid_constant__ Lattice L,
+                                                                  const double *__restrict__ kpts, int32_t n_k, int32_t nb,
+                                                                  int32_t rows, double *__restrict__ hk) {
     extern __shared__ __align__(16) unsigned char dyn[];
     double2 *ph = reinterpret_cast<double2 *>(dyn);          // [n_images][KQ]
     int *off = reinterpret_cast<int *>(ph + (size_t)n_images * KQ);  // [nb + 1] first entry of each function
     int *cur = off + nb + 1;                                 // [nb] fill position
     int2 *ent = reinterpret_cast<int2 *>(cur + nb + ((2 * nb + 1) & 1));  // [n_rs] (real-space function, image)
-    __shared__ int wsum[8];
-    __shared__ double2 ka[KQ][3];  // k.a_c
+    __shared__ int wsum[kBlochThreads / 32];
+    __shared__ double2 ka[KQ][3];             // k.a_c
+    __shared__ double2 red[PARTS ? kBlochThreads : 1];  // the parts' sums
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k0 = blockIdx.y * KQ;
     auto valid = [&](int r, int &i, int &t) {
@@ -97,15 +107,16 @@ __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restric
         const int q = tid / 3, c = tid % 3;
         ka[q][c] = k0 + q < n_k ? k_dot(L, c, kpts + 3 * (int64_t)(k0 + q)) : make_double2(0.0, 0.0);
     }
-    for (int i = tid; i < nb; i += 256) cur[i] = 0;
+    for (int i = tid; i < nb; i += kBlochThreads) cur[i] = 0;
     __syncthreads();
-    for (int x = tid; x < n_images * KQ; x += 256) ph[x] = image_phase2(ka[x % KQ], img_cell + 3 * (int64_t)(x / KQ));
+    for (int x = tid; x < n_images * KQ; x += kBlochThreads)
+        ph[x] = image_phase2(ka[x % KQ], img_cell + 3 * (int64_t)(x / KQ));
     int i, t;
-    for (int r = tid; r < n_rs; r += 256)
+    for (int r = tid; r < n_rs; r += kBlochThreads)
         if (valid(r, i, t)) atomicAdd(cur + i, 1);
     __syncthreads();
     // exclusive prefix sum of the counts: thread t owns `per` consecutive functions
-    const int per = (nb + 255) / 256, lo = min(nb, tid * per), hi = min(nb, lo + per);
+    const int per = (nb + kBlochThreads - 1) / kBlochThreads, lo = min(nb, tid * per), hi = min(nb, lo + per);
     int cnt = 0;
     for (int x = lo; x < hi; x++) cnt += cur[x];
     int incl = cnt;
@@ -123,29 +134,52 @@ __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restric
         off[x] = cur[x] = at;
         at += c;
     }
-    if (tid == 255) off[nb] = at;
+    if (tid == kBlochThreads - 1) off[nb] = at;
     __syncthreads();
-    for (int r = tid; r < n_rs; r += 256)
-        if (valid(r, i, t)) ent[atomicAdd(cur + i, 1)] = make_int2(r, t);
-    __syncthreads();
-    for (int x = tid; x < nb; x += 256)  // a fixed order whatever the atomics' (the lists are short)
-        for (int p = off[x] + 1; p < off[x + 1]; p++) {
-            const int2 e = ent[p];
-            int q = p;
-            for (; q > off[x] && ent[q - 1].x > e.x; q--) ent[q] = ent[q - 1];
-            ent[q] = e;
+    // the entries of every function by increasing r
+    if constexpr (!PARTS) {
+        for (int r = tid; r < n_rs; r += kBlochThreads)
+            if (valid(r, i, t)) ent[atomicAdd(cur + i, 1)] = make_int2(r, t);
+        __syncthreads();
+        for (int x = tid; x < nb; x += kBlochThreads)  // a fixed order whatever the atomics' (with so many functions the lists are short)
+            for (int p = off[x] + 1; p < off[x + 1]; p++) {
+                const int2 e = ent[p];
+                int q = p;
+                for (; q > off[x] && ent[q - 1].x > e.x; q--) ent[q] = ent[q - 1];
+                ent[q] = e;
+            }
+        __syncthreads();
+    } else {
+        // 256 at a time, the warps one after the other, a warp's lanes by rank: lists may hold thousands
+        for (int r0 = 0; r0 < n_rs; r0 += kBlochThreads) {
+            const int r = r0 + tid;
+            if (r >= n_rs || !valid(r, i, t)) i = -1;
+            const unsigned same = __match_any_sync(0xffffffffu, i);
+            const int rank = __popc(same & ((1u << lane) - 1u));
+#pragma unroll 1
+            for (int w = 0; w < kBlochThreads / 32 && r0 + 32 * w < n_rs; w++) {
+                if (w == warp && i >= 0) {
+                    const int p = cur[i];
+                    ent[p + rank] = make_int2(r, t);
+                    __syncwarp(same);
+                    if (rank == 0) cur[i] = p + __popc(same);
+                }
+                __syncthreads();
+            }
         }
-    __syncthreads();
+    }
 
+    const int parts = PARTS ? kBlochThreads / nb : 1;
+    const int part = PARTS ? tid / nb : 0, jt = PARTS ? tid - part * nb : tid;
     const int r1 = min(nb, (int)(blockIdx.x + 1) * rows);
     for (int row = blockIdx.x * rows; row < r1; row++)
-        for (int j0 = 0; j0 < nb; j0 += 256) {
-            const int j = j0 + tid;
+        for (int j0 = 0; j0 < nb; j0 += kBlochThreads) {  // once where PARTS
+            const int j = j0 + jt;
             const int s0 = j < nb ? off[j] : 0, s1 = j < nb ? off[j + 1] : 0;
             double2 acc[KQ];
 #pragma unroll
             for (int q = 0; q < KQ; q++) acc[q] = make_double2(0.0, 0.0);
-            for (int a = off[row]; a < off[row + 1]; a++) {
+            for (int a = part < parts ? off[row] + part : off[row + 1]; a < off[row + 1]; a += parts) {
                 const double *h = huc + (int64_t)ent[a].x * n_rs;
                 double2 G[KQ];
 #pragma unroll
@@ -173,14 +207,25 @@ __global__ void __launch_bounds__(256) bloch_rows_kernel(const double *__restric
                     acc[q].y = fma(w.x, G[q].y, fma(-w.y, G[q].x, acc[q].y));
                 }
             }
-            if (j < nb)
 #pragma unroll
-                for (int q = 0; q < KQ; q++)
-                    if (k0 + q < n_k) {  // as two doubles: hk need not lie on a 16-byte boundary
-                        double *out = hk + 2 * (((int64_t)(k0 + q) * nb + row) * nb + j);
-                        out[0] = acc[q].x;
-                        out[1] = acc[q].y;
-                    }
+            for (int q = 0; q < KQ; q++) {
+                if (PARTS) {
+                    __syncthreads();
+                    red[tid] = acc[q];
+                    __syncthreads();
+                    if (part == 0)
+                        for (int x = 1; x < parts; x++) {
+                            const double2 y = red[x * nb + jt];
+                            acc[q].x += y.x;
+                            acc[q].y += y.y;
+                        }
+                }
+                if (part == 0 && j < nb && k0 + q < n_k) {  // as two doubles: hk need not lie on a 16-byte boundary
+                    double *out = hk + 2 * (((int64_t)(k0 + q) * nb + row) * nb + j);
+                    out[0] = acc[q].x;
+                    out[1] = acc[q].y;
+                }
+            }
         }
 }
 
@@ -229,21 +274,21 @@ size_t bloch_rows_smem(int64_t n_rs, int64_t n_images, int64_t nb, int KQ) {
     return (size_t)n_images * KQ * 16 + 4 * (size_t)(2 * nb + 2) + 8 * (size_t)n_rs;
 }
 
-template <int KQ>
+template <int KQ, bool PARTS>
 cudaError_t launch_bloch_rows(const double *huc, int32_t n_rs, const int32_t *fn_map, const int32_t *fn_image,
                               const int32_t *img_cell, int32_t n_images, const Lattice &L, const double *k, int32_t n_k,
                               int32_t nb, double *hk, cudaStream_t st) {
     const size_t smem = bloch_rows_smem(n_rs, n_images, nb, KQ);
     if (smem > 40 * 1024) {
         const cudaError_t e =
-            cudaFuncSetAttribute(bloch_rows_kernel<KQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlochSmem);
+            cudaFuncSetAttribute(bloch_rows_kernel<KQ, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlochSmem);
         if (e != cudaSuccess) return e;
     }
     // about four CTAs for each of the 152 SMs: more would repeat the lists and phases, fewer leave a
     // tail
     const int nq = (n_k + KQ - 1) / KQ, want = (608 + nq - 1) / nq, rows = (nb + want - 1) / want;
-    bloch_rows_kernel<KQ><<<dim3((nb + rows - 1) / rows, nq), 256, smem, st>>>(huc, n_rs, fn_map, fn_image, img_cell, n_images,
-                                                                               L, k, n_k, nb, rows, hk);
+    bloch_rows_kernel<KQ, PARTS><<<dim3((nb + rows - 1) / rows, nq), kBlochThreads, smem, st>>>(
+        huc, n_rs, fn_map, fn_image, img_cell, n_images, L, k, n_k, nb, rows, hk);
     return cudaGetLastError();
 }
 
@@ -384,9 +429,10 @@ nao_status nao_bloch_sum(const double *h_uc_dev, int64_t n_rs, const int32_t *fn
     const int KQ = n_k >= 8 ? 8 : (n_k >= 4 ? 4 : (n_k >= 2 ? 2 : 1));
     if (e != cudaSuccess) {
     } else if (nb < (1 << 20) && bloch_rows_smem(n_rs, n_images, nb, KQ) <= kBlochSmem) {
-#define NAO_BLOCH(K)                                                                                               \
-    launch_bloch_rows<K>(h_uc_dev, (int32_t)n_rs, fn_map_dev, fn_image_dev, img_cell_dev, n_images, L, k_dev, n_k, \
-                         (int32_t)nb, hk_dev, st)
+#define NAO_BLOCH(K)                                                                             \
+    (nb <= kBlochThreads / 2 ? launch_bloch_rows<K, true> : launch_bloch_rows<K, false>)(        \
+        h_uc_dev, (int32_t)n_rs, fn_map_dev, fn_image_dev, img_cell_dev, n_images, L, k_dev, n_k, \
+        (int32_t)nb, hk_dev, st)
         e = KQ == 8 ? NAO_BLOCH(8) : KQ == 4 ? NAO_BLOCH(4) : KQ == 2 ? NAO_BLOCH(2) : NAO_BLOCH(1);
 #undef NAO_BLOCH
     } else {

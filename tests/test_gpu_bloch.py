@@ -1,4 +1,5 @@
-"""The Bloch sum against complex sums in numpy: an output array on any 8-byte boundary, images far from the origin."""
+"""The Bloch sum against complex sums in numpy: an output array on any 8-byte boundary, images far from the origin,
+cells of few functions with long lists of images."""
 import numpy as np
 import pytest
 
@@ -60,3 +61,16 @@ def test_images_far_from_the_origin(far):
     ref, A = reference(h, fm, fi, cell, lat, k, nb)
     hk = nao.nao_bloch_sum(cuda(h), cuda(fm), cuda(fi), cuda(cell + np.int32(far)), lat, cuda(k), nb).cpu().numpy()
     assert np.max(np.abs(hk - ref) / A) <= 1e-14
+
+
+# on both sides of 128 functions, up to which several threads share a column; lists of up to 500 images
+@pytest.mark.parametrize("n_rs,nb,n_images,n_k", [(500, 1, 40, 3), (1600, 4, 400, 8), (1300, 13, 100, 1), (700, 100, 9, 4),
+                                                 (640, 128, 5, 9), (645, 129, 5, 2)])
+def test_small_cells(n_rs, nb, n_images, n_k):
+    """The sums of a few hundred thousand terms at most, each rounded a few times, and the same twice."""
+    h, fm, fi, cell, lat, k = inputs(n_rs, nb, n_images, n_k)
+    ref, A = reference(h, fm, fi, cell, lat, k, nb)
+    d = [cuda(x) for x in (h, fm, fi, cell)]
+    hk, again = (nao.nao_bloch_sum(*d, lat, cuda(k), nb).cpu().numpy() for _ in range(2))
+    assert np.max(np.abs(hk - ref) / A) <= 1e-13
+    assert np.array_equal(hk, again)
