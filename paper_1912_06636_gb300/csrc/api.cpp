@@ -255,12 +255,6 @@ struct CallEnd {
     }
 };
 
-double factorial(int n) {
-    double f = 1.0;
-    for (int i = 2; i <= n; i++) f *= (double)i;
-    return f;
-}
-
 inline bool finite(double x) { return std::isfinite(x); }
 
 nao_status validate(const nao_system_desc *d, const nao_options &o) {
@@ -679,45 +673,52 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     s.inv_delta = 1.0 / g->delta;
     s.step_m1 = std::expm1(g->delta);
     s.nb = g->nb;
-    // K_lm = sqrt((2l+1)/(4pi) (l-m)!/(l+m)!), times sqrt 2 for m > 0
-    double knorm[NAO_LMAX + 1][NAO_LMAX + 1] = {};
-    for (int l = 0; l <= NAO_LMAX; l++)
-        for (int m = 0; m <= NAO_LMAX; m++) {
-            double k = 0.0;
-            if (m <= l) {
-                k = std::sqrt((2.0 * l + 1.0) / (4.0 * M_PI) * factorial(l - m) / factorial(l + m));
-                if (m > 0) k *= std::sqrt(2.0);
-            }
-            knorm[l][m] = k;
-        }
-    s.s00 = knorm[0][0];
-    s.s00_h = (float)s.s00;
-    s.s00_l = (float)(s.s00 - (double)s.s00_h);
-    // With W_l^m = r^l P_l^m e^{i m phi} (no Condon-Shortley phase): d/dz W_l^m = (l+m) W_{l-1}^m,
-    // (d/dx + i d/dy) W_l^m = -W_{l-1}^{m+1}, (d/dx - i d/dy) W_l^m = (l+m)(l+m-1) W_{l-1}^{m-1} (m >= 1),
-    // and S_l,m = K_lm Re W_l^m, S_l,-m = K_lm Im W_l^m.
+    // Normalised harmonics S_l,m = K_lm Re W_l^m, S_l,-m = K_lm Im W_l^m with W_l^m = r^l P_l^m e^{i m phi} (no
+    // Condon-Shortley phase) and K_lm = sqrt((2l+1)/(4pi) (l-m)!/(l+m)!), times sqrt 2 for m > 0. From
+    // d/dz W_l^m = (l+m) W_{l-1}^m, (d/dx + i d/dy) W_l^m = -W_{l-1}^{m+1} and
+    // (d/dx - i d/dy) W_l^m = (l+m)(l+m-1) W_{l-1}^{m-1} (m >= 1), the coefficients are square roots of rationals:
+    // one division of exact integers and one root each, so within an ulp (as ratios of rounded K_lm they were off by
+    // up to three, a bias that every value of an l then shares).
+    s.s00 = std::sqrt(1.0 / (4.0 * M_PI));
     s.hc = HarmonicCoefs{};
-    double odd = 1.0;  // (2l-1)!!
+    double odd = 1.0, even = 1.0;  // (2l-1)!!, (2l)!!
     for (int l = 1; l <= NAO_LMAX; l++) {
         odd *= 2 * l - 1;
-        s.hc.kl[l] = odd * knorm[l][l];
+        even *= 2 * l;
+        s.hc.kl[l] = std::sqrt((2 * l + 1) * odd / (even * 2.0 * M_PI));  // (2l-1)!! K_ll
         for (int m = 0; m <= l; m++) {
-            const double k = knorm[l][m];
+            auto root = [](int64_t num, int64_t den) { return std::sqrt((double)num / (double)den); };
+            const int64_t a = 2 * l + 1, p = l + m, q = l - m;
             if (m <= l - 1) {
-                s.hc.ra[l][m] = k / knorm[l - 1][m] * (2 * l - 1) / (l - m);
-                s.hc.dz[l][m] = k / knorm[l - 1][m] * (l + m);
+                s.hc.ra[l][m] = root(a * (2 * l - 1), q * p);
+                s.hc.dz[l][m] = root(a * q * p, 2 * l - 1);
             }
             if (m <= l - 2) {
-                s.hc.rb[l][m] = k / knorm[l - 2][m] * (l + m - 1) / (l - m);
-                s.hc.dp[l][m] = (m == 0 ? -1.0 : -0.5) * k / knorm[l - 1][m + 1];
+                s.hc.rb[l][m] = root(a * (p - 1) * (q - 1), (2 * l - 3) * q * p);
+                s.hc.dp[l][m] = -0.5 * root((m == 0 ? 2 : 1) * a * q * (q - 1), 2 * l - 1);
             }
-            if (m >= 1) s.hc.dm[l][m] = 0.5 * (l + m) * (l + m - 1) * k / knorm[l - 1][m - 1];
+            if (m >= 1) s.hc.dm[l][m] = 0.5 * root((m == 1 ? 2 : 1) * a * p * (p - 1), 2 * l - 1);
+        }
+    }
+    // As float-floats the recurrences run on T_lm = S_lm / N_lm, N_lm = K_lm (2l-1)!! / (l-m)!, whose highest power of z
+    // has the coefficient 1: T_lm = z T_{l-1},m - beta r^2 T_{l-2},m, and the derivatives' coefficients take N_{l-1}.
+    double norm[NAO_LMAX + 1][NAO_LMAX + 1] = {};
+    odd = 1.0;
+    for (int l = 0; l <= NAO_LMAX; l++) {
+        odd *= l > 0 ? 2 * l - 1 : 1;
+        for (int m = 0; m <= l; m++) {
+            double f = 4.0 * M_PI;  // 4 pi (l+m)! (l-m)!
+            for (int i = 2; i <= l + m; i++) f *= i;
+            for (int i = 2; i <= l - m; i++) f *= i;
+            norm[l][m] = std::sqrt((m > 0 ? 2.0 : 1.0) * (2 * l + 1) * odd * odd / f);
         }
     }
     for (int l = 0; l <= NAO_LMAX; l++)
-        for (int m = 0; m <= NAO_LMAX; m++) {
-            const double c[6] = {s.hc.ra[l][m], s.hc.rb[l][m], s.hc.dz[l][m], s.hc.dp[l][m], s.hc.dm[l][m], m == 0 ? s.hc.kl[l] : 0.0};
-            for (int i = 0; i < 6; i++) {
+        for (int m = 0; m <= l; m++) {
+            auto at = [&](int k) { return l > 0 && k >= 0 && k <= l - 1 ? norm[l - 1][k] : 0.0; };
+            const double beta = m <= l - 2 ? (double)((l + m - 1) * (l - m - 1)) / (double)((2 * l - 1) * (2 * l - 3)) : 0.0;
+            const double c[5] = {norm[l][m], beta, s.hc.dz[l][m] * at(m), s.hc.dp[l][m] * at(m + 1), s.hc.dm[l][m] * at(m - 1)};
+            for (int i = 0; i < 5; i++) {
                 s.hcf[i][l][m][0] = (float)c[i];
                 s.hcf[i][l][m][1] = (float)(c[i] - (double)s.hcf[i][l][m][0]);
             }

@@ -97,7 +97,8 @@ template <typename H> __device__ __forceinline__ H from_f64(double x);
 template <> __device__ __forceinline__ double from_f64<double>(double x) { return x; }
 template <> __device__ __forceinline__ ffa::F from_f64<ffa::F>(double x) { return ffa::from_double_bits(x); }
 
-// Coefficient c of the harmonics' recurrences (0 ra, 1 rb, 2 dz, 3 dp, 4 dm, 5 kl at m = 0).
+// Coefficient c of the harmonics' recurrences: in FP64 0 ra, 1 rb, 2 dz, 3 dp, 4 dm, 5 kl at m = 0 (DevSystem::hc), as
+// float-floats 0 N, 1 beta, 2 dz, 3 dp, 4 dm (DevSystem::hcf).
 template <typename H, int c>
 __device__ __forceinline__ H coef(const DevSystem &s, int l, int m) {
     if constexpr (std::is_same<H, double>::value)
@@ -106,23 +107,39 @@ __device__ __forceinline__ H coef(const DevSystem &s, int l, int m) {
         return ffa::F{s.hcf[c][l][m][0], s.hcf[c][l][m][1]};
 }
 
-// Entry m = mm - l of the harmonics S_l from those of l - 1 and l - 2 (S1, S2) and, at m = +-l, from
+// Entry m = mm - l of the harmonics of l from those of l - 1 and l - 2 (S1, S2) and, at m = +-l, from
 // A + i B = (x + i y)^l (its rounding at the nodes of cos(l phi) and sin(l phi) is then that of the powers alone).
+// FP64: the normalised S_lm. Float-float: T_lm = S_lm / N_lm, whose highest power of z has the coefficient 1 (T_ll =
+// A or B), multiplied by N_lm where S_lm is used: with the normalisation in every step the errors of S_3m and S_4m
+// were 15 and 7 % larger (5.6e-15 against 4.8e-15 of the norm for l = 3).
 template <int l, typename H, int W>
 __device__ __forceinline__ H harmonic(const DevSystem &s, const H (&x)[3], H r2, H A, H B, const H (&S1)[W], const H (&S2)[W],
                                       int mm) {
     const int m = mm >= l ? mm - l : l - mm, sg = mm >= l ? 1 : -1;
-    if (m == l) return hmul(coef<H, 5>(s, l, 0), sg > 0 ? A : B);
-    const H az = hmul(coef<H, 0>(s, l, m), x[2]);
-    if (m > l - 2) return hmul(az, S1[l - 1 + sg * m]);
-    return hdot(az, S1[l - 1 + sg * m], hneg(hmul(coef<H, 1>(s, l, m), r2)), S2[l - 2 + sg * m]);
+    if constexpr (std::is_same<H, double>::value) {
+        if (m == l) return hmul(coef<H, 5>(s, l, 0), sg > 0 ? A : B);
+        if constexpr (l == 1) return hmul(coef<H, 5>(s, 1, 0), x[2]);  // S_1m = kl (x, y, z): one rounding, not two
+        const H az = hmul(coef<H, 0>(s, l, m), x[2]);
+        if (m > l - 2) return hmul(az, S1[l - 1 + sg * m]);
+        return hdot(az, S1[l - 1 + sg * m], hneg(hmul(coef<H, 1>(s, l, m), r2)), S2[l - 2 + sg * m]);
+    } else {
+        if (m == l) return sg > 0 ? A : B;
+        if constexpr (l == 1) return x[2];
+        if (m > l - 2) return hmul(x[2], S1[l - 1 + sg * m]);
+        return hdot(x[2], S1[l - 1 + sg * m], hneg(hmul(coef<H, 1>(s, l, m), r2)), S2[l - 2 + sg * m]);
+    }
 }
 
-// d/dx, d/dy or d/dz of that entry: at most two harmonics of l - 1 (zero: none).
+// d/dx, d/dy or d/dz of S_lm: at most two harmonics of l - 1 (zero: none).
 template <int l, typename H, int W>
 __device__ __forceinline__ H harmonic_d(const DevSystem &s, const H (&C)[W], int mm, int axis, bool &zero) {
     const int m = mm >= l ? mm - l : l - mm, sg = mm >= l ? 1 : -1;
     constexpr int o = l - 1;
+    if constexpr (l == 1) {  // a constant, kl = N_1m (the product of dz or dm and S_00 would be off in every value)
+        zero = !(axis == 2 ? m == 0 : m == 1 && (axis == 0) == (sg > 0));
+        if constexpr (std::is_same<H, double>::value) return zero ? H{} : coef<H, 5>(s, 1, 0);
+        else return zero ? H{} : coef<H, 0>(s, 1, 0);
+    }
     zero = false;
     if (axis == 2) {
         zero = m > l - 1;
@@ -231,7 +248,7 @@ __device__ __forceinline__ RfnEntry rfn_entry(const DevSystem &s, int ri) {
 
 // The functions of l = L of one atom at one point, then those of L + 1 .. LMAX. The radial functions of an
 // atom are visited in increasing l and share the harmonics; pa + i pb = (x + i y)^L, S1, S2: the harmonics of L - 1,
-// L - 2. ul: u^L.
+// L - 2 (in FP64 the normalised ones, as float-floats those divided by N_lm). ul: u^L.
 template <int L, int LMAX, typename A, bool GRAD, typename OutT, int EXPO>
 __device__ __forceinline__ void eval_level(const DevSystem &s, const AtomGroup &ag, int ri, const Point<A> &pt,
                                            typename A::R ul, typename A::H pa, typename A::H pb,
@@ -239,16 +256,22 @@ __device__ __forceinline__ void eval_level(const DevSystem &s, const AtomGroup &
                                            const typename A::H (&S2)[2 * LMAX + 1], const EvalOut<OutT> &o, int q, int &pt_eb) {
     using H = typename A::H;
     using R = typename A::R;
-    H S[2 * LMAX + 1], G[3][2 * LMAX + 1];
+    H T[2 * LMAX + 1], S[2 * LMAX + 1], G[3][2 * LMAX + 1];
     bool zero[3][2 * LMAX + 1];
     if constexpr (L == 0) {
-        if constexpr (std::is_same<H, double>::value) S[0] = s.s00;
-        else S[0] = H{s.s00_h, s.s00_l};
+        if constexpr (std::is_same<H, double>::value) {
+            T[0] = S[0] = s.s00;
+        } else {
+            T[0] = H{1.0f, 0.0f};
+            S[0] = coef<H, 0>(s, 0, 0);
+        }
         zero[0][0] = zero[1][0] = zero[2][0] = true;
     } else {
 #pragma unroll
         for (int mm = 0; mm < 2 * L + 1; mm++) {
-            S[mm] = harmonic<L>(s, pt.x, pt.r2, pa, pb, S1, S2, mm);
+            T[mm] = harmonic<L>(s, pt.x, pt.r2, pa, pb, S1, S2, mm);
+            if constexpr (std::is_same<H, double>::value) S[mm] = T[mm];
+            else S[mm] = hmul(coef<H, 0>(s, L, mm >= L ? mm - L : L - mm), T[mm]);
             if (GRAD)
 #pragma unroll
                 for (int a = 0; a < 3; a++) G[a][mm] = harmonic_d<L>(s, S1, mm, a, zero[a][mm]);
@@ -311,7 +334,7 @@ __device__ __forceinline__ void eval_level(const DevSystem &s, const AtomGroup &
             else un = ul * pt.u;
             const H na = L == 0 ? pt.x[0] : hdot(pt.x[0], pa, hneg(pt.x[1]), pb);
             const H nb = L == 0 ? pt.x[1] : hdot(pt.x[0], pb, pt.x[1], pa);
-            eval_level<L + 1, LMAX, A, GRAD, OutT, EXPO>(s, ag, ri, pt, un, na, nb, S, S1, o, q, pt_eb);
+            eval_level<L + 1, LMAX, A, GRAD, OutT, EXPO>(s, ag, ri, pt, un, na, nb, T, S1, o, q, pt_eb);
         }
     }
 }

@@ -86,14 +86,15 @@ struct HessLevel {
                 const double bq = m <= L - 2 ? s.hc.rb[L][m] * r2 : 0.0;
 #pragma unroll
                 for (int sg = 1; sg >= (m == 0 ? 1 : -1); sg -= 2) {
-                    const double v = az * S1[L - 1 + sg * m];
+                    const double v = L == 1 ? s.hc.kl[1] * xa[2] : az * S1[L - 1 + sg * m];  // S_1m = kl (x, y, z)
                     S[L + sg * m] = m <= L - 2 ? fma(-bq, S2[L - 2 + sg * m], v) : v;
                 }
             }
 #pragma unroll
             for (int mm = 0; mm < 2 * L + 1; mm++) {
 #pragma unroll
-                for (int a = 0; a < 3; a++) G[a][mm] = harmonic_d<L, LMAX>(s, S1, mm, a);
+                for (int a = 0; a < 3; a++)
+                    G[a][mm] = L > 1 ? harmonic_d<L, LMAX>(s, S1, mm, a) : mm == (a == 0 ? 2 : a == 1 ? 0 : 1) ? s.hc.kl[1] : 0.0;
                 if (!LAP) {
 #pragma unroll
                     for (int kk = 0; kk < 6; kk++) H[kk][mm] = harmonic_d<L, LMAX>(s, G1[pair_a(kk)], mm, pair_b(kk));

@@ -87,13 +87,13 @@ struct DevSystem {
     int64_t nb;               // total basis size over all systems
     SysTables sys;
     double s00;               // S_00 = 1 / sqrt(4 pi)
-    float s00_h, s00_l;       // and as a float-float
-    // The normalised solid harmonics by l (from l - 1 and l - 2) and their derivatives from l - 1
-    // (nao_harmonic_coefficients): S_l,+-m = ra z S_{l-1},+-m - rb r^2 S_{l-2},+-m (m < l), and with
-    // C = S_{l-1}, d/dz S_l,+-m = dz C_{+-m}, d/dx S_l,+-m = dp C_{+-(m+1)} + dm C_{+-(m-1)} and
-    // d/dy S_l,+-m = +-(dp C_{-+(m+1)} - dm C_{-+(m-1)}).
+    // The normalised solid harmonics by l (from l - 1 and l - 2) and their derivatives from l - 1 (filled at create):
+    // S_l,+-m = ra z S_{l-1},+-m - rb r^2 S_{l-2},+-m (m < l), and with C = S_{l-1}, d/dz S_l,+-m = dz C_{+-m},
+    // d/dx S_l,+-m = dp C_{+-(m+1)} + dm C_{+-(m-1)} and d/dy S_l,+-m = +-(dp C_{-+(m+1)} - dm C_{-+(m-1)}).
     HarmonicCoefs hc;
-    float hcf[6][NAO_LMAX + 1][NAO_LMAX + 1][2];  // ra, rb, dz, dp, dm and kl (at m = 0) as float-floats
+    // The same as float-floats for T_lm = S_lm / N_lm: N, beta (T_l = z T_{l-1} - beta r^2 T_{l-2}) and the derivatives'
+    // coefficients dz, dp, dm with C = T_{l-1}
+    float hcf[5][NAO_LMAX + 1][NAO_LMAX + 1][2];
 };
 
 #ifdef __CUDACC__

@@ -71,7 +71,7 @@ __device__ __forceinline__ double2 image_phase2(const double2 *ka, const int32_t
 // is multiplied by e^{-i k.T_i'} and added to h_ij(k) in registers: no atomics, every h(k) element is
 // written once, and its terms are added in the same order on every call. Bound by the FP64 pipe (two lanes per clock
 // and SM); elements that are zero for the whole warp are left out. Periodic silicon, N_rs = 2350, 64 k points:
-// 0.8 ms, against 6.2 ms with one sincos and two atomics per element and k point (bloch_kernel).
+// 0.79 ms, against 6.2 ms with one sincos and two atomics per element and k point (bloch_kernel).
 // With at most 128 unit-cell functions a thread takes every parts-th i' only, parts = 256 / nb, and the parts' sums
 // are added in order: a small cell has long lists (N_rs / nb entries each) and few functions. One thread per j, as
 // with more functions, walked all (N_rs / nb)^2 elements by itself:
