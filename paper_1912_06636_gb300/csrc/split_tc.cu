@@ -716,18 +716,9 @@ __device__ __forceinline__ ffa::F pair_ff(const int (&p)[n_pairs<F>()][8], int c
 template <int F>
 __host__ __device__ constexpr int n_unit() { return (F == NAO_DIGITS_BF16 ? 50 : 47) - 21; }
 
-// A float-float of an FP64 from its bit pattern (the FP64 pipe's conversions would bound the Hessian's
-// epilogue): the 24 leading bits and the next 23, truncated; zero below 2^-100 (of no weight in a density).
+// A float-float of an FP64, zeros (functions beyond their cutoffs) apart.
 __device__ __forceinline__ ffa::F ff_of_bits(double x) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const uint32_t e = (hi >> 20) & 0x7FFu;
-    if (e < 923u || e > 1100u) return e < 923u ? ffa::F{0.0f, 0.0f} : ffa::from_double(x);
-    const uint32_t sg = hi & 0x80000000u, fe = (e - 896u) << 23;
-    const float h = __uint_as_float(sg | fe | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
-    // the next 23 bits as the fraction of a number in [1, 2) 2^(E-23), E the exponent of x, less that power
-    const uint32_t base = sg | (fe - (23u << 23));
-    const float l = __fsub_rn(__uint_as_float(base | ((lo >> 6) & 0x7FFFFFu)), __uint_as_float(base));
-    return ffa::F{h, l};
+    return ((uint32_t)__double2hiint(x) & 0x7FF00000u) == 0u ? ffa::F{0.0f, 0.0f} : ffa::from_double_bits(x);
 }
 // A value that no other thread reads, past L1: shared memory, the same array, is what the MMAs read their operands
 // from (27 atoms with grad n: 4.43 -> 4.01 ms).

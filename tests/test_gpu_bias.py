@@ -29,3 +29,15 @@ def test_gradient_of_p_functions():
             a, x = (g.evaluate_batch(b, prec, True)[1][0, 2].cpu().numpy() for prec in ("split", "fp64"))
             rel.append(a / x - 1.0)
     assert abs(np.mean(np.concatenate(rel))) <= 2.0 ** -49 + 4 * 2.0 ** -48 / np.sqrt(2000.0)
+
+
+@pytest.mark.parametrize("opts", [dict(split_slices=12), dict(split_digits=1, split_slices=14)])
+def test_density_of_the_hessian(opts):
+    """N_e of the split Hessian's density against the FP64 one, from the same evaluation: the values of phi that it
+    multiplies are rounded to nearest, so that over 2000 points their 2^-48 average out."""
+    s = synth.config_water(n_rad=20, n_theta=6, n_phi=7)
+    P = cuda(synth.density_matrix(s, 4))
+    with nao.Grid(s, device=0, max_batch_points=100, **opts) as g:
+        ne = [float(g.density_hessian(P, prec=prec)[3].item()) for prec in ("split", "fp64")]
+        g.sync()
+    assert abs(ne[0] / ne[1] - 1.0) <= 1e-15
