@@ -1489,19 +1489,13 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
     // SM: a small system's launch is as long as one CTA (3-atom molecule, 66 batches: 41 -> 26 us)
     const int tile = (int64_t)(b1 - b0) * max_rt < 2 * 152 ? 16 : 64;
     const dim3 grid(b1 - b0, max_rt * (64 / tile));
-    static_assert(slice_h_smem(NAO_SPLIT_MAX_PPAD, 0) + 1024 <= kSmemOptin && slice_h_smem(NAO_SPLIT_MAX_PPAD, 1) + 1024 <= kSmemOptin,
-                  "the H slicer's rows exceed shared memory");
-    cudaError_t e = cudaSuccess;
-#define NAO_SLICE_H(SS, FF)                                                                                          \
-    {                                                                                                                \
-        if (sm > 48 * 1024)                                                                                          \
-            e = cudaFuncSetAttribute(slice_h_kernel<SS, FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);  \
-        if (e == cudaSuccess)                                                                                        \
-            slice_h_kernel<SS, FF><<<grid, 32 * kSliceWarps, sm, st>>>(s, b0, tile, ev, terms, slices, sl_off, expo, neg16);                    \
-    }
+    static_assert(slice_h_smem(NAO_SPLIT_MAX_PPAD, 0) <= 47 * 1024 && slice_h_smem(NAO_SPLIT_MAX_PPAD, 1) <= 47 * 1024,
+                  "the H slicer's columns exceed the shared memory of a plain launch");
+#define NAO_SLICE_H(SS, FF) \
+    slice_h_kernel<SS, FF><<<grid, 32 * kSliceWarps, sm, st>>>(s, b0, tile, ev, terms, slices, sl_off, expo, neg16)
     NAO_SPLIT_DISPATCH(S, F, NAO_SLICE_H)
 #undef NAO_SLICE_H
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return cudaGetLastError();
 }
 
 cudaError_t launch_h_tc(const DevSystem &s, const HTask *work, int32_t w0, int32_t n_work, const uint8_t *slices,
