@@ -669,6 +669,7 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     s.n_rgrid = g->n_rgrid;
     s.lmax = fn_l.empty() ? 0 : *std::max_element(fn_l.begin(), fn_l.end());
     s.max_ppad = (g->max_P + NAO_PPAD - 1) / NAO_PPAD * NAO_PPAD;
+    NAO_CUDA(cudaDeviceGetAttribute(&s.n_sm, cudaDevAttrMultiProcessorCount, g->device));
     s.r0 = g->r0;
     s.inv_delta = 1.0 / g->delta;
     s.step_m1 = std::expm1(g->delta);
@@ -991,7 +992,7 @@ nao_status split_tune(nao_grid *g, uint32_t terms, cudaStream_t st) {
                 nao_split_h_items(b, g->Pb[b], g->Nb[b], 48, S, tmp, pairs, g->split_F);
                 base48 += (int64_t)tmp.size();
             }
-            const int64_t reps = base48 > 0 ? (8 * 152 + base48 - 1) / base48 : 0;
+            const int64_t reps = base48 > 0 ? (8 * s.n_sm + base48 - 1) / base48 : 0;
             for (int w = 0; w < 2 && rs == NAO_OK && reps > 0; w++) {
                 const int TN = w == 0 ? 48 : 32;
                 std::vector<HTask> items;

@@ -601,7 +601,7 @@ static cudaError_t launch_h_simt_t(const DevSystem &s, const HWork *work, int32_
     // Segments of points, not of K: a point's four components may cancel in phi_i phi_j d and the gradients'
     // product, and a sum over points of h's terms has no larger partial sums than the magnitudes it is measured
     // against. 8-atom cluster (490 batches): H 6.60 -> 5.33 ms.
-    const int kseg = sizeof(T) == 4 || n_work >= 20 * 152 ? 1 : (n_work >= 10 * 152 ? 2 : 4);
+    const int kseg = sizeof(T) == 4 || n_work >= 20 * s.n_sm ? 1 : (n_work >= 10 * s.n_sm ? 2 : 4);
     h_simt_kernel<T><<<dim3(n_work, kseg), 256, dyn, st>>>(s, work, scratch, terms);
     return cudaGetLastError();
 }

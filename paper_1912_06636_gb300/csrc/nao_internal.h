@@ -81,6 +81,7 @@ struct DevSystem {
     const int64_t *scr_off;   // [n_batches] element offset of the batch's block in scratch
     int32_t n_rgrid;
     int32_t max_ppad;         // largest padded batch (points)
+    int32_t n_sm;             // multiprocessors of the handle's device
     int32_t lmax;             // largest angular momentum of the handle's functions
     double r0, inv_delta;
     double step_m1;           // exp(Delta) - 1: r_{k+1} / r_k - 1 of the logarithmic grid

@@ -279,14 +279,17 @@ cudaError_t launch_bloch_rows(const double *huc, int32_t n_rs, const int32_t *fn
                               const int32_t *img_cell, int32_t n_images, const Lattice &L, const double *k, int32_t n_k,
                               int32_t nb, double *hk, cudaStream_t st) {
     const size_t smem = bloch_rows_smem(n_rs, n_images, nb, KQ);
+    cudaError_t e = cudaSuccess;
     if (smem > 40 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(bloch_rows_kernel<KQ, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlochSmem);
+        e = cudaFuncSetAttribute(bloch_rows_kernel<KQ, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlochSmem);
         if (e != cudaSuccess) return e;
     }
-    // about four CTAs for each of the 152 SMs: more would repeat the lists and phases, fewer leave a
-    // tail
-    const int nq = (n_k + KQ - 1) / KQ, want = (608 + nq - 1) / nq, rows = (nb + want - 1) / want;
+    // about four CTAs per SM: more would repeat the lists and phases, fewer leave a tail
+    int dev = 0, n_sm = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int nq = (n_k + KQ - 1) / KQ, want = (4 * n_sm + nq - 1) / nq, rows = (nb + want - 1) / want;
     bloch_rows_kernel<KQ, PARTS><<<dim3((nb + rows - 1) / rows, nq), kBlochThreads, smem, st>>>(
         huc, n_rs, fn_map, fn_image, img_cell, n_images, L, k, n_k, nb, rows, hk);
     return cudaGetLastError();

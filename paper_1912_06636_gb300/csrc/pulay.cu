@@ -287,7 +287,7 @@ cudaError_t launch_pulay(const DevSystem &s, const HWork *work, int32_t w0, int3
         }
         // few items: their points are cut into up to four segments, whose partial sums simply add (an item
         // keeps an SM's FP64 pipe busy for most of a millisecond; at 900 items two segments took 8.44 ms, four 8.30)
-        const int seg = n_work >= 20 * 152 ? 1 : (n_work >= 10 * 152 ? 2 : 4);
+        const int seg = n_work >= 20 * s.n_sm ? 1 : (n_work >= 10 * s.n_sm ? 2 : 4);
         pulay_fp64_kernel<<<dim3(n_work, 2, seg), 256, dyn, st>>>(s, work, w0, static_cast<const double *>(scratch), hoff, M, S, nb);
     }
     return cudaGetLastError();

@@ -1424,15 +1424,6 @@ cudaError_t launch_wait_timeout_probe(long long max_cycles, int32_t *err, cudaSt
     return cudaGetLastError();
 }
 
-// SMs of the current device (the persistent kernels' grid size).
-static int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        n <= 0)
-        return 1;
-    return n;
-}
-
 cudaError_t split_configure() {
     size_t bytes = 0;
     for (int S = 4; S <= NAO_SPLIT_MAX_SLICES; S++) bytes = std::max(bytes, split_smem_bytes(S, NAO_DIGITS_BF16));
@@ -1487,7 +1478,7 @@ cudaError_t launch_slice_h(const DevSystem &s, int32_t b0, int32_t b1, int32_t m
     const size_t sm = slice_h_smem(s.max_ppad, F);
     // 64 rows per CTA (max_rt such tiles cover the largest batch), 16 where that gives fewer than two CTAs per
     // SM: a small system's launch is as long as one CTA (3-atom molecule, 66 batches: 41 -> 26 us)
-    const int tile = (int64_t)(b1 - b0) * max_rt < 2 * 152 ? 16 : 64;
+    const int tile = (int64_t)(b1 - b0) * max_rt < 2 * s.n_sm ? 16 : 64;
     const dim3 grid(b1 - b0, max_rt * (64 / tile));
     static_assert(slice_h_smem(NAO_SPLIT_MAX_PPAD, 0) <= 47 * 1024 && slice_h_smem(NAO_SPLIT_MAX_PPAD, 1) <= 47 * 1024,
                   "the H slicer's columns exceed the shared memory of a plain launch");
@@ -1502,7 +1493,7 @@ cudaError_t launch_h_tc(const DevSystem &s, const HTask *work, int32_t w0, int32
                         const int64_t *sl_off, const int32_t *expo, const int32_t *neg16, int S, int F, int tn,
                         int scatter, int32_t *err, cudaStream_t st) {
     if (n_work <= 0) return cudaSuccess;
-    const int grid = n_work < sm_count() ? n_work : sm_count();  // persistent: one CTA per SM
+    const int grid = n_work < s.n_sm ? n_work : s.n_sm;  // persistent: one CTA per SM
     const size_t sm = split_smem_bytes(S, F);
     if (F == NAO_DIGITS_E4M3 && tn == 32)
         h_tc_kernel<32, 1><<<grid, tc_threads<32>(), sm, st>>>(s, work, w0, n_work, slices, sl_off, expo, neg16, S, scatter, err);
@@ -1571,7 +1562,7 @@ static cudaError_t launch_n_tc_mode(const DevSystem &s, const HWork *work, int32
     if (n_work <= 0) return cudaSuccess;
     if (F == NAO_DIGITS_E4M3 ? tn != 32 : (tn != 32 && !(tn == 48 && S <= 10))) return cudaErrorInvalidValue;
     const size_t sm = split_smem_bytes(S, F);
-    const int grid = n_work < sm_count() ? n_work : sm_count();  // persistent: one CTA per SM
+    const int grid = n_work < s.n_sm ? n_work : s.n_sm;  // persistent: one CTA per SM
 #define NAO_N_TC(TNV, M, FF)                                                                                  \
     n_tc_kernel<TNV, M, FF><<<grid, tc_threads<TNV>(), sm, st>>>(s, work, w0, n_work, slices, sl_off, expo_q, expo_b, ev, eoff, S, hc, \
                                                    hess, err)
