@@ -109,8 +109,9 @@ typedef struct {
                                  below 2^-52); costs 16 bytes of device memory per H
                                  element of every system, taken at create, and two integer atomics
                                  per contribution. n, grad n, the Hessian and N_e have no atomics
-                                 and are reproducible either way; the Pulay matrices and the Bloch
-                                 sum keep FP64 atomics. */
+                                 and are reproducible either way, and so is the Bloch sum
+                                 but for very large cells (see nao_bloch_sum); the Pulay matrices
+                                 keep FP64 atomics. */
     int32_t device;           /* CUDA device ordinal; -1 = the calling thread's current device */
     int64_t scratch_bytes;    /* device scratch for evaluated basis functions; 0 = library default (8 GiB;
                                  the split path's slices take three times this). Memory is taken only
@@ -333,7 +334,11 @@ nao_status nao_pulay_forces(nao_grid *g, const double *n_dev, const double *q_de
  *     h_ij(k_q) = sum_{r -> i, s -> j} h_uc[r*n_rs + s] e^{i k_q . (T_s - T_r)},  T = img_cell A,
  * for the n_k points k_dev [n_k*3] (cartesian, 1/bohr): Eq. Bloch-basis inserted into
  * Eq. HamPeriodic. h_uc_dev [n_rs*n_rs], fn_map_dev/fn_image_dev [n_rs], img_cell_dev [3*n_images]
- * on the device; lattice on the host; hk_dev overwritten. FP64 atomics (one per element and k).
+ * on the device; lattice on the host; hk_dev overwritten (8-byte aligned, as any double array). The
+ * terms are added in a fixed order, and h(k) is bitwise the same from call to call, where the tables of
+ * n_rs entries, nb functions and n_images phases fit in shared memory: 8 (n_rs + nb) + 16 q n_images
+ * bytes, q = 1, 2, 4 or 8 for 1, 2, 4 or 8 k points or more, up to 222 KB. Larger cells take FP64 atomics
+ * (two per element and k), whose order varies.
  * Every fn_map entry must lie in [0, nb) and every fn_image entry in [0, n_images), as
  * nao_periodic_basis_map writes them; the maps live on the device, so the kernel checks them
  * itself: an h^uc element with an out-of-range entry is skipped (nothing outside hk_dev and
@@ -363,7 +368,7 @@ nao_status nao_update_density_host(nao_grid *g, const double *P_host, nao_precis
  * for the batch's q = 0..P_b-1 points in batch order and j = 0..N_b-1 reduced-basis
  * positions. grad_dev may be NULL; for a batch with N_b = 0 nothing is written and both
  * pointers may be NULL. prec selects the evaluation arithmetic
- * (NAO_FP32 evaluates in FP32 and widens; NAO_FP64 and NAO_SPLIT evaluate in FP64).      */
+ * (NAO_FP32 evaluates in FP32 and widens, NAO_FP64 in FP64, NAO_SPLIT in float-float).    */
 nao_status nao_evaluate_batch(nao_grid *g, int64_t batch, nao_precision prec, double *phi_dev, double *grad_dev,
                               void *cuda_stream);
 

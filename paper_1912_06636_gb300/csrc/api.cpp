@@ -513,7 +513,7 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
     // Segments whose cubic is ill-conditioned (coefficient magnitudes above 4x the smaller end
     // value, or above 4x the smaller end slope: the decaying tails of steep functions, the
     // approach to the cutoff, extrema) lose more than a few FP32 ulps to cancellation; the FP32
-    // path evaluates them from the FP64 coefficients.
+    // path evaluates them in float-float, from the coefficients' both halves.
     std::vector<uint8_t> seg64((size_t)g->n_fn * (nr - 1), 0);
     for (size_t q = 0; q < seg64.size(); q++) {
         const double *c = coef.data() + 4 * q;

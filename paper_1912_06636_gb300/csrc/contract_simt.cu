@@ -10,7 +10,8 @@
 //
 // Density (Eq. Density restricted to nnz(B)): n_q = sum_ij phi_iq P_ij phi_jq, evaluated per
 // 64-point tile as the sum over tile pairs I <= J of c_IJ sum_{i in I, j in J} phi_iq P_ij phi_jq
-// with c_II = 1 and c_IJ = 2 (I < J), which reads only P's upper triangle.
+// with c_II = 1 and c_IJ = 2 (I < J), which reads only P's upper triangle; I and J are groups of 64 functions in FP32
+// and of 8 in FP64.
 //
 // FP32: products accumulate in FP32 over chunks of 32 terms; each chunk sum is folded into an
 // FP32 (hi, lo) pair with Knuth's TwoSum, and hi + lo is widened to FP64 for the scatter.

@@ -5,8 +5,8 @@
 // phi_i(r) = R_f(|d|) Y_lm(d/|d|), d = r - R_A, is computed as g(r) S_lm(d) with the real
 // solid harmonic S_lm = r^l Y_lm (a polynomial in x, y, z) and g = R / r^l, so that
 //   grad phi = g'(r) (d/r) S_lm + g grad S_lm,   g' = (R' - l R / r) / r^l.
-// The normalised harmonics of l come from those of l - 1 and l - 2, and their gradients are fixed
-// combinations of at most two harmonics of l - 1 (DevSystem::hc), so that no division by sin(theta)
+// The harmonics of l come from those of l - 1 and l - 2, and their gradients are fixed combinations
+// of at most two harmonics of l - 1 (DevSystem::hc, as float-floats hcf), so that no division by sin(theta)
 // and no derivative recurrence occurs. R_f is the natural cubic spline in s = ln(r/r0)/Delta, evaluated
 // as a per-segment polynomial in t = s - floor(s) (r < r0 uses r0; R = 0 for r >= rc).
 #include <cmath>

@@ -7,16 +7,16 @@
 //   d_a d_b n_q = 2 sum_j (T_qj d_a d_b phi_qj + T_a,qj d_b phi_qj),
 // and the same pass gives n_q = sum_j T_qj phi_qj and d_a n_q = 2 sum_j T_qj d_a phi_qj.
 //
-// Evaluation: one CTA per batch, one thread per (point, atom) as in the other evaluation
-// kernels; phi = g(r) S_lm with g = R / r^l and S_lm the normalised real solid harmonic:
+// Evaluation: four CTAs per batch, one thread per (point, atom); phi = g(r) S_lm with g = R / r^l and
+// S_lm the normalised real solid harmonic:
 //   d_a phi     = g' (x_a / r) S + g d_a S,
 //   d_a d_b phi = (g'' / r^2 - g' / r^3) x_a x_b S + (g' / r)(delta_ab S + x_b d_a S + x_a d_b S)
 //                 + g d_a d_b S,
 //   g' = R' / r^l - l R / r^(l+1),  g'' = R'' / r^l - 2 l R' / r^(l+1) + l (l+1) R / r^(l+2),
 // with R' and R'' from the spline in s = ln(r / r0) / Delta (ds/dr = 1 / (r Delta),
-// d^2s/dr^2 = -1 / (r^2 Delta), all at r0 where r < r0). The harmonics of l come from those of l - 1 and l - 2, and their
-// derivatives are fixed combinations of at most two harmonics of l - 1 (the second ones of the first
-// ones of l - 1), so that an entry takes 3 + 5 + 9 FP64 operations. Every batch's block of scratch holds,
+// d^2s/dr^2 = -1 / (r^2 Delta), all at r0 where r < r0). The harmonics of l come from those of l - 1 and
+// l - 2, and their derivatives are fixed combinations of at most two harmonics of l - 1 (the second ones
+// of the first ones of l - 1), so that an entry takes 3 + 5 + 9 FP64 operations. Every batch's block of scratch holds,
 // per reduced-basis row, 10 rows of Ppad points: phi, d/dx, d/dy, d/dz, xx, xy, xz, yy, yz, zz, in the
 // path's type T (the values are computed in FP64 on both paths; the FP32 path rounds them once when
 // storing). For the Pulay terms (LAP) the fifth row holds the Laplacian instead: S is harmonic and

@@ -67,7 +67,7 @@ struct DevSystem {
     const float *coef_f32;    // same in FP32 (rounded to nearest)
     const float *coef_lo;     // c - coef_f32 rounded to FP32: (coef_f32, coef_lo) is c as a float-float
     const double *inv_rk;     // [n_rgrid] 1 / r_k of the logarithmic grid
-    const uint8_t *seg64;     // [n_fn][n_rgrid-1] 1: the FP32 path evaluates this spline segment in FP64
+    const uint8_t *seg64;     // [n_fn][n_rgrid-1] 1: the FP32 path evaluates this spline segment in float-float
     const double *fn_rc;      // [n_fn]
     const double *px, *py, *pz, *pw;  // points in batch order
     const int32_t *perm;      // batch order -> original index

@@ -39,9 +39,9 @@ constexpr long long kWaitCycles = 400000000LL;  // ~0.2 s at 2 GHz: bounded mbar
 constexpr size_t kSmemOptin = 232448;           // shared memory a CTA may opt into on this GPU (227 KB)
 
 
-// Digit extraction works on FP64 bit patterns with integer instructions: on this GPU the FP64
-// pipe is ~1/60 of the FP32 rate, and a double-to-int64 conversion per element would make the
-// slicing kernels FP64-bound.
+// Digits are cut in FP32 arithmetic from a value's FP32 parts (a float-float's two, an FP64's three, taken from its bit
+// pattern): on this GPU the FP64 pipe is ~1/60 of the FP32 rate, and a double-to-int64 conversion per element would
+// make the slicing kernels FP64-bound.
 using split_bits::abs_bits;
 
 // S balanced base-2^B digits (B = 6: base 64, |d| <= 32, bf16; B = 5: base 32, |d| <= 16, e4m3;
@@ -509,7 +509,8 @@ __global__ void __launch_bounds__(256) slice_np_kernel(const __grid_constant__ D
 }
 
 // ----------------------------------------------------------------------------------------
-// Slice-product pipeline of the persistent contraction kernels, ten warps. Shared memory: a ring of
+// Slice-product pipeline of the persistent contraction kernels, eighteen warps with TN = 32, fourteen with 48 (sixteen
+// or twelve that read the accumulators, the producer, the MMA issuer). Shared memory: a ring of
 // ring_slots(S) A-tile buffers (128 rows of 128 B, 16 KB, one slice of one K chunk each) and two sets
 // of S B-tile buffers (TN rows, TN x 128 B). Producer (second last warp): for each K chunk, the S B
 // slices into B set kc % 2, then the S A slices one by one into the ring, each copy a bulk (TMA)
