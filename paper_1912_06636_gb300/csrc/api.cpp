@@ -524,7 +524,12 @@ nao_status build(nao_grid *g, const nao_system_desc *descs, int32_t n_sys, const
         seg64[q] = (sv > 4.0 * std::min(y0, y1) || sd > 4.0 * std::min(d0, d1)) ? 1 : 0;
     }
     std::vector<double> inv_rk((size_t)nr);
-    for (int k = 0; k < nr; k++) inv_rk[(size_t)k] = 1.0 / (g->r0 * std::exp((double)k * g->delta));
+    // 1 / r_k = exp(-k Delta) / r0, the product k Delta as an unevaluated sum: rounded to FP64 it moves a knot by up to
+    // 9e-16 of itself, and every point of its segment with it
+    for (int k = 0; k < nr; k++) {
+        const double x = k * g->delta, lo = std::fma((double)k, g->delta, -x), i = std::exp(-x) / g->r0;
+        inv_rk[(size_t)k] = std::fma(-i, lo, i);
+    }
 
     // work lists and chunks of batches that fit the scratch
     std::vector<HWork> hw;
