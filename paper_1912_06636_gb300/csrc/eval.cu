@@ -481,8 +481,8 @@ __device__ __forceinline__ EvalOut<T> batch_out(const DevSystem &s, int b, int P
 // One CTA per (batch, 64-point tile); the batch's block of scratch holds, per reduced-basis row j,
 // [phi | d/dx | d/dy | d/dz] over Ppad points each (GRAD) or phi alone, in A's output type.
 // Bound by latency and instruction fetch (dependent float-float or FP64 chains in long unrolled code; 128
-// registers, four CTAs per SM). 45-atom slab, float-float: phi and grad phi 5.15 -> 2.98 ms, phi alone 1.75 ->
-// 1.16 ms, against one CTA of 256 threads and 255 registers per batch, with the argument block copied to every
+// registers, four CTAs per SM). 45-atom slab, float-float: phi and grad phi 5.15 -> 2.96 ms, phi alone 1.75 ->
+// 1.21 ms, against one CTA of 256 threads and 255 registers per batch, with the argument block copied to every
 // thread's stack and derivative recurrences for the harmonics; a 21-atom molecule (227 batches) 0.59 -> 0.28 ms,
 // as the tiles also spread a small system over the SMs.
 template <int LMAX, bool GRAD, typename A>
