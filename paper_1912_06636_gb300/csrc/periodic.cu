@@ -20,9 +20,10 @@ struct Lattice {
     double a[9];  // rows a1, a2, a3
 };
 
-// Shared memory that the row form of the sum may take (227 KB less its static part).
-constexpr size_t kBlochSmem = 222 * 1024;
 constexpr int kBlochThreads = 256;
+// Dynamic shared memory that the row form of the sum may take: 227 KB less its static part, of which the parts' sums
+// (cells of at most 128 functions) are 4 KB.
+constexpr size_t bloch_smem_limit(bool parts) { return (parts ? 222 : 226) * 1024; }
 
 // e^{i k.T} of image (c0, c1, c2).
 __device__ __forceinline__ double2 image_phase(const Lattice &L, const int32_t *c, const double *k) {
@@ -281,7 +282,8 @@ cudaError_t launch_bloch_rows(const double *huc, int32_t n_rs, const int32_t *fn
     const size_t smem = bloch_rows_smem(n_rs, n_images, nb, KQ);
     cudaError_t e = cudaSuccess;
     if (smem > 40 * 1024) {
-        e = cudaFuncSetAttribute(bloch_rows_kernel<KQ, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlochSmem);
+        e = cudaFuncSetAttribute(bloch_rows_kernel<KQ, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)bloch_smem_limit(PARTS));
         if (e != cudaSuccess) return e;
     }
     // about four CTAs per SM: more would repeat the lists and phases, fewer leave a tail
@@ -431,7 +433,7 @@ nao_status nao_bloch_sum(const double *h_uc_dev, int64_t n_rs, const int32_t *fn
     // the row form where its tables fit, with as many k points per CTA as there are, up to 8
     const int KQ = n_k >= 8 ? 8 : (n_k >= 4 ? 4 : (n_k >= 2 ? 2 : 1));
     if (e != cudaSuccess) {
-    } else if (nb < (1 << 20) && bloch_rows_smem(n_rs, n_images, nb, KQ) <= kBlochSmem) {
+    } else if (nb < (1 << 20) && bloch_rows_smem(n_rs, n_images, nb, KQ) <= bloch_smem_limit(nb <= kBlochThreads / 2)) {
 #define NAO_BLOCH(K)                                                                             \
     (nb <= kBlochThreads / 2 ? launch_bloch_rows<K, true> : launch_bloch_rows<K, false>)(        \
         h_uc_dev, (int32_t)n_rs, fn_map_dev, fn_image_dev, img_cell_dev, n_images, L, k_dev, n_k, \

@@ -74,3 +74,15 @@ def test_small_cells(n_rs, nb, n_images, n_k):
     hk, again = (nao.nao_bloch_sum(*d, lat, cuda(k), nb).cpu().numpy() for _ in range(2))
     assert np.max(np.abs(hk - ref) / A) <= 1e-13
     assert np.array_equal(hk, again)
+
+
+# tables just below and just above the row form's shared memory, with 129 functions and with 128
+@pytest.mark.parametrize("nb,kb", [(129, 226), (128, 222)])
+@pytest.mark.parametrize("over", [0, 1])
+def test_largest_tables(nb, kb, over):
+    n_rs, n_k = 140, 8
+    n_images = (kb * 1024 - 8 * (n_rs + nb + 1)) // 128 + over
+    h, fm, fi, cell, lat, k = inputs(n_rs, nb, n_images, n_k)
+    ref, A = reference(h, fm, fi, cell, lat, k, nb)
+    hk = nao.nao_bloch_sum(cuda(h), cuda(fm), cuda(fi), cuda(cell), lat, cuda(k), nb).cpu().numpy()
+    assert np.max(np.abs(hk - ref)) <= 1e-13 * A.max()
