@@ -338,8 +338,7 @@ nao_status nao_pulay_forces(nao_grid *g, const double *n_dev, const double *q_de
  * terms are added in a fixed order, and h(k) is bitwise the same from call to call, where the tables of
  * n_rs entries, nb functions and n_images phases fit in shared memory: 8 (n_rs + nb) + 16 q n_images
  * bytes, q = 1, 2, 4 or 8 for 1, 2, 4 or 8 k points or more, up to 222 KB (226 KB with more than 128
- * functions). Larger cells take FP64 atomics
- * (two per element and k), whose order varies.
+ * functions). Larger cells take FP64 atomics (two per element and k), whose order varies.
  * Every fn_map entry must lie in [0, nb) and every fn_image entry in [0, n_images), as
  * nao_periodic_basis_map writes them; the maps live on the device, so the kernel checks them
  * itself: an h^uc element with an out-of-range entry is skipped (nothing outside hk_dev and
