@@ -7,7 +7,7 @@
 // then, since grad_at phi_i = -grad phi_i for a function on atom at,
 //     F_at,c = 2 sum_{i on at} sum_j (n_ij M^c_ij - q_ij S^c_ij).
 // The batches' basis functions come from the density Hessian's evaluation (10 rows per function:
-// phi, grad phi and, in place of the six second derivatives, lap = xx + yy + zz summed in FP64).
+// phi, grad phi and, in place of the six second derivatives, the Laplacian).
 // Work items are the 64 x 64 tile pairs (I, J) of a batch (all pairs: the matrices are not symmetric);
 // FP64 atomics add each tile into the global matrices.
 // FP64: bound by the FP64 pipe (two lanes per clock and SM), 6 N^2 P products per batch. One CTA takes half
