@@ -690,32 +690,38 @@ template <int F>
 __device__ __forceinline__ int h_unit(int t) {
     return F == NAO_DIGITS_BF16 ? (t == 0 ? 66 : 50) : (t == 0 ? 85 : (t == 1 ? 67 : 47));
 }
-// A density T element from its joined integers, as a float-float in units of 2^(e_q + e_b - n_unit<F>):
-// v + f / 2^10 with the 64-bit integer v = floor(4 hi + lo' / 2^16) (bf16; lo' = lo + lo2 / 2^18) or
-// floor(4 hi + lo / 2^38) (e4m3), |v| < 2^62.1, and the next ten bits f. v's three 21-bit pieces and f
-// become FP32s exactly. n_unit: 50 and 47 bits below, and 21 more because the float-float counts in 2^21.
+// A density T element from its joined integers, as a float-float in units of 2^(e_q + e_b - kTUnit): v + f / 2^10
+// with the 64-bit integer v = floor(4 hi + lo' / 2^16) (bf16; lo' = lo + lo2 / 2^18) or floor(32 hi + lo / 2^35)
+// (e4m3), T in units of 2^-50, and the next ten bits f. |T| < K / 4 keeps |v| < 2^61.1 (K <= 8191). v's three 21-bit
+// pieces and f become FP32s exactly. kTUnit: 50 bits below, and 21 more because the float-float counts in 2^21. The
+// lowest piece and f keep 2^-4 of a unit: with units of 2^-47, where an e4m3 T is about 2^42, that was 2^-46 of T
+// (root mean square error of n against the root of its squared terms' sum, 20 functions: 4.1e-15, now 2.8e-15).
+constexpr int kTUnit = 50 - 21;
 template <int F>
 __device__ __forceinline__ ffa::F pair_ff(const int (&p)[n_pairs<F>()][8], int c) {
     long long w;
-    int r;  // lo' or lo in units of 2^-10 of v's (their part above)
+    int f;
+    uint32_t up;
     if constexpr (F == NAO_DIGITS_E4M3) {
-        r = p[4][c] * 4 + (p[5][c] >> 8);
-        w = (long long)p[1][c] * (1 << 22) + ((long long)p[2][c] * (1 << 12) + (p[3][c] * 4 + (r >> 10)));
+        const long long r = (long long)p[4][c] * 32 + (p[5][c] >> 5);  // lo in units of 2^-10 of v's
+        w = (long long)p[1][c] * (1 << 25) + ((long long)p[2][c] * (1 << 15) + ((long long)p[3][c] * 32 + (r >> 10)));
+        f = (int)r & 1023;
+        up = (uint32_t)p[0][c] * 8u;
     } else {
-        r = p[4][c] + (p[5][c] >> 6) + (p[6][c] >> 18);
+        const int r = p[4][c] + (p[5][c] >> 6) + (p[6][c] >> 18);  // lo', the same
         w = (long long)p[1][c] * (1 << 20) + ((long long)p[2][c] * (1 << 8) + (p[3][c] * 4 + (r >> 10)));
+        f = r & 1023;
+        up = (uint32_t)p[0][c];
     }
     const uint32_t lo = (uint32_t)w;
-    const int hi = (int)((uint32_t)(w >> 32) + (uint32_t)p[0][c]);  // v = hi 2^32 + lo
+    const int hi = (int)((uint32_t)(w >> 32) + up);  // v = hi 2^32 + lo
     auto small = [](uint32_t x) { return __fsub_rn(__uint_as_float(0x4B000000u | x), 8388608.0f); };  // x < 2^23
     const float f2 = __fsub_rn(__int_as_float(0x4B400000 + (hi >> 10)), 12582912.0f);
     const float f1 = small(__funnelshift_r(lo, (uint32_t)hi, 21) & 0x1FFFFFu), f0 = small(lo & 0x1FFFFFu);
     const ffa::F a = ffa::quick(__fmul_rn(f2, 2097152.0f), f1);
-    const float low = __fmaf_rn(small((uint32_t)r & 1023u), 1.0f / 1024.0f, f0);
+    const float low = __fmaf_rn(small((uint32_t)f), 1.0f / 1024.0f, f0);
     return ffa::quick(a.h, __fmaf_rn(low, 1.0f / 2097152.0f, a.l));
 }
-template <int F>
-__host__ __device__ constexpr int n_unit() { return (F == NAO_DIGITS_BF16 ? 50 : 47) - 21; }
 
 // A float-float of an FP64, zeros (functions beyond their cutoffs) apart.
 __device__ __forceinline__ ffa::F ff_of_bits(double x) {
@@ -1324,7 +1330,7 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
             if (part == 0 && row_ok) {
                 const int eq = expo_q[h.p0 + q], eb = split_bits::exponent_of_binade(expo_b[h.b]);
                 const bool live = eq > -10000 && eb > -10000;
-                const double sc = pow2(eq + eb - n_unit<F>());
+                const double sc = pow2(eq + eb - kTUnit);
                 if (MODE <= 2) *n_at(s, h.m, h.p0 + q) = live ? tot[0] * sc : 0.0;
                 if (MODE == 1 || MODE == 2)
 #pragma unroll
