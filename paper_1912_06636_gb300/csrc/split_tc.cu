@@ -742,14 +742,17 @@ __device__ __forceinline__ double load_once(const double *p) {
 __device__ __forceinline__ ffa::F ff_of_value(const FF2 &v) { return v.f(); }
 __device__ __forceinline__ ffa::F ff_of_value(double v) { return ff_of_bits(v); }
 
-// acc += a b (float-floats): the product to 2^-48, added to the unevaluated sum.
-__device__ __forceinline__ void ff_mac(ffa::F &acc, ffa::F a, ffa::F b) {
+// acc + rest += a b (float-floats): the product to 2^-48, added to the unevaluated sum. rest collects the rounding of
+// acc.l, which without it is most of a density's own error (root mean square against the root of the squared terms'
+// sum, 20 functions, 12 bf16 slices: 5.4e-15, with it 2.8e-15; in FP64 with T rounded to 2^-50 of its scale 4.2e-15).
+// It costs 0.6 % of the density contraction, 4 % of a Hessian (13 atoms 4.39 -> 4.60 ms).
+__device__ __forceinline__ void ff_mac(ffa::F &acc, float &rest, ffa::F a, ffa::F b) {
     const float p = __fmul_rn(a.h, b.h);
     float e = __fmaf_rn(a.h, b.h, -p);
     e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
-    const ffa::F t = ffa::two_sum(acc.h, p);
-    acc.h = t.h;
-    acc.l = __fadd_rn(acc.l, __fadd_rn(t.l, e));
+    const ffa::F t = ffa::two_sum(acc.h, p), u = ffa::two_sum(acc.l, __fadd_rn(t.l, e));
+    acc = ffa::F{t.h, u.h};
+    rest = __fadd_rn(rest, u.l);
 }
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
@@ -1291,8 +1294,12 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
 #pragma unroll
                     for (int c8 = 0; c8 < HC; c8 += 8) {
                         ffa::F sum[NC];
+                        float rest[NC];
 #pragma unroll
-                        for (int d = 0; d < NC; d++) sum[d] = ffa::F{0.0f, 0.0f};
+                        for (int d = 0; d < NC; d++) {
+                            sum[d] = ffa::F{0.0f, 0.0f};
+                            rest[d] = 0.0f;
+                        }
 #pragma unroll
                         for (int c = c8; c < c8 + 8; c += CB) {
                             V fv[CB][NC];
@@ -1304,10 +1311,11 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
                             for (int y = 0; y < CB; y++)
 #pragma unroll
                                 for (int d = 0; d < NC; d++)
-                                    if (c + y < jn) ff_mac(sum[d], tv[c + y], ff_of_value(fv[y][d]));
+                                    if (c + y < jn) ff_mac(sum[d], rest[d], tv[c + y], ff_of_value(fv[y][d]));
                         }
 #pragma unroll
-                        for (int d = 0; d < NC; d++) tot[d] += __dadd_rn(ffa::widen(sum[d].h), ffa::widen(sum[d].l));
+                        for (int d = 0; d < NC; d++)
+                            tot[d] += __dadd_rn(ffa::widen(sum[d].h), __dadd_rn(ffa::widen(sum[d].l), ffa::widen(rest[d])));
                     }
                 }
                 __syncwarp();

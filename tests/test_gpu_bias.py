@@ -75,3 +75,32 @@ def test_radial_coordinate():
             shift.append((phi / (R / np.sqrt(4 * np.arccos(ld(-1)))) - 1) / slope)
     shift = np.concatenate(shift).astype(float)
     assert np.sqrt(np.mean(shift * shift)) <= 3e-16
+
+
+@pytest.mark.parametrize("opts", [dict(split_slices=12), dict(split_digits=1, split_slices=15)])
+def test_density_sums(opts):
+    """n = sum_j T_j phi_j of the split path from its own phi, with T = P phi: T, the product and its addition are
+    rounded to a few 2^-49 of a term, independently, so that the error is at most 2^-48 of the root of the sum of the
+    squared terms in the root mean square (one atom with 20 functions; points outside the sphere evaluated in FP64)."""
+    ld = np.longdouble
+    if np.finfo(ld).nmant < 60:
+        pytest.skip("no extended precision on this host")
+    rng = np.random.Generator(np.random.PCG64(7))
+    sp = synth.Species(ls=[0, 0, 1, 1, 2, 3], alphas=[0.4, 1.5, 0.6, 1.1, 0.8, 0.9], Z=6.0)
+    s = synth.make_system([[0.1, -0.2, 0.3]], [0], [sp], n_rad=1, n_theta=1, n_phi=1)
+    assert s.n_basis == 20
+    d = rng.normal(size=(2000, 3))
+    s.pt_xyz = np.ascontiguousarray(s.atom_xyz[0] + d * (rng.uniform(0.15, 4.0, 2000) / np.linalg.norm(d, axis=1))[:, None])
+    s.pt_w = np.full(2000, 0.01)
+    P = synth.density_matrix(s, 5)
+    err = []
+    with nao.Grid(s, device=0, max_batch_points=200, **opts) as g:
+        n = g.update_density(cuda(P), prec="split")[0].cpu().numpy()
+        g.sync()
+        off, perm, rel_off, rel = g.batches()
+        for b in range(len(off) - 1):
+            phi = g.evaluate_batch(b, "split", False)[0].cpu().numpy().astype(ld)
+            i = rel[rel_off[b]:rel_off[b + 1]]
+            t = (P[np.ix_(i, i)].astype(ld) @ phi) * phi
+            err.append((n[perm[off[b]:off[b + 1]]] - t.sum(axis=0)) / np.sqrt((t * t).sum(axis=0)))
+    assert np.sqrt(np.mean(np.concatenate(err).astype(float) ** 2)) <= 2.0 ** -48
