@@ -742,15 +742,22 @@ __device__ __forceinline__ double load_once(const double *p) {
 __device__ __forceinline__ ffa::F ff_of_value(const FF2 &v) { return v.f(); }
 __device__ __forceinline__ ffa::F ff_of_value(double v) { return ff_of_bits(v); }
 
-// acc + rest += a b (float-floats): the product to 2^-48, added to the unevaluated sum. rest collects the rounding of
-// acc.l, which without it is most of a density's own error (root mean square against the root of the squared terms'
-// sum, 20 functions, 12 bf16 slices: 5.4e-15, with it 2.8e-15; in FP64 with T rounded to 2^-50 of its scale 4.2e-15).
-// It costs 0.6 % of the density contraction, 4 % of a Hessian (13 atoms 4.39 -> 4.60 ms).
-__device__ __forceinline__ void ff_mac(ffa::F &acc, float &rest, ffa::F a, ffa::F b) {
+// p + e = a b (float-floats) to 2^-48
+__device__ __forceinline__ float ff_product(ffa::F a, ffa::F b, float &e) {
     const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
-    const ffa::F t = ffa::two_sum(acc.h, p), u = ffa::two_sum(acc.l, __fadd_rn(t.l, e));
+    e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
+    return p;
+}
+// acc + rest += a0 b0 + a1 b1 (float-floats), unevaluated. rest collects the rounding of acc.l, which without it is most
+// of a density's own error (root mean square against the root of the squared terms' sum, 20 functions, 12 bf16 slices:
+// 5.4e-15, with it 2.8e-15; in FP64 with T rounded to 2^-50 of its scale 4.2e-15). Two products at a time: n and
+// grad n of 125 atoms, 14 e4m3 slices, 41.8 ms without rest, 44.3 one by one, 42.7 in pairs (12 bf16 slices 52.4,
+// 51.3, 50.3).
+__device__ __forceinline__ void ff_mac2(ffa::F &acc, float &rest, ffa::F a0, ffa::F b0, ffa::F a1, ffa::F b1) {
+    float e0, e1;
+    const float p0 = ff_product(a0, b0, e0), p1 = ff_product(a1, b1, e1);
+    const ffa::F s = ffa::two_sum(p0, p1), t = ffa::two_sum(acc.h, s.h);
+    const ffa::F u = ffa::two_sum(acc.l, __fadd_rn(__fadd_rn(t.l, s.l), __fadd_rn(e0, e1)));
     acc = ffa::F{t.h, u.h};
     rest = __fadd_rn(rest, u.l);
 }
@@ -1308,10 +1315,15 @@ __global__ void __launch_bounds__(tc_threads<TN>(), 1)
 #pragma unroll
                                 for (int d = 0; d < NC; d++) fv[y][d] = MODE == 0 ? f0[MODE == 0 ? c + y : 0] : (c + y < jn ? load_once(f + (c + y) * ld + d * h.Ppad) : V(0));
 #pragma unroll
-                            for (int y = 0; y < CB; y++)
+                            for (int y = 0; y < CB; y += 2) {
+                                // (of an odd last column's neighbour the value is zero and T, whatever integers it
+                                // came from, finite)
+                                if (c + y < jn)
 #pragma unroll
-                                for (int d = 0; d < NC; d++)
-                                    if (c + y < jn) ff_mac(sum[d], rest[d], tv[c + y], ff_of_value(fv[y][d]));
+                                    for (int d = 0; d < NC; d++)
+                                        ff_mac2(sum[d], rest[d], tv[c + y], ff_of_value(fv[y][d]), tv[c + y + 1],
+                                                ff_of_value(fv[y + 1][d]));
+                            }
                         }
 #pragma unroll
                         for (int d = 0; d < NC; d++)
